@@ -73,7 +73,8 @@ extern "C" {
 #define CG_OPT_ILP          5  /* 1..4: generators whose probe sequences one thread advances
                                   together, probing one slot per step; 9..12: the same with
                                   ILP = value - 8, probing a whole 32-byte sector per step;
-                                  0: library chooses                                          */
+                                  0: library chooses.  Hash tables only: the rank-bitmap kernels
+                                  have one form, whatever the value                           */
 #define CG_OPT_SWEEP_ORDER  9  /* CG_STRATEGY_SWEEP: order in which a round takes the layer's
                                   nonempty 1024-rank blocks.  0 = auto (rank order when they
                                   fill at least a quarter of S_n and the visited bitmap, n!/8

@@ -262,51 +262,100 @@ __device__ __forceinline__ uint64_t perm_rank(uint64_t key, int n) {
     return (uint64_t)top * 479001600ull + low;
 }
 
-// The rank with n known at run time but the same for a whole warp (one job): the loop compiled
-// for that n, through a switch.
-__device__ __forceinline__ uint64_t perm_rank_uniform(uint64_t key, int n) {
-    switch (n) {
-        case 2: return perm_rank_n<2>(key);
-        case 3: return perm_rank_n<3>(key);
-        case 4: return perm_rank_n<4>(key);
-        case 5: return perm_rank_n<5>(key);
-        case 6: return perm_rank_n<6>(key);
-        case 7: return perm_rank_n<7>(key);
-        case 8: return perm_rank_n<8>(key);
-        case 9: return perm_rank_n<9>(key);
-        case 10: return perm_rank_n<10>(key);
-        case 11: return perm_rank_n<11>(key);
-        case 12: return perm_rank_n<12>(key);
-        case 13: return perm_rank_n<13>(key);
-        case 14: return perm_rank_n<14>(key);
-        default: return perm_rank(key, n);
+// A permutation of N <= 16 elements held as one byte per element (byte_word, byte_slot): what the
+// byte-permute generators (GenSM::sel) act on and what rank_bytes reads an element from in one
+// instruction.
+template <int N>
+struct ByteState {
+    static constexpr int kWords = N <= 8 ? 2 : N <= 12 ? 3 : 4;
+    uint32_t w[kWords];
+};
+
+// The bytes of a packed key; a parent-edge tag in bits 60..63 (N <= 15) is dropped.
+template <int N>
+__device__ __forceinline__ ByteState<N> unpack_bytes(uint64_t key) {
+    const uint32_t lo = (uint32_t)key, hi = (uint32_t)(key >> 32);
+    ByteState<N> s;
+    s.w[0] = lo & 0x0F0F0F0Fu;
+    s.w[1] = (lo >> 4) & 0x0F0F0F0Fu;
+    if constexpr (N > 8 && N <= 12) {
+        const uint32_t x = __byte_perm(hi, 0, 0x1100);
+        s.w[2] = (x & 0x000F000Fu) | ((x >> 4) & 0x0F000F00u);
     }
+    if constexpr (N > 12) {
+        s.w[2] = hi & 0x0F0F0F0Fu;
+        s.w[3] = (hi >> 4) & (N <= 15 ? 0x000F0F0Fu : 0x0F0F0F0Fu);
+    }
+    return s;
 }
 
-// Visited test-and-set of G keys in a rank-indexed bitmap (one bit per element of S_n): one
-// atomicOr per key, whose returned word says whether the bit was already set (a single L2
-// round trip whether the key is new or not).  res[i] = 1 if this call set the bit, 0 if it
-// was set, -1 if the rank fell outside the bitmap (not a permutation of 0..n-1).
-template <int G, int N = 0>
-__device__ __forceinline__ void bitmap_insert_multi(unsigned* bm, uint64_t words, int n,
-                                                    const uint64_t (&key)[G], int (&res)[G],
-                                                    unsigned vmask) {
-    uint64_t w[G];
-    unsigned bit[G], old[G];
-#pragma unroll
-    for (int i = 0; i < G; ++i) {
-        res[i] = 0;
-        const uint64_t r = N > 0 ? perm_rank_n<(N > 0 ? N : 1)>(key[i]) : perm_rank_uniform(key[i], n);
-        w[i] = r >> 5;
-        bit[i] = 1u << (unsigned)(r & 31u);
-        if ((vmask >> i & 1u) && w[i] >= words) res[i] = -1;
+// The packed key of a byte state, as its two halves.
+template <int N>
+__device__ __forceinline__ void pack_bytes(const ByteState<N>& s, uint32_t& lo, uint32_t& hi) {
+    lo = s.w[0] | (s.w[1] << 4);
+    hi = 0;
+    if constexpr (N > 8 && N <= 12) {
+        const uint32_t x = s.w[2] | (s.w[2] >> 4);
+        hi = __byte_perm(x, 0, 0x4420);
     }
+    if constexpr (N > 12) hi = s.w[2] | (s.w[3] << 4);
+}
+
+// t[i] = s[g[i]] with the generator's selectors (16-byte aligned); *head receives sel[0], whose
+// top four bits are the inverse's tag.
+template <int N>
+__device__ __forceinline__ ByteState<N> apply_selectors(const uint32_t* sel, const ByteState<N>& s, uint32_t* head) {
+    ByteState<N> t;
+    if constexpr (N <= 8) {
+        const uint2 a = *reinterpret_cast<const uint2*>(sel);
+        *head = a.x;
+        t.w[0] = __byte_perm(s.w[0], s.w[1], a.x);
+        t.w[1] = __byte_perm(s.w[0], s.w[1], a.y);
+    } else if constexpr (N <= 12) {
+        const uint4 a = *reinterpret_cast<const uint4*>(sel);
+        const uint2 b = *reinterpret_cast<const uint2*>(sel + 4);
+        *head = a.x;
+        t.w[0] = __byte_perm(__byte_perm(s.w[0], s.w[1], a.x), s.w[2], a.y);
+        t.w[1] = __byte_perm(__byte_perm(s.w[0], s.w[1], a.z), s.w[2], a.w);
+        t.w[2] = __byte_perm(__byte_perm(s.w[0], s.w[1], b.x), s.w[2], b.y);
+    } else {
+        const uint4 a = *reinterpret_cast<const uint4*>(sel);
+        const uint4 b = *reinterpret_cast<const uint4*>(sel + 4);
+        const uint4 c = *reinterpret_cast<const uint4*>(sel + 8);
+        *head = a.x;
+        t.w[0] = __byte_perm(__byte_perm(s.w[0], s.w[1], a.x), __byte_perm(s.w[2], s.w[3], a.y), a.z);
+        t.w[1] = __byte_perm(__byte_perm(s.w[0], s.w[1], a.w), __byte_perm(s.w[2], s.w[3], b.x), b.y);
+        t.w[2] = __byte_perm(__byte_perm(s.w[0], s.w[1], b.z), __byte_perm(s.w[2], s.w[3], b.w), c.x);
+        t.w[3] = __byte_perm(__byte_perm(s.w[0], s.w[1], c.y), __byte_perm(s.w[2], s.w[3], c.z), c.w);
+    }
+    return t;
+}
+
+// perm_rank_n of a byte state.  A digit is d_i = v_i - (N-1-i) + #{j > i : s_j > v_i}; with the
+// values to the right as bits 0..15 of `right` and ones above them, the arithmetic shift
+// right >> v_i holds 16 + v_i + #{j > i : s_j > v_i} ones, so one popc gives d_i plus a constant
+// and the constants of all positions come off at the end: six instructions a position.
+template <int N>
+__device__ __forceinline__ uint64_t rank_bytes(const ByteState<N>& s) {
+    int right = (int)0xFFFF0000u;
+    unsigned top = 0, low = 0, ctop = 0, clow = 0;
 #pragma unroll
-    for (int i = 0; i < G; ++i)
-        if ((vmask >> i & 1u) && res[i] == 0) old[i] = atomicOr(bm + w[i], bit[i]);
-#pragma unroll
-    for (int i = 0; i < G; ++i)
-        if ((vmask >> i & 1u) && res[i] == 0) res[i] = (old[i] & bit[i]) ? 0 : 1;
+    for (int i = N - 1; i >= 1; --i) {
+        const unsigned v = __byte_perm(s.w[byte_word(N, i)], 0, 0x4440u | (unsigned)byte_slot(N, i));
+        // (the top position has nothing to its right: its digit is its value)
+        const unsigned p = i == N - 1 ? v : (unsigned)__popc((unsigned)(right >> v));
+        const unsigned c = i == N - 1 ? 0u : 16u + (unsigned)(N - 1 - i);
+        if (i >= 12) {
+            top = top * (unsigned)(i + 1) + p;
+            ctop = ctop * (unsigned)(i + 1) + c;
+        } else {
+            low = low * (unsigned)(i + 1) + p;
+            clow = clow * (unsigned)(i + 1) + c;
+        }
+        right |= 1 << v;
+    }
+    if (N > 12) return (uint64_t)(top - ctop) * 479001600ull + (low - clow);   // 12!
+    return low - clow;
 }
 
 __device__ __forceinline__ unsigned atom_add_acq_rel(unsigned* p, unsigned v) {

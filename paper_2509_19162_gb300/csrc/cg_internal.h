@@ -23,6 +23,14 @@ constexpr int kMaxLayers = 16384;    // device layer-size array per job
 // with its bits reversed), the bits of every element put back in order, and the result shifted
 // so that element e lands on a + b - e: t = (s & ~mask[0]) | (shift(rev(s), rev_shift) & mask[0]).
 // Other generators of more than kMaxTerms offsets are not supported (CG_EINVAL at create).
+//
+// sel: permutations of n <= 16 elements (4 bits each) also as byte-permute selectors, for the
+// kernels that hold a state as one byte per element (ByteState in cg_device.cuh): one prmt per
+// output word for n <= 8, two for n <= 12, three for n <= 16, whatever the generator (the
+// shift-and-mask form costs about ten instructions a term).  The inverse's tag sits in bits
+// 28..31 of sel[0], above the selector bits prmt reads.  All zero for other vectors.
+constexpr int kSelWords = 12;
+
 struct GenSM {
     uint32_t nterms;
     uint32_t inv_tag;   // 1 + index of this generator's inverse in the set (< 15), or 0
@@ -31,7 +39,37 @@ struct GenSM {
     int16_t rev_shift;  // kind 1: right shift (bits) of the reversed key; negative: left shift
     uint8_t rot[kMaxTerms];
     uint64_t mask[kMaxTerms];
+    alignas(16) uint32_t sel[kSelWords];
 };
+static_assert(offsetof(GenSM, sel) % 16 == 0 && sizeof(GenSM) % 16 == 0, "GenSM: sel is read in 16-byte vectors");
+
+// Where a state held as bytes keeps element p of n: word and byte (elements 0..7 alternate between
+// words 0 and 1, which is how a packed key's nibbles fall apart under one mask; elements 8..11 are
+// word 2, or, when n > 12, elements 8..15 alternate between words 2 and 3).
+constexpr int byte_word(int n, int p) { return p < 8 ? (p & 1) : n <= 12 ? 2 : 2 + (p & 1); }
+constexpr int byte_slot(int n, int p) { return p < 8 ? (p >> 1) : n <= 12 ? p - 8 : (p - 8) >> 1; }
+
+// Byte-permute selectors of the gather t[i] = s[g[i]] on n <= 16 elements (GenSM::sel, without
+// the tag).  Positions past n (zero bytes) stay where they are.
+inline void make_selectors(const uint8_t* g, int n, uint32_t* sel) {
+    for (int i = 0; i < kSelWords; ++i) sel[i] = 0;
+    const int words = n <= 8 ? 2 : n <= 12 ? 3 : 4, elems = words * 4;
+    for (int p = 0; p < elems; ++p) {
+        const int q = p < n ? g[p] : p;
+        const uint32_t o = (uint32_t)byte_word(n, p), b = (uint32_t)byte_slot(n, p);
+        const uint32_t sw = (uint32_t)byte_word(n, q), sb = (uint32_t)byte_slot(n, q);
+        if (words == 2) {
+            sel[o] |= (sw * 4 + sb) << (4 * b);
+        } else if (words == 3) {        // from words 0, 1; then from that and word 2
+            sel[2 * o] |= (sw < 2 ? sw * 4 + sb : 0) << (4 * b);
+            sel[2 * o + 1] |= (sw < 2 ? b : 4 + sb) << (4 * b);
+        } else {                        // from words 0, 1; from words 2, 3; then from both
+            sel[3 * o] |= (sw < 2 ? sw * 4 + sb : 0) << (4 * b);
+            sel[3 * o + 1] |= (sw >= 2 ? (sw - 2) * 4 + sb : 0) << (4 * b);
+            sel[3 * o + 2] |= (sw < 2 ? b : 4 + b) << (4 * b);
+        }
+    }
+}
 
 // Keys of more than 64 bits (two words): vectors of n elements of w bits with 64 < n w <= 128 --
 // coset vectors of 4-bit values up to n = 32, 2-bit up to 64, 1-bit up to 128, and permutations
@@ -95,6 +133,11 @@ constexpr uint64_t kKeyBits60 = (1ull << 60) - 1;
 constexpr int kVisitHash = 0;
 constexpr int kVisitBitmap = 2;
 
+// Generators beyond the parent edge from which a rank-bitmap job reads a visited word before its
+// atomic as long as nothing better is known (a single job decides by its last round's yield, see
+// bitmap_test_first in hash_path.cu).
+constexpr int kTestMinDegree = 4;
+
 enum JobStatus : int {
     kRunning = 0,
     kDone = 1,          // empty next layer: growth complete
@@ -129,6 +172,8 @@ struct alignas(128) JobDev {
     int tagged;                // 1: keys leave bits 60-63 free for the parent-edge tag
     int closed;                // 1: every generator's inverse is in the set (every state but
                                //    the start carries a parent-edge tag)
+    int test;                  // rank bitmap, one job: the launch's first round reads visited
+                               //    words before its atomics (later rounds decide themselves)
     // dynamic, updated between rounds by block 0
     alignas(128) unsigned long long lo;     // frontier = keys[lo, hi)
     unsigned long long hi;

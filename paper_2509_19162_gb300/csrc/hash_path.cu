@@ -339,11 +339,20 @@ __device__ void close_round_single(JobDev* jobs, unsigned long long* ubeg, Ctl* 
     __syncthreads();
 }
 
-// Per-warp staging of newly found states in shared memory: a warp appends its winners to
-// its own buffer and reserves room in the job's key array with one atomic per flush, which
-// turns a per-unit atomic on one global counter into one per ~kStage/32 units and writes the
-// keys out coalesced.
-constexpr int kStage = 512;
+// Per-warp staging of newly found states in shared memory (dynamic, JobConst::stage entries a
+// warp): a warp appends its winners to its own buffer and reserves room in the job's key array with
+// one atomic per flush, which turns a per-unit atomic on one global counter into one per ~stage/32
+// units and writes the keys out coalesced.  A flush waits for that atomic, behind whatever the L2
+// has queued: with half the entries a growth bound by random DRAM accesses ran 15 % longer (S_14,
+// six random generators to radius 12: 20.1 against 23.2 ms), while a rank-bitmap launch that reads
+// visited words before its atomics finds few new states and has the better use of the room as L1
+// (S_12 pancake 28.9 against 30.3 ms).  Launches of several jobs keep selectors or generators per
+// warp as well and have to stay within 48 KB, or a quarter of the SM.
+constexpr int kStage = 512, kStageTest = 256, kStageMulti = 448;
+
+__host__ __device__ __forceinline__ int stage_entries(bool multi, bool bitmap, bool test) {
+    return multi ? (bitmap ? kStageTest : kStageMulti) : (bitmap && test ? kStageTest : kStage);
+}
 
 // The static fields of one job as the work loops use them.  A single-job launch receives them
 // as a kernel parameter (read from the constant bank: no load, no register, nothing to reload
@@ -360,9 +369,21 @@ struct JobConst {
     int tagged;
     int mode;
     int closed;
+    int test;              // rank bitmap: read the visited word before the atomic (bitmap_test_first)
+    int stage;             // staged states a warp holds
 };
 
-__device__ __forceinline__ JobConst job_const(const JobDev* J) {
+// Rank bitmap, read before the atomic or not: with `fresh` new states out of `expanded` last round,
+// whether less than a quarter of the candidates were new.  A read costs L2 about half of what an
+// atomic does (287 G/s against 133 G/s on a bitmap in L2), so it pays while most bits are found set:
+// S_12 pancake 28.8 ms, 41.2 ms without; S_11 under L, R, X, half of whose candidates are new, 1.04 ms
+// by this rule and 1.13 ms with the line at a half.
+__host__ __device__ __forceinline__ bool bitmap_test_first(unsigned long long fresh, unsigned long long expanded,
+                                                           int k, int closed) {
+    return 4 * fresh < expanded * (unsigned long long)(k - (closed ? 1 : 0));
+}
+
+__device__ __forceinline__ JobConst job_const(const JobDev* J, int stage) {
     JobConst c;
     c.keys = J->keys;
     c.keys_cap = J->keys_cap;
@@ -374,6 +395,8 @@ __device__ __forceinline__ JobConst job_const(const JobDev* J) {
     c.tagged = J->tagged;
     c.mode = J->mode;
     c.closed = J->closed;
+    c.test = c.k - (c.closed ? 1 : 0) >= kTestMinDegree;     // several jobs: by the out-degree alone
+    c.stage = stage;
     return c;
 }
 
@@ -438,12 +461,11 @@ __device__ __forceinline__ void stage_flush_block(uint64_t* buf, int& cnt, JobDe
 // leads back to its parent, which is already visited.  When every active lane of the warp holds
 // a tagged state, each lane runs only the other k - 1 generators (the generator index depends on
 // the lane), so the parent edge costs neither a probe nor the expansion and index arithmetic.
-template <int kProbeILP, int kMode, int kN = 0>
+template <int kProbeILP, int kMode>
 __device__ __forceinline__ void do_unit(JobDev* J, const JobConst& c, const GenSM* gens,
                                         unsigned long long idx, unsigned long long hi, uint64_t* buf,
                                         int& cnt, int lane, bool& overflow_seen, uint64_t s) {
     const bool active = idx < hi;
-    const int n = c.n;
     const bool tagged = c.tagged != 0;
     unsigned tag = 0;                       // 1 + generator that leads back to the parent
     if (tagged) {
@@ -465,13 +487,10 @@ __device__ __forceinline__ void do_unit(JobDev* J, const JobConst& c, const GenS
             // skipping: generators 0..tag-2 keep their slot, the rest move up by one (inactive
             // lanes have tag 0 and take j + 1 <= k - 1)
             gi[i] = (skip && (int)tag - 1 <= j) ? j + 1 : j;
-            t[i] = (i < ng) ? apply_gen<kMode != kVisitBitmap>(gens[gi[i]], s) : 0;
+            t[i] = (i < ng) ? apply_gen(gens[gi[i]], s) : 0;
             if (active && i < ng && tag != (unsigned)(gi[i] + 1)) vmask |= 1u << i;
         }
-        if (kMode == kVisitBitmap)
-            bitmap_insert_multi<kProbeILP, kN>(reinterpret_cast<unsigned*>(c.table), c.bitmap_words,
-                                               n, t, res, vmask);
-        else if (kMode == 1)
+        if (kMode == 1)
             table_insert_multi_sector<kProbeILP>(c.table, c.table_mask, t, res, vmask, kMaxProbe);
         else
             table_insert_multi_slot<kProbeILP>(c.table, c.table_mask, t, res, vmask, kMaxProbe);
@@ -491,7 +510,7 @@ __device__ __forceinline__ void do_unit(JobDev* J, const JobConst& c, const GenS
             }
             cnt += __popc(fresh);
             __syncwarp();
-            if (cnt > kStage - 32) stage_flush(buf, cnt, J, c, lane);
+            if (cnt > c.stage - 32) stage_flush(buf, cnt, J, c, lane);
         }
     }
 }
@@ -501,7 +520,7 @@ __device__ __forceinline__ void do_unit(JobDev* J, const JobConst& c, const GenS
 // and its non-parent generator number l mod (k - 1) (lslot), so that the k - 1 probes of a state
 // are in flight together rather than one after the other.  Every state must carry its parent-edge
 // tag (the set is closed under inverses and the frontier is not the start).
-template <int kMode, int kN = 0>
+template <int kMode>
 __device__ __forceinline__ void do_unit_split(JobDev* J, const JobConst& c, const GenSM* gens, bool active,
                                               uint64_t s, int lslot, uint64_t* buf, int& cnt, int lane,
                                               bool& overflow_seen) {
@@ -511,11 +530,9 @@ __device__ __forceinline__ void do_unit_split(JobDev* J, const JobConst& c, cons
     const int gi = (active && lslot >= (int)tag - 1) ? lslot + 1 : lslot;
     uint64_t t[1];
     int res[1];
-    t[0] = apply_gen<kMode != kVisitBitmap>(gens[gi], s);
+    t[0] = apply_gen(gens[gi], s);
     const unsigned vmask = active ? 1u : 0u;
-    if (kMode == kVisitBitmap)
-        bitmap_insert_multi<1, kN>(reinterpret_cast<unsigned*>(c.table), c.bitmap_words, c.n, t, res, vmask);
-    else if (kMode == 1)
+    if (kMode == 1)
         table_insert_multi_sector<1>(c.table, c.table_mask, t, res, vmask, kMaxProbe);
     else
         table_insert_multi_slot<1>(c.table, c.table_mask, t, res, vmask, kMaxProbe);
@@ -527,7 +544,127 @@ __device__ __forceinline__ void do_unit_split(JobDev* J, const JobConst& c, cons
     if (res[0] == 1) buf[cnt + __popc(fresh & lanemask_lt())] = t[0] | (uint64_t)gens[gi].inv_tag << 60;
     cnt += __popc(fresh);
     __syncwarp();
-    if (cnt > kStage - 32) stage_flush(buf, cnt, J, c, lane);
+    if (cnt > c.stage - 32) stage_flush(buf, cnt, J, c, lane);
+}
+
+// ---- rank bitmap: candidates, probes, staging ------------------------------------------------
+// A growth on a bitmap in L2 is bound by instructions (the expansion and the rank of a candidate)
+// and by the L2 rate of returned atomics (133 G/s).  So a state is expanded as bytes (six permutes a
+// generator for n <= 12 where the shift-and-mask form took about ten instructions a term, six
+// instructions a rank position where it took nine), a candidate's visited word is looked at one
+// candidate later, and rounds that find mostly visited states read the word before any atomic.
+// S_12 pancake: 55.8 ms before, 41.2 ms with byte states, 28.8 ms reading first; S_11 under L, R, X
+// 1.17 to 1.01 ms; 1024 random groups 47.5 to 36.3 ms.
+// One candidate per lane whose visited word has been asked for but not yet looked at: the next
+// candidate is computed while the word is on its way.  w: word index, b: bit (its low five bits),
+// word: the visited word as the probe saw it.  Word indices fit 32 bits (n <= 14: 2.8e9 words).
+// Every index lies inside the bitmap: frontier keys are permutations of 0..n-1 (the start is, and
+// generators permute), and the rank of a permutation is below n!.
+struct BitmapCand {
+    uint32_t lo, hi, w, b, word;
+    bool live;
+};
+
+// Candidates whose visited bit was clear when they read it, waiting for their atomicOr (test first
+// only): at most 63 between calls, popped 32 at a time so that the atomics run on full warps.
+constexpr int kPend = 64;
+
+__device__ __forceinline__ void stage_push(bool fresh, uint32_t klo, uint32_t khi, uint64_t* buf, int& cnt,
+                                           JobDev* J, const JobConst& c, int lane) {
+    const unsigned m = __ballot_sync(0xffffffffu, fresh);
+    if (fresh) buf[cnt + __popc(m & lanemask_lt())] = (uint64_t)khi << 32 | klo;
+    cnt += __popc(m);
+    __syncwarp();
+    if (cnt > c.stage - 32) stage_flush(buf, cnt, J, c, lane);
+}
+
+// Claim the last `take` (<= 32) pending candidates: the ones whose bit this atomicOr set are new.
+__device__ __forceinline__ void pend_claim(uint4* pend, int& pcnt, int take, uint64_t* buf, int& cnt, JobDev* J,
+                                           const JobConst& c, int lane) {
+    pcnt -= take;
+    bool fresh = false;
+    uint4 e = make_uint4(0u, 0u, 0u, 0u);
+    if (lane < take) {
+        e = pend[pcnt + lane];
+        const unsigned bit = 1u << (e.w & 31u);
+        fresh = !(atomicOr(reinterpret_cast<unsigned*>(c.table) + e.z, bit) & bit);
+    }
+    __syncwarp();
+    stage_push(fresh, e.x, e.y, buf, cnt, J, c, lane);
+}
+
+// Ask for a candidate's visited word.  Test first: a plain load, which may hit this SM's L1; bits
+// are only ever set, so a set bit is the truth and a stale clear one is caught by the atomicOr of
+// pend_claim.  Otherwise the atomicOr itself, whose returned word decides.
+__device__ __forceinline__ void bitmap_probe(BitmapCand& a, const JobConst& c, bool test) {
+    unsigned* p = reinterpret_cast<unsigned*>(c.table) + a.w;
+    if (test) {
+        if (a.live) asm volatile("ld.relaxed.cta.global.b32 %0, [%1];" : "=r"(a.word) : "l"(p));
+    } else {
+        if (a.live) a.word = atomicOr(p, 1u << (a.b & 31u));
+    }
+}
+
+__device__ __forceinline__ void bitmap_settle(const BitmapCand& a, uint64_t* buf, int& cnt, uint4* pend, int& pcnt,
+                                              JobDev* J, const JobConst& c, bool test, int lane) {
+    const bool clear = a.live && !(a.word >> (a.b & 31u) & 1u);
+    if (!test) {
+        stage_push(clear, a.lo, a.hi, buf, cnt, J, c, lane);
+        return;
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, clear);
+    if (m == 0) return;
+    if (clear) pend[pcnt + __popc(m & lanemask_lt())] = make_uint4(a.lo, a.hi, a.w, a.b);
+    pcnt += __popc(m);
+    __syncwarp();
+    if (pcnt >= 32) pend_claim(pend, pcnt, 32, buf, cnt, J, c, lane);
+}
+
+// Candidate t = generator gi of state s.
+template <int N>
+__device__ __forceinline__ void bitmap_candidate(BitmapCand& a, const ByteState<N>& s, const uint32_t* sel,
+                                                 bool live) {
+    uint32_t head;
+    const ByteState<N> t = apply_selectors<N>(sel, s, &head);
+    const uint64_t r = rank_bytes<N>(t);
+    pack_bytes<N>(t, a.lo, a.hi);
+    a.hi |= head & 0xF0000000u;         // the parent-edge tag: the generator's inverse
+    a.w = (uint32_t)(r >> 5);
+    a.b = (uint32_t)r;
+    a.live = live;
+}
+
+// One group of 32 frontier states (one per lane), every generator applied to each.  `prev` is the
+// candidate still waiting for its visited word.  sel: generator 0's selectors, `stride` words from
+// one generator to the next.
+template <int N>
+__device__ __forceinline__ void bitmap_unit(JobDev* J, const JobConst& c, const uint32_t* sel, int stride,
+                                            bool test, bool active, uint64_t key, BitmapCand& prev, uint64_t* buf,
+                                            int& cnt, uint4* pend, int& pcnt, int lane) {
+    const unsigned tag = (unsigned)(key >> 60);   // 1 + generator that leads back to the parent
+    const ByteState<N> s = unpack_bytes<N>(key);
+    const int k = c.k;
+    const bool skip = __all_sync(0xffffffffu, !active || tag != 0);
+    const int iters = skip ? k - 1 : k;
+    // skipping: generators 0..tag-2 keep their slot, the rest move up by one (inactive lanes take
+    // j + 1 <= k - 1)
+    const int from = skip ? (int)tag - 1 : k;
+    for (int j = 0; j < iters; ++j) {
+        const int gi = j + (j >= from ? 1 : 0);
+        BitmapCand a;
+        bitmap_candidate<N>(a, s, sel + gi * stride, active && tag != (unsigned)(gi + 1));
+        bitmap_probe(a, c, test);
+        bitmap_settle(prev, buf, cnt, pend, pcnt, J, c, test, lane);
+        prev = a;
+    }
+}
+
+// Look at the last candidate and claim what is pending (before the job changes or a round ends).
+__device__ __forceinline__ void bitmap_drain(BitmapCand& prev, uint64_t* buf, int& cnt, uint4* pend, int& pcnt,
+                                             JobDev* J, const JobConst& c, bool test, int lane) {
+    bitmap_settle(prev, buf, cnt, pend, pcnt, J, c, test, lane);
+    prev.live = false;
+    if (pcnt > 0) pend_claim(pend, pcnt, pcnt, buf, cnt, J, c, lane);
 }
 
 // Next work unit of the block for the calling warp (one shared-memory atomic per warp).
@@ -544,7 +681,7 @@ __device__ __forceinline__ unsigned long long draw_unit(unsigned long long& coun
 // flush of newly found states (every thread of the block calls this).  The job's overflow flag
 // (buffers full: the host grows them and redoes the layer) is read every 16 units, one unit
 // before its value is needed.
-template <int kProbeILP, int kMode, int kN = 0>
+template <int kProbeILP, int kMode>
 __device__ __forceinline__ void phase_single(JobDev* J, const JobConst& c, const GenSM* gens,
                                              unsigned long long w0, unsigned long long W, uint64_t* buf,
                                              int lane, unsigned long long lo, unsigned long long hi) {
@@ -561,7 +698,7 @@ __device__ __forceinline__ void phase_single(JobDev* J, const JobConst& c, const
             const unsigned long long idx = lo + u * (unsigned long long)sp + (unsigned long long)lstate;
             const bool active = lstate < sp && idx < hi;
             const uint64_t s = active ? __ldcg(c.keys + idx) : 0;
-            do_unit_split<kMode, kN>(J, c, gens, active, s, lslot, buf, cnt, lane, overflow_seen);
+            do_unit_split<kMode>(J, c, gens, active, s, lslot, buf, cnt, lane, overflow_seen);
             if (overflow_seen) break;
         }
         stage_flush_block(buf, cnt, J, c, lane);
@@ -576,12 +713,86 @@ __device__ __forceinline__ void phase_single(JobDev* J, const JobConst& c, const
         s_next = (nu < total && lo + (nu << 5) + lane < hi) ? __ldcg(c.keys + lo + (nu << 5) + lane) : 0;
         const bool check = (iter & 15u) == 15u;
         if ((iter & 15u) == 14u) ov = ld_relaxed_int(&J->overflow);
-        do_unit<kProbeILP, kMode, kN>(J, c, gens, lo + (u << 5) + lane, hi, buf, cnt, lane, overflow_seen, s_cur);
+        do_unit<kProbeILP, kMode>(J, c, gens, lo + (u << 5) + lane, hi, buf, cnt, lane, overflow_seen, s_cur);
         if (check && __any_sync(0xffffffffu, ov)) overflow_seen = true;
         if (overflow_seen) break;
         u = nu;
     }
     stage_flush_block(buf, cnt, J, c, lane);
+}
+
+// phase_single of a rank-bitmap job.  A small round (at most one unit a warp) takes a lane per
+// (state, generator) pair, as do_unit_split, with one atomicOr each.
+template <int N>
+__device__ __forceinline__ void phase_bitmap(JobDev* J, const JobConst& c, const uint32_t* sel, int stride,
+                                             bool test, unsigned long long w0, unsigned long long W, uint64_t* buf,
+                                             uint4* pend, int lane, unsigned long long lo, unsigned long long hi) {
+    int cnt = 0, pcnt = 0;
+    const unsigned long long total = (hi - lo + 31) >> 5;
+    const int m = c.k - 1;                      // generators a tagged state expands
+    if (total <= W && c.closed && lo > 0 && m >= 1 && m <= 32) {
+        const int sp = 32 / m;
+        const int lstate = lane / m, lslot = lane - lstate * m;
+        const unsigned long long ts = (hi - lo + (unsigned long long)sp - 1) / (unsigned long long)sp;
+        for (unsigned long long u = w0; u < ts; u += W) {
+            const unsigned long long idx = lo + u * (unsigned long long)sp + (unsigned long long)lstate;
+            const bool active = lstate < sp && idx < hi;
+            const uint64_t key = active ? __ldcg(c.keys + idx) : 0;
+            const unsigned tag = (unsigned)(key >> 60);
+            // generators 0..tag-2 keep their number, the rest move up by one (idle lanes: lslot itself)
+            const int gi = (active && lslot >= (int)tag - 1) ? lslot + 1 : lslot;
+            BitmapCand a;
+            bitmap_candidate<N>(a, unpack_bytes<N>(key), sel + gi * stride, active);
+            bool fresh = false;
+            if (active) {
+                const unsigned bit = 1u << (a.b & 31u);
+                fresh = !(atomicOr(reinterpret_cast<unsigned*>(c.table) + a.w, bit) & bit);
+            }
+            stage_push(fresh, a.lo, a.hi, buf, cnt, J, c, lane);
+        }
+        stage_flush_block(buf, cnt, J, c, lane);
+        return;
+    }
+    BitmapCand prev;
+    prev.live = false;
+    prev.lo = prev.hi = prev.w = prev.b = prev.word = 0;
+    // units fit 32 bits (at most 14!/32); the last one may be partly empty
+    const unsigned units = (unsigned)total, step = (unsigned)W;
+    const unsigned last = (unsigned)(hi - lo - 1) & 31u;        // last lane of the last unit
+    const uint64_t* from = c.keys + lo + lane;
+    unsigned u = (unsigned)w0;
+    bool act = u < units && (u + 1 < units || lane <= (int)last);
+    uint64_t s_next = act ? __ldcg(from + ((unsigned long long)u << 5)) : 0;
+    int ov = 0;
+    for (unsigned iter = 0; u < units; ++iter) {
+        const uint64_t s_cur = s_next;
+        const bool active = act;
+        const unsigned nu = u + step;
+        act = nu < units && nu > u && (nu + 1 < units || lane <= (int)last);
+        s_next = act ? __ldcg(from + ((unsigned long long)nu << 5)) : 0;
+        const bool check = (iter & 15u) == 15u;
+        if ((iter & 15u) == 14u) ov = ld_relaxed_int(&J->overflow);
+        bitmap_unit<N>(J, c, sel, stride, test, active, s_cur, prev, buf, cnt, pend, pcnt, lane);
+        if (check && __any_sync(0xffffffffu, ov)) break;
+        if (nu < u) break;              // past the last unit (the counter wrapped)
+        u = nu;
+    }
+    bitmap_drain(prev, buf, cnt, pend, pcnt, J, c, test, lane);
+    stage_flush_block(buf, cnt, J, c, lane);
+}
+
+// bitmap_unit with n known at run time but the same for a whole warp (one job): compiled for
+// that n, through a switch.
+__device__ __forceinline__ void bitmap_unit_n(JobDev* J, const JobConst& c, const uint32_t* sel, int stride,
+                                              bool active, uint64_t key, BitmapCand& prev, uint64_t* buf, int& cnt,
+                                              uint4* pend, int& pcnt, int lane) {
+    switch (c.n) {
+#define CG_UNIT(n) case n: bitmap_unit<n>(J, c, sel, stride, c.test != 0, active, key, prev, buf, cnt, pend, pcnt, lane); break;
+        CG_UNIT(2) CG_UNIT(3) CG_UNIT(4) CG_UNIT(5) CG_UNIT(6) CG_UNIT(7) CG_UNIT(8) CG_UNIT(9) CG_UNIT(10)
+        CG_UNIT(11) CG_UNIT(12) CG_UNIT(13) CG_UNIT(14)
+#undef CG_UNIT
+        default: break;                 // no bitmap for other n
+    }
 }
 
 // Barrier payload of a single-job round: the next frontier's size, with this bit set when the
@@ -596,26 +807,52 @@ constexpr int kSmemGens = 32;
 // Several jobs: each warp keeps the generators of its current job in shared memory when the job
 // has at most this many.
 constexpr int kWarpGens = 10;
+// Rank bitmap: selectors of a single job's generators in shared memory when there are at most
+// this many; of a warp's current job, as many as fit where its kWarpGens generators would go.
+constexpr int kSmemSels = 64;
+constexpr int kWarpSels = kWarpGens * (int)sizeof(GenSM) / (kSelWords * 4);
+constexpr int kGenStride = (int)sizeof(GenSM) / 4;
 
 // kMulti = false: the launch has exactly one job (the single-job path only is compiled, which
-// keeps registers low), whose static fields are `jc`; true: any number of jobs (`jc` unused).
+// keeps registers low), whose static fields are `jc`; true: any number of jobs (of `jc` only the
+// stage size is used).
 template <int kProbeILP, int kMode, bool kMulti, int kN = 0>
 __global__ void __launch_bounds__(kGrowBlock, kMode == 2 ? 4 : ((kMode == 1 && kProbeILP >= 3) ? 2 : 3))
 hash_grow_kernel(JobDev* jobs, int njobs, unsigned long long* ubeg, Ctl* ctl, int max_rounds,
                  uint64_t timeout_ns, const AdmitDev* adm, const JobConst jc) {
-    __shared__ uint64_t s_stage[kGrowBlock / 32][kStage];
-    __shared__ GenSM s_gens[kSmemGens];
+    constexpr bool kBitmap = kMode == kVisitBitmap;
+    extern __shared__ uint64_t s_stage[];       // jc.stage entries a warp
+    __shared__ uint4 s_pend[kBitmap ? kGrowBlock / 32 : 1][kBitmap ? kPend : 1];
+    __shared__ GenSM s_gens[!kMulti && !kBitmap ? kSmemGens : 1];
+    __shared__ alignas(16) uint32_t s_selw[!kMulti && kBitmap ? kSmemSels * kSelWords : 4];
     __shared__ unsigned long long s_unit;
     __shared__ JobConst s_jc[kMulti ? kGrowBlock / 32 : 1];
     __shared__ GenSM s_wgens[kMulti ? kGrowBlock / 32 : 1][kMulti ? kWarpGens : 1];
     const GenSM* single_gens = jobs[0].gens;
-    if (!kMulti && jobs[0].k <= kSmemGens) {
+    if (!kMulti && !kBitmap && jobs[0].k <= kSmemGens) {
         for (int j = threadIdx.x; j < jobs[0].k; j += blockDim.x) s_gens[j] = jobs[0].gens[j];
         __syncthreads();
         single_gens = s_gens;
     }
+    if (!kMulti && kBitmap && jc.k <= kSmemSels) {
+        for (int i = threadIdx.x; i < jc.k * kSelWords; i += blockDim.x)
+            s_selw[i] = jobs[0].gens[i / kSelWords].sel[i % kSelWords];
+        __syncthreads();
+    }
     const int lane = threadIdx.x & 31;
-    uint64_t* buf = s_stage[threadIdx.x >> 5];
+    uint64_t* buf = s_stage + (threadIdx.x >> 5) * jc.stage;
+    uint4* pend = s_pend[kBitmap ? threadIdx.x >> 5 : 0];
+    // one round's work of a single job
+    auto single_phase = [&](bool test, unsigned long long w0, unsigned long long W, unsigned long long lo,
+                            unsigned long long hi) {
+        if constexpr (kBitmap && !kMulti) {
+            const bool smem = jc.k <= kSmemSels;
+            phase_bitmap<kN>(jobs, jc, smem ? s_selw : single_gens->sel, smem ? kSelWords : kGenStride, test, w0, W,
+                             buf, pend, lane, lo, hi);
+        } else if constexpr (!kMulti) {
+            phase_single<kProbeILP, kMode>(jobs, jc, single_gens, w0, W, buf, lane, lo, hi);
+        }
+    };
     // One job: every block keeps the frontier bounds itself.  They are read once here; after
     // each barrier the releasing block hands every block the size of the next frontier in the
     // barrier word, so no block reloads them.  (Several jobs: the round's layout is read from
@@ -629,6 +866,12 @@ hash_grow_kernel(JobDev* jobs, int njobs, unsigned long long* ubeg, Ctl* ctl, in
     }
 
     unsigned nbar = 0;                      // grid barriers this block has passed
+    // Single job: while the frontier stays small the block that closed a round runs the next ones
+    // alone, with __syncthreads for a barrier; the others wait until it releases them, with the
+    // word it arrived on.
+    bool solo = false;
+    unsigned long long word = 0;
+    bool test = !kMulti && jc.test != 0;    // rank bitmap: this round reads before its atomics
     for (int round = 0; round < max_rounds; ++round) {
         if (threadIdx.x == 0) {
             s_total = kMulti ? ld_relaxed_ull(&ctl->total_units) : (s_hi - s_lo + 31) >> 5;
@@ -653,9 +896,10 @@ hash_grow_kernel(JobDev* jobs, int njobs, unsigned long long* ubeg, Ctl* ctl, in
         bool overflow_seen = false;
         if (!kMulti) {
             // unit u goes to block u mod grid, so that a small round spreads over every SM
-            const unsigned long long W = (unsigned long long)gridDim.x * (blockDim.x >> 5);
-            const unsigned long long w0 = (unsigned long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
-            phase_single<kProbeILP, kMode, kN>(jobs, jc, single_gens, w0, W, buf, lane, lo, hi);
+            const unsigned long long W = (solo ? 1ull : (unsigned long long)gridDim.x) * (blockDim.x >> 5);
+            const unsigned long long w0 = solo ? (unsigned long long)(threadIdx.x >> 5)
+                                               : (unsigned long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+            single_phase(test, w0, W, lo, hi);
         } else {
             int cur = -1;
             JobDev* J = nullptr;
@@ -663,6 +907,13 @@ hash_grow_kernel(JobDev* jobs, int njobs, unsigned long long* ubeg, Ctl* ctl, in
             // used, which keeps them out of the registers)
             JobConst& c = s_jc[threadIdx.x >> 5];
             const GenSM* jg = nullptr;              // the current job's generators
+            const uint32_t* jsel = nullptr;         // or, for a rank-bitmap job, their selectors
+            int jstride = 0;
+            bool jbitmap = false;
+            BitmapCand prev;
+            prev.live = false;
+            prev.lo = prev.hi = prev.w = prev.b = prev.word = 0;
+            int pcnt = 0;
             int ovf = 0;                            // the current job's overflow flag, read a unit ago
             unsigned long long lo = 0, hi = 0, u0 = 0;
             const unsigned long long ue = stat * (blockIdx.x + 1) / gridDim.x;
@@ -696,14 +947,29 @@ hash_grow_kernel(JobDev* jobs, int njobs, unsigned long long* ubeg, Ctl* ctl, in
                     // same job as the previous unit
                 } else {
                     const int slot = find_job(ubeg, nj, u);
-                    if (J) stage_flush(buf, cnt, J, c, lane);
+                    if (J) {
+                        if (jbitmap) bitmap_drain(prev, buf, cnt, pend, pcnt, J, c, c.test != 0, lane);
+                        stage_flush(buf, cnt, J, c, lane);
+                    }
                     cur = slot;
                     J = jobs + (act ? __ldcg(act + slot) : slot);
-                    if (lane == 0) c = job_const(J);
+                    if (lane == 0) c = job_const(J, jc.stage);
                     __syncwarp();
                     ovf = 0;
                     jg = J->gens;
-                    if (kMulti && c.k <= kWarpGens) {
+                    jbitmap = kBitmap && c.mode == kVisitBitmap;
+                    if (jbitmap) {
+                        jsel = jg->sel;
+                        jstride = kGenStride;
+                        if (c.k <= kWarpSels) {
+                            uint32_t* to = reinterpret_cast<uint32_t*>(s_wgens[threadIdx.x >> 5]);
+                            for (int i = lane; i < c.k * kSelWords; i += 32)
+                                to[i] = jg[i / kSelWords].sel[i % kSelWords];
+                            __syncwarp();
+                            jsel = to;
+                            jstride = kSelWords;
+                        }
+                    } else if (c.k <= kWarpGens) {
                         // copy them into this warp's shared slots, word by word across the lanes
                         GenSM* dst = s_wgens[threadIdx.x >> 5];
                         const unsigned words = (unsigned)c.k * (unsigned)(sizeof(GenSM) / 4);
@@ -733,58 +999,63 @@ hash_grow_kernel(JobDev* jobs, int njobs, unsigned long long* ubeg, Ctl* ctl, in
                     const unsigned long long nf = first + 32;
                     s_nx = (sub + 1 < umult && nf + lane < hi) ? __ldcg(c.keys + nf + lane) : 0;
                     // In the rank-bitmap variant a launch may mix jobs of both visited-set kinds.
-                    if (kMode == kVisitBitmap && c.mode != kVisitBitmap)
-                        do_unit<kProbeILP, kVisitHash>(J, c, jg, idx, hi, buf, cnt, lane, overflow_seen, s0);
+                    if (kBitmap && jbitmap)
+                        bitmap_unit_n(J, c, jsel, jstride, idx < hi, s0, prev, buf, cnt, pend, pcnt, lane);
                     else
-                        do_unit<kProbeILP, kMode>(J, c, jg, idx, hi, buf, cnt, lane, overflow_seen, s0);
+                        do_unit<kProbeILP, kBitmap ? kVisitHash : kMode>(J, c, jg, idx, hi, buf, cnt, lane,
+                                                                         overflow_seen, s0);
                     first = nf;
                 }
             }
-            if (J) stage_flush(buf, cnt, J, c, lane);
+            if (J) {
+                if (jbitmap) bitmap_drain(prev, buf, cnt, pend, pcnt, J, c, c.test != 0, lane);
+                stage_flush(buf, cnt, J, c, lane);
+            }
         }
         // One barrier per round: the last block to finish the round closes it (layer counts,
         // stop tests, next round's work layout) and then releases the others.
-        unsigned long long word = 0;
-        const int arrive = grid_arrive(ctl, timeout_ns, word, nbar++);
+        int arrive = 1;
+        if (solo) __syncthreads();
+        else arrive = grid_arrive(ctl, timeout_ns, word, nbar++);
         if (arrive < 0) return;
         if (arrive == 1) {
             if (!kMulti) {
                 close_round_single(jobs, ubeg, ctl, &s_fresh, &s_lo, &s_hi);
-                // While the frontier stays small this block runs the next rounds alone, with
-                // __syncthreads for a barrier; the other blocks wait until it releases them.
-                bool solo = false;
-                for (;;) {
-                    const unsigned long long t = (s_fresh + 31) >> 5;
-                    if (t == 0 || t > kSoloUnits || round + 1 >= max_rounds) break;
-                    ++round;
+                const unsigned long long fresh = s_fresh;
+                const unsigned long long t = (fresh + 31) >> 5;
+                test = bitmap_test_first(fresh, hi - lo, jc.k, jc.closed);
+                const bool more = t != 0 && t <= kSoloUnits && round + 1 < max_rounds;
+                if (more) {
                     solo = true;
-                    const unsigned long long slo = s_lo, shi = s_hi;
-                    phase_single<kProbeILP, kMode, kN>(jobs, jc, single_gens, threadIdx.x >> 5,
-                                                       blockDim.x >> 5, buf, lane, slo, shi);
-                    __syncthreads();
-                    close_round_single(jobs, ubeg, ctl, &s_fresh, &s_lo, &s_hi);
+                    continue;
                 }
-                if (threadIdx.x == 0 && s_fresh == 0) s_hi = s_lo;   // stop: empty frontier
+                __syncthreads();                                    // everyone has read s_fresh
+                if (threadIdx.x == 0 && fresh == 0) s_hi = s_lo;    // stop: empty frontier
                 // payload: the next frontier's size, and whether this block ran rounds alone (the
                 // others' bounds are then stale and they reload them)
-                grid_release(ctl, word, s_fresh | (solo ? kReloadFlag : 0ull));
+                grid_release(ctl, word, fresh | (solo ? kReloadFlag : 0ull));
+                solo = false;
             } else {
                 if (adm) close_round_admit(jobs, ubeg, ctl, adm);
                 else close_round(jobs, njobs, ubeg, ctl);
                 grid_release(ctl, word, 0);
             }
-        } else if (!kMulti && threadIdx.x == 0) {
+        } else if (!kMulti) {
             // the next frontier follows this one in the key array (size 0: the growth stops)
             const unsigned long long payload = word >> kGenBits;
             const unsigned long long fresh = payload & ~kReloadFlag;
-            if (fresh == 0) {
-                s_lo = s_hi;
-            } else if (payload & kReloadFlag) {
-                s_lo = ld_relaxed_ull(&jobs[0].lo);
-                s_hi = ld_relaxed_ull(&jobs[0].hi);
-            } else {
-                s_lo = s_hi;
-                s_hi = s_hi + fresh;
+            // (after rounds run by one block the frontier is small and either way will do)
+            test = bitmap_test_first(fresh, hi - lo, jc.k, jc.closed);
+            if (threadIdx.x == 0) {
+                if (fresh == 0) {
+                    s_lo = s_hi;
+                } else if (payload & kReloadFlag) {
+                    s_lo = ld_relaxed_ull(&jobs[0].lo);
+                    s_hi = ld_relaxed_ull(&jobs[0].hi);
+                } else {
+                    s_lo = s_hi;
+                    s_hi = s_hi + fresh;
+                }
             }
         }
     }
@@ -932,10 +1203,7 @@ GrowFn grow_fn_t(int variant) {
         case 10: return hash_grow_kernel<2, 1, M>;
         case 11: return hash_grow_kernel<3, 1, M>;
         case 12: return hash_grow_kernel<4, 1, M>;
-        case 17: return hash_grow_kernel<1, 2, M>;
-        case 18: return hash_grow_kernel<2, 2, M>;
-        case 19: return hash_grow_kernel<3, 2, M>;
-        default: return hash_grow_kernel<4, 2, M>;
+        default: return hash_grow_kernel<1, 2, M, M ? 0 : 14>;   // (single jobs: grow_fn_bitmap_n)
     }
 }
 
@@ -951,7 +1219,7 @@ GrowFn grow_fn_bitmap_n(int n, std::integer_sequence<int, Ns...>) {
 }
 
 GrowFn grow_fn(int variant, bool multi, int n) {
-    if (variant == 17 && !multi && n >= 2 && n <= 14)
+    if (variant >= 17 && !multi && n >= 2 && n <= 14)
         return grow_fn_bitmap_n<1>(n, std::make_integer_sequence<int, 13>{});
     return grow_fn(variant, multi);
 }
@@ -960,7 +1228,8 @@ GrowFn grow_fn(int variant, bool multi, int n) {
 int hash_grow_max_grid(int device, int ilp, bool multi) {
     int sms = 0, per_sm = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, grow_fn(ilp, multi), kGrowBlock, 0) !=
+    const size_t smem = (size_t)(kGrowBlock / 32) * stage_entries(multi, ilp >= 16, false) * sizeof(uint64_t);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, grow_fn(ilp, multi), kGrowBlock, smem) !=
         cudaSuccess)
         return 0;
     return sms * per_sm;
@@ -996,6 +1265,7 @@ cudaError_t launch_hash_grow(JobDev* d_jobs, int njobs, unsigned long long* d_ub
     // copy of them, one job runs through the general kernel.
     const bool multi = njobs > 1 || d_adm != nullptr || host_job == nullptr;
     JobConst jc = {};
+    jc.stage = stage_entries(multi, ilp >= 16, !multi && host_job->test != 0);
     if (!multi) {
         jc.keys = host_job->keys;
         jc.keys_cap = host_job->keys_cap;
@@ -1007,11 +1277,12 @@ cudaError_t launch_hash_grow(JobDev* d_jobs, int njobs, unsigned long long* d_ub
         jc.tagged = host_job->tagged;
         jc.mode = host_job->mode;
         jc.closed = host_job->closed;
+        jc.test = host_job->test;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kGrowBlock);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = (size_t)(kGrowBlock / 32) * jc.stage * sizeof(uint64_t);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;

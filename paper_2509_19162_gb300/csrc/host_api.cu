@@ -217,6 +217,10 @@ std::vector<GenSM> make_gensms(const std::vector<std::vector<uint8_t>>& rows, in
         for (int i = 0; i < n; ++i) inv[rows[j][i]] = (uint8_t)i;
         for (size_t m = 0; m < rows.size() && m < 15; ++m)
             if (rows[m] == inv) { out[j].inv_tag = (uint32_t)(m + 1); break; }
+        if (w == 4 && n <= cg::kMaxN) {
+            cg::make_selectors(rows[j].data(), n, out[j].sel);
+            out[j].sel[0] |= out[j].inv_tag << 28;
+        }
     }
     return out;
 }
@@ -551,6 +555,7 @@ void fill_static(cg_growth* h, JobDev& J) {
     J.tagged = h->n * h->width <= 60 ? 1 : 0;
     J.closed = 1;
     for (const GenSM& g : h->gsm) J.closed &= g.inv_tag != 0 ? 1 : 0;
+    J.test = h->k - J.closed >= cg::kTestMinDegree ? 1 : 0;
 }
 
 int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
@@ -646,6 +651,8 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
                 }
             }
         }
+        const uint64_t expanded = J.hi - J.lo;
+        const int test = J.test;
         if ((e = cg::launch_hash_grow(h->d_job, 1, h->d_ubeg, h->d_ctl, grid,
                                       order_frontier ? 1 : cg::kMaxLayers + 1, kTimeoutNs, ilp, st, h->n,
                                       nullptr, &J)) != cudaSuccess)
@@ -664,6 +671,8 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
         if (ctl.err) return ctl.err;
         if (sort_err) return sort_err;
         if (order_frontier && J.status == cg::kRunning) {
+            // as the kernel decides between its own rounds (bitmap_test_first)
+            J.test = 4 * (J.hi - J.lo) < expanded * (uint64_t)(h->k - J.closed) ? 1 : 0;
             // the next round, in its own launch
             if ((e = cg::launch_resume_units(h->d_job, 1, h->d_ubeg, h->d_ctl, st)) != cudaSuccess)
                 return cuda_rc(e);
@@ -685,6 +694,7 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
                                               grid_max, st);
         if (e != cudaSuccess) return cuda_rc(e);
         fill_static(h, J);
+        J.test = test;                      // the layer is redone as it was begun
         J.tail = J.hi;
         J.overflow = 0;
         J.status = cg::kRunning;
