@@ -558,6 +558,29 @@ void fill_static(cg_growth* h, JobDev& J) {
     J.test = h->k - J.closed >= cg::kTestMinDegree ? 1 : 0;
 }
 
+// Before a round on a frontier of J (host copy, current): room for the next layer as the last two
+// predict it -- F * (F / Fprev) and a quarter more, at most every candidate, never past the states
+// there can be.  A layer that comes out larger still ends the round early (kNeedMem) and is redone in
+// a larger store; so is one whose predicted room could not be allocated.  Cutting rounds off at 2^24,
+// 2^26, ... states, redoing them and rebuilding the bitmap took 24 of S_14's 44 ms under six random
+// generators to 3.6e8 states, and 180 of whole S_13 pancake's 864 ms.
+int grow_for_next_layer(cg_growth* h, JobDev& J, uint64_t Fprev, uint64_t max_cap, cudaStream_t st) {
+    const double F = (double)(J.hi - J.lo);
+    const double all = F * (double)h->k, ratio = Fprev > 0 ? 1.25 * F / (double)Fprev : (double)h->k;
+    const uint64_t next = (uint64_t)std::min(all, F * ratio) + 1;
+    const uint64_t left = h->states_bound - std::min(h->states_bound, (uint64_t)J.hi);
+    const uint64_t need = J.hi + std::min(next, left);
+    if (need <= h->keys_cap || h->keys_cap >= max_cap) return CG_OK;
+    const uint64_t cap = std::min(max_cap, std::max(need, 2 * h->keys_cap));
+    const int rc = resize_state(h, cap, J.hi, st);
+    if (rc == CG_ENOMEM) return CG_OK;
+    if (rc) return rc;
+    J.keys = h->d_keys;
+    J.keys_cap = h->keys_cap;
+    h->stats.h2d_bytes += sizeof(J);
+    return cuda_rc(cudaMemcpyAsync(h->d_job, &J, sizeof(J), cudaMemcpyHostToDevice, st));
+}
+
 int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
     // buffers of an earlier run that switched to the sorted step are not needed
     if (h->d_cand || h->d_L[0]) h->release_sort(st);
@@ -615,22 +638,29 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
         if ((e = cudaEventCreate(&h->ev0)) != cudaSuccess) return cuda_rc(e);
         if ((e = cudaEventCreate(&h->ev1)) != cudaSuccess) return cuda_rc(e);
     }
-    // A rank bitmap larger than L2 takes its random atomics from DRAM.  Keys in ascending order are
-    // in Lehmer-rank order (the value at position n - 1 is the top rank digit, and so on down), and
-    // a generator that moves only positions below j sends a state within j! ranks of it: a frontier
-    // grouped by its top four elements keeps the visited words of most images inside the group's
-    // stretch of the bitmap, which L2 holds while the grid works through it.  Such a growth runs
-    // one round per launch, and a frontier of at least kOrderMinStates states is first put in order
-    // of key bits [4n - 16, 4n) (two stable 8-bit passes; the parent-edge tags ride along), when
-    // the sort's scratch fits beside the job's buffers within mem_cap.
+    // A rank bitmap larger than L2 takes its random atomics from DRAM.  Such a growth runs one round
+    // per launch, which the host uses twice.  (1) The key store is grown before a round that may
+    // outgrow it, by the last layers' ratio (grow_for_next_layer), so that no round is cut off, redone
+    // and preceded by a rebuild of the bitmap.  (2) Keys in ascending order are in Lehmer-rank order
+    // (the value at position n - 1 is the top rank digit, and so on down), and a generator that moves
+    // only positions below j sends a state within j! ranks of it: a frontier grouped by its top four
+    // elements keeps the visited words of such images inside the group's stretch of the bitmap, which
+    // L2 holds while the grid works through it.  So when some generator leaves the top two positions
+    // alone, a frontier of at least kOrderMinStates states is first put in order of key bits
+    // [4n - 16, 4n) (two stable 8-bit passes; the parent-edge tags ride along), when the sort's
+    // scratch fits beside the job's buffers within mem_cap.
     int l2 = 0;
     if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, h->device) != cudaSuccess) {
         (void)cudaGetLastError();
         l2 = 0;
     }
-    const bool order_frontier = bitmap && h->start_is_perm && h->width == 4 && h->n >= 8 && l2 > 0 &&
-                                bm_bytes > (uint64_t)l2;
+    const bool by_round = bitmap && h->start_is_perm && h->width == 4 && h->n >= 8 && l2 > 0 &&
+                          bm_bytes > (uint64_t)l2;
+    bool order_frontier = false;
+    for (const auto& r : h->rows) order_frontier |= by_round && r[h->n - 1] == h->n - 1 && r[h->n - 2] == h->n - 2;
+    uint64_t Fprev = 0;                         // size of the layer before the frontier
     for (;;) {
+        if (by_round && J.hi > 0 && (rc = grow_for_next_layer(h, J, Fprev, max_cap, st))) return rc;
         if ((e = cudaEventRecord(h->ev0, st)) != cudaSuccess) return cuda_rc(e);
         int sort_err = 0;
         if (order_frontier) {
@@ -654,7 +684,7 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
         const uint64_t expanded = J.hi - J.lo;
         const int test = J.test;
         if ((e = cg::launch_hash_grow(h->d_job, 1, h->d_ubeg, h->d_ctl, grid,
-                                      order_frontier ? 1 : cg::kMaxLayers + 1, kTimeoutNs, ilp, st, h->n,
+                                      by_round ? 1 : cg::kMaxLayers + 1, kTimeoutNs, ilp, st, h->n,
                                       nullptr, &J)) != cudaSuccess)
             return cuda_rc(e);
         if ((e = cudaEventRecord(h->ev1, st)) != cudaSuccess) return cuda_rc(e);
@@ -670,7 +700,8 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
         h->stats.rounds += ctl.rounds;
         if (ctl.err) return ctl.err;
         if (sort_err) return sort_err;
-        if (order_frontier && J.status == cg::kRunning) {
+        if (by_round && J.status == cg::kRunning) {
+            Fprev = expanded;
             // as the kernel decides between its own rounds (bitmap_test_first)
             J.test = 4 * (J.hi - J.lo) < expanded * (uint64_t)(h->k - J.closed) ? 1 : 0;
             // the next round, in its own launch
