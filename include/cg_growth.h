@@ -47,8 +47,9 @@ extern "C" {
                                   cg_growth_run_noalloc (CG_NOALLOC_MAX_*)                    */
 
 /* ---- strategies (cg_growth_set_option(h, CG_OPT_STRATEGY, ...)) --------------------- */
-#define CG_STRATEGY_AUTO    0  /* library chooses: BITMAP when eligible, SWEEP when the states
-                                  of BITMAP do not fit but the sweep's bitmaps do, else HASH  */
+#define CG_STRATEGY_AUTO    0  /* library chooses: SWEEP for whole growths of large dense groups
+                                  (n >= 10) and when the states of BITMAP do not fit but the
+                                  sweep's bitmaps do, else BITMAP when eligible, else HASH     */
 #define CG_STRATEGY_HASH    1  /* visited open-addressing hash set; any generating set        */
 #define CG_STRATEGY_SORT    2  /* sorted layers, radix sort + unique + merge-path difference
                                   against layers r and r-1; inverse-closed sets only          */
@@ -62,7 +63,9 @@ extern "C" {
                                   element of S_n, nothing per state), so the whole of S_14 fits
                                   in 33.4 GB; any generating set; start with distinct values;
                                   needs n <= 14 and the bitmaps within mem_cap (else CG_EINVAL
-                                  at run)                                                      */
+                                  at run).  For 10 <= n, when a fourth bit fits (43.8 GB for
+                                  S_14), the states are expanded in blocks that the generators
+                                  move together                                                */
 
 /* ---- options ------------------------------------------------------------------------ */
 #define CG_OPT_STRATEGY     1  /* one of CG_STRATEGY_*                                        */
@@ -79,8 +82,8 @@ extern "C" {
                                   nonempty 1024-rank blocks.  0 = auto (rank order when they
                                   fill at least a quarter of S_n and the visited bitmap, n!/8
                                   bytes, is larger than L2; else the order of discovery);
-                                  1 = order of discovery; 2 = rank order.  The layers are the
-                                  same in every order                                          */
+                                  1 = order of discovery; 2 = rank order (both state by state,
+                                  never in blocks).  The layers are the same in every order    */
 /* batch options (cg_batch_set_option; CG_OPT_ILP and CG_OPT_GRID apply there too, 1..4)      */
 #define CG_OPT_BATCH_WAVE_L2 6 /* cap on the summed visited-set bytes of one launch:
                                   0 = half of L2 (default), -1 = none                          */

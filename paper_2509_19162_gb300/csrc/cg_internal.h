@@ -219,6 +219,33 @@ struct alignas(128) SweepDev {
     int status;                // JobStatus
 };
 
+// One growth in blocks of 2^M states that the generators move together (block_path.cu): the visited
+// set and three layers, one bit per element of S_n each, as one word per block; layer r lives in
+// N[r % 3].  flag[i][g] is nonzero when one of the blocks 32 g .. 32 g + 31 may have bits in N[i].
+constexpr int block_pairs(int n) { return n >= 12 ? 6 : n / 2; }
+constexpr int kBlockMinN = 10, kBlockMaxN = 14;
+constexpr int kBlockSmemGens = 128;
+struct alignas(128) BlockDev {
+    // static, written by the host
+    void* V;                   // 64-bit words for M = 6, 32-bit words for M = 5
+    void* N[3];
+    unsigned char* flag[3];
+    uint2* top;                // unranking tables (block_tables_kernel)
+    unsigned* bottom;
+    const uint4* maps;         // k generators: byte q = the position that position q's value goes to
+    uint64_t* layer_sizes;     // layers_cap entries; [0] = 1
+    uint64_t stop_above;       // 0: none
+    uint64_t start;            // the start state's packed key
+    unsigned nblocks, ngroups, ntop;
+    int k, n;
+    int layers_cap;
+    int max_radius;            // < 0: unlimited
+    // dynamic, updated during a run
+    alignas(128) unsigned long long fresh;  // states found in the round
+    int radius;                // radius of the frontier layer
+    int status;                // JobStatus
+};
+
 // Admission of many jobs into one persistent launch (a batch): the jobs are grown in index
 // order, at most max_active at a time and with the visited sets of the active jobs summing to at
 // most `window` bytes, so that their random accesses stay in L2.  Whenever jobs end, the block

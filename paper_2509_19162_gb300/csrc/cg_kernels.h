@@ -66,6 +66,17 @@ cudaError_t launch_sweep_init(SweepDev* d, cudaStream_t st);
 constexpr int kSweepOrderAuto = 0, kSweepOrderList = 1, kSweepOrderRank = 2;
 cudaError_t launch_sweep_grow(SweepDev* d, Ctl* ctl, int grid, int max_rounds, uint64_t timeout_ns,
                               int ilp, int n, int order, cudaStream_t st);
+// sweep strategy in blocks of states (block_path.cu): n in kBlockMinN .. kBlockMaxN
+int block_max_grid(int device, int n);
+cudaError_t launch_block_tables(const BlockDev& host, cudaStream_t st);
+cudaError_t launch_block_init(BlockDev* d, int n, cudaStream_t st);
+cudaError_t launch_block_grow(BlockDev* d, Ctl* ctl, int n, int grid, int max_rounds, uint64_t timeout_ns,
+                              cudaStream_t st);
+// Packed keys of the layer in N[which] into out[0, cap); *count (zeroed by the caller) receives their
+// number.
+cudaError_t launch_block_export(const BlockDev& host, int which, uint64_t* out, unsigned long long cap,
+                                unsigned long long* count, int grid, cudaStream_t st);
+
 // Unrank the states of one layer (bitmap F, block list L[0, nlist)) into out[0, cap); *count
 // (zeroed by the caller) receives the number of states.
 cudaError_t launch_sweep_export(const unsigned* F, const unsigned* L, unsigned long long nlist, int n,

@@ -21,6 +21,7 @@
 #include "group_order.h"
 #include "sort_kernels.h"
 
+using cg::BlockDev;
 using cg::Ctl;
 using cg::GenSM;
 using cg::JobDev;
@@ -286,6 +287,28 @@ uint64_t sweep_bytes(int n) {
     return 4 * (3 * words + 2 * sum + 2 * nb) + 4096;
 }
 
+// Sweep in blocks of states (block_path.cu) over S_n: layout of the one allocation
+// V | N0 N1 N2 | flags of the three | top table | bottom table | generator maps.
+struct BlockLayout {
+    uint64_t nblocks, ngroups, ntop, words, flags, o_flags, o_top, o_bottom, o_maps, bytes;
+};
+BlockLayout block_layout(int n, int k) {
+    BlockLayout L;
+    const int M = cg::block_pairs(n);
+    const uint64_t word = M == 6 ? 8 : 4;
+    L.nblocks = factorial(n) >> M;
+    L.ngroups = (L.nblocks + 31) / 32;
+    L.ntop = L.nblocks / 2520;
+    L.words = (L.nblocks * word + 255) & ~255ull;
+    L.flags = (L.ngroups + 255) & ~255ull;
+    L.o_flags = 4 * L.words;
+    L.o_top = L.o_flags + 3 * L.flags;
+    L.o_bottom = L.o_top + ((L.ntop * 8 + 255) & ~255ull);
+    L.o_maps = L.o_bottom + ((2520 * 4 + 255) & ~255ull);
+    L.bytes = L.o_maps + (uint64_t)k * 16;
+    return L;
+}
+
 // 32-bit words of a rank bitmap over S_n, rounded up to whole 8-byte slots.
 uint64_t bitmap_words(int n) { return ((factorial(n) + 63) / 64) * 2; }
 
@@ -437,6 +460,10 @@ struct cg_growth {
     uint64_t sw_bytes = 0;
     SweepDev host_sweep{};
     bool last_is_sweep = false;
+    BlockDev* d_block = nullptr;                 // sweep in blocks of states
+    char* d_blk = nullptr;                       // one allocation (BlockLayout)
+    BlockDev host_block{};
+    bool last_is_block = false;
 
     JobDev host_job{};
     bool have_last = false;
@@ -459,6 +486,10 @@ struct cg_growth {
         d_sweep = nullptr;
         d_sw = nullptr;
         sw_bytes = 0;
+        dev_free(d_block, st);
+        dev_free(d_blk, st);
+        d_block = nullptr;
+        d_blk = nullptr;
         dev_free(d_wgens, st);
         dev_free(d_wjob, st);
         dev_free(d_wkeys, st);
@@ -891,17 +922,115 @@ int run_wide(cg_growth* h, cudaStream_t st, int* final_status) {
 // Bitmaps over S_n for the visited set and two layers (sweep_path.cu: 3 bits per element); one
 // persistent launch runs every layer step.  Needs a start with distinct values and n <= 14.
 
-// AUTO takes the sweep for the whole growth (no radius or layer-size limit) of a dense subgroup
-// of S_n whose states, stored as keys beside a rank bitmap, would not fit the memory cap while
-// the sweep's bitmaps do.  With a limit the key-list path runs first: it is faster while the
-// states it stores fit, and grows its buffers as the layers come.
+bool block_fits(const cg_growth* h) {
+    const uint64_t mem = h->mem_cap ? h->mem_cap : kDefaultMemCap;
+    return h->start_is_perm && h->width == 4 && h->n >= cg::kBlockMinN && h->n <= cg::kBlockMaxN && h->k > 0 &&
+           block_layout(h->n, h->k).bytes + (1 << 20) <= mem;
+}
+
+// AUTO takes the sweep for the whole growth (no radius or layer-size limit) of a dense subgroup of
+// S_n in two cases.  (1) Its block form fits the memory cap and the group fills most of its blocks
+// (index at most 4): one expansion serves all states of a block in the layer.  Whole growths, the
+// key-list path against it: S_12 under LRX 10.4 / 5.7 ms, star 29 / 4.0, adjacent transpositions
+// 28 / 5.9, all transpositions 169 / 16.5, S_13 pancake 688 / 52; in smaller groups a round's fixed
+// cost (12 us) counts and the line is the generators' number: S_11 LRX 1.00 / 1.28 ms (k = 3),
+// adjacent transpositions 2.59 / 1.51 (k = 10), S_10 adjacent transpositions 0.53 / 0.59 (k = 9),
+// pancake 0.30 / 0.19 (k = 9), all transpositions 1.01 / 0.31 (k = 45).  (2) The states, stored as
+// keys beside a rank bitmap, would not fit the memory cap while the sweep's bitmaps do.
+// With a limit the key-list path runs first: most limits stop a growth while its layers are sparse,
+// one state to a block.
 bool sweep_preferred(const cg_growth* h) {
     const uint64_t mem = h->mem_cap ? h->mem_cap : kDefaultMemCap;
     if (!h->start_is_perm || h->n > 14 || h->n < 2) return false;
     if (h->max_radius >= 0 || h->stop_above > 0) return false;
+    const int min_k = h->n >= 12 ? 1 : h->n == 11 ? 6 : 10;
+    if (block_fits(h) && h->order * 4 >= factorial(h->n) && h->k >= min_k) return true;
     if (h->order * 512 < factorial(h->n)) return false;
     if (sweep_bytes(h->n) > mem) return false;
     return h->states_bound * 8 + bitmap_words(h->n) * 4 > mem;
+}
+
+int run_block(cg_growth* h, cudaStream_t st, int* final_status) {
+    int rc = ensure_small_buffers(h, st);
+    if (rc) return rc;
+    const BlockLayout L = block_layout(h->n, h->k);
+    const int n = h->n;
+    cudaError_t e = cudaSuccess;
+    BlockDev D;
+    std::memset(&D, 0, sizeof(D));
+    const bool fresh_alloc = h->d_blk == nullptr;
+    if (fresh_alloc) {
+        h->d_blk = (char*)dev_alloc(L.bytes, st);
+        h->d_block = (BlockDev*)dev_alloc(sizeof(BlockDev), st);
+        if (!h->d_blk || !h->d_block) return CG_ENOMEM;
+    }
+    D.V = h->d_blk;
+    for (int i = 0; i < 3; ++i) {
+        D.N[i] = h->d_blk + (uint64_t)(i + 1) * L.words;
+        D.flag[i] = reinterpret_cast<unsigned char*>(h->d_blk + L.o_flags + (uint64_t)i * L.flags);
+    }
+    D.top = reinterpret_cast<uint2*>(h->d_blk + L.o_top);
+    D.bottom = reinterpret_cast<unsigned*>(h->d_blk + L.o_bottom);
+    D.maps = reinterpret_cast<const uint4*>(h->d_blk + L.o_maps);
+    D.layer_sizes = h->d_layers;
+    D.stop_above = h->stop_above;
+    D.nblocks = (unsigned)L.nblocks;
+    D.ngroups = (unsigned)L.ngroups;
+    D.ntop = (unsigned)L.ntop;
+    D.k = h->k;
+    D.n = n;
+    D.layers_cap = cg::kMaxLayers;
+    D.max_radius = h->max_radius;
+    for (int i = 0; i < n; ++i) {
+        const uint64_t v = h->use_start ? (h->start_key >> (4 * i)) & 15u : (uint64_t)i;
+        D.start |= v << (4 * i);
+    }
+    if (fresh_alloc) {                   // tables and generators stay with the handle
+        std::vector<uint8_t> maps((size_t)h->k * 16, 0);
+        for (int j = 0; j < h->k; ++j)
+            for (int i = 0; i < n; ++i) maps[(size_t)j * 16 + h->rows[j][i]] = (uint8_t)i;
+        if ((e = cudaMemcpyAsync(h->d_blk + L.o_maps, maps.data(), maps.size(), cudaMemcpyHostToDevice, st)) != cudaSuccess)
+            return cuda_rc(e);
+        if ((e = cg::launch_block_tables(D, st)) != cudaSuccess) return cuda_rc(e);
+        h->stats.launches += 1;
+        h->stats.h2d_bytes += maps.size();
+    }
+    if ((e = cudaMemsetAsync(h->d_blk, 0, L.o_top, st)) != cudaSuccess) return cuda_rc(e);
+    if ((e = cudaMemcpyAsync(h->d_block, &D, sizeof(D), cudaMemcpyHostToDevice, st)) != cudaSuccess) return cuda_rc(e);
+    if ((e = cudaMemsetAsync(h->d_ctl, 0, sizeof(Ctl), st)) != cudaSuccess) return cuda_rc(e);
+    if ((e = cg::launch_block_init(h->d_block, n, st)) != cudaSuccess) return cuda_rc(e);
+    h->stats.h2d_bytes += sizeof(D);
+    int grid = cg::block_max_grid(h->device, n);
+    if (grid <= 0) return CG_ECUDA;
+    if (h->grid_override > 0) grid = std::min(grid, h->grid_override);
+    if (!h->ev0) {
+        if ((e = cudaEventCreate(&h->ev0)) != cudaSuccess) return cuda_rc(e);
+        if ((e = cudaEventCreate(&h->ev1)) != cudaSuccess) return cuda_rc(e);
+    }
+    if ((e = cudaEventRecord(h->ev0, st)) != cudaSuccess) return cuda_rc(e);
+    if ((e = cg::launch_block_grow(h->d_block, h->d_ctl, n, grid, cg::kMaxLayers + 1, kSweepTimeoutNs, st)) != cudaSuccess)
+        return cuda_rc(e);
+    if ((e = cudaEventRecord(h->ev1, st)) != cudaSuccess) return cuda_rc(e);
+    h->stats.launches += 2;
+    Ctl ctl;
+    if ((e = cudaMemcpyAsync(&D, h->d_block, sizeof(D), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return cuda_rc(e);
+    if ((e = cudaMemcpyAsync(&ctl, h->d_ctl, sizeof(ctl), cudaMemcpyDeviceToHost, st)) != cudaSuccess)
+        return cuda_rc(e);
+    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_rc(e);
+    h->stats.d2h_bytes += sizeof(D) + sizeof(ctl);
+    h->stats.kernel_ms += elapsed_ms(h->ev0, h->ev1);
+    h->stats.rounds += ctl.rounds;
+    if (ctl.err) return ctl.err;
+    h->stats.state_capacity = factorial(n);
+    h->stats.table_slots = L.words / 8;
+    h->stats.strategy_used = CG_STRATEGY_SWEEP;
+    h->stats.probe_variant = 1;
+    h->host_block = D;
+    std::memset(&h->host_job, 0, sizeof(h->host_job));
+    h->host_job.radius = D.radius;
+    h->host_job.status = D.status;
+    *final_status = D.status;
+    return CG_OK;
 }
 
 int run_sweep(cg_growth* h, cudaStream_t st, int* final_status) {
@@ -909,6 +1038,8 @@ int run_sweep(cg_growth* h, cudaStream_t st, int* final_status) {
     if (!h->start_is_perm || h->n > 14 || h->n < 1) return CG_EINVAL;
     const uint64_t bytes = sweep_bytes(h->n);
     if (bytes > mem) return CG_EINVAL;
+    h->last_is_block = h->sweep_order == cg::kSweepOrderAuto && block_fits(h);
+    if (h->last_is_block) return run_block(h, st, final_status);
     int rc = ensure_small_buffers(h, st);
     if (rc) return rc;
     const uint64_t nb = sweep_blocks(h->n);
@@ -1570,6 +1701,30 @@ int cg_growth_last_layer(cg_growth_t h, uint64_t* keys_out, uint64_t cap, uint64
         if (e == cudaSuccess && D.tagged)
             for (uint64_t i = 0; i < cnt; ++i) keys_out[2 * i + 1] &= (1ull << 60) - 1;
         return cuda_rc(e);
+    }
+    if (h->last_is_sweep && h->last_is_block) {
+        const BlockDev& D = h->host_block;
+        uint64_t cnt = 0;
+        cudaError_t e = cudaMemcpy(&cnt, h->d_layers + D.radius, 8, cudaMemcpyDeviceToHost);
+        if (e != cudaSuccess) return cuda_rc(e);
+        *count_out = cnt;
+        if (cap < cnt || (!keys_out && cnt > 0)) return CG_EINVAL;
+        if (cnt == 0) return CG_OK;
+        uint64_t* d_out = (uint64_t*)dev_alloc(cnt * 8 + 64, nullptr);
+        if (!d_out) return CG_ENOMEM;
+        unsigned long long* d_count = (unsigned long long*)(d_out + cnt);
+        int sms = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+        e = cudaMemsetAsync(d_count, 0, 8, nullptr);
+        if (e == cudaSuccess)
+            e = cg::launch_block_export(D, D.radius % 3, d_out, cnt, d_count, std::max(sms, 1) * 16, nullptr);
+        unsigned long long got = 0;
+        if (e == cudaSuccess) e = cudaMemcpy(&got, d_count, 8, cudaMemcpyDeviceToHost);
+        if (e == cudaSuccess) e = cudaMemcpy(keys_out, d_out, cnt * 8, cudaMemcpyDeviceToHost);
+        dev_free(d_out, nullptr);
+        cudaStreamSynchronize(nullptr);
+        if (e != cudaSuccess) return cuda_rc(e);
+        return got == cnt ? CG_OK : CG_EDEVICE;
     }
     if (h->last_is_sweep) {
         // unrank the last layer's bitmap (layer R lives in F[R & 1], its blocks in L[R & 1])

@@ -1,0 +1,84 @@
+"""GPU tests of the sweep strategy in blocks of states (n = 10..14): layers and last layer against
+the key-list strategies and closed forms, from the identity and from other states, with limits, with
+more generators than shared memory holds and for subgroups that fill half of every block.  Whole
+numbers: every comparison is exact."""
+
+import math
+
+import numpy as np
+import pytest
+
+import workloads as w
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def cg():
+    import torch
+    assert torch.cuda.is_available()
+    import paper_2509_19162_gb300 as p
+    p.build()
+    return p
+
+
+def gens_of(kind, n, seed):
+    rng = np.random.default_rng(seed)
+    if kind == "random":
+        return w.random_perms(rng, n, 2)
+    if kind == "random_inv":
+        return w.inverse_closure(w.random_perms(rng, n, 2))
+    if kind == "even":                  # three-cycles: A_n, half of every block's bits
+        return w.cycles_01i_inv(n)
+    return w.FAMILIES[kind](n)
+
+
+@pytest.mark.parametrize("n", [10, 11])
+@pytest.mark.parametrize("kind", ["lrx", "lx", "pancake", "random", "random_inv", "even", "star"])
+def test_whole_growth_and_antipodes(cg, n, kind):
+    gens = gens_of(kind, n, 40 + n)
+    start = np.random.default_rng(n).permutation(n).tolist()
+    with cg.Growth(n, gens, strategy="hash", start=start) as g:
+        want, far = g.run(), np.sort(g.last_layer())
+    for s in ("sweep", "auto"):
+        with cg.Growth(n, gens, strategy=s, start=start) as g:
+            for _ in range(2):          # a handle is run again
+                got = g.run()
+                assert (got.status, got.layers) == (want.status, want.layers)
+                assert np.array_equal(np.sort(g.last_layer()), far)
+
+
+@pytest.mark.parametrize("n,radius", [(12, 8), (13, 7), (14, 6)])
+@pytest.mark.parametrize("kind", ["pancake", "random", "random_inv"])
+def test_limited_growth_and_last_layer(cg, n, radius, kind):
+    gens = gens_of(kind, n, 60 + n)
+    with cg.Growth(n, gens, strategy="hash", max_radius=radius) as g:
+        want, far = g.run(), np.sort(g.last_layer())
+    with cg.Growth(n, gens, strategy="sweep", max_radius=radius) as g:
+        got = g.run()
+        assert (got.status, got.layers) == (want.status, want.layers)
+        assert np.array_equal(np.sort(g.last_layer()), far)
+    stop = want.layers[-2]
+    r = cg.growth(n, gens, strategy="sweep", stop_above=stop - 1)
+    assert r.status == 3 and r.layers == want.layers[:len(r.layers)] and r.layers[-1] >= stop
+
+
+def test_mahonian_and_memory(cg):
+    row = [1]
+    for j in range(2, 13):              # inversions of S_12
+        new = [0] * (len(row) + j - 1)
+        for i, x in enumerate(row):
+            for t in range(j):
+                new[i + t] += x
+        row = new
+    assert cg.growth(12, w.coxeter(12)).layers == row
+    # 1/4 GiB holds the three-bit sweep but not the blocks' four bits; the layers are the same
+    assert cg.growth(12, w.coxeter(12), mem_cap=1 << 28).layers == row
+    assert cg.growth(12, w.coxeter(12), strategy="sweep", mem_cap=1 << 28).layers == row
+
+
+def test_more_generators_than_shared_memory_holds(cg):
+    gens = w.three_cycles(10)           # 240
+    got = cg.growth(10, gens, strategy="sweep")
+    assert got.layers == cg.growth(10, gens, strategy="hash").layers
+    assert sum(got.layers) == math.factorial(10) // 2
