@@ -270,8 +270,49 @@ __global__ void block_init_kernel(BlockDev* Dp) {
     D.flag[0][idx >> 5] = 1;
     D.layer_sizes[0] = 1;
     D.fresh = 0;
+    D.states = 1;
     D.radius = 0;
     D.status = D.max_radius == 0 ? kTruncRadius : kRunning;
+}
+
+// The stored states of a key-list growth: keys[0, hi), of which keys[lo, hi) are layer D.radius, set in
+// the (cleared) visited words and that layer's words.  A stored key s = s0 w gives w^-1: the place i
+// of s0's value v in s is the place of v in w.
+template <int N>
+__global__ void block_import_kernel(BlockDev* Dp, const uint64_t* __restrict__ keys, unsigned long long lo,
+                                    unsigned long long hi, int* err) {
+    using Word = typename BlockShape<N>::Word;
+    const BlockDev& D = *Dp;
+    const int which = D.radius % 3;
+    Word* V = static_cast<Word*>(D.V);
+    Word* F = static_cast<Word*>(D.N[which]);
+    unsigned char* flag = D.flag[which];
+    uint64_t place = 0;                                // nibble x: the v with s0[v] = x
+    for (int v = 0; v < N; ++v) place |= (uint64_t)v << (4 * ((D.start >> (4 * v)) & 15u));
+    const unsigned long long step = (unsigned long long)gridDim.x * blockDim.x;
+    for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < hi; i += step) {
+        const uint64_t s = __ldcg(keys + i);
+        uint64_t inv = 0;                              // nibble v: position of v in w
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            const unsigned v = (unsigned)(place >> (4 * ((unsigned)(s >> (4 * j)) & 15u))) & 15u;
+            inv |= (uint64_t)j << (4 * v);
+        }
+        uint32_t q[BlockShape<N>::kWords] = {};
+#pragma unroll
+        for (int v = 0; v < N; ++v) q[v >> 2] |= (uint32_t)((inv >> (4 * v)) & 15u) << (8 * (v & 3));
+        unsigned m;
+        const unsigned idx = block_rank<N>(q, m);
+        if (idx >= D.nblocks) {                        // not a permutation: never expected
+            atomicExch(err, CG_EDEVICE);
+            continue;
+        }
+        atomicOr(V + idx, (Word)1 << m);
+        if (i >= lo) {
+            atomicOr(F + idx, (Word)1 << m);
+            flag[idx >> 5] = 1;
+        }
+    }
 }
 
 // ---- the persistent kernel ---------------------------------------------------------------------------
@@ -281,8 +322,11 @@ __device__ void block_close(BlockDev& D, Ctl* ctl) {
     const unsigned long long fresh = ld_relaxed_ull(&D.fresh);
     if (fresh == 0) {
         W.status = kDone;
+    } else if (D.max_states > 0 && W.states + fresh > D.max_states) {
+        W.status = kNeedMem;                // the layer is past the states the job may keep
     } else {
         const int r1 = W.radius + 1;
+        W.states = W.states + fresh;
         D.layer_sizes[r1] = fresh;
         W.radius = r1;
         if (D.max_radius >= 0 && r1 >= D.max_radius) W.status = kTruncRadius;
@@ -527,6 +571,19 @@ cudaError_t launch_block_init(BlockDev* d, int n, cudaStream_t st) {
         case 12: block_init_kernel<12><<<1, 32, 0, st>>>(d); break;
         case 13: block_init_kernel<13><<<1, 32, 0, st>>>(d); break;
         default: block_init_kernel<14><<<1, 32, 0, st>>>(d); break;
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_block_import(BlockDev* d, int n, const uint64_t* keys, unsigned long long lo,
+                                unsigned long long hi, int* d_err, int grid, cudaStream_t st) {
+    (void)cudaGetLastError();   // clear a stale error: the check after the launch is about this one
+    switch (n) {
+        case 10: block_import_kernel<10><<<grid, 256, 0, st>>>(d, keys, lo, hi, d_err); break;
+        case 11: block_import_kernel<11><<<grid, 256, 0, st>>>(d, keys, lo, hi, d_err); break;
+        case 12: block_import_kernel<12><<<grid, 256, 0, st>>>(d, keys, lo, hi, d_err); break;
+        case 13: block_import_kernel<13><<<grid, 256, 0, st>>>(d, keys, lo, hi, d_err); break;
+        default: block_import_kernel<14><<<grid, 256, 0, st>>>(d, keys, lo, hi, d_err); break;
     }
     return cudaGetLastError();
 }

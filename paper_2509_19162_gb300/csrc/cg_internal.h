@@ -236,12 +236,14 @@ struct alignas(128) BlockDev {
     uint64_t* layer_sizes;     // layers_cap entries; [0] = 1
     uint64_t stop_above;       // 0: none
     uint64_t start;            // the start state's packed key
+    uint64_t max_states;       // > 0: a layer that takes the states past this ends the growth (kNeedMem)
     unsigned nblocks, ngroups, ntop;
     int k, n;
     int layers_cap;
     int max_radius;            // < 0: unlimited
     // dynamic, updated during a run
     alignas(128) unsigned long long fresh;  // states found in the round
+    unsigned long long states;              // states of the layers so far
     int radius;                // radius of the frontier layer
     int status;                // JobStatus
 };

@@ -70,6 +70,9 @@ cudaError_t launch_sweep_grow(SweepDev* d, Ctl* ctl, int grid, int max_rounds, u
 int block_max_grid(int device, int n);
 cudaError_t launch_block_tables(const BlockDev& host, cudaStream_t st);
 cudaError_t launch_block_init(BlockDev* d, int n, cudaStream_t st);
+// Take over a key-list growth at layer d->radius: its states keys[0, hi), that layer keys[lo, hi).
+cudaError_t launch_block_import(BlockDev* d, int n, const uint64_t* keys, unsigned long long lo,
+                                unsigned long long hi, int* d_err, int grid, cudaStream_t st);
 cudaError_t launch_block_grow(BlockDev* d, Ctl* ctl, int n, int grid, int max_rounds, uint64_t timeout_ns,
                               cudaStream_t st);
 // Packed keys of the layer in N[which] into out[0, cap); *count (zeroed by the caller) receives their

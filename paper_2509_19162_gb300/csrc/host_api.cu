@@ -464,6 +464,7 @@ struct cg_growth {
     char* d_blk = nullptr;                       // one allocation (BlockLayout)
     BlockDev host_block{};
     bool last_is_block = false;
+    bool served = false;                         // grown for a server: the share bounds its states
 
     JobDev host_job{};
     bool have_last = false;
@@ -486,10 +487,7 @@ struct cg_growth {
         d_sweep = nullptr;
         d_sw = nullptr;
         sw_bytes = 0;
-        dev_free(d_block, st);
-        dev_free(d_blk, st);
-        d_block = nullptr;
-        d_blk = nullptr;
+        release_block(st);
         dev_free(d_wgens, st);
         dev_free(d_wjob, st);
         dev_free(d_wkeys, st);
@@ -500,6 +498,13 @@ struct cg_growth {
         have_last = false;                 // the last layer lived in the freed buffers
         last_layer_ptr = nullptr;
         last_layer_n = 0;
+    }
+
+    void release_block(cudaStream_t st) {
+        dev_free(d_block, st);
+        dev_free(d_blk, st);
+        d_block = nullptr;
+        d_blk = nullptr;
     }
 
     void release_sort(cudaStream_t st) {
@@ -589,6 +594,130 @@ void fill_static(cg_growth* h, JobDev& J) {
     J.test = h->k - J.closed >= cg::kTestMinDegree ? 1 : 0;
 }
 
+bool block_fits(const cg_growth* h) {
+    const uint64_t mem = h->mem_cap ? h->mem_cap : kDefaultMemCap;
+    return h->start_is_perm && h->width == 4 && h->n >= cg::kBlockMinN && h->n <= cg::kBlockMaxN && h->k > 0 &&
+           block_layout(h->n, h->k).bytes + (1 << 20) <= mem;
+}
+
+// The sweep in blocks of states, from the start state or, with `from`, on from a key-list growth's
+// last layer (its states are in d_keys; `from` is the host's copy of its descriptor).  max_states > 0:
+// a layer that takes the states past it ends the growth as one that does not fit (kNeedMem).
+int run_block(cg_growth* h, cudaStream_t st, int* final_status, const JobDev* from = nullptr,
+              uint64_t max_states = 0) {
+    int rc = ensure_small_buffers(h, st);
+    if (rc) return rc;
+    const BlockLayout L = block_layout(h->n, h->k);
+    const int n = h->n;
+    cudaError_t e = cudaSuccess;
+    BlockDev D;
+    std::memset(&D, 0, sizeof(D));
+    const bool fresh_alloc = h->d_blk == nullptr;
+    if (fresh_alloc) {
+        h->d_blk = (char*)dev_alloc(L.bytes, st);
+        h->d_block = (BlockDev*)dev_alloc(sizeof(BlockDev), st);
+        if (!h->d_blk || !h->d_block) return CG_ENOMEM;
+    }
+    D.V = h->d_blk;
+    for (int i = 0; i < 3; ++i) {
+        D.N[i] = h->d_blk + (uint64_t)(i + 1) * L.words;
+        D.flag[i] = reinterpret_cast<unsigned char*>(h->d_blk + L.o_flags + (uint64_t)i * L.flags);
+    }
+    D.top = reinterpret_cast<uint2*>(h->d_blk + L.o_top);
+    D.bottom = reinterpret_cast<unsigned*>(h->d_blk + L.o_bottom);
+    D.maps = reinterpret_cast<const uint4*>(h->d_blk + L.o_maps);
+    D.layer_sizes = h->d_layers;
+    D.stop_above = h->stop_above;
+    D.nblocks = (unsigned)L.nblocks;
+    D.ngroups = (unsigned)L.ngroups;
+    D.ntop = (unsigned)L.ntop;
+    D.k = h->k;
+    D.n = n;
+    D.layers_cap = cg::kMaxLayers;
+    D.max_radius = h->max_radius;
+    D.max_states = max_states;
+    for (int i = 0; i < n; ++i) {
+        const uint64_t v = h->use_start ? (h->start_key >> (4 * i)) & 15u : (uint64_t)i;
+        D.start |= v << (4 * i);
+    }
+    if (fresh_alloc) {                   // tables and generators stay with the handle
+        std::vector<uint8_t> maps((size_t)h->k * 16, 0);
+        for (int j = 0; j < h->k; ++j)
+            for (int i = 0; i < n; ++i) maps[(size_t)j * 16 + h->rows[j][i]] = (uint8_t)i;
+        if ((e = cudaMemcpyAsync(h->d_blk + L.o_maps, maps.data(), maps.size(), cudaMemcpyHostToDevice, st)) != cudaSuccess)
+            return cuda_rc(e);
+        if ((e = cg::launch_block_tables(D, st)) != cudaSuccess) return cuda_rc(e);
+        h->stats.launches += 1;
+        h->stats.h2d_bytes += maps.size();
+    }
+    if ((e = cudaMemsetAsync(h->d_blk, 0, L.o_top, st)) != cudaSuccess) return cuda_rc(e);
+    if (from) {
+        D.radius = from->radius;
+        D.states = from->hi;
+        D.status = cg::kRunning;
+    }
+    if ((e = cudaMemcpyAsync(h->d_block, &D, sizeof(D), cudaMemcpyHostToDevice, st)) != cudaSuccess) return cuda_rc(e);
+    if ((e = cudaMemsetAsync(h->d_ctl, 0, sizeof(Ctl), st)) != cudaSuccess) return cuda_rc(e);
+    if (!from) e = cg::launch_block_init(h->d_block, n, st);
+    else e = cg::launch_block_import(h->d_block, n, h->d_keys, from->lo, from->hi, &h->d_ctl->err, 152 * 8, st);
+    if (e != cudaSuccess) return cuda_rc(e);
+    h->stats.h2d_bytes += sizeof(D);
+    int grid = cg::block_max_grid(h->device, n);
+    if (grid <= 0) return CG_ECUDA;
+    if (h->grid_override > 0) grid = std::min(grid, h->grid_override);
+    if (!h->ev0) {
+        if ((e = cudaEventCreate(&h->ev0)) != cudaSuccess) return cuda_rc(e);
+        if ((e = cudaEventCreate(&h->ev1)) != cudaSuccess) return cuda_rc(e);
+    }
+    if ((e = cudaEventRecord(h->ev0, st)) != cudaSuccess) return cuda_rc(e);
+    if ((e = cg::launch_block_grow(h->d_block, h->d_ctl, n, grid, cg::kMaxLayers + 1, kSweepTimeoutNs, st)) != cudaSuccess)
+        return cuda_rc(e);
+    if ((e = cudaEventRecord(h->ev1, st)) != cudaSuccess) return cuda_rc(e);
+    h->stats.launches += 2;
+    Ctl ctl;
+    if ((e = cudaMemcpyAsync(&D, h->d_block, sizeof(D), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return cuda_rc(e);
+    if ((e = cudaMemcpyAsync(&ctl, h->d_ctl, sizeof(ctl), cudaMemcpyDeviceToHost, st)) != cudaSuccess)
+        return cuda_rc(e);
+    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_rc(e);
+    h->stats.d2h_bytes += sizeof(D) + sizeof(ctl);
+    h->stats.kernel_ms += elapsed_ms(h->ev0, h->ev1);
+    h->stats.rounds += ctl.rounds;
+    if (ctl.err) return ctl.err;
+    h->stats.state_capacity = factorial(n);
+    h->stats.table_slots = L.words / 8;
+    h->stats.strategy_used = CG_STRATEGY_SWEEP;
+    h->stats.probe_variant = 1;
+    h->host_block = D;
+    std::memset(&h->host_job, 0, sizeof(h->host_job));
+    h->host_job.radius = D.radius;
+    h->host_job.status = D.status;
+    *final_status = D.status;
+    return CG_OK;
+}
+
+// A key-list growth with a radius limit goes on in blocks of states when its layers get dense enough:
+// whether the frontier's size F (layer r, after a layer of Fprev) says that the last layer will hold
+// a state per block of 64.  Checked when a layer reaches 1/4096 of the group, early enough for the
+// stored states to be few, and two million states, when the rounds to come are worth the 0.05 ms of
+// looking.  Kernels, list against blocks: S_13 pancake to radius 12 290 / 31 ms, S_12 adjacent
+// transpositions to radius 20 1.09 / 0.49 ms, S_12 LRX to radius 40 3.21 / 2.21 ms (dense); to radius
+// 30 0.43 / 0.58 ms, S_14 under six random generators to radius 12 18.6 / 38.6 ms (sparse).
+uint64_t block_check(const cg_growth* h) { return std::max<uint64_t>(h->order / 4096, 1ull << 21); }
+bool blocks_will_fill(const cg_growth* h, uint64_t F, uint64_t Fprev, int r) {
+    if (Fprev == 0 || h->max_radius < 0) return false;
+    const double full = (double)h->order, ratio = (double)F / (double)Fprev;
+    double layer = (double)F;
+    for (int q = r; q < h->max_radius && layer * 64.0 < full && ratio > 1.0; ++q) layer *= ratio;
+    return layer * 64.0 >= full;
+}
+
+// Groups the block form takes: at least index 4 in S_n, and, in the smaller ones, generators enough
+// for a round to be worth its fixed cost (sweep_preferred).
+bool block_group(const cg_growth* h) {
+    const int min_k = h->n >= 12 ? 1 : h->n == 11 ? 6 : 10;
+    return block_fits(h) && h->order * 4 >= factorial(h->n) && h->k >= min_k;
+}
+
 // Before a round on a frontier of J (host copy, current): room for the next layer as the last two
 // predict it -- F * (F / Fprev) and a quarter more, at most every candidate, never past the states
 // there can be.  A layer that comes out larger still ends the round early (kNeedMem) and is redone in
@@ -631,19 +760,28 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
                       ? cg::kVisitBitmap : cg::kVisitHash;
     }
     const bool bitmap = h->mode == cg::kVisitBitmap;
+    h->last_is_block = false;
     const int ilp = (h->ilp_override > 0 ? h->ilp_override : default_ilp(h->k, bitmap)) + (bitmap ? 16 : 0);
     const uint64_t avail = mem > (1 << 20) ? mem - (1 << 20) : mem;
     const uint64_t bm_bytes = bitmap ? bitmap_words(h->n) * 4 : 0;
     const uint64_t max_cap = std::min<uint64_t>(
         h->states_bound, bitmap ? (avail > bm_bytes ? (avail - bm_bytes) / 8 : 0) : max_cap_for_mem(avail));
     if (max_cap < 1) return CG_ENOMEM;
+    // radius limit: a growth that may go on in blocks of states (blocks_will_fill) begins with room
+    // for its sparse layers, beside which the blocks have to fit
+    const uint64_t first_cap = std::min<uint64_t>(max_cap, std::max<uint64_t>(h->order / 64, 1ull << 24));
+    bool may_block = bitmap && h->max_radius > 0 && (h->strategy == CG_STRATEGY_AUTO || h->served) &&
+                     (h->stop_above == 0 || h->stop_above >= std::max(h->order / 64, block_check(h))) &&
+                     block_group(h) &&
+                     block_layout(h->n, h->k).bytes + bm_bytes + first_cap * 8 + (1 << 20) <= mem;
+    uint64_t list_cap = h->states_bound;
+    {
+        const uint64_t need = bitmap ? list_cap * 8 + bm_bytes : bytes_for(list_cap);
+        if (need > std::min<uint64_t>(mem, kExactAllocLimit)) list_cap = std::min<uint64_t>(max_cap, 1ull << 24);
+        list_cap = std::max<uint64_t>(std::min(list_cap, max_cap), 1);
+    }
     if (!h->d_keys) {
-        uint64_t start = h->states_bound;
-        const uint64_t need = bitmap ? start * 8 + bm_bytes : bytes_for(start);
-        if (need > std::min<uint64_t>(mem, kExactAllocLimit))
-            start = std::min<uint64_t>(max_cap, 1ull << 24);
-        start = std::min(start, max_cap);
-        rc = resize_state(h, std::max<uint64_t>(start, 1), 0, st);
+        rc = resize_state(h, may_block ? std::min<uint64_t>(first_cap, 1ull << 28) : list_cap, 0, st);
         if (rc) return rc;
     }
     const int grid_max = grow_grid(h->device, ilp);
@@ -658,6 +796,8 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
     JobDev J;
     std::memset(&J, 0, sizeof(J));
     fill_static(h, J);
+    const uint64_t check = block_check(h);
+    if (may_block) J.stop_above = check;        // (not above the caller's)
     if ((e = cudaMemcpyAsync(h->d_job, &J, sizeof(J), cudaMemcpyHostToDevice, st)) != cudaSuccess)
         return cuda_rc(e);
     if ((e = cudaMemsetAsync(h->d_ctl, 0, sizeof(Ctl), st)) != cudaSuccess) return cuda_rc(e);
@@ -731,6 +871,47 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
         h->stats.rounds += ctl.rounds;
         if (ctl.err) return ctl.err;
         if (sort_err) return sort_err;
+        if (may_block && J.status == cg::kTruncAbove) {
+            // the first layer past the check: go on in blocks, or on the list without further checks
+            const uint64_t F = J.hi - J.lo;
+            uint64_t last[2] = {0, 0};
+            if (J.radius > 0) {
+                if ((e = cudaMemcpyAsync(last, h->d_layers + J.radius - 1, sizeof(last), cudaMemcpyDeviceToHost, st)) !=
+                    cudaSuccess)
+                    return cuda_rc(e);
+                if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_rc(e);
+                h->stats.d2h_bytes += sizeof(last);
+            }
+            may_block = false;
+            const bool over = h->stop_above > 0 && F > h->stop_above;
+            if (!over && blocks_will_fill(h, F, last[0], J.radius) &&
+                block_layout(h->n, h->k).bytes + bm_bytes + h->keys_cap * 8 + (1 << 20) <= mem) {
+                h->last_is_block = true;
+                rc = run_block(h, st, final_status, &J, h->served ? max_cap : 0);
+                if (rc != CG_ENOMEM) return rc;
+                h->last_is_block = false;       // no room on the device: stay on the list
+                h->release_block(st);
+            }
+            if (!over) {
+                if (h->keys_cap < list_cap) {   // room for the whole list, as without the check
+                    rc = resize_state(h, list_cap, J.hi, st);
+                    if (rc && rc != CG_ENOMEM) return rc;
+                    J.keys = h->d_keys;
+                    J.keys_cap = h->keys_cap;
+                }
+                J.stop_above = h->stop_above;
+                J.status = cg::kRunning;
+                if ((e = cudaMemcpyAsync(h->d_job, &J, sizeof(J), cudaMemcpyHostToDevice, st)) != cudaSuccess)
+                    return cuda_rc(e);
+                h->stats.h2d_bytes += sizeof(J);
+                if (!by_round) {
+                    if ((e = cg::launch_resume_units(h->d_job, 1, h->d_ubeg, h->d_ctl, st)) != cudaSuccess)
+                        return cuda_rc(e);
+                    h->stats.launches += 1;
+                    continue;
+                }
+            }
+        }
         if (by_round && J.status == cg::kRunning) {
             Fprev = expanded;
             // as the kernel decides between its own rounds (bitmap_test_first)
@@ -757,6 +938,7 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
         if (e != cudaSuccess) return cuda_rc(e);
         fill_static(h, J);
         J.test = test;                      // the layer is redone as it was begun
+        if (may_block) J.stop_above = check;
         J.tail = J.hi;
         J.overflow = 0;
         J.status = cg::kRunning;
@@ -922,12 +1104,6 @@ int run_wide(cg_growth* h, cudaStream_t st, int* final_status) {
 // Bitmaps over S_n for the visited set and two layers (sweep_path.cu: 3 bits per element); one
 // persistent launch runs every layer step.  Needs a start with distinct values and n <= 14.
 
-bool block_fits(const cg_growth* h) {
-    const uint64_t mem = h->mem_cap ? h->mem_cap : kDefaultMemCap;
-    return h->start_is_perm && h->width == 4 && h->n >= cg::kBlockMinN && h->n <= cg::kBlockMaxN && h->k > 0 &&
-           block_layout(h->n, h->k).bytes + (1 << 20) <= mem;
-}
-
 // AUTO takes the sweep for the whole growth (no radius or layer-size limit) of a dense subgroup of
 // S_n in two cases.  (1) Its block form fits the memory cap and the group fills most of its blocks
 // (index at most 4): one expansion serves all states of a block in the layer.  Whole growths, the
@@ -937,100 +1113,17 @@ bool block_fits(const cg_growth* h) {
 // adjacent transpositions 2.59 / 1.51 (k = 10), S_10 adjacent transpositions 0.53 / 0.59 (k = 9),
 // pancake 0.30 / 0.19 (k = 9), all transpositions 1.01 / 0.31 (k = 45).  (2) The states, stored as
 // keys beside a rank bitmap, would not fit the memory cap while the sweep's bitmaps do.
-// With a limit the key-list path runs first: most limits stop a growth while its layers are sparse,
-// one state to a block.
+// A layer-size limit of at least a state per block does not change (1): S_14 pancake to the first layer
+// above 2^31 142 / 58 ms.  With a lower one, or a radius limit, the key-list path runs first: most such
+// growths stop while their layers are sparse (and see blocks_will_fill).
 bool sweep_preferred(const cg_growth* h) {
     const uint64_t mem = h->mem_cap ? h->mem_cap : kDefaultMemCap;
     if (!h->start_is_perm || h->n > 14 || h->n < 2) return false;
+    if (h->max_radius < 0 && (h->stop_above == 0 || h->stop_above >= h->order / 64) && block_group(h)) return true;
     if (h->max_radius >= 0 || h->stop_above > 0) return false;
-    const int min_k = h->n >= 12 ? 1 : h->n == 11 ? 6 : 10;
-    if (block_fits(h) && h->order * 4 >= factorial(h->n) && h->k >= min_k) return true;
     if (h->order * 512 < factorial(h->n)) return false;
     if (sweep_bytes(h->n) > mem) return false;
     return h->states_bound * 8 + bitmap_words(h->n) * 4 > mem;
-}
-
-int run_block(cg_growth* h, cudaStream_t st, int* final_status) {
-    int rc = ensure_small_buffers(h, st);
-    if (rc) return rc;
-    const BlockLayout L = block_layout(h->n, h->k);
-    const int n = h->n;
-    cudaError_t e = cudaSuccess;
-    BlockDev D;
-    std::memset(&D, 0, sizeof(D));
-    const bool fresh_alloc = h->d_blk == nullptr;
-    if (fresh_alloc) {
-        h->d_blk = (char*)dev_alloc(L.bytes, st);
-        h->d_block = (BlockDev*)dev_alloc(sizeof(BlockDev), st);
-        if (!h->d_blk || !h->d_block) return CG_ENOMEM;
-    }
-    D.V = h->d_blk;
-    for (int i = 0; i < 3; ++i) {
-        D.N[i] = h->d_blk + (uint64_t)(i + 1) * L.words;
-        D.flag[i] = reinterpret_cast<unsigned char*>(h->d_blk + L.o_flags + (uint64_t)i * L.flags);
-    }
-    D.top = reinterpret_cast<uint2*>(h->d_blk + L.o_top);
-    D.bottom = reinterpret_cast<unsigned*>(h->d_blk + L.o_bottom);
-    D.maps = reinterpret_cast<const uint4*>(h->d_blk + L.o_maps);
-    D.layer_sizes = h->d_layers;
-    D.stop_above = h->stop_above;
-    D.nblocks = (unsigned)L.nblocks;
-    D.ngroups = (unsigned)L.ngroups;
-    D.ntop = (unsigned)L.ntop;
-    D.k = h->k;
-    D.n = n;
-    D.layers_cap = cg::kMaxLayers;
-    D.max_radius = h->max_radius;
-    for (int i = 0; i < n; ++i) {
-        const uint64_t v = h->use_start ? (h->start_key >> (4 * i)) & 15u : (uint64_t)i;
-        D.start |= v << (4 * i);
-    }
-    if (fresh_alloc) {                   // tables and generators stay with the handle
-        std::vector<uint8_t> maps((size_t)h->k * 16, 0);
-        for (int j = 0; j < h->k; ++j)
-            for (int i = 0; i < n; ++i) maps[(size_t)j * 16 + h->rows[j][i]] = (uint8_t)i;
-        if ((e = cudaMemcpyAsync(h->d_blk + L.o_maps, maps.data(), maps.size(), cudaMemcpyHostToDevice, st)) != cudaSuccess)
-            return cuda_rc(e);
-        if ((e = cg::launch_block_tables(D, st)) != cudaSuccess) return cuda_rc(e);
-        h->stats.launches += 1;
-        h->stats.h2d_bytes += maps.size();
-    }
-    if ((e = cudaMemsetAsync(h->d_blk, 0, L.o_top, st)) != cudaSuccess) return cuda_rc(e);
-    if ((e = cudaMemcpyAsync(h->d_block, &D, sizeof(D), cudaMemcpyHostToDevice, st)) != cudaSuccess) return cuda_rc(e);
-    if ((e = cudaMemsetAsync(h->d_ctl, 0, sizeof(Ctl), st)) != cudaSuccess) return cuda_rc(e);
-    if ((e = cg::launch_block_init(h->d_block, n, st)) != cudaSuccess) return cuda_rc(e);
-    h->stats.h2d_bytes += sizeof(D);
-    int grid = cg::block_max_grid(h->device, n);
-    if (grid <= 0) return CG_ECUDA;
-    if (h->grid_override > 0) grid = std::min(grid, h->grid_override);
-    if (!h->ev0) {
-        if ((e = cudaEventCreate(&h->ev0)) != cudaSuccess) return cuda_rc(e);
-        if ((e = cudaEventCreate(&h->ev1)) != cudaSuccess) return cuda_rc(e);
-    }
-    if ((e = cudaEventRecord(h->ev0, st)) != cudaSuccess) return cuda_rc(e);
-    if ((e = cg::launch_block_grow(h->d_block, h->d_ctl, n, grid, cg::kMaxLayers + 1, kSweepTimeoutNs, st)) != cudaSuccess)
-        return cuda_rc(e);
-    if ((e = cudaEventRecord(h->ev1, st)) != cudaSuccess) return cuda_rc(e);
-    h->stats.launches += 2;
-    Ctl ctl;
-    if ((e = cudaMemcpyAsync(&D, h->d_block, sizeof(D), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return cuda_rc(e);
-    if ((e = cudaMemcpyAsync(&ctl, h->d_ctl, sizeof(ctl), cudaMemcpyDeviceToHost, st)) != cudaSuccess)
-        return cuda_rc(e);
-    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_rc(e);
-    h->stats.d2h_bytes += sizeof(D) + sizeof(ctl);
-    h->stats.kernel_ms += elapsed_ms(h->ev0, h->ev1);
-    h->stats.rounds += ctl.rounds;
-    if (ctl.err) return ctl.err;
-    h->stats.state_capacity = factorial(n);
-    h->stats.table_slots = L.words / 8;
-    h->stats.strategy_used = CG_STRATEGY_SWEEP;
-    h->stats.probe_variant = 1;
-    h->host_block = D;
-    std::memset(&h->host_job, 0, sizeof(h->host_job));
-    h->host_job.radius = D.radius;
-    h->host_job.status = D.status;
-    *final_status = D.status;
-    return CG_OK;
 }
 
 int run_sweep(cg_growth* h, cudaStream_t st, int* final_status) {
@@ -1673,6 +1766,7 @@ int cg_growth_run(cg_growth_t h, void* cuda_stream, uint64_t* layer_sizes_out, i
     }
     const bool sorted = use_sort || h->stats.switched_to_sort;
     h->last_is_sweep = use_sweep;
+    if (use_sort || h->stats.switched_to_sort) h->last_is_block = false;
     const int layers = h->host_job.radius + 1;
     *num_layers_out = layers;
     if (cap < layers) return CG_EINVAL;
@@ -1702,7 +1796,7 @@ int cg_growth_last_layer(cg_growth_t h, uint64_t* keys_out, uint64_t cap, uint64
             for (uint64_t i = 0; i < cnt; ++i) keys_out[2 * i + 1] &= (1ull << 60) - 1;
         return cuda_rc(e);
     }
-    if (h->last_is_sweep && h->last_is_block) {
+    if (h->last_is_block) {
         const BlockDev& D = h->host_block;
         uint64_t cnt = 0;
         cudaError_t e = cudaMemcpy(&cnt, h->d_layers + D.radius, 8, cudaMemcpyDeviceToHost);
@@ -2704,6 +2798,7 @@ int server_run_solo(cg_server* s, cudaStream_t st) {
                               J.mode == cg::kVisitBitmap ? CG_STRATEGY_BITMAP : CG_STRATEGY_HASH);
     std::vector<uint64_t> layers(kSrvLayers);
     int nl = 0;
+    g->served = true;                       // states past the share end the job, however they are kept
     if (rc == CG_OK) rc = cg_growth_run(g, st, layers.data(), kSrvLayers, &nl);
     cg_growth_destroy(g);
     if (rc < 0) return rc;

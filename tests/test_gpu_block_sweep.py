@@ -82,3 +82,46 @@ def test_more_generators_than_shared_memory_holds(cg):
     got = cg.growth(10, gens, strategy="sweep")
     assert got.layers == cg.growth(10, gens, strategy="hash").layers
     assert sum(got.layers) == math.factorial(10) // 2
+
+
+@pytest.mark.parametrize("n,kind,radius", [(11, "pancake", 9), (12, "coxeter", 24), (12, "lrx", 38),
+                                           (12, "random_inv", 16), (12, "random", 27), (13, "pancake", 10)])
+def test_radius_limited_growth_goes_on_in_blocks(cg, n, kind, radius):
+    # the key list hands over to the blocks when the last layer is predicted to be dense
+    gens = gens_of(kind, n, 80 + n)
+    start = np.random.default_rng(n).permutation(n).tolist()
+    with cg.Growth(n, gens, strategy="bitmap", max_radius=radius, start=start) as g:
+        want, far = g.run(), np.sort(g.last_layer())
+    with cg.Growth(n, gens, max_radius=radius, start=start) as g:
+        for _ in range(2):
+            got = g.run()
+            assert g.stats()["strategy_used"] == 4 and g.stats()["launches"] > 3
+            assert (got.status, got.layers) == (want.status, want.layers)
+            assert np.array_equal(np.sort(g.last_layer()), far)
+
+
+@pytest.mark.parametrize("n,kind,radius", [(11, "pancake", 5), (12, "lrx", 29), (13, "random_inv", 15), (12, "star", 6)])
+def test_radius_limited_growth_that_stays_sparse(cg, n, kind, radius):
+    gens = gens_of(kind, n, 80 + n)
+    with cg.Growth(n, gens, strategy="hash", max_radius=radius) as g:
+        want, far = g.run(), np.sort(g.last_layer())
+    with cg.Growth(n, gens, max_radius=radius) as g:
+        got = g.run()
+        assert g.stats()["strategy_used"] == 3
+        assert (got.status, got.layers) == (want.status, want.layers)
+        assert np.array_equal(np.sort(g.last_layer()), far)
+
+
+@pytest.mark.parametrize("kind,radius", [("pancake", 12), ("coxeter", 34), ("coxeter", 64)])
+def test_served_job_over_its_share_keeps_its_layers(cg, kind, radius):
+    # a served job that would store more states than its share holds stops there, in blocks as on the list
+    n, share = 12, 1 << 30
+    gens = w.FAMILIES[kind](n)
+    want = cg.growth(n, gens, strategy="bitmap", max_radius=radius, mem_cap=share)
+    from paper_2509_19162_gb300.serve import Server
+    with Server(job_mem_cap=share) as s:
+        i = s.submit(n, gens, max_radius=radius)
+        while i not in s.finished():
+            s.step()
+        got = s.result(i)
+    assert (got.status, got.layers) == (want.status, want.layers)
