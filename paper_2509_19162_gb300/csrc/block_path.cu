@@ -33,6 +33,7 @@
 //
 // Measured against the state-by-state rank bitmap and sweep kernels it takes the place of: see
 // block_preferred in host_api.cu.
+#include <cooperative_groups.h>
 #include <cstdio>
 #include <type_traits>
 #include <utility>
@@ -47,7 +48,14 @@ namespace {
 constexpr int kBlkThreads = 256;
 constexpr int kBlkWarps = kBlkThreads / 32;
 constexpr int kBlkQueue = 64;          // queued blocks per warp, and claims per warp
+constexpr int kPairBlocks = 8;         // at most this many blocks are expanded a lane per pair
 constexpr unsigned kBottom = 2520;     // arrangements of the pairs 0..3 among eight positions
+
+constexpr unsigned block_count(int n) {
+    unsigned long long f = 1;
+    for (int i = 2; i <= n; ++i) f *= (unsigned long long)i;
+    return (unsigned)(f >> block_pairs(n));
+}
 
 template <int N>
 struct BlockShape {
@@ -473,9 +481,31 @@ block_grow_kernel(BlockDev* Dp, Ctl* ctl, int max_rounds, uint64_t timeout_ns) {
             }
             if (32ull * W + base > 0xffffffffull) break;
         }
-        if (qn > 0) expand(qn);
+        if (qn > kPairBlocks) expand(qn);
         settle();
         pf = 0;
+        // a short remainder, a lane per (block, generator) pair (as in cluster_grow)
+        for (int first = 0; first < qn * k; first += 32) {
+            const int pair = first + lane;
+            const bool live = pair < qn * k;
+            const int b = live ? pair / k : 0, g = live ? pair - b * k : 0;
+            const BlockPerm<N> P = block_unrank<N>(tops, bottoms, live ? qidx[b] : 0u);
+            uint32_t q[BlockShape<N>::kWords];
+            block_map<N>(maps[g], P, q);
+            unsigned m;
+            const unsigned i = block_rank<N>(q, m);
+            if (live && i < nblocks) {
+                const Word f = xor_bits(qf[b], m);
+                const Word neu = f & ~(Word)atomicOr(V + i, f);
+                if (neu) {
+                    fresh += popc_word(neu);
+                    if (atomicOr(X + i, neu) == 0) fnxt[i >> 5] = 1;
+                }
+            } else if (live) {
+                atomicCAS(&ctl->err, 0, CG_EDEVICE);
+            }
+        }
+        qn = 0;
         if (cn > 0) claim(cn);
         found += fresh;
 #pragma unroll
@@ -532,6 +562,345 @@ __global__ void block_export_kernel(BlockDev D, int which, uint64_t* out, unsign
     }
 }
 
+// ---- small groups: a thread-block cluster per growth ---------------------------------------------------
+// Batches of growths of S_n for n <= 10, each in blocks of states by one cluster: a round ends with the
+// cluster's hardware barrier instead of a grid barrier through L2, many growths run side by side
+// without a common round, and a cluster that finishes one takes the next from the queue.  (1024
+// random groups of n in 6..10: 36.2 ms as key lists in one launch with a grid barrier per round,
+// 6.3 ms here.)  All words of a layer are looked at every round (113,400 for n = 10,
+// 454 KB), no flags.  The words live in L2: 38 clusters of eight blocks hold 69 MB of them.
+// Decisions are taken by every thread from the same counts, which the blocks write into each
+// other's shared memory before the barrier.
+namespace cgr = cooperative_groups;
+
+constexpr int kClThreads = 512;
+constexpr int kClMaxCluster = 16;
+
+template <int T>
+struct ClusterShared {
+    static constexpr int kClWarps = T / 32;
+    uint4 map[kClusterGens];
+    unsigned qidx[kClWarps][kBlkQueue];
+    unsigned qf[kClWarps][kBlkQueue];
+    unsigned cidx[kClWarps][kBlkQueue];
+    unsigned cf[kClWarps][kBlkQueue];
+    unsigned acc[2];                       // states the block found, this round and (cleared) the next
+    unsigned cnt[2][kClMaxCluster];        // states each block of the cluster found, by round parity
+    int job;
+};
+
+template <int N>
+__device__ __forceinline__ BlockPerm<N> cluster_unrank(const uint64_t* table, unsigned idx) {
+    const uint64_t p = table[idx];
+    BlockPerm<N> P;
+    lookup_form((uint32_t)p & 0xFFFFu, P.sel[0], P.high[0]);
+    if constexpr (N > 4) lookup_form((uint32_t)p >> 16, P.sel[1], P.high[1]);
+    if constexpr (N > 8) lookup_form((uint32_t)(p >> 32), P.sel[2], P.high[2]);
+    return P;
+}
+
+// The barrier of a growth's blocks.
+template <bool kSm>
+__device__ __forceinline__ void growth_sync(const cgr::cluster_group& cl) {
+    if (kSm) __syncthreads();
+    else cl.sync();
+}
+
+// A word of the growth that its blocks change: from shared memory, or through L2 (this SM's L1 may
+// hold words of the growth before).
+template <bool kSm>
+__device__ __forceinline__ unsigned growth_word(const unsigned* p) {
+    return kSm ? *(const volatile unsigned*)p : __ldcg(p);
+}
+
+// kSm: one block grows the job alone, words and table in its shared memory.  T threads a block.
+template <int N, bool kSm, int T>
+__device__ __forceinline__ void cluster_grow(ClusterShared<T>& S, const ClusterArgs& A, JobDev& J, unsigned* ws,
+                                             const uint64_t* table, const cgr::cluster_group& cl) {
+    constexpr unsigned kBlocks = block_count(N);
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const unsigned size = kSm ? 1u : cl.num_blocks(), rank = kSm ? 0u : cl.block_rank();
+    const int k = J.k;
+    const GenSM* gens = J.gens;
+    const bool smem = k <= kClusterGens;
+    unsigned* V = ws;
+    unsigned* qidx = S.qidx[wid];
+    unsigned* qf = S.qf[wid];
+    unsigned* cidx = S.cidx[wid];
+    unsigned* cf = S.cf[wid];
+    // the words of this growth, empty
+    const unsigned all = size * T, me = rank * T + tid;
+    for (unsigned i = me; i < 4 * kBlocks; i += all) ws[i] = 0;
+    if (smem)
+        for (int j = tid; j < k; j += T) S.map[j] = *reinterpret_cast<const uint4*>(gens[j].map);
+    if (tid < 2) S.acc[tid] = 0;
+    growth_sync<kSm>(cl);
+    if (me == 0) {
+        uint32_t q[BlockShape<N>::kWords] = {};
+        for (int v = 0; v < N; ++v) q[v >> 2] |= (uint32_t)v << (8 * (v & 3));      // the identity
+        unsigned m = 0;
+        const unsigned idx = block_rank<N>(q, m);
+        V[idx] = 1u << m;
+        ws[kBlocks + idx] = 1u << m;
+        J.layer_sizes[0] = 1;
+    }
+    growth_sync<kSm>(cl);
+    int radius = 0, status = kRunning;
+    unsigned long long states = 1;
+    const int max_radius = J.max_radius, layers_cap = J.layers_cap;
+    const unsigned long long max_states = J.keys_cap, stop_above = J.stop_above;
+    while (status == kRunning) {
+        const unsigned* F = ws + kBlocks * (1u + (unsigned)radius % 3u);
+        unsigned* X = ws + kBlocks * (1u + (unsigned)(radius + 1) % 3u);
+        unsigned* O = ws + kBlocks * (1u + (unsigned)(radius + 2) % 3u);
+        const int par = radius & 1;
+        unsigned found = 0;
+        int qn = 0, cn = 0;
+        unsigned pidx = 0, pf = 0, pv = 0;
+        auto claim = [&](int take) {
+            cn -= take;
+            if (lane < take) {
+                const unsigned i = cidx[cn + lane], f = cf[cn + lane];
+                const unsigned neu = f & ~atomicOr(V + i, f);
+                if (neu) {
+                    found += __popc(neu);
+                    atomicOr(X + i, neu);
+                }
+            }
+            __syncwarp();
+        };
+        auto settle = [&]() {
+            const unsigned neu = pf & ~pv;
+            const unsigned b = __ballot_sync(0xffffffffu, neu != 0);
+            if (b == 0) return;
+            if (neu) {
+                const int at = cn + __popc(b & lanemask_lt());
+                cidx[at] = pidx;
+                cf[at] = neu;
+            }
+            cn += __popc(b);
+            __syncwarp();
+            if (cn >= 32) claim(32);
+        };
+        auto expand = [&](int take) {
+            qn -= take;
+            const bool active = lane < take;
+            const unsigned idx = active ? qidx[qn + lane] : 0u;
+            const unsigned f = active ? qf[qn + lane] : 0u;
+            __syncwarp();
+            const BlockPerm<N> P = cluster_unrank<N>(table, idx);
+            for (int g = 0; g < k; ++g) {
+                uint32_t q[BlockShape<N>::kWords];
+                block_map<N>(smem ? S.map[g] : *reinterpret_cast<const uint4*>(gens[g].map), P, q);
+                unsigned m;
+                const unsigned i = block_rank<N>(q, m);
+                // (as in block_grow_kernel: never past the words, whatever the tables hold)
+                const bool live = active && i < kBlocks;
+                if (active && !live) atomicCAS(&A.ctl->err, 0, CG_EDEVICE);
+                const unsigned t = xor_bits32(f, m);
+                unsigned v = 0;
+                if (live) v = growth_word<kSm>(V + i);
+                settle();
+                pidx = i;
+                pf = live ? t : 0u;
+                pv = v;
+            }
+        };
+        for (unsigned base = me - lane; base < kBlocks; base += all) {
+            const unsigned i = base + lane;
+            unsigned f = 0;
+            if (i < kBlocks) {
+                f = growth_word<kSm>(F + i);
+                O[i] = 0;
+            }
+            const unsigned have = __ballot_sync(0xffffffffu, f != 0);
+            if (have == 0) continue;
+            if (f) {
+                const int at = qn + __popc(have & lanemask_lt());
+                qidx[at] = i;
+                qf[at] = f;
+            }
+            qn += __popc(have);
+            __syncwarp();
+            if (qn >= 32) expand(32);
+        }
+        if (qn > kPairBlocks) expand(qn);
+        settle();
+        pf = 0;
+        // A short remainder (in a small round all there is): a lane per (block, generator) pair instead
+        // of per block, so that the lookups of a block are on their way together, and no look at the
+        // visited word before the atomic.
+        for (int first = 0; first < qn * k; first += 32) {
+            const int pair = first + lane;
+            const bool live = pair < qn * k;
+            const int b = live ? pair / k : 0, g = live ? pair - b * k : 0;
+            const BlockPerm<N> P = cluster_unrank<N>(table, live ? qidx[b] : 0u);
+            uint32_t q[BlockShape<N>::kWords];
+            block_map<N>(smem ? S.map[g] : *reinterpret_cast<const uint4*>(gens[g].map), P, q);
+            unsigned m;
+            const unsigned i = block_rank<N>(q, m);
+            if (live && i < kBlocks) {
+                const unsigned f = xor_bits32(qf[b], m);
+                const unsigned neu = f & ~atomicOr(V + i, f);
+                if (neu) {
+                    found += __popc(neu);
+                    atomicOr(X + i, neu);
+                }
+            } else if (live) {
+                atomicCAS(&A.ctl->err, 0, CG_EDEVICE);
+            }
+        }
+        qn = 0;
+        if (cn > 0) claim(cn);
+#pragma unroll
+        for (int o = 16; o; o >>= 1) found += __shfl_xor_sync(0xffffffffu, found, o);
+        if (lane == 0 && found) atomicAdd(&S.acc[par], found);
+        __syncthreads();
+        if (kSm) {
+            if (tid == 0) S.cnt[par][0] = S.acc[par];
+        } else if (tid < (int)size) {
+            *cl.map_shared_rank(&S.cnt[par][rank], tid) = S.acc[par];
+        }
+        if (tid == 0) S.acc[par ^ 1] = 0;
+        growth_sync<kSm>(cl);
+        unsigned long long fresh = 0;
+        for (unsigned q = 0; q < size; ++q) fresh += S.cnt[par][q];
+        if (fresh == 0) {
+            status = kDone;
+        } else if (states + fresh > max_states) {
+            status = kNeedMem;              // the layer is past the states the job may keep
+        } else {
+            states += fresh;
+            ++radius;
+            if (me == 0) J.layer_sizes[radius] = fresh;
+            if (max_radius >= 0 && radius >= max_radius) status = kTruncRadius;
+            else if (stop_above > 0 && fresh > stop_above) status = kTruncAbove;
+            else if (radius + 1 >= layers_cap) status = kTruncRadius;
+        }
+    }
+    if (me == 0) {
+        J.radius = radius;
+        J.status = status;
+    }
+    if (kSm && A.last) {
+        const unsigned* F = ws + kBlocks * (1u + (unsigned)radius % 3u);
+        for (unsigned i = tid; i < kBlocks; i += T) A.last[i] = F[i];
+    }
+}
+
+__global__ void __launch_bounds__(kClThreads, 2) cluster_grow_kernel(const ClusterArgs A) {
+    __shared__ ClusterShared<kClThreads> S;
+    const cgr::cluster_group cl = cgr::this_cluster();
+    const unsigned size = cl.num_blocks();
+    unsigned* ws = A.words + (uint64_t)(blockIdx.x / size) * A.stride;
+    for (;;) {
+        if (cl.block_rank() == 0 && threadIdx.x < size) {
+            int j = 0;
+            if (threadIdx.x == 0) j = (int)atomicAdd(&A.ctl->total_units, 1ull);
+            j = __shfl_sync((1u << size) - 1u, j, 0);
+            *cl.map_shared_rank(&S.job, threadIdx.x) = j;
+        }
+        cl.sync();
+        const int job = S.job;
+        if (job >= A.njobs) break;
+        JobDev& J = A.jobs[job];
+        switch (J.n) {
+#define CG_CLUSTER(n) case n: cluster_grow<n, false, kClThreads>(S, A, J, ws, A.table[n], cl); break;
+            CG_CLUSTER(2) CG_CLUSTER(3) CG_CLUSTER(4) CG_CLUSTER(5) CG_CLUSTER(6) CG_CLUSTER(7) CG_CLUSTER(8)
+            CG_CLUSTER(9) CG_CLUSTER(10)
+#undef CG_CLUSTER
+            default: break;                 // planned for n in 2..10 only
+        }
+        cl.sync();                          // everyone is done with this job's shared state
+    }
+}
+
+// Growths of n <= kClusterSmemN by one block each, words (40 KB for n = 8) and unranking table in its
+// shared memory: a round costs shared-memory latencies and a block barrier, no trip to L2 (one growth
+// of S_6 under adjacent transpositions 49 us on the grid, 29 us here; S_7 86 / 55, S_8 161 / 146, where
+// one SM's issue rate takes over and more than ten generators are faster on the grid).  The jobs
+// [A.first, A.njobs) of the queue (the first ones are the larger, for cluster_grow_kernel).
+// 512 threads a block, two to an SM, for many jobs; 1024 for one, whose rounds they share.
+template <int T>
+__global__ void __launch_bounds__(T, 1024 / T) cluster_grow_small_kernel(const ClusterArgs A) {
+    __shared__ ClusterShared<T> S;
+    extern __shared__ uint64_t s_words[];
+    const cgr::cluster_group cl = cgr::this_cluster();
+    unsigned* ws = reinterpret_cast<unsigned*>(s_words);
+    uint64_t* table = s_words + 2 * block_count(kClusterSmemN);
+    int have = 0;                           // the n whose table is in shared memory
+    for (;;) {
+        if (threadIdx.x == 0) S.job = A.first + (int)atomicAdd(&A.ctl->dyn_next, 1ull);
+        __syncthreads();
+        const int job = S.job;
+        if (job >= A.njobs) break;
+        JobDev& J = A.jobs[job];
+        const int n = J.n;
+        if (n != have && n >= 2 && n <= kClusterSmemN) {
+            for (unsigned i = threadIdx.x; i < block_count(n); i += T) table[i] = A.table[n][i];
+            have = n;
+        }
+        switch (n) {
+#define CG_CLUSTER(n) case n: cluster_grow<n, true, T>(S, A, J, ws, table, cl); break;
+            CG_CLUSTER(2) CG_CLUSTER(3) CG_CLUSTER(4) CG_CLUSTER(5) CG_CLUSTER(6) CG_CLUSTER(7) CG_CLUSTER(8)
+#undef CG_CLUSTER
+            default: break;                 // planned for n in 2..8 only
+        }
+        __syncthreads();                    // everyone is done with this job's shared state
+    }
+}
+
+// Unranking tables of the cluster kernels, one for each n asked for: block idx -> nibble v = position
+// of value v.
+__global__ void cluster_prepare_kernel(const ClusterArgs A, unsigned want) {
+    for (int n = 2; n <= kClusterMaxN; ++n) {
+        if (!(want >> n & 1u)) continue;
+        uint64_t* out = const_cast<uint64_t*>(A.table[n]);
+        const int M = block_pairs(n);
+        const unsigned count = block_count(n);
+        for (unsigned b = blockIdx.x * blockDim.x + threadIdx.x; b < count; b += gridDim.x * blockDim.x) {
+            unsigned pairs = 1;
+            for (int i = 0; i < M; ++i) pairs *= (unsigned)((2 * i + 2) * (2 * i + 1) / 2);
+            unsigned char place[16];
+            arrange_pairs(b % pairs, M, place);
+            unsigned char free_[16];
+            for (int i = 0; i < n; ++i) free_[i] = (unsigned char)i;
+            uint64_t key = 0;
+            if (n > 2 * M) {                // the single top value (n odd)
+                const unsigned d = b / pairs;
+                key |= (uint64_t)d << (4 * (n - 1));
+                for (int j = (int)d; j + 1 < n; ++j) free_[j] = free_[j + 1];
+            }
+            for (int v = 0; v < 2 * M; ++v) key |= (uint64_t)free_[place[v]] << (4 * v);
+            out[b] = key;
+        }
+    }
+}
+
+// Packed keys of one layer of a cluster growth (words F), in no particular order; see
+// block_export_kernel.
+__global__ void cluster_export_kernel(const unsigned* F, const uint64_t* table, int n, uint64_t start, uint64_t* out,
+                                      unsigned long long cap, unsigned long long* count) {
+    const unsigned total = block_count(n);
+    const int M = block_pairs(n);
+    for (unsigned b = blockIdx.x * blockDim.x + threadIdx.x; b < total; b += gridDim.x * blockDim.x) {
+        const unsigned f = F[b];
+        if (!f) continue;
+        const uint64_t p = table[b];
+        unsigned long long o = atomicAdd(count, (unsigned long long)__popc(f));
+        for (int e = 0; e < 1 << M; ++e) {
+            if (!(f >> e & 1u)) continue;
+            uint64_t key = 0;
+            for (int v = 0; v < n; ++v) {
+                const int u = v < 2 * M && (e >> (v >> 1) & 1) ? (v ^ 1) : v;
+                key |= ((start >> (4 * v)) & 15ull) << (4 * ((p >> (4 * u)) & 15ull));
+            }
+            if (o < cap) out[o] = key;
+            ++o;
+        }
+    }
+}
+
 using block_fn = void (*)(BlockDev*, Ctl*, int, uint64_t);
 
 block_fn block_kernel(int n) {
@@ -545,6 +914,84 @@ block_fn block_kernel(int n) {
 }
 
 }  // namespace
+
+uint64_t cluster_words(int n) { return 4ull * block_count(n); }
+uint64_t cluster_table_entries(int n) { return block_count(n); }
+
+cudaError_t launch_cluster_prepare(const ClusterArgs& A, unsigned want, cudaStream_t st) {
+    (void)cudaGetLastError();   // clear a stale error: the check after the launch is about this one
+    cluster_prepare_kernel<<<152, 256, 0, st>>>(A, want);
+    return cudaGetLastError();
+}
+
+int cluster_max_clusters(int device, int size) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)size);
+    cfg.blockDim = dim3(kClThreads);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim = {(unsigned)size, 1, 1};
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    (void)device;
+    if (size > 8 &&
+        cudaFuncSetAttribute(cluster_grow_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, cluster_grow_kernel, &cfg) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    return n;
+}
+
+cudaError_t launch_cluster_grow(const ClusterArgs& A, int clusters, int size, cudaStream_t st) {
+    (void)cudaGetLastError();   // clear a stale error: the check after the launch is about this one
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(clusters * size));
+    cfg.blockDim = dim3(kClThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim = {(unsigned)size, 1, 1};
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, cluster_grow_kernel, A);
+}
+
+namespace {
+constexpr size_t small_smem() { return (size_t)block_count(kClusterSmemN) * (4 * 4 + 8); }
+}
+
+int cluster_small_blocks(int device) {
+    int sms = 0, per_sm = 0;
+    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    if (cudaFuncSetAttribute(cluster_grow_small_kernel<512>, at, (int)small_smem()) != cudaSuccess ||
+        cudaFuncSetAttribute(cluster_grow_small_kernel<1024>, at, (int)small_smem()) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cluster_grow_small_kernel<512>, 512, small_smem()) !=
+            cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    return sms * per_sm;
+}
+
+cudaError_t launch_cluster_small(const ClusterArgs& A, int blocks, cudaStream_t st) {
+    (void)cudaGetLastError();   // clear a stale error: the check after the launch is about this one
+    if (blocks == 1) cluster_grow_small_kernel<1024><<<1, 1024, small_smem(), st>>>(A);
+    else cluster_grow_small_kernel<512><<<blocks, 512, small_smem(), st>>>(A);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_cluster_export(const unsigned* F, const uint64_t* table, int n, uint64_t start, uint64_t* out,
+                                  unsigned long long cap, unsigned long long* count, cudaStream_t st) {
+    (void)cudaGetLastError();   // clear a stale error: the check after the launch is about this one
+    cluster_export_kernel<<<152, 256, 0, st>>>(F, table, n, start, out, cap, count);
+    return cudaGetLastError();
+}
 
 int block_max_grid(int device, int n) {
     int sms = 0, per_sm = 0;

@@ -40,6 +40,7 @@ struct GenSM {
     uint8_t rot[kMaxTerms];
     uint64_t mask[kMaxTerms];
     alignas(16) uint32_t sel[kSelWords];
+    uint8_t map[16];    // the inverse, byte q = the i with g[i] = q: how a generator moves position q
 };
 static_assert(offsetof(GenSM, sel) % 16 == 0 && sizeof(GenSM) % 16 == 0, "GenSM: sel is read in 16-byte vectors");
 
@@ -246,6 +247,23 @@ struct alignas(128) BlockDev {
     unsigned long long states;              // states of the layers so far
     int radius;                // radius of the frontier layer
     int status;                // JobStatus
+};
+
+// Growths of S_n, n <= kClusterMaxN, one thread-block cluster each (block_path.cu).  Of a JobDev the
+// kernel reads gens (GenSM::map), k, n, layer_sizes, layers_cap, max_radius, stop_above and keys_cap
+// (the states the job may hold) and writes layer_sizes, radius and status.
+struct Ctl;
+constexpr int kClusterMaxN = 10;
+constexpr int kClusterSmemN = 8;            // up to this n one block each, all in its shared memory
+constexpr int kClusterGens = 64;            // generators kept in shared memory
+struct ClusterArgs {
+    JobDev* jobs;                           // in the order they are taken
+    int first, njobs;                       // cluster_grow_kernel: [0, njobs); the small kernel: [first, njobs)
+    unsigned* words;                        // per cluster `stride` words: visited and three layers
+    uint64_t stride;
+    const uint64_t* table[kClusterMaxN + 1];
+    unsigned* last;                         // small kernel, one job: receives the last layer's words, or null
+    Ctl* ctl;                               // zeroed: total_units and dyn_next, the two queues; err
 };
 
 // Admission of many jobs into one persistent launch (a batch): the jobs are grown in index

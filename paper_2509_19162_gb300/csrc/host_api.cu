@@ -221,6 +221,7 @@ std::vector<GenSM> make_gensms(const std::vector<std::vector<uint8_t>>& rows, in
         if (w == 4 && n <= cg::kMaxN) {
             cg::make_selectors(rows[j].data(), n, out[j].sel);
             out[j].sel[0] |= out[j].inv_tag << 28;
+            for (int i = 0; i < n; ++i) out[j].map[rows[j][i]] = (uint8_t)i;
         }
     }
     return out;
@@ -386,6 +387,23 @@ int grow_grid(int dev, int ilp, bool multi = false) {
     return c;
 }
 
+// Clusters of `size` blocks of the cluster kernel that device `dev` runs at once (0: none).
+int cluster_cache[64][17] = {};
+int cluster_clusters(int dev, int size) {
+    if (dev < 0 || dev >= 64 || size < 1 || size > 16) return 0;
+    int& c = cluster_cache[dev][size];
+    if (!c) c = 1 + cg::cluster_max_clusters(dev, size);
+    return c - 1;
+}
+
+// Blocks of the small cluster kernel that device `dev` runs at once.
+int small_cache[64] = {};
+int small_blocks(int dev) {
+    if (dev < 0 || dev >= 64) return 0;
+    if (!small_cache[dev]) small_cache[dev] = 1 + cg::cluster_small_blocks(dev);
+    return small_cache[dev] - 1;
+}
+
 // Generators probed together per thread.  Hash tables (random DRAM probes): all of them when
 // k <= 4, else 4.  Rank bitmap (L2-resident, one atomic per probe): 1 -- measured fastest, and
 // the only bitmap variant that fits 64 registers without spilling.
@@ -464,6 +482,8 @@ struct cg_growth {
     char* d_blk = nullptr;                       // one allocation (BlockLayout)
     BlockDev host_block{};
     bool last_is_block = false;
+    unsigned* d_cl = nullptr;                    // one-block growth: last layer's words, unranking table
+    bool last_is_cluster = false;
     bool served = false;                         // grown for a server: the share bounds its states
 
     JobDev host_job{};
@@ -488,6 +508,8 @@ struct cg_growth {
         d_sw = nullptr;
         sw_bytes = 0;
         release_block(st);
+        dev_free(d_cl, st);
+        d_cl = nullptr;
         dev_free(d_wgens, st);
         dev_free(d_wjob, st);
         dev_free(d_wkeys, st);
@@ -716,6 +738,70 @@ bool blocks_will_fill(const cg_growth* h, uint64_t F, uint64_t Fprev, int r) {
 bool block_group(const cg_growth* h) {
     const int min_k = h->n >= 12 ? 1 : h->n == 11 ? 6 : 10;
     return block_fits(h) && h->order * 4 >= factorial(h->n) && h->k >= min_k;
+}
+
+// A growth of S_n, n <= kClusterSmemN, by one block in its shared memory (block_path.cu).  AUTO takes it
+// for groups of index at most 4 whose key list would have fitted mem_cap (so that nothing else would
+// have stopped or handed over).
+bool cluster_preferred(const cg_growth* h) {
+    const uint64_t mem = h->mem_cap ? h->mem_cap : kDefaultMemCap;
+    if (h->strategy != CG_STRATEGY_AUTO || !h->start_is_perm || h->width != 4 || h->n < 2 ||
+        h->n > cg::kClusterSmemN || h->grid_override > 0 || h->ilp_override > 0)
+        return false;
+    if (h->order * 4 < factorial(h->n) || (h->n == cg::kClusterSmemN && h->k > 10)) return false;
+    return h->states_bound * 8 + bitmap_words(h->n) * 4 + (2 << 20) <= mem;
+}
+
+int run_cluster(cg_growth* h, cudaStream_t st, int* final_status) {
+    int rc = ensure_small_buffers(h, st);
+    if (rc) return rc;
+    cudaError_t e = cudaSuccess;
+    const uint64_t words = (cg::cluster_words(h->n) / 4 + 63) & ~63ull;    // of one layer: the last
+    const bool fresh_alloc = h->d_cl == nullptr;
+    if (fresh_alloc) {
+        h->d_cl = (unsigned*)dev_alloc(words * 4 + cg::cluster_table_entries(h->n) * 8, st);
+        if (!h->d_cl) return CG_ENOMEM;
+    }
+    JobDev J;
+    std::memset(&J, 0, sizeof(J));
+    fill_static(h, J);
+    J.keys_cap = ~0ull;
+    cg::ClusterArgs A{};
+    A.jobs = h->d_job;
+    A.njobs = 1;
+    A.last = h->d_cl;
+    A.table[h->n] = reinterpret_cast<const uint64_t*>(h->d_cl + words);
+    A.ctl = h->d_ctl;
+    if ((e = cudaMemcpyAsync(h->d_job, &J, sizeof(J), cudaMemcpyHostToDevice, st)) != cudaSuccess) return cuda_rc(e);
+    if ((e = cudaMemsetAsync(h->d_ctl, 0, sizeof(Ctl), st)) != cudaSuccess) return cuda_rc(e);
+    if (fresh_alloc) {
+        if ((e = cg::launch_cluster_prepare(A, 1u << h->n, st)) != cudaSuccess) return cuda_rc(e);
+        h->stats.launches += 1;
+    }
+    if (!h->ev0) {
+        if ((e = cudaEventCreate(&h->ev0)) != cudaSuccess) return cuda_rc(e);
+        if ((e = cudaEventCreate(&h->ev1)) != cudaSuccess) return cuda_rc(e);
+    }
+    if ((e = cudaEventRecord(h->ev0, st)) != cudaSuccess) return cuda_rc(e);
+    if ((e = cg::launch_cluster_small(A, 1, st)) != cudaSuccess) return cuda_rc(e);
+    if ((e = cudaEventRecord(h->ev1, st)) != cudaSuccess) return cuda_rc(e);
+    Ctl ctl;
+    if ((e = cudaMemcpyAsync(&J, h->d_job, sizeof(J), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return cuda_rc(e);
+    if ((e = cudaMemcpyAsync(&ctl, h->d_ctl, sizeof(ctl), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return cuda_rc(e);
+    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_rc(e);
+    h->stats.launches += 1;
+    h->stats.h2d_bytes += sizeof(J);
+    h->stats.d2h_bytes += sizeof(J) + sizeof(ctl);
+    h->stats.kernel_ms += elapsed_ms(h->ev0, h->ev1);
+    h->stats.rounds += J.radius + 1;
+    if (ctl.err) return ctl.err;
+    h->stats.state_capacity = factorial(h->n);
+    h->stats.table_slots = words / 2;
+    h->stats.strategy_used = CG_STRATEGY_SWEEP;
+    h->stats.probe_variant = 1;
+    h->host_job = J;
+    *final_status = J.status;
+    return CG_OK;
 }
 
 // Before a round on a frontier of J (host copy, current): room for the next layer as the last two
@@ -1755,18 +1841,21 @@ int cg_growth_run(cg_growth_t h, void* cuda_stream, uint64_t* layer_sizes_out, i
         return status_to_rc(status);
     }
     const bool use_sort = h->strategy == CG_STRATEGY_SORT;
-    const bool use_sweep = h->strategy == CG_STRATEGY_SWEEP ||
-                           (h->strategy == CG_STRATEGY_AUTO && sweep_preferred(h));
-    int rc = use_sort ? run_sort(h, st, &status)
+    const bool use_cluster = cluster_preferred(h) && small_blocks(dev) > 0;
+    const bool use_sweep = !use_cluster && (h->strategy == CG_STRATEGY_SWEEP ||
+                                            (h->strategy == CG_STRATEGY_AUTO && sweep_preferred(h)));
+    h->last_is_cluster = use_cluster;
+    int rc = use_cluster ? run_cluster(h, st, &status)
+             : use_sort ? run_sort(h, st, &status)
                       : use_sweep ? run_sweep(h, st, &status) : run_hash(h, st, &status);
     if (rc) return rc;
-    if (!use_sort && !use_sweep && status == cg::kNeedMem && h->strategy == CG_STRATEGY_AUTO &&
+    if (!use_cluster && !use_sort && !use_sweep && status == cg::kNeedMem && h->strategy == CG_STRATEGY_AUTO &&
         h->inverse_closed) {
         if ((rc = continue_sorted(h, st, &status))) return rc;
     }
     const bool sorted = use_sort || h->stats.switched_to_sort;
     h->last_is_sweep = use_sweep;
-    if (use_sort || h->stats.switched_to_sort) h->last_is_block = false;
+    if (use_cluster || use_sort || h->stats.switched_to_sort) h->last_is_block = false;
     const int layers = h->host_job.radius + 1;
     *num_layers_out = layers;
     if (cap < layers) return CG_EINVAL;
@@ -1796,10 +1885,11 @@ int cg_growth_last_layer(cg_growth_t h, uint64_t* keys_out, uint64_t cap, uint64
             for (uint64_t i = 0; i < cnt; ++i) keys_out[2 * i + 1] &= (1ull << 60) - 1;
         return cuda_rc(e);
     }
-    if (h->last_is_block) {
+    if (h->last_is_block || h->last_is_cluster) {
         const BlockDev& D = h->host_block;
+        const int radius = h->host_job.radius;
         uint64_t cnt = 0;
-        cudaError_t e = cudaMemcpy(&cnt, h->d_layers + D.radius, 8, cudaMemcpyDeviceToHost);
+        cudaError_t e = cudaMemcpy(&cnt, h->d_layers + radius, 8, cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) return cuda_rc(e);
         *count_out = cnt;
         if (cap < cnt || (!keys_out && cnt > 0)) return CG_EINVAL;
@@ -1810,7 +1900,13 @@ int cg_growth_last_layer(cg_growth_t h, uint64_t* keys_out, uint64_t cap, uint64
         int sms = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
         e = cudaMemsetAsync(d_count, 0, 8, nullptr);
-        if (e == cudaSuccess)
+        if (e == cudaSuccess && h->last_is_cluster) {
+            const uint64_t words = (cg::cluster_words(h->n) / 4 + 63) & ~63ull;
+            uint64_t id = 0;
+            for (int i = 0; i < h->n; ++i) id |= (uint64_t)i << (4 * i);
+            e = cg::launch_cluster_export(h->d_cl, reinterpret_cast<const uint64_t*>(h->d_cl + words), h->n,
+                                          h->use_start ? h->start_key : id, d_out, cnt, d_count, nullptr);
+        } else if (e == cudaSuccess)
             e = cg::launch_block_export(D, D.radius % 3, d_out, cnt, d_count, std::max(sms, 1) * 16, nullptr);
         unsigned long long got = 0;
         if (e == cudaSuccess) e = cudaMemcpy(&got, d_count, 8, cudaMemcpyDeviceToHost);
@@ -2056,9 +2152,17 @@ struct cg_batch {
         uint64_t order = 1;
         uint64_t cap = 1;          // states the job may store
         int mode = cg::kVisitHash; // rank bitmap for small dense groups, else hash table
+        bool cluster = false;      // small rank-bitmap group: grown by one thread-block cluster
     };
     struct Wave {
         std::vector<int> ids;
+        bool cluster = false;      // jobs grown by clusters (ClusterArgs):
+        int clusters = 0;          //   the first `large` by this many clusters of csize blocks,
+        int csize = 1;
+        int large = 0;
+        int small_blocks = 0;      //   the others by this many blocks
+        unsigned want = 0;         // clusters: the n that occur, a bit each
+        int max_n = 0;
         bool admit = false;        // one launch admitting its jobs by the L2 window (AdmitDev)
         char* base = nullptr;      // resident plans: the wave's device buffer
         uint64_t bytes = 0;
@@ -2184,6 +2288,62 @@ void layout_wave(cg_batch* b, cg_batch::Wave& w, int lcap) {
     }
 }
 
+// A wave of cluster jobs: gens | jobs | order | ctl | layers | unranking tables | words per cluster.
+// The largest jobs are taken first.
+void layout_cluster_wave(cg_batch* b, cg_batch::Wave& w, int lcap) {
+    std::stable_sort(w.ids.begin(), w.ids.end(), [&](int x, int y) {
+        const auto &X = b->jobs[x], &Y = b->jobs[y];
+        return X.n != Y.n ? X.n > Y.n : X.k > Y.k;
+    });
+    const int nj = (int)w.ids.size();
+    uint64_t ngens = 0;
+    w.hg.clear();
+    w.hj.assign(nj, JobDev{});
+    for (int i = 0; i < nj; ++i) {
+        const auto& J = b->jobs[w.ids[i]];
+        JobDev& D = w.hj[i];
+        std::memset(&D, 0, sizeof(D));
+        D.keys_cap = J.cap;
+        D.gens = reinterpret_cast<const GenSM*>(ngens * sizeof(GenSM));      // offsets until bound
+        D.layer_sizes = reinterpret_cast<uint64_t*>((uint64_t)i * lcap * 8);
+        D.k = J.k;
+        D.n = J.n;
+        D.layers_cap = lcap;
+        D.max_radius = J.max_radius;
+        ngens += J.gsm.size();
+        w.hg.insert(w.hg.end(), J.gsm.begin(), J.gsm.end());
+        w.want |= 1u << J.n;
+        w.max_n = std::max(w.max_n, J.n);
+    }
+    w.o_gens = 0;
+    w.o_jobs = al256(ngens * sizeof(GenSM));
+    w.o_ctl = al256(w.o_jobs + nj * sizeof(JobDev));
+    w.o_lay = al256(w.o_ctl + sizeof(Ctl));
+    w.o_tab = al256(w.o_lay + (uint64_t)nj * lcap * 8);
+    uint64_t tables = 0;
+    for (int n = 2; n <= cg::kClusterMaxN; ++n)
+        if (w.want >> n & 1u) tables += al256(cg::cluster_table_entries(n) * 8);
+    w.o_keys = al256(w.o_tab + tables);
+    w.bytes = al256(w.o_keys + std::max<uint64_t>((uint64_t)w.clusters * cg::cluster_words(w.max_n) * 4, 256));
+}
+
+cg::ClusterArgs cluster_args(const cg_batch::Wave& w, char* base) {
+    cg::ClusterArgs A{};
+    A.jobs = reinterpret_cast<JobDev*>(base + w.o_jobs);
+    A.first = w.large;
+    A.njobs = (int)w.ids.size();
+    A.words = reinterpret_cast<unsigned*>(base + w.o_keys);
+    A.stride = cg::cluster_words(w.max_n);
+    uint64_t o = w.o_tab;
+    for (int n = 2; n <= cg::kClusterMaxN; ++n)
+        if (w.want >> n & 1u) {
+            A.table[n] = reinterpret_cast<const uint64_t*>(base + o);
+            o += al256(cg::cluster_table_entries(n) * 8);
+        }
+    A.ctl = reinterpret_cast<Ctl*>(base + w.o_ctl);
+    return A;
+}
+
 // Turn the offsets of the wave's descriptors into device addresses of `base` and upload the
 // static part (generators and descriptors).
 cudaError_t bind_wave(cg_batch::Wave& w, char* base, cudaStream_t st) {
@@ -2199,6 +2359,7 @@ cudaError_t bind_wave(cg_batch::Wave& w, char* base, cudaStream_t st) {
                                            cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(base + w.o_jobs, hj.data(), hj.size() * sizeof(JobDev), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess && w.cluster) e = cg::launch_cluster_prepare(cluster_args(w, base), w.want, st);
     cg::AdmitDev A{};
     if (w.admit) {
         A.act[0] = reinterpret_cast<int*>(base + w.o_act);
@@ -2234,7 +2395,12 @@ cudaError_t enqueue_wave(cg_batch* b, cg_batch::Wave& w, char* base, char* hout,
     unsigned long long* d_ubeg = reinterpret_cast<unsigned long long*>(base + w.o_ubeg);
     Ctl* d_ctl = reinterpret_cast<Ctl*>(base + w.o_ctl);
     if (e == cudaSuccess) e = cudaMemsetAsync(d_ctl, 0, sizeof(Ctl), st);
-    if (w.admit) {
+    if (w.cluster) {
+        cg::ClusterArgs A = cluster_args(w, base);
+        if (e == cudaSuccess && w.small_blocks) e = cg::launch_cluster_small(A, w.small_blocks, st);
+        A.njobs = w.large;
+        if (e == cudaSuccess && w.large) e = cg::launch_cluster_grow(A, w.clusters, w.csize, st);
+    } else if (w.admit) {
         // one launch for the whole batch: jobs are admitted (and set up) as the window allows
         const cg::AdmitDev* d_adm = reinterpret_cast<const cg::AdmitDev*>(base + w.o_adm);
         if (e == cudaSuccess) e = cg::launch_admit_first(d_jobs, d_ubeg, d_ctl, d_adm, st);
@@ -2268,6 +2434,7 @@ int collect_wave(cg_batch* b, const cg_batch::Wave& w, const char* hres, int lca
     for (int i = 0; i < nj; ++i) {
         const int j = w.ids[i];
         const int layers = hj[i].radius + 1;
+        if (w.cluster) b->stats.rounds += layers;
         int st_rc = status_to_rc(hj[i].status);
         if (layers > cap) { st_rc = CG_EINVAL; rc = CG_EINVAL; }
         nl_out[j] = layers;
@@ -2276,6 +2443,42 @@ int collect_wave(cg_batch* b, const cg_batch::Wave& w, const char* hres, int lca
         if (st_rc < 0 && rc == CG_OK) rc = st_rc;
     }
     return rc;
+}
+
+// The wave of the jobs marked `cluster` (b->waves[0]), in at most `bytes` of device memory; false when
+// it cannot be had.  Jobs of n <= kClusterSmemN take a block each, the larger ones a cluster: eight
+// blocks for S_10, whose rounds go through 113,400 words and of which then few enough run at once for
+// their words (1.8 MB each) to share L2, four when n = 9 is the largest.  1024 random groups of n in
+// 6..10: 36.2 ms as key lists in one launch, 6.9 ms as clusters, 6.3 ms with the small ones apart.
+bool plan_cluster_wave(cg_batch* b, int dev, int lcap, uint64_t bytes) {
+    cg_batch::Wave w;
+    int max_n = 0;
+    for (int j = 0; j < (int)b->jobs.size(); ++j)
+        if (b->jobs[j].cluster) {
+            w.ids.push_back(j);
+            w.large += b->jobs[j].n > cg::kClusterSmemN ? 1 : 0;
+            max_n = std::max(max_n, b->jobs[j].n);
+        }
+    if (w.ids.empty()) return true;
+    w.cluster = true;
+    w.csize = max_n >= 10 ? 8 : 4;
+    int fit = w.large ? cluster_clusters(dev, w.csize) : 0, small_fit = small_blocks(dev);
+    if (b->grid_override > 0) {
+        fit = std::min(fit, std::max(1, b->grid_override / w.csize));
+        small_fit = std::min(small_fit, b->grid_override);
+    }
+    w.clusters = std::min<int>(fit, w.large);
+    w.small_blocks = std::min<int>(small_fit, (int)w.ids.size() - w.large);
+    if ((w.large && w.clusters < 1) || (w.large < (int)w.ids.size() && w.small_blocks < 1)) return false;
+    layout_cluster_wave(b, w, lcap);
+    if (w.bytes > bytes) {
+        const uint64_t each = cg::cluster_words(w.max_n) * 4, fixed = w.bytes - (uint64_t)w.clusters * each;
+        if (fixed + (w.large ? each : 0) + 256 > bytes) return false;
+        w.clusters = (int)((bytes - fixed - 256) / each);
+        layout_cluster_wave(b, w, lcap);
+    }
+    b->waves.push_back(std::move(w));
+    return true;
 }
 
 // Choose visited sets, kernel variant, grid and waves; allocate the waves' buffers when they
@@ -2301,7 +2504,7 @@ int plan_batch(cg_batch* b, int dev, int cap, cudaStream_t st) {
     const int grid_max = grow_grid(dev, b->ilp, true);
     if (grid_max <= 0) return CG_ECUDA;
     b->grid = b->grid_override > 0 ? std::min(grid_max, b->grid_override) : grid_max;
-    const uint64_t budget = b->mem_cap;
+    uint64_t budget = b->mem_cap;
     const uint64_t per_job_max = max_cap_for_mem(budget / 2);
     uint64_t l2_cap = b->wave_l2;
     if (l2_cap == 0) {
@@ -2328,6 +2531,8 @@ int plan_batch(cg_batch* b, int dev, int cap, cudaStream_t st) {
         J.cap = std::max<uint64_t>(1, std::min<uint64_t>(J.order, per_job_max));
         const uint64_t set_bytes = J.mode == cg::kVisitBitmap ? bitmap_words(J.n) * 4
                                                                : table_slots_for(J.cap) * 8;
+        J.cluster = J.mode == cg::kVisitBitmap && J.n >= 2 && J.n <= cg::kClusterMaxN;
+        if (J.cluster) continue;
         need_of[j] = J.cap * 8 + set_bytes + sizeof(GenSM) * J.gsm.size() + sizeof(JobDev) +
                      (uint64_t)lcap * 8 + 1024;
         vis_of[j] = set_bytes <= l2_cap ? set_bytes : 0;
@@ -2335,6 +2540,23 @@ int plan_batch(cg_batch* b, int dev, int cap, cudaStream_t st) {
         ++with_work;
     }
     uint64_t total_bytes = 0;
+    if (!plan_cluster_wave(b, dev, lcap, budget / 2)) {
+        for (int j = 0; j < (int)b->jobs.size(); ++j) {      // no clusters to be had: with the others
+            auto& J = b->jobs[j];
+            if (!J.cluster) continue;
+            J.cluster = false;
+            const uint64_t set_bytes = bitmap_words(J.n) * 4;
+            need_of[j] = J.cap * 8 + set_bytes + sizeof(GenSM) * J.gsm.size() + sizeof(JobDev) +
+                         (uint64_t)lcap * 8 + 1024;
+            vis_of[j] = set_bytes <= l2_cap ? set_bytes : 0;
+            all_need += need_of[j] + 16;
+            ++with_work;
+        }
+    } else if (!b->waves.empty()) {
+        total_bytes = b->waves[0].bytes;
+        budget -= total_bytes;
+    }
+    const uint64_t cluster_bytes = total_bytes;
     if (with_work > 0 && all_need + (4ull << 20) <= budget) {
         cg_batch::Wave w;
         w.admit = true;
@@ -2347,7 +2569,7 @@ int plan_batch(cg_batch* b, int dev, int cap, cudaStream_t st) {
                 w.vis.push_back(vis_of[j]);
             }
         layout_wave(b, w, lcap);
-        total_bytes = w.bytes;
+        total_bytes = cluster_bytes + w.bytes;
         b->waves.push_back(std::move(w));
     } else {
         cg_batch::Wave cur;
@@ -2384,7 +2606,7 @@ int plan_batch(cg_batch* b, int dev, int cap, cudaStream_t st) {
         b->h_bytes = hb;
     }
     // resident when all waves fit the budget together
-    b->resident = total_bytes <= budget;
+    b->resident = total_bytes <= b->mem_cap;
     if (b->resident) {
         for (auto& w : b->waves) {
             w.base = (char*)dev_alloc(w.bytes, st);
@@ -2512,7 +2734,8 @@ int cg_batch_run(cg_batch_t b, void* cuda_stream, uint64_t* layer_sizes_out, int
         }
         b->stats.kernel_ms += elapsed_ms(b->ev0, b->ev1);
         for (auto& w : b->waves) {
-            b->stats.launches += w.admit ? 2 : 3;     // (admit_first | init_jobs + init_units) + grow
+            b->stats.launches += w.cluster ? (w.large > 0) + (w.small_blocks > 0)
+                                           : w.admit ? 2 : 3;     // (admit_first | init_jobs + init_units) + grow
             b->stats.d2h_bytes += wave_result_bytes(w, lcap);
             int r = collect_wave(b, w, b->h_pinned + w.h_off, lcap, cap, layer_sizes_out,
                                  num_layers_out, status_out);

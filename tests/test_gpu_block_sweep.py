@@ -125,3 +125,47 @@ def test_served_job_over_its_share_keeps_its_layers(cg, kind, radius):
             s.step()
         got = s.result(i)
     assert (got.status, got.layers) == (want.status, want.layers)
+
+
+@pytest.mark.parametrize("n", range(2, 9))
+@pytest.mark.parametrize("kind", ["random", "random_inv", "coxeter", "lx"])
+def test_one_block_growth_every_small_n(cg, n, kind):
+    gens = gens_of(kind, n, 20 + n) if n > 2 or kind in ("random", "random_inv") else [[1, 0]]
+    start = np.random.default_rng(n).permutation(n).tolist()
+    for lim in ({}, {"max_radius": 3}, {"stop_above": 4}):
+        with cg.Growth(n, gens, strategy="hash", start=start, **lim) as g:
+            want, far = g.run(), np.sort(g.last_layer())
+        with cg.Growth(n, gens, start=start, **lim) as g:
+            for _ in range(2):
+                got = g.run()
+                assert (got.status, got.layers) == (want.status, want.layers)
+                assert np.array_equal(np.sort(g.last_layer()), far)
+
+
+@pytest.mark.parametrize("cap", [1 << 20, 24 << 20, 0])
+def test_batch_of_clusters(cg, cap):
+    # n = 2..12 in one batch: a block each up to 8, a cluster each for 9 and 10, the rest as key lists;
+    # with too little memory for clusters everything is a key list
+    jobs = []
+    for n in range(2, 13):
+        for kind in ("random", "random_inv", "coxeter", "lx"):
+            gens = gens_of(kind, n, 300 + n) if n > 2 or kind in ("random", "random_inv") else [[1, 0]]
+            inv = kind in ("random_inv", "coxeter") or n == 2
+            jobs.append((n, gens, inv, -1 if n <= 10 else 7))
+            jobs.append((n, gens, inv, 5))
+    with cg.Batch(jobs, mem_cap=cap) as b:
+        first, again = b.run(), b.run()
+    assert [(r.layers, r.status) for r in first] == [(r.layers, r.status) for r in again]
+    for (n, gens, inv, rad), r in zip(jobs, first):
+        want = cg.growth(n, gens, inv, rad, strategy="hash")
+        if cap and r.status == 2:       # cut off by the batch's memory: exact so far
+            assert r.layers == want.layers[:len(r.layers)]
+        else:
+            assert (r.layers, r.status) == (want.layers, want.status)
+
+
+def test_batch_with_more_generators_than_shared_memory_holds(cg):
+    gens = w.three_cycles(8)            # 112
+    for r in cg.Batch([(8, gens, True, -1), (9, w.three_cycles(9), True, -1)]).run():
+        assert r.status == 0
+    assert cg.Batch([(8, gens, True, -1)]).run()[0].layers == cg.growth(8, gens, strategy="hash").layers
