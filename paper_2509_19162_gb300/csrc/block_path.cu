@@ -599,6 +599,42 @@ __device__ __forceinline__ BlockPerm<N> cluster_unrank(const uint64_t* table, un
     return P;
 }
 
+// Nibble v = position of value v in the canonical member of block b (the inverse of block_rank), in
+// registers: the free positions are kept ascending in nibbles.
+template <int N>
+__device__ __forceinline__ uint64_t small_unrank(unsigned b) {
+    constexpr int M = BlockShape<N>::M;
+    uint32_t avail = 0x76543210u;           // N <= 8
+    uint32_t key = 0;
+    auto take = [&](unsigned at) {
+        const unsigned sh = 4u * at;
+        const uint32_t v = (avail >> sh) & 15u;
+        const uint32_t below = (1u << sh) - 1u;
+        avail = (avail & below) | ((avail >> 4) & ~below);
+        return v;
+    };
+    constexpr unsigned pairs = N > 2 * M ? block_count(N) / N : block_count(N);
+    if (N > 2 * M) {
+        key |= take(b / pairs) << (4 * (N - 1));
+        b %= pairs;
+    }
+    unsigned radix = pairs;
+#pragma unroll
+    for (int i = M - 1; i >= 1; --i) {
+        radix /= (unsigned)((2 * i + 2) * (2 * i + 1) / 2);
+        const unsigned d = b / radix;
+        b -= d * radix;
+        unsigned hi = 1;
+#pragma unroll
+        for (int h = 2; h < 2 * i + 2; ++h) hi += (unsigned)(h * (h - 1) / 2) <= d ? 1u : 0u;
+        const unsigned lo = d - hi * (hi - 1u) / 2u;
+        key |= take(hi) << (4 * (2 * i + 1));           // the larger place first: the smaller keeps its own
+        key |= take(lo) << (4 * (2 * i));
+    }
+    key |= (avail & 15u) | (avail & 0xF0u);             // pair 0: the two free positions, ascending
+    return key;
+}
+
 // The barrier of a growth's blocks.
 template <bool kSm>
 __device__ __forceinline__ void growth_sync(const cgr::cluster_group& cl) {
@@ -616,7 +652,8 @@ __device__ __forceinline__ unsigned growth_word(const unsigned* p) {
 // kSm: one block grows the job alone, words and table in its shared memory.  T threads a block.
 template <int N, bool kSm, int T>
 __device__ __forceinline__ void cluster_grow(ClusterShared<T>& S, const ClusterArgs& A, JobDev& J, unsigned* ws,
-                                             const uint64_t* table, const cgr::cluster_group& cl) {
+                                             std::conditional_t<kSm, uint64_t*, const uint64_t*> table, bool build,
+                                             const cgr::cluster_group& cl) {
     constexpr unsigned kBlocks = block_count(N);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const unsigned size = kSm ? 1u : cl.num_blocks(), rank = kSm ? 0u : cl.block_rank();
@@ -631,6 +668,10 @@ __device__ __forceinline__ void cluster_grow(ClusterShared<T>& S, const ClusterA
     // the words of this growth, empty
     const unsigned all = size * T, me = rank * T + tid;
     for (unsigned i = me; i < 4 * kBlocks; i += all) ws[i] = 0;
+    if constexpr (kSm) {
+        if (build)
+            for (unsigned i = tid; i < kBlocks; i += T) table[i] = small_unrank<N>(i);
+    }
     if (smem)
         for (int j = tid; j < k; j += T) S.map[j] = *reinterpret_cast<const uint4*>(gens[j].map);
     if (tid < 2) S.acc[tid] = 0;
@@ -782,9 +823,31 @@ __device__ __forceinline__ void cluster_grow(ClusterShared<T>& S, const ClusterA
         J.radius = radius;
         J.status = status;
     }
-    if (kSm && A.last) {
+    if constexpr (kSm) {
+        // the last layer's packed keys, in no particular order: the value v of a state stands for the
+        // start state's (see block_export_kernel)
+        if (A.last == nullptr) return;
+        constexpr int M = BlockShape<N>::M;
         const unsigned* F = ws + kBlocks * (1u + (unsigned)radius % 3u);
-        for (unsigned i = tid; i < kBlocks; i += T) A.last[i] = F[i];
+        __syncthreads();                    // (everyone has read the last round's counts)
+        if (tid == 0) S.cnt[0][0] = 0;
+        __syncthreads();
+        for (unsigned i = tid; i < kBlocks; i += T) {
+            unsigned f = F[i];
+            if (!f) continue;
+            const uint32_t p = (uint32_t)table[i];
+            unsigned at = atomicAdd(&S.cnt[0][0], (unsigned)__popc(f));
+            for (; f; f &= f - 1u) {
+                const int e = __ffs(f) - 1;
+                uint64_t key = 0;
+#pragma unroll
+                for (int v = 0; v < N; ++v) {
+                    const int swapped = v < 2 * M ? (e >> (v >> 1)) & 1 : 0;
+                    key |= ((A.start >> (4 * v)) & 15ull) << (4u * ((p >> (4 * (v ^ swapped))) & 15u));
+                }
+                A.last[at++] = key;
+            }
+        }
     }
 }
 
@@ -805,7 +868,7 @@ __global__ void __launch_bounds__(kClThreads, 2) cluster_grow_kernel(const Clust
         if (job >= A.njobs) break;
         JobDev& J = A.jobs[job];
         switch (J.n) {
-#define CG_CLUSTER(n) case n: cluster_grow<n, false, kClThreads>(S, A, J, ws, A.table[n], cl); break;
+#define CG_CLUSTER(n) case n: cluster_grow<n, false, kClThreads>(S, A, J, ws, A.table[n], false, cl); break;
             CG_CLUSTER(2) CG_CLUSTER(3) CG_CLUSTER(4) CG_CLUSTER(5) CG_CLUSTER(6) CG_CLUSTER(7) CG_CLUSTER(8)
             CG_CLUSTER(9) CG_CLUSTER(10)
 #undef CG_CLUSTER
@@ -836,12 +899,10 @@ __global__ void __launch_bounds__(T, 1024 / T) cluster_grow_small_kernel(const C
         if (job >= A.njobs) break;
         JobDev& J = A.jobs[job];
         const int n = J.n;
-        if (n != have && n >= 2 && n <= kClusterSmemN) {
-            for (unsigned i = threadIdx.x; i < block_count(n); i += T) table[i] = A.table[n][i];
-            have = n;
-        }
+        const bool build = n != have;
+        have = n;
         switch (n) {
-#define CG_CLUSTER(n) case n: cluster_grow<n, true, T>(S, A, J, ws, table, cl); break;
+#define CG_CLUSTER(n) case n: cluster_grow<n, true, T>(S, A, J, ws, table, build, cl); break;
             CG_CLUSTER(2) CG_CLUSTER(3) CG_CLUSTER(4) CG_CLUSTER(5) CG_CLUSTER(6) CG_CLUSTER(7) CG_CLUSTER(8)
 #undef CG_CLUSTER
             default: break;                 // planned for n in 2..8 only
@@ -873,30 +934,6 @@ __global__ void cluster_prepare_kernel(const ClusterArgs A, unsigned want) {
             }
             for (int v = 0; v < 2 * M; ++v) key |= (uint64_t)free_[place[v]] << (4 * v);
             out[b] = key;
-        }
-    }
-}
-
-// Packed keys of one layer of a cluster growth (words F), in no particular order; see
-// block_export_kernel.
-__global__ void cluster_export_kernel(const unsigned* F, const uint64_t* table, int n, uint64_t start, uint64_t* out,
-                                      unsigned long long cap, unsigned long long* count) {
-    const unsigned total = block_count(n);
-    const int M = block_pairs(n);
-    for (unsigned b = blockIdx.x * blockDim.x + threadIdx.x; b < total; b += gridDim.x * blockDim.x) {
-        const unsigned f = F[b];
-        if (!f) continue;
-        const uint64_t p = table[b];
-        unsigned long long o = atomicAdd(count, (unsigned long long)__popc(f));
-        for (int e = 0; e < 1 << M; ++e) {
-            if (!(f >> e & 1u)) continue;
-            uint64_t key = 0;
-            for (int v = 0; v < n; ++v) {
-                const int u = v < 2 * M && (e >> (v >> 1) & 1) ? (v ^ 1) : v;
-                key |= ((start >> (4 * v)) & 15ull) << (4 * ((p >> (4 * u)) & 15ull));
-            }
-            if (o < cap) out[o] = key;
-            ++o;
         }
     }
 }
@@ -983,13 +1020,6 @@ cudaError_t launch_cluster_small(const ClusterArgs& A, int blocks, cudaStream_t 
     (void)cudaGetLastError();   // clear a stale error: the check after the launch is about this one
     if (blocks == 1) cluster_grow_small_kernel<1024><<<1, 1024, small_smem(), st>>>(A);
     else cluster_grow_small_kernel<512><<<blocks, 512, small_smem(), st>>>(A);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_cluster_export(const unsigned* F, const uint64_t* table, int n, uint64_t start, uint64_t* out,
-                                  unsigned long long cap, unsigned long long* count, cudaStream_t st) {
-    (void)cudaGetLastError();   // clear a stale error: the check after the launch is about this one
-    cluster_export_kernel<<<152, 256, 0, st>>>(F, table, n, start, out, cap, count);
     return cudaGetLastError();
 }
 

@@ -83,7 +83,7 @@ cudaError_t launch_block_export(const BlockDev& host, int which, uint64_t* out, 
 // growths of small groups, a cluster each: words of a growth of S_n, entries of its unranking table,
 // the tables of the n in the bit set `want`, clusters of `size` blocks that run at once (0: not
 // available), the growths of the queue (on a zeroed control block), blocks of the small kernel that run
-// at once and its growths, the keys of a layer
+// at once and its growths
 uint64_t cluster_words(int n);
 uint64_t cluster_table_entries(int n);
 cudaError_t launch_cluster_prepare(const ClusterArgs& A, unsigned want, cudaStream_t st);
@@ -91,8 +91,6 @@ int cluster_max_clusters(int device, int size);
 cudaError_t launch_cluster_grow(const ClusterArgs& A, int clusters, int size, cudaStream_t st);
 int cluster_small_blocks(int device);
 cudaError_t launch_cluster_small(const ClusterArgs& A, int blocks, cudaStream_t st);
-cudaError_t launch_cluster_export(const unsigned* F, const uint64_t* table, int n, uint64_t start, uint64_t* out,
-                                  unsigned long long cap, unsigned long long* count, cudaStream_t st);
 
 // Unrank the states of one layer (bitmap F, block list L[0, nlist)) into out[0, cap); *count
 // (zeroed by the caller) receives the number of states.

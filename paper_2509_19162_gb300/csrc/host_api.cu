@@ -482,8 +482,8 @@ struct cg_growth {
     char* d_blk = nullptr;                       // one allocation (BlockLayout)
     BlockDev host_block{};
     bool last_is_block = false;
-    unsigned* d_cl = nullptr;                    // one-block growth: last layer's words, unranking table
-    bool last_is_cluster = false;
+    char* d_cl = nullptr;                        // one-block growth: its one buffer (run_cluster)
+    std::vector<uint64_t> cl_layers;             // and its layer sizes
     bool served = false;                         // grown for a server: the share bounds its states
 
     JobDev host_job{};
@@ -752,32 +752,37 @@ bool cluster_preferred(const cg_growth* h) {
     return h->states_bound * 8 + bitmap_words(h->n) * 4 + (2 << 20) <= mem;
 }
 
+// One buffer, one copy each way: control block | descriptor | layer sizes | generators | last layer's
+// keys.  (The call to S_8 under adjacent transpositions takes @@ us; with the growth's usual buffers, a
+// table kernel and an export kernel it took 326 us, on the grid 312 us.)
 int run_cluster(cg_growth* h, cudaStream_t st, int* final_status) {
-    int rc = ensure_small_buffers(h, st);
-    if (rc) return rc;
+    constexpr uint64_t kHostLayers = 256;                       // come back with the first copy
+    const uint64_t o_job = al_up(sizeof(Ctl)), o_layers = o_job + al_up(sizeof(JobDev));
+    const uint64_t o_gens = o_layers + cg::kMaxLayers * sizeof(uint64_t);
+    const uint64_t o_last = o_gens + al_up(sizeof(GenSM) * h->k);
     cudaError_t e = cudaSuccess;
-    const uint64_t words = (cg::cluster_words(h->n) / 4 + 63) & ~63ull;    // of one layer: the last
     const bool fresh_alloc = h->d_cl == nullptr;
     if (fresh_alloc) {
-        h->d_cl = (unsigned*)dev_alloc(words * 4 + cg::cluster_table_entries(h->n) * 8, st);
+        h->d_cl = (char*)dev_alloc(o_last + factorial(h->n) * 8, st);
         if (!h->d_cl) return CG_ENOMEM;
+        if ((e = cudaMemcpyAsync(h->d_cl + o_gens, h->gsm.data(), sizeof(GenSM) * h->k, cudaMemcpyHostToDevice, st)) !=
+            cudaSuccess)
+            return cuda_rc(e);
+        h->stats.h2d_bytes += sizeof(GenSM) * h->k;
     }
-    JobDev J;
-    std::memset(&J, 0, sizeof(J));
+    std::vector<char> head(o_layers + kHostLayers * sizeof(uint64_t), 0);
+    JobDev& J = *reinterpret_cast<JobDev*>(head.data() + o_job);
     fill_static(h, J);
+    J.gens = reinterpret_cast<const GenSM*>(h->d_cl + o_gens);
+    J.layer_sizes = reinterpret_cast<uint64_t*>(h->d_cl + o_layers);
     J.keys_cap = ~0ull;
     cg::ClusterArgs A{};
-    A.jobs = h->d_job;
+    A.jobs = reinterpret_cast<JobDev*>(h->d_cl + o_job);
     A.njobs = 1;
-    A.last = h->d_cl;
-    A.table[h->n] = reinterpret_cast<const uint64_t*>(h->d_cl + words);
-    A.ctl = h->d_ctl;
-    if ((e = cudaMemcpyAsync(h->d_job, &J, sizeof(J), cudaMemcpyHostToDevice, st)) != cudaSuccess) return cuda_rc(e);
-    if ((e = cudaMemsetAsync(h->d_ctl, 0, sizeof(Ctl), st)) != cudaSuccess) return cuda_rc(e);
-    if (fresh_alloc) {
-        if ((e = cg::launch_cluster_prepare(A, 1u << h->n, st)) != cudaSuccess) return cuda_rc(e);
-        h->stats.launches += 1;
-    }
+    A.last = reinterpret_cast<uint64_t*>(h->d_cl + o_last);
+    for (int i = 0; i < h->n; ++i) A.start |= (h->use_start ? (h->start_key >> (4 * i)) & 15u : (uint64_t)i) << (4 * i);
+    A.ctl = reinterpret_cast<Ctl*>(h->d_cl);
+    if ((e = cudaMemcpyAsync(h->d_cl, head.data(), o_layers, cudaMemcpyHostToDevice, st)) != cudaSuccess) return cuda_rc(e);
     if (!h->ev0) {
         if ((e = cudaEventCreate(&h->ev0)) != cudaSuccess) return cuda_rc(e);
         if ((e = cudaEventCreate(&h->ev1)) != cudaSuccess) return cuda_rc(e);
@@ -785,21 +790,32 @@ int run_cluster(cg_growth* h, cudaStream_t st, int* final_status) {
     if ((e = cudaEventRecord(h->ev0, st)) != cudaSuccess) return cuda_rc(e);
     if ((e = cg::launch_cluster_small(A, 1, st)) != cudaSuccess) return cuda_rc(e);
     if ((e = cudaEventRecord(h->ev1, st)) != cudaSuccess) return cuda_rc(e);
-    Ctl ctl;
-    if ((e = cudaMemcpyAsync(&J, h->d_job, sizeof(J), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return cuda_rc(e);
-    if ((e = cudaMemcpyAsync(&ctl, h->d_ctl, sizeof(ctl), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return cuda_rc(e);
+    if ((e = cudaMemcpyAsync(head.data(), h->d_cl, head.size(), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return cuda_rc(e);
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_rc(e);
     h->stats.launches += 1;
-    h->stats.h2d_bytes += sizeof(J);
-    h->stats.d2h_bytes += sizeof(J) + sizeof(ctl);
+    h->stats.h2d_bytes += o_layers;
+    h->stats.d2h_bytes += head.size();
     h->stats.kernel_ms += elapsed_ms(h->ev0, h->ev1);
     h->stats.rounds += J.radius + 1;
+    const Ctl& ctl = *reinterpret_cast<const Ctl*>(head.data());
     if (ctl.err) return ctl.err;
+    if (J.radius < 0 || J.radius >= cg::kMaxLayers) return CG_EDEVICE;
+    const uint64_t* sizes = reinterpret_cast<const uint64_t*>(head.data() + o_layers);
+    h->cl_layers.assign(sizes, sizes + std::min<uint64_t>((uint64_t)J.radius + 1, kHostLayers));
+    if ((uint64_t)J.radius + 1 > kHostLayers) {
+        h->cl_layers.resize((size_t)J.radius + 1);
+        if ((e = cudaMemcpyAsync(h->cl_layers.data(), J.layer_sizes, sizeof(uint64_t) * h->cl_layers.size(),
+                                 cudaMemcpyDeviceToHost, st)) != cudaSuccess)
+            return cuda_rc(e);
+        if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_rc(e);
+    }
     h->stats.state_capacity = factorial(h->n);
-    h->stats.table_slots = words / 2;
+    h->stats.table_slots = 0;
     h->stats.strategy_used = CG_STRATEGY_SWEEP;
     h->stats.probe_variant = 1;
     h->host_job = J;
+    h->last_layer_ptr = A.last;
+    h->last_layer_n = h->cl_layers.back();
     *final_status = J.status;
     return CG_OK;
 }
@@ -1844,7 +1860,6 @@ int cg_growth_run(cg_growth_t h, void* cuda_stream, uint64_t* layer_sizes_out, i
     const bool use_cluster = cluster_preferred(h) && small_blocks(dev) > 0;
     const bool use_sweep = !use_cluster && (h->strategy == CG_STRATEGY_SWEEP ||
                                             (h->strategy == CG_STRATEGY_AUTO && sweep_preferred(h)));
-    h->last_is_cluster = use_cluster;
     int rc = use_cluster ? run_cluster(h, st, &status)
              : use_sort ? run_sort(h, st, &status)
                       : use_sweep ? run_sweep(h, st, &status) : run_hash(h, st, &status);
@@ -1859,6 +1874,11 @@ int cg_growth_run(cg_growth_t h, void* cuda_stream, uint64_t* layer_sizes_out, i
     const int layers = h->host_job.radius + 1;
     *num_layers_out = layers;
     if (cap < layers) return CG_EINVAL;
+    if (use_cluster) {
+        std::copy(h->cl_layers.begin(), h->cl_layers.end(), layer_sizes_out);
+        h->have_last = true;
+        return status_to_rc(status);
+    }
     if (sorted) {
         for (int r = 0; r < layers; ++r) layer_sizes_out[r] = h->sort_layers[r];
     } else {
@@ -1885,7 +1905,7 @@ int cg_growth_last_layer(cg_growth_t h, uint64_t* keys_out, uint64_t cap, uint64
             for (uint64_t i = 0; i < cnt; ++i) keys_out[2 * i + 1] &= (1ull << 60) - 1;
         return cuda_rc(e);
     }
-    if (h->last_is_block || h->last_is_cluster) {
+    if (h->last_is_block) {
         const BlockDev& D = h->host_block;
         const int radius = h->host_job.radius;
         uint64_t cnt = 0;
@@ -1900,13 +1920,7 @@ int cg_growth_last_layer(cg_growth_t h, uint64_t* keys_out, uint64_t cap, uint64
         int sms = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
         e = cudaMemsetAsync(d_count, 0, 8, nullptr);
-        if (e == cudaSuccess && h->last_is_cluster) {
-            const uint64_t words = (cg::cluster_words(h->n) / 4 + 63) & ~63ull;
-            uint64_t id = 0;
-            for (int i = 0; i < h->n; ++i) id |= (uint64_t)i << (4 * i);
-            e = cg::launch_cluster_export(h->d_cl, reinterpret_cast<const uint64_t*>(h->d_cl + words), h->n,
-                                          h->use_start ? h->start_key : id, d_out, cnt, d_count, nullptr);
-        } else if (e == cudaSuccess)
+        if (e == cudaSuccess)
             e = cg::launch_block_export(D, D.radius % 3, d_out, cnt, d_count, std::max(sms, 1) * 16, nullptr);
         unsigned long long got = 0;
         if (e == cudaSuccess) e = cudaMemcpy(&got, d_count, 8, cudaMemcpyDeviceToHost);
