@@ -604,12 +604,13 @@ __device__ __forceinline__ BlockPerm<N> cluster_unrank(const uint64_t* table, un
 template <int N>
 __device__ __forceinline__ uint64_t small_unrank(unsigned b) {
     constexpr int M = BlockShape<N>::M;
-    uint32_t avail = 0x76543210u;           // N <= 8
-    uint32_t key = 0;
+    using Nibbles = std::conditional_t<(N > 8), uint64_t, uint32_t>;
+    Nibbles avail = (Nibbles)0x9876543210ull;
+    Nibbles key = 0;
     auto take = [&](unsigned at) {
         const unsigned sh = 4u * at;
-        const uint32_t v = (avail >> sh) & 15u;
-        const uint32_t below = (1u << sh) - 1u;
+        const Nibbles v = (avail >> sh) & 15u;
+        const Nibbles below = ((Nibbles)1 << sh) - 1u;
         avail = (avail & below) | ((avail >> 4) & ~below);
         return v;
     };
@@ -631,69 +632,87 @@ __device__ __forceinline__ uint64_t small_unrank(unsigned b) {
         key |= take(hi) << (4 * (2 * i + 1));           // the larger place first: the smaller keeps its own
         key |= take(lo) << (4 * (2 * i));
     }
-    key |= (avail & 15u) | (avail & 0xF0u);             // pair 0: the two free positions, ascending
-    return key;
+    return key | (avail & 0xFFu);                       // pair 0: the two free positions, ascending
 }
 
+// Where a growth's words live: in L2 (its blocks share them through a cluster), in the shared memory of
+// the one block that grows it, or spread over the shared memory of its cluster (word i in block
+// i mod size).
+constexpr int kInL2 = 0, kInBlock = 1, kInCluster = 2;
+
 // The barrier of a growth's blocks.
-template <bool kSm>
+template <int kWhere>
 __device__ __forceinline__ void growth_sync(const cgr::cluster_group& cl) {
-    if (kSm) __syncthreads();
+    if (kWhere == kInBlock) __syncthreads();
     else cl.sync();
 }
 
 // A word of the growth that its blocks change: from shared memory, or through L2 (this SM's L1 may
 // hold words of the growth before).
-template <bool kSm>
+template <int kWhere>
 __device__ __forceinline__ unsigned growth_word(const unsigned* p) {
-    return kSm ? *(const volatile unsigned*)p : __ldcg(p);
+    return kWhere == kInL2 ? __ldcg(p) : *(const volatile unsigned*)p;
 }
 
-// kSm: one block grows the job alone, words and table in its shared memory.  T threads a block.
-template <int N, bool kSm, int T>
+// One growth by one cluster of blocks of T threads.  In shared memory (kInBlock, kInCluster) a block
+// keeps the words of its share of the blocks of states, and their unranking table, and expands them.
+template <int N, int kWhere, int T>
 __device__ __forceinline__ void cluster_grow(ClusterShared<T>& S, const ClusterArgs& A, JobDev& J, unsigned* ws,
-                                             std::conditional_t<kSm, uint64_t*, const uint64_t*> table, bool build,
+                                             std::conditional_t<kWhere != kInL2, uint64_t*, const uint64_t*> table, bool build,
                                              const cgr::cluster_group& cl) {
     constexpr unsigned kBlocks = block_count(N);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const unsigned size = kSm ? 1u : cl.num_blocks(), rank = kSm ? 0u : cl.block_rank();
+    const unsigned size = kWhere == kInBlock ? 1u : cl.num_blocks();
+    const unsigned rank = kWhere == kInBlock ? 0u : cl.block_rank();
+    // the words one array of ws holds (kInCluster: this block's share; sizes are powers of two)
+    const int sh = kWhere == kInCluster ? __ffs((int)size) - 1 : 0;
+    const unsigned held = kWhere == kInCluster ? (kBlocks + size - 1u) >> sh : kBlocks;
+    // word i of array `arr` (0: visited, 1..3: layers), wherever it is
+    auto word = [&](unsigned arr, unsigned i) -> unsigned* {
+        if constexpr (kWhere == kInCluster) return cl.map_shared_rank(ws + arr * held + (i >> sh), i & (size - 1u));
+        else return ws + arr * kBlocks + i;
+    };
     const int k = J.k;
     const GenSM* gens = J.gens;
     const bool smem = k <= kClusterGens;
-    unsigned* V = ws;
     unsigned* qidx = S.qidx[wid];
     unsigned* qf = S.qf[wid];
     unsigned* cidx = S.cidx[wid];
     unsigned* cf = S.cf[wid];
     // the words of this growth, empty
     const unsigned all = size * T, me = rank * T + tid;
-    for (unsigned i = me; i < 4 * kBlocks; i += all) ws[i] = 0;
-    if constexpr (kSm) {
+    if (kWhere == kInCluster) {
+        for (unsigned i = tid; i < 4 * held; i += T) ws[i] = 0;
+    } else {
+        for (unsigned i = me; i < 4 * kBlocks; i += all) ws[i] = 0;
+    }
+    if constexpr (kWhere != kInL2) {
         if (build)
-            for (unsigned i = tid; i < kBlocks; i += T) table[i] = small_unrank<N>(i);
+            for (unsigned i = tid; i < held; i += T)
+                table[i] = (i << sh) + rank < kBlocks ? small_unrank<N>((i << sh) + rank) : 0;
     }
     if (smem)
         for (int j = tid; j < k; j += T) S.map[j] = *reinterpret_cast<const uint4*>(gens[j].map);
     if (tid < 2) S.acc[tid] = 0;
-    growth_sync<kSm>(cl);
+    growth_sync<kWhere>(cl);
     if (me == 0) {
         uint32_t q[BlockShape<N>::kWords] = {};
         for (int v = 0; v < N; ++v) q[v >> 2] |= (uint32_t)v << (8 * (v & 3));      // the identity
         unsigned m = 0;
         const unsigned idx = block_rank<N>(q, m);
-        V[idx] = 1u << m;
-        ws[kBlocks + idx] = 1u << m;
+        *word(0, idx) = 1u << m;
+        *word(1, idx) = 1u << m;
         J.layer_sizes[0] = 1;
     }
-    growth_sync<kSm>(cl);
+    growth_sync<kWhere>(cl);
     int radius = 0, status = kRunning;
     unsigned long long states = 1;
     const int max_radius = J.max_radius, layers_cap = J.layers_cap;
     const unsigned long long max_states = J.keys_cap, stop_above = J.stop_above;
     while (status == kRunning) {
-        const unsigned* F = ws + kBlocks * (1u + (unsigned)radius % 3u);
-        unsigned* X = ws + kBlocks * (1u + (unsigned)(radius + 1) % 3u);
-        unsigned* O = ws + kBlocks * (1u + (unsigned)(radius + 2) % 3u);
+        const unsigned* F = ws + held * (1u + (unsigned)radius % 3u);
+        unsigned* O = ws + held * (1u + (unsigned)(radius + 2) % 3u);
+        const unsigned next = 1u + (unsigned)(radius + 1) % 3u;
         const int par = radius & 1;
         unsigned found = 0;
         int qn = 0, cn = 0;
@@ -702,10 +721,10 @@ __device__ __forceinline__ void cluster_grow(ClusterShared<T>& S, const ClusterA
             cn -= take;
             if (lane < take) {
                 const unsigned i = cidx[cn + lane], f = cf[cn + lane];
-                const unsigned neu = f & ~atomicOr(V + i, f);
+                const unsigned neu = f & ~atomicOr(word(0, i), f);
                 if (neu) {
                     found += __popc(neu);
-                    atomicOr(X + i, neu);
+                    atomicOr(word(next, i), neu);
                 }
             }
             __syncwarp();
@@ -740,18 +759,19 @@ __device__ __forceinline__ void cluster_grow(ClusterShared<T>& S, const ClusterA
                 if (active && !live) atomicCAS(&A.ctl->err, 0, CG_EDEVICE);
                 const unsigned t = xor_bits32(f, m);
                 unsigned v = 0;
-                if (live) v = growth_word<kSm>(V + i);
+                if (live) v = growth_word<kWhere>(word(0, i));
                 settle();
                 pidx = i;
                 pf = live ? t : 0u;
                 pv = v;
             }
         };
-        for (unsigned base = me - lane; base < kBlocks; base += all) {
+        const unsigned start = kWhere == kInCluster ? (unsigned)tid : me, step = kWhere == kInCluster ? (unsigned)T : all;
+        for (unsigned base = start - lane; base < held; base += step) {
             const unsigned i = base + lane;
             unsigned f = 0;
-            if (i < kBlocks) {
-                f = growth_word<kSm>(F + i);
+            if (i < held) {
+                f = growth_word<kWhere>(F + i);
                 O[i] = 0;
             }
             const unsigned have = __ballot_sync(0xffffffffu, f != 0);
@@ -782,10 +802,10 @@ __device__ __forceinline__ void cluster_grow(ClusterShared<T>& S, const ClusterA
             const unsigned i = block_rank<N>(q, m);
             if (live && i < kBlocks) {
                 const unsigned f = xor_bits32(qf[b], m);
-                const unsigned neu = f & ~atomicOr(V + i, f);
+                const unsigned neu = f & ~atomicOr(word(0, i), f);
                 if (neu) {
                     found += __popc(neu);
-                    atomicOr(X + i, neu);
+                    atomicOr(word(next, i), neu);
                 }
             } else if (live) {
                 atomicCAS(&A.ctl->err, 0, CG_EDEVICE);
@@ -797,13 +817,13 @@ __device__ __forceinline__ void cluster_grow(ClusterShared<T>& S, const ClusterA
         for (int o = 16; o; o >>= 1) found += __shfl_xor_sync(0xffffffffu, found, o);
         if (lane == 0 && found) atomicAdd(&S.acc[par], found);
         __syncthreads();
-        if (kSm) {
+        if (kWhere == kInBlock) {
             if (tid == 0) S.cnt[par][0] = S.acc[par];
         } else if (tid < (int)size) {
             *cl.map_shared_rank(&S.cnt[par][rank], tid) = S.acc[par];
         }
         if (tid == 0) S.acc[par ^ 1] = 0;
-        growth_sync<kSm>(cl);
+        growth_sync<kWhere>(cl);
         unsigned long long fresh = 0;
         for (unsigned q = 0; q < size; ++q) fresh += S.cnt[par][q];
         if (fresh == 0) {
@@ -823,27 +843,24 @@ __device__ __forceinline__ void cluster_grow(ClusterShared<T>& S, const ClusterA
         J.radius = radius;
         J.status = status;
     }
-    if constexpr (kSm) {
+    if constexpr (kWhere != kInL2) {
         // the last layer's packed keys, in no particular order: the value v of a state stands for the
         // start state's (see block_export_kernel)
         if (A.last == nullptr) return;
         constexpr int M = BlockShape<N>::M;
-        const unsigned* F = ws + kBlocks * (1u + (unsigned)radius % 3u);
-        __syncthreads();                    // (everyone has read the last round's counts)
-        if (tid == 0) S.cnt[0][0] = 0;
-        __syncthreads();
-        for (unsigned i = tid; i < kBlocks; i += T) {
+        const unsigned* F = ws + held * (1u + (unsigned)radius % 3u);
+        for (unsigned i = tid; i < held; i += T) {
             unsigned f = F[i];
             if (!f) continue;
-            const uint32_t p = (uint32_t)table[i];
-            unsigned at = atomicAdd(&S.cnt[0][0], (unsigned)__popc(f));
+            const uint64_t p = table[i];
+            unsigned at = (unsigned)atomicAdd(&A.ctl->adm.vis_used, (unsigned long long)__popc(f));
             for (; f; f &= f - 1u) {
                 const int e = __ffs(f) - 1;
                 uint64_t key = 0;
 #pragma unroll
                 for (int v = 0; v < N; ++v) {
                     const int swapped = v < 2 * M ? (e >> (v >> 1)) & 1 : 0;
-                    key |= ((A.start >> (4 * v)) & 15ull) << (4u * ((p >> (4 * (v ^ swapped))) & 15u));
+                    key |= ((A.start >> (4 * v)) & 15ull) << (4u * ((unsigned)(p >> (4 * (v ^ swapped))) & 15u));
                 }
                 A.last[at++] = key;
             }
@@ -868,7 +885,7 @@ __global__ void __launch_bounds__(kClThreads, 2) cluster_grow_kernel(const Clust
         if (job >= A.njobs) break;
         JobDev& J = A.jobs[job];
         switch (J.n) {
-#define CG_CLUSTER(n) case n: cluster_grow<n, false, kClThreads>(S, A, J, ws, A.table[n], false, cl); break;
+#define CG_CLUSTER(n) case n: cluster_grow<n, kInL2, kClThreads>(S, A, J, ws, A.table[n], false, cl); break;
             CG_CLUSTER(2) CG_CLUSTER(3) CG_CLUSTER(4) CG_CLUSTER(5) CG_CLUSTER(6) CG_CLUSTER(7) CG_CLUSTER(8)
             CG_CLUSTER(9) CG_CLUSTER(10)
 #undef CG_CLUSTER
@@ -902,13 +919,34 @@ __global__ void __launch_bounds__(T, 1024 / T) cluster_grow_small_kernel(const C
         const bool build = n != have;
         have = n;
         switch (n) {
-#define CG_CLUSTER(n) case n: cluster_grow<n, true, T>(S, A, J, ws, table, build, cl); break;
+#define CG_CLUSTER(n) case n: cluster_grow<n, kInBlock, T>(S, A, J, ws, table, build, cl); break;
             CG_CLUSTER(2) CG_CLUSTER(3) CG_CLUSTER(4) CG_CLUSTER(5) CG_CLUSTER(6) CG_CLUSTER(7) CG_CLUSTER(8)
 #undef CG_CLUSTER
             default: break;                 // planned for n in 2..8 only
         }
         __syncthreads();                    // everyone is done with this job's shared state
     }
+}
+
+// One growth of S_8 or S_9 by one cluster with everything in its shared memory: the issue rate of as
+// many SMs, and rounds without a trip to L2 (which blocks take part, and for which sizes: spread_blocks
+// in host_api.cu).
+constexpr int kSpreadThreads = 1024;
+__global__ void __launch_bounds__(kSpreadThreads, 1) cluster_grow_spread_kernel(const ClusterArgs A) {
+    __shared__ ClusterShared<kSpreadThreads> S;
+    extern __shared__ uint64_t s_words[];
+    const cgr::cluster_group cl = cgr::this_cluster();
+    JobDev& J = A.jobs[0];
+    const unsigned size = cl.num_blocks();
+    const unsigned held = ((J.n == 8 ? block_count(8) : block_count(9)) + size - 1u) / size;
+    unsigned* ws = reinterpret_cast<unsigned*>(s_words);
+    uint64_t* table = s_words + 2 * held;
+    switch (J.n) {
+        case 8: cluster_grow<8, kInCluster, kSpreadThreads>(S, A, J, ws, table, true, cl); break;
+        case 9: cluster_grow<9, kInCluster, kSpreadThreads>(S, A, J, ws, table, true, cl); break;
+        default: break;                     // planned for n = 8, 9 only
+    }
+    cl.sync();                              // nobody leaves while its words are in use
 }
 
 // Unranking tables of the cluster kernels, one for each n asked for: block idx -> nibble v = position
@@ -1000,6 +1038,44 @@ cudaError_t launch_cluster_grow(const ClusterArgs& A, int clusters, int size, cu
 
 namespace {
 constexpr size_t small_smem() { return (size_t)block_count(kClusterSmemN) * (4 * 4 + 8); }
+}
+
+namespace {
+size_t spread_smem(int n, int size) { return (size_t)((block_count(n) + size - 1) / size) * (4 * 4 + 8); }
+cudaLaunchConfig_t spread_config(int n, int size, cudaLaunchAttribute* attr) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)size);
+    cfg.blockDim = dim3(kSpreadThreads);
+    cfg.dynamicSmemBytes = spread_smem(n, size);
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim = {(unsigned)size, 1, 1};
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+}
+
+bool cluster_spread_ok(int n, int size) {
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = spread_config(n, size, &attr);
+    int clusters = 0;
+    if (cudaFuncSetAttribute(cluster_grow_spread_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)spread_smem(9, 4)) != cudaSuccess ||
+        cudaFuncSetAttribute(cluster_grow_spread_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&clusters, cluster_grow_spread_kernel, &cfg) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return clusters > 0;
+}
+
+cudaError_t launch_cluster_spread(const ClusterArgs& A, int n, int size, cudaStream_t st) {
+    (void)cudaGetLastError();   // clear a stale error: the check after the launch is about this one
+    cudaLaunchAttribute attr;
+    cudaLaunchConfig_t cfg = spread_config(n, size, &attr);
+    cfg.stream = st;
+    return cudaLaunchKernelEx(&cfg, cluster_grow_spread_kernel, A);
 }
 
 int cluster_small_blocks(int device) {

@@ -262,7 +262,7 @@ struct ClusterArgs {
     unsigned* words;                        // per cluster `stride` words: visited and three layers
     uint64_t stride;
     const uint64_t* table[kClusterMaxN + 1];    // unranking tables (cluster_grow_kernel)
-    uint64_t* last;                         // small kernel, one job: receives the last layer's keys (n! fit), or null
+    uint64_t* last;                         // one job in shared memory: receives the last layer's keys (n! fit), or null
     uint64_t start;                         // the start state's packed key, for `last`
     Ctl* ctl;                               // zeroed: total_units and dyn_next, the two queues; err
 };

@@ -90,6 +90,9 @@ cudaError_t launch_cluster_prepare(const ClusterArgs& A, unsigned want, cudaStre
 int cluster_max_clusters(int device, int size);
 cudaError_t launch_cluster_grow(const ClusterArgs& A, int clusters, int size, cudaStream_t st);
 int cluster_small_blocks(int device);
+// one growth of n = 8 or 9 by a cluster of `size` blocks, and whether the device runs such a cluster
+bool cluster_spread_ok(int n, int size);
+cudaError_t launch_cluster_spread(const ClusterArgs& A, int n, int size, cudaStream_t st);
 cudaError_t launch_cluster_small(const ClusterArgs& A, int blocks, cudaStream_t st);
 
 // Unrank the states of one layer (bitmap F, block list L[0, nlist)) into out[0, cap); *count

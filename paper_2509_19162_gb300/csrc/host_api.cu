@@ -404,6 +404,20 @@ int small_blocks(int dev) {
     return small_cache[dev] - 1;
 }
 
+// Blocks of the cluster that grows S_n under k generators by itself, its words and tables in shared
+// memory (0: another path).  Kernels, key list on the grid against 16 / 8 / 4 blocks: S_8 adjacent
+// transpositions 165 against 96 / 98 / 110 us, all transpositions (k = 28) 141 against 75 / 79 / 95; S_9
+// L, X 262 against 162 / 190 / 262, adjacent transpositions 258 against 198 / 247 / 364, all
+// transpositions (k = 36) 236 against 309 (sixteen SMs' issue rate); S_10 L, X 395 against 490 / - / -.
+int spread_cache[64][2] = {};
+int spread_blocks(int dev, int n, int k) {
+    if (dev < 0 || dev >= 64 || n < 8 || n > 9 || (n == 9 && k > 12)) return 0;
+    const int size = n == 8 ? 8 : 16;
+    int& c = spread_cache[dev][n - 8];
+    if (!c) c = cg::cluster_spread_ok(n, size) ? 1 : -1;
+    return c > 0 ? size : 0;
+}
+
 // Generators probed together per thread.  Hash tables (random DRAM probes): all of them when
 // k <= 4, else 4.  Rank bitmap (L2-resident, one atomic per probe): 1 -- measured fastest, and
 // the only bitmap variant that fits 64 registers without spilling.
@@ -740,21 +754,22 @@ bool block_group(const cg_growth* h) {
     return block_fits(h) && h->order * 4 >= factorial(h->n) && h->k >= min_k;
 }
 
-// A growth of S_n, n <= kClusterSmemN, by one block in its shared memory (block_path.cu).  AUTO takes it
+// A growth of S_n, n <= 9, by one block or one cluster in its shared memory (block_path.cu).  AUTO takes it
 // for groups of index at most 4 whose key list would have fitted mem_cap (so that nothing else would
 // have stopped or handed over).
 bool cluster_preferred(const cg_growth* h) {
     const uint64_t mem = h->mem_cap ? h->mem_cap : kDefaultMemCap;
     if (h->strategy != CG_STRATEGY_AUTO || !h->start_is_perm || h->width != 4 || h->n < 2 ||
-        h->n > cg::kClusterSmemN || h->grid_override > 0 || h->ilp_override > 0)
+        h->n > cg::kClusterMaxN || h->grid_override > 0 || h->ilp_override > 0)
         return false;
-    if (h->order * 4 < factorial(h->n) || (h->n == cg::kClusterSmemN && h->k > 10)) return false;
+    if (h->order * 4 < factorial(h->n)) return false;
+    if (h->n >= cg::kClusterSmemN && spread_blocks(h->device, h->n, h->k) == 0) return false;
     return h->states_bound * 8 + bitmap_words(h->n) * 4 + (2 << 20) <= mem;
 }
 
 // One buffer, one copy each way: control block | descriptor | layer sizes | generators | last layer's
-// keys.  (The call to S_8 under adjacent transpositions takes @@ us; with the growth's usual buffers, a
-// table kernel and an export kernel it took 326 us, on the grid 312 us.)
+// keys.  (The call to S_8 under adjacent transpositions, with the antipodes: 312 us on the grid; by one
+// block 326 us with the growth's usual buffers, a table kernel and an export kernel, 255 us so.)
 int run_cluster(cg_growth* h, cudaStream_t st, int* final_status) {
     constexpr uint64_t kHostLayers = 256;                       // come back with the first copy
     const uint64_t o_job = al_up(sizeof(Ctl)), o_layers = o_job + al_up(sizeof(JobDev));
@@ -788,7 +803,9 @@ int run_cluster(cg_growth* h, cudaStream_t st, int* final_status) {
         if ((e = cudaEventCreate(&h->ev1)) != cudaSuccess) return cuda_rc(e);
     }
     if ((e = cudaEventRecord(h->ev0, st)) != cudaSuccess) return cuda_rc(e);
-    if ((e = cg::launch_cluster_small(A, 1, st)) != cudaSuccess) return cuda_rc(e);
+    const int spread = spread_blocks(h->device, h->n, h->k);
+    e = spread ? cg::launch_cluster_spread(A, h->n, spread, st) : cg::launch_cluster_small(A, 1, st);
+    if (e != cudaSuccess) return cuda_rc(e);
     if ((e = cudaEventRecord(h->ev1, st)) != cudaSuccess) return cuda_rc(e);
     if ((e = cudaMemcpyAsync(head.data(), h->d_cl, head.size(), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return cuda_rc(e);
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_rc(e);
@@ -1216,12 +1233,14 @@ int run_wide(cg_growth* h, cudaStream_t st, int* final_status) {
 // pancake 0.30 / 0.19 (k = 9), all transpositions 1.01 / 0.31 (k = 45).  (2) The states, stored as
 // keys beside a rank bitmap, would not fit the memory cap while the sweep's bitmaps do.
 // A layer-size limit of at least a state per block does not change (1): S_14 pancake to the first layer
-// above 2^31 142 / 58 ms.  With a lower one, or a radius limit, the key-list path runs first: most such
+// above 2^31 142 / 58 ms; with a bitmap in L2 (n <= 12) it takes more, S_12 under six random generators
+// to the first layer above 2^24 0.83 / 1.20 ms, above 2^27 8.8 / 2.3 ms.  With a lower one, or a radius limit, the key-list path runs first: most such
 // growths stop while their layers are sparse (and see blocks_will_fill).
 bool sweep_preferred(const cg_growth* h) {
     const uint64_t mem = h->mem_cap ? h->mem_cap : kDefaultMemCap;
     if (!h->start_is_perm || h->n > 14 || h->n < 2) return false;
-    if (h->max_radius < 0 && (h->stop_above == 0 || h->stop_above >= h->order / 64) && block_group(h)) return true;
+    const uint64_t dense = h->order / (h->n >= 13 ? 64 : 8);
+    if (h->max_radius < 0 && (h->stop_above == 0 || h->stop_above >= dense) && block_group(h)) return true;
     if (h->max_radius >= 0 || h->stop_above > 0) return false;
     if (h->order * 512 < factorial(h->n)) return false;
     if (sweep_bytes(h->n) > mem) return false;

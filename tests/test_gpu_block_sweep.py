@@ -127,9 +127,9 @@ def test_served_job_over_its_share_keeps_its_layers(cg, kind, radius):
     assert (got.status, got.layers) == (want.status, want.layers)
 
 
-@pytest.mark.parametrize("n", range(2, 9))
+@pytest.mark.parametrize("n", range(2, 10))
 @pytest.mark.parametrize("kind", ["random", "random_inv", "coxeter", "lx"])
-def test_one_block_growth_every_small_n(cg, n, kind):
+def test_shared_memory_growth_every_small_n(cg, n, kind):
     gens = gens_of(kind, n, 20 + n) if n > 2 or kind in ("random", "random_inv") else [[1, 0]]
     start = np.random.default_rng(n).permutation(n).tolist()
     for lim in ({}, {"max_radius": 3}, {"stop_above": 4}):
