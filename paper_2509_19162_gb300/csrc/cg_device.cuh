@@ -358,6 +358,24 @@ __device__ __forceinline__ uint64_t rank_bytes(const ByteState<N>& s) {
     return low - clow;
 }
 
+// Rank of a binary vector of n elements with m ones among all C(n, m): sum over its ones p_1 < p_2 < ..
+// of C(p_t, t) (the combinatorial number system), six elements at a time: row c of group j holds, for
+// every value of the elements 6j .. 6j+5, their part of the sum when c ones come before them
+// (make_comb_table in host_api.cu lays the rows out, min(6j, m) + 1 of group j).  Moving elements below
+// position j leaves the parts of the ones above it alone, as with perm_rank.
+__device__ __forceinline__ uint32_t comb_rank(const uint32_t* table, uint64_t v, int n, int m) {
+    uint32_t r = 0;
+    unsigned c = 0, row = 0;
+    for (int j = 0; j < n; j += 6) {
+        const unsigned x = (unsigned)v & 63u;
+        v >>= 6;
+        r += table[(row + c) * 64u + x];
+        c += __popc(x);
+        row += (unsigned)min(j, m) + 1u;
+    }
+    return r;
+}
+
 __device__ __forceinline__ unsigned atom_add_acq_rel(unsigned* p, unsigned v) {
     unsigned old;
     asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");

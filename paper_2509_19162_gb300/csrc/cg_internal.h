@@ -133,6 +133,9 @@ constexpr uint64_t kKeyBits60 = (1ull << 60) - 1;
 
 constexpr int kVisitHash = 0;
 constexpr int kVisitBitmap = 2;
+constexpr int kVisitComb = 3;           // bitmap over the C(n, m) binary vectors (comb_rank)
+constexpr int kVariantComb = 21;        // its kernel variant
+constexpr int kCombMaxWords = 6144;     // ranking table: at most 96 rows of 64
 
 // Generators beyond the parent edge from which a rank-bitmap job reads a visited word before its
 // atomic as long as nothing better is known (a single job decides by its last round's yield, see
@@ -175,6 +178,9 @@ struct alignas(128) JobDev {
                                //    the start carries a parent-edge tag)
     int test;                  // rank bitmap, one job: the launch's first round reads visited
                                //    words before its atomics (later rounds decide themselves)
+    int ones;                  // kVisitComb: ones of a vector, ranking table and its words
+    const uint32_t* comb;
+    int comb_words;
     // dynamic, updated between rounds by block 0
     alignas(128) unsigned long long lo;     // frontier = keys[lo, hi)
     unsigned long long hi;

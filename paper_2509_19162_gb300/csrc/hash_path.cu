@@ -370,6 +370,9 @@ struct JobConst {
     int mode;
     int closed;
     int test;              // rank bitmap: read the visited word before the atomic (bitmap_test_first)
+    const uint32_t* comb;  // binary vectors (kVisitComb): ranking table, its words, ones in a vector
+    int comb_words;
+    int ones;
     int stage;             // staged states a warp holds
 };
 
@@ -620,29 +623,58 @@ __device__ __forceinline__ void bitmap_settle(const BitmapCand& a, uint64_t* buf
     if (pcnt >= 32) pend_claim(pend, pcnt, 32, buf, cnt, J, c, lane);
 }
 
-// Candidate t = generator gi of state s.
+// How a rank-bitmap job's states are read, expanded and ranked.  Permutations of N <= 14 elements:
+// byte states; sel: generator 0's selectors, `stride` words from one generator to the next.
 template <int N>
-__device__ __forceinline__ void bitmap_candidate(BitmapCand& a, const ByteState<N>& s, const uint32_t* sel,
-                                                 bool live) {
-    uint32_t head;
-    const ByteState<N> t = apply_selectors<N>(sel, s, &head);
-    const uint64_t r = rank_bytes<N>(t);
-    pack_bytes<N>(t, a.lo, a.hi);
-    a.hi |= head & 0xF0000000u;         // the parent-edge tag: the generator's inverse
-    a.w = (uint32_t)(r >> 5);
-    a.b = (uint32_t)r;
-    a.live = live;
-}
+struct PermExpand {
+    using State = ByteState<N>;
+    const uint32_t* sel;
+    int stride;
+    __device__ __forceinline__ unsigned tag(uint64_t key) const { return (unsigned)(key >> 60); }
+    __device__ __forceinline__ State load(uint64_t key) const { return unpack_bytes<N>(key); }
+    __device__ __forceinline__ void candidate(BitmapCand& a, const State& s, int gi, bool live) const {
+        uint32_t head;
+        const ByteState<N> t = apply_selectors<N>(sel + gi * stride, s, &head);
+        const uint64_t r = rank_bytes<N>(t);
+        pack_bytes<N>(t, a.lo, a.hi);
+        a.hi |= head & 0xF0000000u;         // the parent-edge tag: the generator's inverse
+        a.w = (uint32_t)(r >> 5);
+        a.b = (uint32_t)r;
+        a.live = live;
+    }
+};
+
+// Binary vectors of n <= 64 elements with m ones: packed keys, ranked among the C(n, m) < 2^32 of them
+// (comb_rank).
+struct CombExpand {
+    using State = uint64_t;
+    const GenSM* gens;
+    const uint32_t* comb;
+    int n, ones;
+    bool tagged;                            // n <= 60
+    __device__ __forceinline__ unsigned tag(uint64_t key) const { return tagged ? (unsigned)(key >> 60) : 0u; }
+    __device__ __forceinline__ State load(uint64_t key) const { return tagged ? key & kKeyBits60 : key; }
+    __device__ __forceinline__ void candidate(BitmapCand& a, State s, int gi, bool live) const {
+        const GenSM& g = gens[gi];
+        uint64_t t = apply_gen(g, s);
+        const uint32_t r = comb_rank(comb, t, n, ones);
+        if (tagged) t |= (uint64_t)g.inv_tag << 60;
+        a.lo = (uint32_t)t;
+        a.hi = (uint32_t)(t >> 32);
+        a.w = r >> 5;
+        a.b = r;
+        a.live = live;
+    }
+};
 
 // One group of 32 frontier states (one per lane), every generator applied to each.  `prev` is the
-// candidate still waiting for its visited word.  sel: generator 0's selectors, `stride` words from
-// one generator to the next.
-template <int N>
-__device__ __forceinline__ void bitmap_unit(JobDev* J, const JobConst& c, const uint32_t* sel, int stride,
-                                            bool test, bool active, uint64_t key, BitmapCand& prev, uint64_t* buf,
-                                            int& cnt, uint4* pend, int& pcnt, int lane) {
-    const unsigned tag = (unsigned)(key >> 60);   // 1 + generator that leads back to the parent
-    const ByteState<N> s = unpack_bytes<N>(key);
+// candidate still waiting for its visited word.
+template <class X>
+__device__ __forceinline__ void bitmap_unit(JobDev* J, const JobConst& c, const X& x, bool test, bool active,
+                                            uint64_t key, BitmapCand& prev, uint64_t* buf, int& cnt, uint4* pend,
+                                            int& pcnt, int lane) {
+    const unsigned tag = x.tag(key);        // 1 + generator that leads back to the parent
+    const typename X::State s = x.load(key);
     const int k = c.k;
     const bool skip = __all_sync(0xffffffffu, !active || tag != 0);
     const int iters = skip ? k - 1 : k;
@@ -652,7 +684,7 @@ __device__ __forceinline__ void bitmap_unit(JobDev* J, const JobConst& c, const 
     for (int j = 0; j < iters; ++j) {
         const int gi = j + (j >= from ? 1 : 0);
         BitmapCand a;
-        bitmap_candidate<N>(a, s, sel + gi * stride, active && tag != (unsigned)(gi + 1));
+        x.candidate(a, s, gi, active && tag != (unsigned)(gi + 1));
         bitmap_probe(a, c, test);
         bitmap_settle(prev, buf, cnt, pend, pcnt, J, c, test, lane);
         prev = a;
@@ -723,14 +755,14 @@ __device__ __forceinline__ void phase_single(JobDev* J, const JobConst& c, const
 
 // phase_single of a rank-bitmap job.  A small round (at most one unit a warp) takes a lane per
 // (state, generator) pair, as do_unit_split, with one atomicOr each.
-template <int N>
-__device__ __forceinline__ void phase_bitmap(JobDev* J, const JobConst& c, const uint32_t* sel, int stride,
-                                             bool test, unsigned long long w0, unsigned long long W, uint64_t* buf,
+template <class X>
+__device__ __forceinline__ void phase_bitmap(JobDev* J, const JobConst& c, const X& x, bool test,
+                                             unsigned long long w0, unsigned long long W, uint64_t* buf,
                                              uint4* pend, int lane, unsigned long long lo, unsigned long long hi) {
     int cnt = 0, pcnt = 0;
     const unsigned long long total = (hi - lo + 31) >> 5;
     const int m = c.k - 1;                      // generators a tagged state expands
-    if (total <= W && c.closed && lo > 0 && m >= 1 && m <= 32) {
+    if (total <= W && c.tagged && c.closed && lo > 0 && m >= 1 && m <= 32) {
         const int sp = 32 / m;
         const int lstate = lane / m, lslot = lane - lstate * m;
         const unsigned long long ts = (hi - lo + (unsigned long long)sp - 1) / (unsigned long long)sp;
@@ -738,11 +770,11 @@ __device__ __forceinline__ void phase_bitmap(JobDev* J, const JobConst& c, const
             const unsigned long long idx = lo + u * (unsigned long long)sp + (unsigned long long)lstate;
             const bool active = lstate < sp && idx < hi;
             const uint64_t key = active ? __ldcg(c.keys + idx) : 0;
-            const unsigned tag = (unsigned)(key >> 60);
+            const unsigned tag = x.tag(key);
             // generators 0..tag-2 keep their number, the rest move up by one (idle lanes: lslot itself)
             const int gi = (active && lslot >= (int)tag - 1) ? lslot + 1 : lslot;
             BitmapCand a;
-            bitmap_candidate<N>(a, unpack_bytes<N>(key), sel + gi * stride, active);
+            x.candidate(a, x.load(key), gi, active);
             bool fresh = false;
             if (active) {
                 const unsigned bit = 1u << (a.b & 31u);
@@ -772,7 +804,7 @@ __device__ __forceinline__ void phase_bitmap(JobDev* J, const JobConst& c, const
         s_next = act ? __ldcg(from + ((unsigned long long)nu << 5)) : 0;
         const bool check = (iter & 15u) == 15u;
         if ((iter & 15u) == 14u) ov = ld_relaxed_int(&J->overflow);
-        bitmap_unit<N>(J, c, sel, stride, test, active, s_cur, prev, buf, cnt, pend, pcnt, lane);
+        bitmap_unit(J, c, x, test, active, s_cur, prev, buf, cnt, pend, pcnt, lane);
         if (check && __any_sync(0xffffffffu, ov)) break;
         if (nu < u) break;              // past the last unit (the counter wrapped)
         u = nu;
@@ -787,7 +819,10 @@ __device__ __forceinline__ void bitmap_unit_n(JobDev* J, const JobConst& c, cons
                                               bool active, uint64_t key, BitmapCand& prev, uint64_t* buf, int& cnt,
                                               uint4* pend, int& pcnt, int lane) {
     switch (c.n) {
-#define CG_UNIT(n) case n: bitmap_unit<n>(J, c, sel, stride, c.test != 0, active, key, prev, buf, cnt, pend, pcnt, lane); break;
+#define CG_UNIT(n) \
+        case n: \
+            bitmap_unit(J, c, PermExpand<n>{sel, stride}, c.test != 0, active, key, prev, buf, cnt, pend, pcnt, lane); \
+            break;
         CG_UNIT(2) CG_UNIT(3) CG_UNIT(4) CG_UNIT(5) CG_UNIT(6) CG_UNIT(7) CG_UNIT(8) CG_UNIT(9) CG_UNIT(10)
         CG_UNIT(11) CG_UNIT(12) CG_UNIT(13) CG_UNIT(14)
 #undef CG_UNIT
@@ -817,12 +852,12 @@ constexpr int kGenStride = (int)sizeof(GenSM) / 4;
 // keeps registers low), whose static fields are `jc`; true: any number of jobs (of `jc` only the
 // stage size is used).
 template <int kProbeILP, int kMode, bool kMulti, int kN = 0>
-__global__ void __launch_bounds__(kGrowBlock, kMode == 2 ? 4 : ((kMode == 1 && kProbeILP >= 3) ? 2 : 3))
+__global__ void __launch_bounds__(kGrowBlock, kMode >= 2 ? 4 : ((kMode == 1 && kProbeILP >= 3) ? 2 : 3))
 hash_grow_kernel(JobDev* jobs, int njobs, unsigned long long* ubeg, Ctl* ctl, int max_rounds,
                  uint64_t timeout_ns, const AdmitDev* adm, const JobConst jc) {
-    constexpr bool kBitmap = kMode == kVisitBitmap;
+    constexpr bool kBitmap = kMode == kVisitBitmap, kComb = kMode == kVisitComb;
     extern __shared__ uint64_t s_stage[];       // jc.stage entries a warp
-    __shared__ uint4 s_pend[kBitmap ? kGrowBlock / 32 : 1][kBitmap ? kPend : 1];
+    __shared__ uint4 s_pend[kBitmap || kComb ? kGrowBlock / 32 : 1][kBitmap || kComb ? kPend : 1];
     __shared__ GenSM s_gens[!kMulti && !kBitmap ? kSmemGens : 1];
     __shared__ alignas(16) uint32_t s_selw[!kMulti && kBitmap ? kSmemSels * kSelWords : 4];
     __shared__ unsigned long long s_unit;
@@ -841,14 +876,26 @@ hash_grow_kernel(JobDev* jobs, int njobs, unsigned long long* ubeg, Ctl* ctl, in
     }
     const int lane = threadIdx.x & 31;
     uint64_t* buf = s_stage + (threadIdx.x >> 5) * jc.stage;
-    uint4* pend = s_pend[kBitmap ? threadIdx.x >> 5 : 0];
+    uint4* pend = s_pend[kBitmap || kComb ? threadIdx.x >> 5 : 0];
+    // binary vectors: the ranking table, behind the staged states
+    const uint32_t* comb = nullptr;
+    if constexpr (kComb) {
+        uint32_t* to = reinterpret_cast<uint32_t*>(s_stage + (kGrowBlock / 32) * jc.stage);
+        for (int i = threadIdx.x; i < jc.comb_words; i += blockDim.x) to[i] = jc.comb[i];
+        __syncthreads();
+        comb = to;
+    }
     // one round's work of a single job
     auto single_phase = [&](bool test, unsigned long long w0, unsigned long long W, unsigned long long lo,
                             unsigned long long hi) {
         if constexpr (kBitmap && !kMulti) {
             const bool smem = jc.k <= kSmemSels;
-            phase_bitmap<kN>(jobs, jc, smem ? s_selw : single_gens->sel, smem ? kSelWords : kGenStride, test, w0, W,
-                             buf, pend, lane, lo, hi);
+            phase_bitmap(jobs, jc,
+                         PermExpand<kN>{smem ? s_selw : single_gens->sel, smem ? kSelWords : kGenStride}, test, w0, W,
+                         buf, pend, lane, lo, hi);
+        } else if constexpr (kComb && !kMulti) {
+            phase_bitmap(jobs, jc, CombExpand{single_gens, comb, jc.n, jc.ones, jc.tagged != 0}, test, w0, W, buf,
+                         pend, lane, lo, hi);
         } else if constexpr (!kMulti) {
             phase_single<kProbeILP, kMode>(jobs, jc, single_gens, w0, W, buf, lane, lo, hi);
         }
@@ -1073,6 +1120,9 @@ __device__ void init_job(JobDev& J) {
     if (J.mode == kVisitBitmap) {
         const uint64_t r = perm_rank(id, J.n);
         atomicOr(reinterpret_cast<unsigned*>(J.table) + (r >> 5), 1u << (unsigned)(r & 31u));
+    } else if (J.mode == kVisitComb) {
+        const uint32_t r = comb_rank(J.comb, id, J.n, J.ones);
+        atomicOr(reinterpret_cast<unsigned*>(J.table) + (r >> 5), 1u << (r & 31u));
     } else {
         table_insert(J.table, J.table_mask, id, kMaxProbe);
     }
@@ -1203,6 +1253,7 @@ GrowFn grow_fn_t(int variant) {
         case 10: return hash_grow_kernel<2, 1, M>;
         case 11: return hash_grow_kernel<3, 1, M>;
         case 12: return hash_grow_kernel<4, 1, M>;
+        case kVariantComb: return hash_grow_kernel<1, M ? 2 : kVisitComb, M, 0>;    // (single jobs only)
         default: return hash_grow_kernel<1, 2, M, M ? 0 : 14>;   // (single jobs: grow_fn_bitmap_n)
     }
 }
@@ -1219,7 +1270,7 @@ GrowFn grow_fn_bitmap_n(int n, std::integer_sequence<int, Ns...>) {
 }
 
 GrowFn grow_fn(int variant, bool multi, int n) {
-    if (variant >= 17 && !multi && n >= 2 && n <= 14)
+    if (variant >= 17 && variant != kVariantComb && !multi && n >= 2 && n <= 14)
         return grow_fn_bitmap_n<1>(n, std::make_integer_sequence<int, 13>{});
     return grow_fn(variant, multi);
 }
@@ -1228,7 +1279,14 @@ GrowFn grow_fn(int variant, bool multi, int n) {
 int hash_grow_max_grid(int device, int ilp, bool multi) {
     int sms = 0, per_sm = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
-    const size_t smem = (size_t)(kGrowBlock / 32) * stage_entries(multi, ilp >= 16, false) * sizeof(uint64_t);
+    const size_t smem = ilp == kVariantComb
+                            ? (size_t)(kGrowBlock / 32) * kStageTest * sizeof(uint64_t) + (size_t)kCombMaxWords * 4
+                            : (size_t)(kGrowBlock / 32) * stage_entries(multi, ilp >= 16, false) * sizeof(uint64_t);
+    if (ilp == kVariantComb &&
+        cudaFuncSetAttribute(grow_fn(ilp, multi), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, grow_fn(ilp, multi), kGrowBlock, smem) !=
         cudaSuccess)
         return 0;
@@ -1265,7 +1323,7 @@ cudaError_t launch_hash_grow(JobDev* d_jobs, int njobs, unsigned long long* d_ub
     // copy of them, one job runs through the general kernel.
     const bool multi = njobs > 1 || d_adm != nullptr || host_job == nullptr;
     JobConst jc = {};
-    jc.stage = stage_entries(multi, ilp >= 16, !multi && host_job->test != 0);
+    jc.stage = ilp == kVariantComb ? kStageTest : stage_entries(multi, ilp >= 16, !multi && host_job->test != 0);
     if (!multi) {
         jc.keys = host_job->keys;
         jc.keys_cap = host_job->keys_cap;
@@ -1278,11 +1336,14 @@ cudaError_t launch_hash_grow(JobDev* d_jobs, int njobs, unsigned long long* d_ub
         jc.mode = host_job->mode;
         jc.closed = host_job->closed;
         jc.test = host_job->test;
+        jc.comb = host_job->comb;
+        jc.comb_words = host_job->comb_words;
+        jc.ones = host_job->ones;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kGrowBlock);
-    cfg.dynamicSmemBytes = (size_t)(kGrowBlock / 32) * jc.stage * sizeof(uint64_t);
+    cfg.dynamicSmemBytes = (size_t)(kGrowBlock / 32) * jc.stage * sizeof(uint64_t) + (size_t)jc.comb_words * 4;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;

@@ -326,6 +326,25 @@ bool bitmap_eligible(int n, uint64_t order, uint64_t mem) {
     return bitmap_fits(n, mem) && order * 512 >= factorial(n);
 }
 
+// Ranking table of binary vectors of n elements with m ones (comb_rank in cg_device.cuh).
+std::vector<uint32_t> make_comb_table(int n, int m) {
+    uint64_t C[65][65] = {};                // C(i, j), saturated at 2^32: larger ones are in no rank
+    for (int i = 0; i <= 64; ++i)
+        for (int j = 0; j <= i; ++j)
+            C[i][j] = j == 0 ? 1 : std::min<uint64_t>(C[i - 1][j - 1] + (j < i ? C[i - 1][j] : 0), 1ull << 32);
+    std::vector<uint32_t> t;
+    for (int j = 0; j < n; j += 6)
+        for (int c = 0; c <= std::min(j, m); ++c)
+            for (unsigned x = 0; x < 64; ++x) {
+                uint64_t sum = 0;
+                int q = c;
+                for (int i = 0; i < 6; ++i)
+                    if (x >> i & 1u) { ++q; sum += j + i <= 64 && q <= 64 ? C[j + i][q] : 0; }
+                t.push_back((uint32_t)sum);
+            }
+    return t;
+}
+
 // Largest state capacity whose keys + table fit in `mem` bytes.
 uint64_t max_cap_for_mem(uint64_t mem) {
     uint64_t best = 0;
@@ -381,7 +400,7 @@ int device_grid_cache[64][32][2] = {};
 // Blocks of the persistent kernel that fit co-resident on device `dev` (variant: ILP 1..4, +8
 // for whole-sector table probing, +16 for the rank bitmap; multi: several jobs per launch).
 int grow_grid(int dev, int ilp, bool multi = false) {
-    if (dev < 0 || dev >= 64 || ilp < 1 || ilp > 20) return 0;
+    if (dev < 0 || dev >= 64 || ilp < 1 || ilp > cg::kVariantComb) return 0;
     int& c = device_grid_cache[dev][ilp][multi ? 1 : 0];
     if (!c) c = cg::hash_grow_max_grid(dev, ilp, multi);
     return c;
@@ -450,6 +469,9 @@ struct cg_growth {
     uint64_t start_key = 0;
     bool start_is_perm = true;                   // the start vector has distinct entries
     uint64_t states_bound = 1;                   // states the growth can reach (orbit bound)
+    uint64_t rearrangements = 0;                 // of the start vector (saturating)
+    uint32_t* d_comb = nullptr;                  // binary vectors: ranking table
+    std::vector<uint32_t> comb;
     uint64_t order = 1;
     int device = -1;
     cudaStream_t alloc_stream = nullptr;
@@ -513,6 +535,8 @@ struct cg_growth {
         dev_free(d_layers, st);
         dev_free(d_keys, st);
         dev_free(d_table, st);
+        dev_free(d_comb, st);
+        d_comb = nullptr;
         d_gens = nullptr; d_job = nullptr; d_ctl = nullptr; d_ubeg = nullptr;
         d_layers = nullptr; d_keys = nullptr; d_table = nullptr;
         keys_cap = table_slots = 0;
@@ -573,13 +597,27 @@ int ensure_small_buffers(cg_growth* h, cudaStream_t st) {
     return CG_OK;
 }
 
+// Bitmap over the rearrangements of a binary start vector.
+uint64_t comb_bytes(const cg_growth* h) { return (h->rearrangements + 63) / 64 * 8; }
+
+// The orbit of a binary vector in one word, most of whose rearrangements it may reach: the visited set
+// is a bitmap over them, a bit each where the hash table takes 16 bytes a state, and fits L2 to n = 32
+// (75 MB; the table 16 GB).  Only where the hash table and every state would have fitted as well, so
+// that nothing else would have stopped the growth or handed it over.
+bool comb_preferred(const cg_growth* h, uint64_t mem) {
+    if (h->strategy != CG_STRATEGY_AUTO || !h->use_start || h->start_is_perm || h->wide || h->width != 1) return false;
+    if (h->rearrangements >> 32 || h->rearrangements > 512 * h->states_bound) return false;
+    if (bytes_for(h->states_bound) + (2 << 20) > mem) return false;
+    return h->states_bound * 8 + comb_bytes(h) <= std::min<uint64_t>(mem, kExactAllocLimit);
+}
+
 // (Re)allocate keys + table for `cap` states, keeping the first `keep` keys.
 int resize_state(cg_growth* h, uint64_t cap, uint64_t keep, cudaStream_t st) {
     uint64_t* keys = (uint64_t*)dev_alloc(cap * 8, st);
     if (!keys) return CG_ENOMEM;
-    if (h->mode == cg::kVisitBitmap) {   // the bitmap has a fixed size: allocate it once
+    if (h->mode == cg::kVisitBitmap || h->mode == cg::kVisitComb) {   // of a fixed size: allocate it once
         if (!h->d_table) {
-            h->table_slots = bitmap_words(h->n) / 2;
+            h->table_slots = h->mode == cg::kVisitComb ? comb_bytes(h) / 8 : bitmap_words(h->n) / 2;
             h->d_table = (uint64_t*)dev_alloc(h->table_slots * 8, st);
             if (!h->d_table) { dev_free(keys, st); return CG_ENOMEM; }
         }
@@ -628,6 +666,9 @@ void fill_static(cg_growth* h, JobDev& J) {
     J.closed = 1;
     for (const GenSM& g : h->gsm) J.closed &= g.inv_tag != 0 ? 1 : 0;
     J.test = h->k - J.closed >= cg::kTestMinDegree ? 1 : 0;
+    J.comb = h->d_comb;
+    J.comb_words = (int)h->comb.size();
+    J.ones = __builtin_popcountll(h->start_key);
 }
 
 bool block_fits(const cg_growth* h) {
@@ -876,15 +917,22 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
         h->mode = (h->strategy == CG_STRATEGY_BITMAP ||
                    (h->strategy == CG_STRATEGY_AUTO && h->start_is_perm &&
                     bitmap_eligible(h->n, h->order, mem)))
-                      ? cg::kVisitBitmap : cg::kVisitHash;
+                      ? cg::kVisitBitmap : comb_preferred(h, mem) ? cg::kVisitComb : cg::kVisitHash;
+        h->comb.clear();
+        if (h->mode == cg::kVisitComb) {
+            h->comb = make_comb_table(h->n, __builtin_popcountll(h->start_key));
+            if (h->comb.size() > (size_t)cg::kCombMaxWords) h->mode = cg::kVisitHash;
+        }
     }
-    const bool bitmap = h->mode == cg::kVisitBitmap;
+    const bool bitmap = h->mode == cg::kVisitBitmap, comb = h->mode == cg::kVisitComb;
     h->last_is_block = false;
-    const int ilp = (h->ilp_override > 0 ? h->ilp_override : default_ilp(h->k, bitmap)) + (bitmap ? 16 : 0);
+    const int ilp = comb ? cg::kVariantComb
+                         : (h->ilp_override > 0 ? h->ilp_override : default_ilp(h->k, bitmap)) + (bitmap ? 16 : 0);
     const uint64_t avail = mem > (1 << 20) ? mem - (1 << 20) : mem;
     const uint64_t bm_bytes = bitmap ? bitmap_words(h->n) * 4 : 0;
     const uint64_t max_cap = std::min<uint64_t>(
-        h->states_bound, bitmap ? (avail > bm_bytes ? (avail - bm_bytes) / 8 : 0) : max_cap_for_mem(avail));
+        h->states_bound, comb ? h->states_bound
+                         : bitmap ? (avail > bm_bytes ? (avail - bm_bytes) / 8 : 0) : max_cap_for_mem(avail));
     if (max_cap < 1) return CG_ENOMEM;
     // radius limit: a growth that may go on in blocks of states (blocks_will_fill) begins with room
     // for its sparse layers, beside which the blocks have to fit
@@ -895,13 +943,20 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
                      block_layout(h->n, h->k).bytes + bm_bytes + first_cap * 8 + (1 << 20) <= mem;
     uint64_t list_cap = h->states_bound;
     {
-        const uint64_t need = bitmap ? list_cap * 8 + bm_bytes : bytes_for(list_cap);
+        const uint64_t need = comb ? 0 : bitmap ? list_cap * 8 + bm_bytes : bytes_for(list_cap);
         if (need > std::min<uint64_t>(mem, kExactAllocLimit)) list_cap = std::min<uint64_t>(max_cap, 1ull << 24);
         list_cap = std::max<uint64_t>(std::min(list_cap, max_cap), 1);
     }
     if (!h->d_keys) {
         rc = resize_state(h, may_block ? std::min<uint64_t>(first_cap, 1ull << 28) : list_cap, 0, st);
         if (rc) return rc;
+    }
+    if (comb && !h->d_comb) {
+        h->d_comb = (uint32_t*)dev_alloc(h->comb.size() * 4, st);
+        if (!h->d_comb) return CG_ENOMEM;
+        const cudaError_t ec = cudaMemcpyAsync(h->d_comb, h->comb.data(), h->comb.size() * 4, cudaMemcpyHostToDevice, st);
+        if (ec != cudaSuccess) return cuda_rc(ec);
+        h->stats.h2d_bytes += h->comb.size() * 4;
     }
     const int grid_max = grow_grid(h->device, ilp);
     if (grid_max <= 0) return CG_ECUDA;
@@ -910,7 +965,7 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
     int grid = (int)std::min<uint64_t>((uint64_t)grid_max, std::max<uint64_t>(want, 1));
     if (h->grid_override > 0) grid = std::min(grid_max, h->grid_override);
 
-    cudaError_t e = cudaMemsetAsync(h->d_table, bitmap ? 0 : 0xFF, h->table_slots * 8, st);
+    cudaError_t e = cudaMemsetAsync(h->d_table, bitmap || comb ? 0 : 0xFF, h->table_slots * 8, st);
     if (e != cudaSuccess) return cuda_rc(e);
     JobDev J;
     std::memset(&J, 0, sizeof(J));
@@ -1042,6 +1097,7 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
             continue;
         }
         if (J.status != cg::kNeedMem) break;
+        if (comb) return CG_EDEVICE;        // every state has its place: never expected
         if (h->keys_cap >= max_cap) break;  // cannot grow: truncated by mem_cap
         // Grow: keep layers 0..radius (keys[0, hi)), rebuild the visited table from them.
         const uint64_t keep = J.hi;
@@ -1070,7 +1126,7 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
     }
     h->stats.state_capacity = h->keys_cap;
     h->stats.table_slots = h->table_slots;
-    h->stats.strategy_used = bitmap ? CG_STRATEGY_BITMAP : CG_STRATEGY_HASH;
+    h->stats.strategy_used = bitmap || comb ? CG_STRATEGY_BITMAP : CG_STRATEGY_HASH;
     h->stats.probe_variant = ilp;
     h->host_job = J;
     *final_status = J.status;
@@ -1800,6 +1856,7 @@ int cg_growth_set_start(cg_growth_t h, const uint8_t* start) {
     else { h->wgsm = wg; h->gsm.clear(); }
     h->wstart = wkey;
     h->states_bound = std::min(h->order, rearr);
+    h->rearrangements = rearr;
     return CG_OK;
 }
 

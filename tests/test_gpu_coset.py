@@ -154,3 +154,24 @@ def test_long_vector_limits(cg):
     # 62 elements of 2 bits take two-word keys: the orbit of 3 0^61 is the 62 positions of the 3
     r = cg.growth(62, w.coxeter(62), start=[3] + [0] * 61)
     assert r.layers == [1] * 62
+
+
+@pytest.mark.parametrize("n,m", [(2, 1), (6, 3), (7, 1), (12, 6), (13, 4), (18, 9), (19, 12), (24, 12), (31, 5), (60, 3), (61, 3),
+                                 (64, 3)])
+@pytest.mark.parametrize("family", ["lrx", "lx", "pancake", "consecutive_4cycles"])
+def test_binary_cosets_on_the_arrangement_bitmap(cg, n, m, family):
+    # AUTO's bitmap over the C(n, m) arrangements against the hash table; n = 61..64 leave no tag bits
+    if n < 5 and family == "consecutive_4cycles":
+        pytest.skip("needs four elements")
+    gens = w.FAMILIES[family](n)
+    start = np.random.default_rng(n * 100 + m).permutation([1] * m + [0] * (n - m)).tolist()
+    with cg.Growth(n, gens, strategy="hash", start=start) as g:
+        want, far = g.run(), np.sort(g.last_layer())
+    with cg.Growth(n, gens, start=start) as g:
+        for _ in range(2):
+            got = g.run()
+            assert (got.status, got.layers) == (want.status, want.layers)
+            assert np.array_equal(np.sort(g.last_layer()), far)
+        assert g.stats()["strategy_used"] == 3
+        g.set_start([1 - v for v in start] if m != 1 else start[::-1])    # another vector on the same handle
+        assert sum(g.run().layers) <= math.comb(n, m)
