@@ -362,8 +362,13 @@ __device__ __forceinline__ uint64_t rank_bytes(const ByteState<N>& s) {
 // of C(p_t, t) (the combinatorial number system), six elements at a time: row c of group j holds, for
 // every value of the elements 6j .. 6j+5, their part of the sum when c ones come before them
 // (make_comb_table in host_api.cu lays the rows out, min(6j, m) + 1 of group j).  Moving elements below
-// position j leaves the parts of the ones above it alone, as with perm_rank.
+// position j leaves the parts of the ones above it alone, as with perm_rank.  m < 0: the vector has -m
+// zeros, and they are ranked.
 __device__ __forceinline__ uint32_t comb_rank(const uint32_t* table, uint64_t v, int n, int m) {
+    if (m < 0) {
+        v ^= n >= 64 ? ~0ull : (1ull << n) - 1ull;
+        m = -m;
+    }
     uint32_t r = 0;
     unsigned c = 0, row = 0;
     for (int j = 0; j < n; j += 6) {

@@ -98,6 +98,15 @@ struct WideGen {
     uint64_t mhi[kMaxWideTerms];
 };
 
+// Ranking of a start vector's arrangements (wide_rank in wide_path.cu): `steps` steps of `bits` key
+// bits, `states` rows of 1 << bits words a step.  table: 1 << bits count increments, then the rows.
+// steps = 0: none.
+constexpr int kWideRankWords = 12288;       // at most 48 KB
+struct WideRank {
+    const uint32_t* table;
+    int steps, bits, states, words;
+};
+
 // One growth with two-word keys (hash strategy): every layer back to back in `keys`, the visited
 // set an open-addressing table of 16-byte slots (empty = all ones).  A state found by generator g
 // carries the tag (1 + index of g's inverse) in bits 124-127 when n w <= 124.
@@ -178,7 +187,7 @@ struct alignas(128) JobDev {
                                //    the start carries a parent-edge tag)
     int test;                  // rank bitmap, one job: the launch's first round reads visited
                                //    words before its atomics (later rounds decide themselves)
-    int ones;                  // kVisitComb: ones of a vector, ranking table and its words
+    int ones;                  // kVisitComb: ones of a vector (< 0: zeros), ranking table and its words
     const uint32_t* comb;
     int comb_words;
     // dynamic, updated between rounds by block 0

@@ -50,9 +50,9 @@ cudaError_t launch_owner_partition(const GenSM* d_gens, int k, const uint64_t* i
                                    cudaStream_t st);
 
 // two-word keys (wide_path.cu): one growth of vectors of more than 64 bits
-int wide_max_grid(int device);
-cudaError_t launch_wide_init(WideDev* d, cudaStream_t st);
-cudaError_t launch_wide_grow(WideDev* d, Ctl* ctl, int grid, int max_rounds, uint64_t timeout_ns,
+int wide_max_grid(int device, const WideRank& R);
+cudaError_t launch_wide_init(WideDev* d, const WideRank& R, cudaStream_t st);
+cudaError_t launch_wide_grow(WideDev* d, Ctl* ctl, const WideRank& R, int grid, int max_rounds, uint64_t timeout_ns,
                              cudaStream_t st);
 cudaError_t launch_wide_rebuild(const Key128* keys, unsigned long long count, Key128* table, uint64_t mask,
                                 int tagged, int* d_err, int grid, cudaStream_t st);

@@ -373,6 +373,7 @@ struct JobConst {
     const uint32_t* comb;  // binary vectors (kVisitComb): ranking table, its words, ones in a vector
     int comb_words;
     int ones;
+    uint64_t start;
     int stage;             // staged states a warp holds
 };
 
@@ -652,8 +653,13 @@ struct CombExpand {
     const uint32_t* comb;
     int n, ones;
     bool tagged;                            // n <= 60
+    uint64_t start;
     __device__ __forceinline__ unsigned tag(uint64_t key) const { return tagged ? (unsigned)(key >> 60) : 0u; }
-    __device__ __forceinline__ State load(uint64_t key) const { return tagged ? key & kKeyBits60 : key; }
+    // (a lane without a state, key 0, takes the start's: comb_rank looks up only vectors with `ones` ones)
+    __device__ __forceinline__ State load(uint64_t key) const {
+        const uint64_t s = tagged ? key & kKeyBits60 : key;
+        return s ? s : start;
+    }
     __device__ __forceinline__ void candidate(BitmapCand& a, State s, int gi, bool live) const {
         const GenSM& g = gens[gi];
         uint64_t t = apply_gen(g, s);
@@ -894,7 +900,7 @@ hash_grow_kernel(JobDev* jobs, int njobs, unsigned long long* ubeg, Ctl* ctl, in
                          PermExpand<kN>{smem ? s_selw : single_gens->sel, smem ? kSelWords : kGenStride}, test, w0, W,
                          buf, pend, lane, lo, hi);
         } else if constexpr (kComb && !kMulti) {
-            phase_bitmap(jobs, jc, CombExpand{single_gens, comb, jc.n, jc.ones, jc.tagged != 0}, test, w0, W, buf,
+            phase_bitmap(jobs, jc, CombExpand{single_gens, comb, jc.n, jc.ones, jc.tagged != 0, jc.start}, test, w0, W, buf,
                          pend, lane, lo, hi);
         } else if constexpr (!kMulti) {
             phase_single<kProbeILP, kMode>(jobs, jc, single_gens, w0, W, buf, lane, lo, hi);
@@ -1339,6 +1345,7 @@ cudaError_t launch_hash_grow(JobDev* d_jobs, int njobs, unsigned long long* d_ub
         jc.comb = host_job->comb;
         jc.comb_words = host_job->comb_words;
         jc.ones = host_job->ones;
+        jc.start = host_job->start_key;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);

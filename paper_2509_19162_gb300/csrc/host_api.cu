@@ -8,6 +8,7 @@
 // (within mem_cap), rebuilds the visited table from the stored states and relaunches.
 #include <algorithm>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <mutex>
 #include <new>
@@ -345,6 +346,79 @@ std::vector<uint32_t> make_comb_table(int n, int m) {
     return t;
 }
 
+// Ranking tables of the arrangements of vector v (n elements of w bits in two words; wide_rank in
+// wide_path.cu), for the widest step whose tables fit: {bits, steps, states} or an empty table when
+// none does.  The most frequent value is left out of the counts (position minus the others).
+std::vector<uint32_t> make_wide_rank(const uint8_t* v, int n, int w, cg::WideRank& R) {
+    int count[16] = {0}, base = 0;
+    for (int i = 0; i < n; ++i) count[v[i]]++;
+    for (int x = 1; x < 16; ++x)
+        if (count[x] > count[base]) base = x;
+    uint64_t stride[16] = {0}, states = 1;
+    for (int x = 0; x < 16; ++x)
+        if (x != base && count[x]) { stride[x] = states; states *= (uint64_t)count[x] + 1; if (states > 65536) return {}; }
+    std::vector<uint64_t> C(129 * 129, 0);        // binomials, saturated at 2^32
+    for (int i = 0; i <= n; ++i)
+        for (int j = 0; j <= i; ++j)
+            C[(size_t)i * 129 + j] =
+                j == 0 ? 1 : std::min<uint64_t>(C[(size_t)(i - 1) * 129 + j - 1] + C[(size_t)(i - 1) * 129 + j], 1ull << 32);
+    for (int bits = 8; bits >= 4; bits -= 4) {
+        const int per = bits / w, steps = (n + per - 1) / per;
+        const uint64_t words = (1ull << bits) * (1 + (uint64_t)steps * states);
+        if (words > (uint64_t)cg::kWideRankWords) continue;
+        std::vector<uint32_t> t(words, 0);
+        // arrangements of positions that hold c[x] of each value: a multinomial as a product of
+        // binomials, 2^32 and above (in no rank) as 2^32
+        auto multinomial = [&](const int* c) {
+            uint64_t r = 1;
+            int placed = 0;
+            for (int x = 0; x < 16 && !(r >> 32); ++x) {
+                if (c[x] == 0) continue;
+                placed += c[x];
+                r *= C[(size_t)placed * 129 + (size_t)c[x]];         // (both factors at most 2^32)
+            }
+            return r >> 32 ? 1ull << 32 : r;
+        };
+        for (unsigned x = 0; x < 1u << bits; ++x) {
+            uint64_t add = 0;
+            for (int q = 0; q < per; ++q) add += stride[(x >> (w * q)) & ((1u << w) - 1u)];
+            t[x] = (uint32_t)add;
+        }
+        for (int s = 0; s < steps; ++s)
+            for (uint64_t id = 0; id < states; ++id) {
+                int before[16] = {0};
+                int known = 0;
+                for (int x = 0; x < 16; ++x)
+                    if (stride[x]) { before[x] = (int)(id / stride[x] % ((uint64_t)count[x] + 1)); known += before[x]; }
+                before[base] = s * per - known;
+                if (before[base] < 0 || before[base] > count[base]) continue;       // no vector comes here
+                for (unsigned x = 0; x < 1u << bits; ++x) {
+                    int c[16];
+                    std::memcpy(c, before, sizeof(c));
+                    uint64_t sum = 0;
+                    bool ok = true;
+                    for (int q = 0; q < per && s * per + q < n && ok; ++q) {
+                        const int val = (int)((x >> (w * q)) & ((1u << w) - 1u));
+                        ok = ++c[val] <= count[val];
+                        for (int u = 0; u < val && ok; ++u) {
+                            if (c[u] == 0) continue;
+                            c[u]--;
+                            sum += multinomial(c);
+                            c[u]++;
+                        }
+                    }
+                    if (ok) t[(1ull << bits) + (((uint64_t)s * states + id) << bits) + x] = (uint32_t)sum;
+                }
+            }
+        R.bits = bits;
+        R.steps = steps;
+        R.states = (int)states;
+        R.words = (int)words;
+        return t;
+    }
+    return {};
+}
+
 // Largest state capacity whose keys + table fit in `mem` bytes.
 uint64_t max_cap_for_mem(uint64_t mem) {
     uint64_t best = 0;
@@ -507,6 +581,10 @@ struct cg_growth {
     cg::Key128* d_wtable = nullptr;
     uint64_t wtable_slots = 0;
     cg::WideDev host_wide{};
+    cg::WideRank wrank{};                        // arrangement bitmap instead of the table (steps > 0)
+    std::vector<uint32_t> wrank_table;
+    std::vector<uint8_t> start_values;
+    uint32_t* d_wrank = nullptr;
 
     // sweep strategy: visited bitmap, two layer bitmaps with block bits and block lists
     SweepDev* d_sweep = nullptr;
@@ -552,6 +630,8 @@ struct cg_growth {
         dev_free(d_wjob, st);
         dev_free(d_wkeys, st);
         dev_free(d_wtable, st);
+        dev_free(d_wrank, st);
+        d_wrank = nullptr;
         d_wgens = nullptr; d_wjob = nullptr; d_wkeys = nullptr; d_wtable = nullptr;
         wkeys_cap = wtable_slots = 0;
         release_sort(st);
@@ -595,6 +675,12 @@ int ensure_small_buffers(cg_growth* h, cudaStream_t st) {
         if (e != cudaSuccess) return cuda_rc(e);
     }
     return CG_OK;
+}
+
+// What comb_rank counts: the ones of a binary start vector, or, negative, its zeros when they are fewer.
+int comb_ones(const cg_growth* h) {
+    const int m = __builtin_popcountll(h->start_key);
+    return 2 * m > h->n ? m - h->n : m;
 }
 
 // Bitmap over the rearrangements of a binary start vector.
@@ -668,7 +754,7 @@ void fill_static(cg_growth* h, JobDev& J) {
     J.test = h->k - J.closed >= cg::kTestMinDegree ? 1 : 0;
     J.comb = h->d_comb;
     J.comb_words = (int)h->comb.size();
-    J.ones = __builtin_popcountll(h->start_key);
+    J.ones = comb_ones(h);
 }
 
 bool block_fits(const cg_growth* h) {
@@ -920,8 +1006,11 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
                       ? cg::kVisitBitmap : comb_preferred(h, mem) ? cg::kVisitComb : cg::kVisitHash;
         h->comb.clear();
         if (h->mode == cg::kVisitComb) {
-            h->comb = make_comb_table(h->n, __builtin_popcountll(h->start_key));
-            if (h->comb.size() > (size_t)cg::kCombMaxWords) h->mode = cg::kVisitHash;
+            h->comb = make_comb_table(h->n, std::abs(comb_ones(h)));
+            if (h->comb.size() > (size_t)cg::kCombMaxWords) {
+                h->comb.clear();
+                h->mode = cg::kVisitHash;
+            }
         }
     }
     const bool bitmap = h->mode == cg::kVisitBitmap, comb = h->mode == cg::kVisitComb;
@@ -1143,7 +1232,7 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
 // (Re)allocate states and table for `cap` states keeping the first `keep` states.
 int resize_wide(cg_growth* h, uint64_t cap, uint64_t keep, cudaStream_t st) {
     auto* keys = (cg::Key128*)dev_alloc(cap * 16, st);
-    const uint64_t slots = table_slots_for(cap);
+    const uint64_t slots = h->wrank.steps ? (h->rearrangements + 127) / 128 : table_slots_for(cap);   // (of 16 bytes)
     auto* table = (cg::Key128*)dev_alloc(slots * 16, st);
     if (!keys || !table) { dev_free(keys, st); dev_free(table, st); return CG_ENOMEM; }
     if (keep > 0) {
@@ -1183,10 +1272,29 @@ int run_wide(cg_growth* h, cudaStream_t st, int* final_status) {
         if (e != cudaSuccess) return cuda_rc(e);
         h->stats.h2d_bytes += sizeof(cg::WideGen) * h->k;
     }
+    // The visited set of a start vector most of whose arrangements the growth may reach is a bitmap over
+    // them where their number and the ranking tables allow it, and only where the hash table and every
+    // state would have fitted as well, so that nothing else would have stopped the growth.  40 elements
+    // of four values under L, R, X: 19.7 M states, 2.5 MB of bitmap in L2 for a table of 1 GB, kernel 3.68 / 2.20 ms.
+    const bool whole = h->states_bound <= max_cap && h->states_bound * 48 <= std::min<uint64_t>(mem, kExactAllocLimit);
+    if (!h->d_wkeys) {
+        h->wrank = cg::WideRank{};
+        if (h->strategy == CG_STRATEGY_AUTO && h->use_start && whole && !(h->rearrangements >> 32) &&
+            h->rearrangements <= 512 * h->states_bound)
+            h->wrank_table = make_wide_rank(h->start_values.data(), h->n, h->width, h->wrank);
+    }
+    if (h->wrank.steps && !h->d_wrank) {
+        h->d_wrank = (uint32_t*)dev_alloc(h->wrank_table.size() * 4, st);
+        if (!h->d_wrank) return CG_ENOMEM;
+        const cudaError_t ec = cudaMemcpyAsync(h->d_wrank, h->wrank_table.data(), h->wrank_table.size() * 4,
+                                               cudaMemcpyHostToDevice, st);
+        if (ec != cudaSuccess) return cuda_rc(ec);
+        h->wrank.table = h->d_wrank;
+        h->stats.h2d_bytes += h->wrank_table.size() * 4;
+    }
     if (!h->d_wkeys) {
         uint64_t start = std::min<uint64_t>(max_cap, 1ull << 22);
-        if (h->states_bound <= max_cap && h->states_bound * 48 <= std::min<uint64_t>(mem, kExactAllocLimit))
-            start = h->states_bound;
+        if (whole) start = h->states_bound;
         if ((rc = resize_wide(h, std::max<uint64_t>(start, 1), 0, st))) return rc;
     }
     const int tagged = h->n * h->width <= 124 ? 1 : 0;
@@ -1208,10 +1316,10 @@ int run_wide(cg_growth* h, cudaStream_t st, int* final_status) {
     cg::WideDev D;
     std::memset(&D, 0, sizeof(D));
     fill(D);
-    cudaError_t e = cudaMemsetAsync(h->d_wtable, 0xFF, h->wtable_slots * 16, st);
+    cudaError_t e = cudaMemsetAsync(h->d_wtable, h->wrank.steps ? 0 : 0xFF, h->wtable_slots * 16, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_wjob, &D, sizeof(D), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->d_ctl, 0, sizeof(Ctl), st);
-    if (e == cudaSuccess) e = cg::launch_wide_init(h->d_wjob, st);
+    if (e == cudaSuccess) e = cg::launch_wide_init(h->d_wjob, h->wrank, st);
     if (e != cudaSuccess) return cuda_rc(e);
     h->stats.launches += 1;
     h->stats.h2d_bytes += sizeof(D);
@@ -1219,14 +1327,14 @@ int run_wide(cg_growth* h, cudaStream_t st, int* final_status) {
         if ((e = cudaEventCreate(&h->ev0)) != cudaSuccess) return cuda_rc(e);
         if ((e = cudaEventCreate(&h->ev1)) != cudaSuccess) return cuda_rc(e);
     }
-    const int grid_max = cg::wide_max_grid(h->device);
+    const int grid_max = cg::wide_max_grid(h->device, h->wrank);
     if (grid_max <= 0) return CG_ECUDA;
     int grid = (int)std::min<uint64_t>((uint64_t)grid_max, h->states_bound / 512 + 1);
     if (h->grid_override > 0) grid = std::min(grid_max, h->grid_override);
     for (;;) {
         if ((e = cudaMemsetAsync(h->d_ctl, 0, sizeof(Ctl), st)) != cudaSuccess) return cuda_rc(e);
         if ((e = cudaEventRecord(h->ev0, st)) != cudaSuccess) return cuda_rc(e);
-        if ((e = cg::launch_wide_grow(h->d_wjob, h->d_ctl, grid, cg::kMaxLayers + 1, kTimeoutNs, st)) != cudaSuccess)
+        if ((e = cg::launch_wide_grow(h->d_wjob, h->d_ctl, h->wrank, grid, cg::kMaxLayers + 1, kTimeoutNs, st)) != cudaSuccess)
             return cuda_rc(e);
         if ((e = cudaEventRecord(h->ev1, st)) != cudaSuccess) return cuda_rc(e);
         h->stats.launches += 1;
@@ -1241,6 +1349,7 @@ int run_wide(cg_growth* h, cudaStream_t st, int* final_status) {
         h->stats.rounds += ctl.rounds;
         if (ctl.err) return ctl.err;
         if (D.status != cg::kNeedMem) break;
+        if (h->wrank.steps) return CG_EDEVICE;    // every state has its place: never expected
         if (h->wkeys_cap >= max_cap) break;   // cannot grow: truncated by mem_cap
         const uint64_t keep = D.hi;
         const uint64_t newcap = std::min<uint64_t>(max_cap, std::max<uint64_t>(h->wkeys_cap * 4, keep + 1));
@@ -1265,7 +1374,7 @@ int run_wide(cg_growth* h, cudaStream_t st, int* final_status) {
     }
     h->stats.state_capacity = h->wkeys_cap;
     h->stats.table_slots = h->wtable_slots;
-    h->stats.strategy_used = CG_STRATEGY_HASH;
+    h->stats.strategy_used = h->wrank.steps ? CG_STRATEGY_BITMAP : CG_STRATEGY_HASH;
     h->stats.probe_variant = 1;
     h->host_wide = D;
     std::memset(&h->host_job, 0, sizeof(h->host_job));
@@ -1857,6 +1966,7 @@ int cg_growth_set_start(cg_growth_t h, const uint8_t* start) {
     h->wstart = wkey;
     h->states_bound = std::min(h->order, rearr);
     h->rearrangements = rearr;
+    h->start_values.assign(start, start + h->n);
     return CG_OK;
 }
 

@@ -115,6 +115,36 @@ __device__ __forceinline__ int table_insert128(Key128* table, uint64_t mask, con
     return -1;
 }
 
+// Rank of a vector among the arrangements of its values (fewer than 2^32 of them), `bits` key bits (one
+// or more elements) a step from element 0 up: the sum over positions i of the arrangements of elements
+// 0..i that agree in their counts and hold a lower value at i.  What a step adds depends on its bits and
+// on how many of each value came before: row `id` of the step, id = sum of the counts times strides, to
+// which a step adds its bits' own counts (WideRank, make_wide_rank in host_api.cu).
+__device__ __forceinline__ uint32_t wide_rank(const uint32_t* s_rank, const WideRank& R, const Key128& t) {
+    const uint32_t* row = s_rank + (1u << R.bits);      // behind the 1 << bits count increments
+    const unsigned mask = (1u << R.bits) - 1u, rows = (unsigned)R.states << R.bits;
+    uint32_t r = 0, id = 0;
+    uint64_t v = t.lo;
+    for (int s = 0; s < R.steps; ++s) {
+        if (s * R.bits == 64) v = t.hi;
+        const unsigned x = (unsigned)v & mask;
+        v >>= R.bits;
+        r += row[(id << R.bits) + x];
+        id += s_rank[x];
+        row += rows;
+    }
+    return r;
+}
+
+// A candidate whose visited word (an atomicOr on the arrangement bitmap) has been asked for but not yet
+// looked at: the next one is computed meanwhile.
+struct WideCand {
+    Key128 t;                 // tagged
+    uint32_t r;
+    unsigned old;
+    bool live;
+};
+
 __device__ __forceinline__ void wide_flush(Key128* buf, int& cnt, WideDev* J, int lane) {
     if (cnt == 0) return;
     unsigned long long base = 0;
@@ -173,6 +203,50 @@ __device__ __forceinline__ void wide_unit(WideDev* J, const WideGen* gens, unsig
     }
 }
 
+__device__ __forceinline__ void wide_settle(const WideCand& a, Key128* buf, int& cnt, WideDev* J, int lane) {
+    const bool neu = a.live && !(a.old >> (a.r & 31u) & 1u);
+    const unsigned fresh = __ballot_sync(0xffffffffu, neu);
+    if (neu) buf[cnt + __popc(fresh & lanemask_lt())] = a.t;
+    cnt += __popc(fresh);
+    __syncwarp();
+    if (cnt > kWideStage - 32) wide_flush(buf, cnt, J, lane);
+}
+
+// wide_unit on an arrangement bitmap.
+__device__ __forceinline__ void wide_unit_rank(WideDev* J, const WideGen* gens, const uint32_t* s_rank, const WideRank& R,
+                                               unsigned* bitmap, unsigned long long idx, unsigned long long hi,
+                                               WideCand& prev, Key128* buf, int& cnt, int lane) {
+    const bool active = idx < hi;
+    Key128 s = J->start;        // (a lane without a state: wide_rank looks up only arrangements of the start)
+    if (active) {
+        const ulonglong2 v = __ldcg(reinterpret_cast<const ulonglong2*>(J->keys + idx));
+        s.lo = v.x;
+        s.hi = v.y;
+    }
+    const bool tagged = J->tagged != 0;
+    unsigned tag = 0;
+    if (tagged && active) {
+        tag = (unsigned)(s.hi >> 60);
+        s.hi &= kTag124;
+    }
+    const int k = J->k;
+    const bool skip = tagged && __all_sync(0xffffffffu, !active || tag != 0);
+    const int iters = skip ? k - 1 : k;
+    for (int j = 0; j < iters; ++j) {
+        // (lanes without a state have tag 0 and take j + 1 <= k - 1)
+        const int g = (skip && (int)tag - 1 <= j) ? j + 1 : j;
+        WideCand a;
+        a.t = apply_wide(gens[g], s);
+        a.r = wide_rank(s_rank, R, a.t);
+        a.live = active && tag != (unsigned)(g + 1);
+        a.old = 0;
+        if (a.live) a.old = atomicOr(bitmap + (a.r >> 5), 1u << (a.r & 31u));
+        if (tagged) a.t.hi |= (uint64_t)gens[g].inv_tag << 60;
+        wide_settle(prev, buf, cnt, J, lane);
+        prev = a;
+    }
+}
+
 // Close a layer (one thread of the block that arrived last): |L_{r+1}| = tail - hi, stop tests.
 __device__ void wide_close(WideDev* J, Ctl* ctl) {
     volatile WideDev* V = J;
@@ -201,8 +275,12 @@ __device__ void wide_close(WideDev* J, Ctl* ctl) {
     __threadfence();
 }
 
+// kRank: the visited set is a bitmap over the arrangements of the start vector's values (R; its tables
+// in dynamic shared memory), else the table of 16-byte slots.
+template <bool kRank>
 __global__ void __launch_bounds__(kWideBlock, 2)
-wide_grow_kernel(WideDev* J, Ctl* ctl, int max_rounds, uint64_t timeout_ns) {
+wide_grow_kernel(WideDev* J, Ctl* ctl, int max_rounds, uint64_t timeout_ns, const WideRank R) {
+    extern __shared__ uint32_t s_rank[];
     __shared__ Key128 s_stage[kWideBlock / 32][kWideStage];
     __shared__ WideGen s_gens[kWideSmemGens];
     __shared__ unsigned long long s_lo, s_hi, s_unit;
@@ -213,6 +291,11 @@ wide_grow_kernel(WideDev* J, Ctl* ctl, int max_rounds, uint64_t timeout_ns) {
         __syncthreads();
         gens = s_gens;
     }
+    if (kRank) {
+        for (int i = threadIdx.x; i < R.words; i += blockDim.x) s_rank[i] = R.table[i];
+        __syncthreads();
+    }
+    unsigned* bitmap = reinterpret_cast<unsigned*>(J->table);
     const int lane = threadIdx.x & 31;
     Key128* buf = s_stage[threadIdx.x >> 5];
     unsigned nbar = 0;                      // grid barriers this block has passed
@@ -230,14 +313,19 @@ wide_grow_kernel(WideDev* J, Ctl* ctl, int max_rounds, uint64_t timeout_ns) {
         if (threadIdx.x == 0) s_unit = ub;
         __syncthreads();
         int cnt = 0;
+        WideCand prev{{0, 0}, 0, 0, false};
         for (;;) {
             unsigned long long u = 0;
             if (lane == 0) u = atomicAdd(&s_unit, 1ull);
             u = __shfl_sync(0xffffffffu, u, 0);
             if (u >= ue) break;
-            wide_unit(J, gens, lo + (u << 5) + lane, hi, buf, cnt, lane);
+            if (kRank)
+                wide_unit_rank(J, gens, s_rank, R, bitmap, lo + (u << 5) + lane, hi, prev, buf, cnt, lane);
+            else
+                wide_unit(J, gens, lo + (u << 5) + lane, hi, buf, cnt, lane);
             if (__any_sync(0xffffffffu, ld_relaxed_int(&J->overflow))) break;
         }
+        if (kRank) wide_settle(prev, buf, cnt, J, lane);
         wide_flush(buf, cnt, J, lane);
         unsigned long long word = 0;
         const int arrive = grid_arrive(ctl, timeout_ns, word, nbar++);
@@ -249,10 +337,15 @@ wide_grow_kernel(WideDev* J, Ctl* ctl, int max_rounds, uint64_t timeout_ns) {
     }
 }
 
-__global__ void wide_init_kernel(WideDev* J) {
+__global__ void wide_init_kernel(WideDev* J, const WideRank R) {
     if (blockIdx.x != 0 || threadIdx.x != 0) return;
     J->keys[0] = J->start;
-    table_insert128(J->table, J->table_mask, J->start, kWideMaxProbe);
+    if (R.steps) {
+        const uint32_t r = wide_rank(R.table, R, J->start);
+        atomicOr(reinterpret_cast<unsigned*>(J->table) + (r >> 5), 1u << (r & 31u));
+    } else {
+        table_insert128(J->table, J->table_mask, J->start, kWideMaxProbe);
+    }
     J->layer_sizes[0] = 1;
     J->lo = 0;
     J->hi = 1;
@@ -275,33 +368,43 @@ __global__ void wide_rebuild_kernel(const Key128* keys, unsigned long long count
 
 }  // namespace
 
-int wide_max_grid(int device) {
+namespace {
+using WideFn = void (*)(WideDev*, Ctl*, int, uint64_t, const WideRank);
+WideFn wide_fn(const WideRank& R) { return R.steps ? wide_grow_kernel<true> : wide_grow_kernel<false>; }
+}
+
+int wide_max_grid(int device, const WideRank& R) {
     int sms = 0, per_sm = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wide_grow_kernel, kWideBlock, 0) != cudaSuccess)
+    const size_t smem = R.steps ? (size_t)kWideRankWords * 4 : 0;
+    if (smem && cudaFuncSetAttribute(wide_fn(R), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+        (void)cudaGetLastError();
         return 0;
+    }
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wide_fn(R), kWideBlock, smem) != cudaSuccess) return 0;
     return sms * per_sm;
 }
 
-cudaError_t launch_wide_init(WideDev* d, cudaStream_t st) {
+cudaError_t launch_wide_init(WideDev* d, const WideRank& R, cudaStream_t st) {
     (void)cudaGetLastError();   // clear a stale error: the check after the launch is about this one
-    wide_init_kernel<<<1, 32, 0, st>>>(d);
+    wide_init_kernel<<<1, 32, 0, st>>>(d, R);
     return cudaGetLastError();
 }
 
-cudaError_t launch_wide_grow(WideDev* d, Ctl* ctl, int grid, int max_rounds, uint64_t timeout_ns,
+cudaError_t launch_wide_grow(WideDev* d, Ctl* ctl, const WideRank& R, int grid, int max_rounds, uint64_t timeout_ns,
                              cudaStream_t st) {
     (void)cudaGetLastError();   // clear a stale error: the check after the launch is about this one
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kWideBlock);
+    cfg.dynamicSmemBytes = R.steps ? (size_t)R.words * 4 : 0;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, wide_grow_kernel, d, ctl, max_rounds, timeout_ns);
+    return cudaLaunchKernelEx(&cfg, wide_fn(R), d, ctl, max_rounds, timeout_ns, R);
 }
 
 cudaError_t launch_wide_rebuild(const Key128* keys, unsigned long long count, Key128* table, uint64_t mask,

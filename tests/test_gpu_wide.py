@@ -158,3 +158,24 @@ def test_two_word_memcap_truncation_and_last_layer(cg):
 def test_constant_start_vector_is_fixed(cg):
     assert cg.growth(32, w.lrx(32), start=[15] * 32).layers == [1]
     assert cg.growth(64, w.coxeter(64)[:3], start=[3] * 64).layers == [1]
+
+
+@pytest.mark.parametrize("counts", [(33, 2, 1), (40, 2, 1, 1), (62, 3), (3, 62), (64, 2), (16, 2, 0, 0, 0, 1),
+                                    (0, 30, 2, 1)])
+@pytest.mark.parametrize("family", ["lrx", "lx"])
+def test_two_word_arrangement_bitmap(cg, counts, family):
+    # AUTO's bitmap over the arrangements of the start vector against the table of 16-byte slots
+    start = [v for v, c in enumerate(counts) for _ in range(c)]
+    n = len(start)
+    start = np.random.default_rng(n).permutation(start).tolist()
+    gens = w.FAMILIES[family](n)
+    with cg.Growth(n, gens, strategy="hash", start=start) as g:
+        want, far = g.run(), g.last_layer()
+        assert g.stats()["strategy_used"] == 1
+    with cg.Growth(n, gens, start=start) as g:
+        for _ in range(2):
+            got, last = g.run(), g.last_layer()
+            assert (got.status, got.layers) == (want.status, want.layers)
+            assert sorted(map(tuple, last.tolist())) == sorted(map(tuple, far.tolist()))
+        if g.key_words == 2:
+            assert g.stats()["strategy_used"] == 3
