@@ -416,16 +416,14 @@ __device__ __forceinline__ int grid_arrive(Ctl* ctl, uint64_t timeout_ns, unsign
     __syncthreads();
     if (threadIdx.x == 0) {
         gen &= (unsigned)kGenMask;
-        const unsigned g = blockIdx.x % kBarGroups;
-        const unsigned gsize = (gridDim.x - g + kBarGroups - 1) / kBarGroups;
-        const unsigned ngroups = gridDim.x < (unsigned)kBarGroups ? gridDim.x : (unsigned)kBarGroups;
         int state = 0;
         unsigned long long w = gen;
-        // The counters only grow (zeroed before each launch): barrier `gen` is complete in a
-        // group when its counter reaches gsize * (gen + 1), so nothing is reset on the way.
-        if (atom_add_acq_rel(&ctl->group[g].count, 1u) == gsize * (gen + 1) - 1) {
-            if (atom_add_acq_rel(&ctl->bar_count, 1u) == ngroups * (gen + 1) - 1) state = 1;
-        }
+        // The counter only grows (zeroed before each launch): barrier `gen` is complete when it reaches
+        // gridDim.x * (gen + 1), so nothing is reset on the way.  One counter for every block: the last
+        // arrival is one L2 round trip from the release, and 608 additions queue for less than the second
+        // trip that a level of group counters costs (S_10 under L, X, 59 rounds: 0.401 ms with 32 groups,
+        // 0.360 ms so; S_11 under L, R, X 1.016 / 0.981 ms).
+        if (atom_add_acq_rel(&ctl->bar_count, 1u) == gridDim.x * (gen + 1) - 1) state = 1;
         if (state == 0) {
             const uint64_t t0 = globaltimer_ns();
             unsigned spins = 0;

@@ -298,10 +298,8 @@ struct AdmitDev {
 };
 
 // Control block of the persistent kernel (device memory, zero-initialised by the host).
-// Blocks arrive at the grid barrier on kBarGroups group counters, the last of each group on
-// the top counter; every counter and the generation word that waiting blocks poll sit in
-// their own 128-byte line, so neither arrivals nor polling queue at one L2 slice.
-constexpr int kBarGroups = 32;
+// The counter on which blocks arrive at the grid barrier and the generation word that waiting blocks
+// poll sit in their own 128-byte lines, so arrivals and polling do not queue at one L2 slice.
 constexpr int kGenBits = 20;
 constexpr unsigned long long kGenMask = (1ull << kGenBits) - 1;
 
@@ -321,10 +319,6 @@ struct alignas(128) Ctl {
     // second half, which blocks that finish their range draw from this counter.
     unsigned long long dyn_next;
     unsigned int pad3[30];
-    struct alignas(128) Group {
-        unsigned int count;
-        unsigned int pad[31];
-    } group[kBarGroups];
     // Admission of a batch into one launch (AdmitDev), updated by the block that closes a round.
     struct alignas(128) Admit {
         int act_sel;                    // AdmitDev::act[act_sel] lists the active jobs
