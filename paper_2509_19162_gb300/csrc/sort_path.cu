@@ -50,7 +50,7 @@ __device__ __forceinline__ unsigned long long make_desc(unsigned epoch, unsigned
 // (independent loads), sums aggregates in order and stops at the first inclusive prefix; a
 // window with an unpublished descriptor is read again from there.  Sets *err and returns 0 if
 // a predecessor never publishes in time.
-constexpr int kWindow = 8;
+constexpr int kWindow = 4;       // (a growth of S_11 under L, R, X: 13.3 ms with 4, 14.4 with 8, 19 with 32)
 
 __device__ unsigned long long look_back(unsigned long long* desc, int stride, int tile, unsigned long long agg,
                                         unsigned epoch, int* err) {
@@ -94,6 +94,48 @@ __device__ unsigned long long look_back(unsigned long long* desc, int stride, in
     return prefix;
 }
 
+// look_back for one chain by one whole warp: the lanes read 32 predecessors' descriptors at once.
+// Every lane returns the exclusive prefix.
+__device__ unsigned long long look_back_warp(unsigned long long* desc, int tile, unsigned long long agg, unsigned epoch,
+                                             int* err, int lane) {
+    if (tile == 0) {
+        if (lane == 0) atomicExch(desc, make_desc(epoch, 2, agg));
+        return 0;
+    }
+    if (lane == 0) atomicExch(desc + tile, make_desc(epoch, 1, agg));
+    unsigned long long prefix = 0;
+    int t = tile - 1;
+    const uint64_t t0 = globaltimer_ns();
+    unsigned spins = 0;
+    for (;;) {
+        const unsigned long long d = t - lane >= 0 ? ld_relaxed_ull(desc + (t - lane)) : 0;
+        const unsigned status = t - lane >= 0 && (unsigned)(d >> 60) == epoch ? (unsigned)(d >> 58) & 3u : 0u;
+        const unsigned missing = __ballot_sync(0xffffffffu, status == 0);
+        const unsigned whole = __ballot_sync(0xffffffffu, status == 2);
+        // the descriptors before the first unpublished one, and not past the first inclusive prefix
+        int use = missing ? __ffs((int)missing) - 1 : 32;
+        const int stop = whole ? __ffs((int)whole) - 1 : 32;
+        const bool done = stop < use;
+        if (done) use = stop + 1;
+        unsigned long long v = lane < use ? d & kValMask : 0;
+#pragma unroll
+        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        prefix += v;
+        t -= use;
+        if (done || t < 0) break;           // (t < 0 never comes first: tile 0 publishes an inclusive prefix)
+        if (use == 0 && (++spins & 7u) == 0) {
+            const bool late = globaltimer_ns() - t0 > kSpinTimeoutNs;
+            if (__any_sync(0xffffffffu, *(volatile int*)err != 0)) return 0;
+            if (__any_sync(0xffffffffu, late)) {
+                if (lane == 0) atomicCAS(err, 0, CG_ETIMEOUT);
+                return 0;
+            }
+        }
+    }
+    if (lane == 0) atomicExch(desc + tile, make_desc(epoch, 2, prefix + agg));
+    return prefix;
+}
+
 // Block-wide exclusive scan of one value per thread (kBlock threads); *total = block sum.
 template <typename T>
 __device__ __forceinline__ T block_excl_scan(T v, T* total) {
@@ -123,9 +165,17 @@ __device__ __forceinline__ T block_excl_scan(T v, T* total) {
     return excl;
 }
 
+// Candidate number i, given the generator `first` of an earlier one: a division per tile instead of one
+// per candidate.
+__device__ __forceinline__ uint64_t gen_candidate_from(const ExpandSrc& src, unsigned long long i, unsigned first) {
+    unsigned long long off = i - (unsigned long long)first * src.F;
+    unsigned g = first;
+    while (off >= src.F) { off -= src.F; ++g; }
+    return apply_gen(src.gens[g], src.frontier[off]);
+}
+
 __device__ __forceinline__ uint64_t gen_candidate(const ExpandSrc& src, unsigned long long i) {
-    const unsigned g = (unsigned)(i / src.F);
-    return apply_gen(src.gens[g], src.frontier[i - (unsigned long long)g * src.F]);
+    return gen_candidate_from(src, i, (unsigned)(i / src.F));
 }
 
 // ---- expand (standalone: the step-level cg_expand and the memory hand-off) ----------------
@@ -149,6 +199,7 @@ __global__ void expand_all_kernel(const GenSM* __restrict__ gens, int k, const u
 }
 
 // ---- digit histograms of every pass in one read ------------------------------------------
+// kGen: the candidates of src, a state's k together (one read of the frontier).
 template <bool kGen>
 __global__ void __launch_bounds__(kBlock)
 hist_all_kernel(const uint64_t* __restrict__ keys, ExpandSrc src, unsigned long long n, int passes, int lo,
@@ -157,9 +208,14 @@ hist_all_kernel(const uint64_t* __restrict__ keys, ExpandSrc src, unsigned long 
     for (int i = threadIdx.x; i < kSortMaxPasses * kDigits; i += kBlock) (&s_h[0][0])[i] = 0;
     __syncthreads();
     const unsigned long long stride = (unsigned long long)gridDim.x * kBlock;
-    for (unsigned long long i = blockIdx.x * (unsigned long long)kBlock + threadIdx.x; i < n; i += stride) {
-        const uint64_t key = kGen ? gen_candidate(src, i) : keys[i];
-        for (int p = 0; p < passes; ++p) atomicAdd(&s_h[p][(key >> (lo + kRadixBits * p)) & (kDigits - 1)], 1u);
+    const unsigned long long items = kGen ? src.F : n;
+    const int each = kGen ? src.k : 1;
+    for (unsigned long long i = blockIdx.x * (unsigned long long)kBlock + threadIdx.x; i < items; i += stride) {
+        const uint64_t in = kGen ? src.frontier[i] : keys[i];
+        for (int g = 0; g < each; ++g) {
+            const uint64_t key = kGen ? apply_gen(src.gens[g], in) : in;
+            for (int p = 0; p < passes; ++p) atomicAdd(&s_h[p][(key >> (lo + kRadixBits * p)) & (kDigits - 1)], 1u);
+        }
     }
     __syncthreads();
     for (int i = threadIdx.x; i < passes * kDigits; i += kBlock) {
@@ -172,7 +228,7 @@ hist_all_kernel(const uint64_t* __restrict__ keys, ExpandSrc src, unsigned long 
 // Warp w of a tile holds the tile's keys w*512 + r*32 + lane (r < kItems), so row-major order
 // is input order and the ranks are stable.
 template <bool kGen>
-__global__ void __launch_bounds__(kBlock, 2)
+__global__ void __launch_bounds__(kBlock, 3)
 onesweep_kernel(const uint64_t* __restrict__ in, ExpandSrc src, uint64_t* __restrict__ out, unsigned long long n,
                 int shift, const unsigned long long* __restrict__ ghist_p, unsigned long long* desc,
                 unsigned* ticket, unsigned epoch, int* err) {
@@ -181,8 +237,12 @@ onesweep_kernel(const uint64_t* __restrict__ in, ExpandSrc src, uint64_t* __rest
     __shared__ unsigned long long s_base[kDigits];
     __shared__ uint64_t s_stage[kTile];
     __shared__ int s_tile;
+    __shared__ unsigned s_gen;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    if (tid == 0) s_tile = (int)atomicAdd(ticket, 1u);
+    if (tid == 0) {
+        s_tile = (int)atomicAdd(ticket, 1u);
+        s_gen = kGen ? (unsigned)((unsigned long long)s_tile * kTile / src.F) : 0u;    // of the tile's first candidate
+    }
     for (int i = tid; i < kWarps * kDigits; i += kBlock) (&s_whist[0][0])[i] = 0;
     __syncthreads();
     const int tile = s_tile;
@@ -192,19 +252,29 @@ onesweep_kernel(const uint64_t* __restrict__ in, ExpandSrc src, uint64_t* __rest
 #pragma unroll
     for (int r = 0; r < kItems; ++r) {
         const unsigned long long idx = base + (unsigned)(wid * (kItems * 32) + r * 32 + lane);
-        key[r] = idx < n ? (kGen ? gen_candidate(src, idx) : in[idx]) : 0;
+        key[r] = idx < n ? (kGen ? gen_candidate_from(src, idx, s_gen) : in[idx]) : 0;
     }
+    // A key's rank among the warp's keys of its digit.  The lanes of a row that share a digit are found
+    // with a vote per digit bit, their first lane
+    // adds their number to the warp's count, and the rows' additions, in program order, need not wait
+    // for one another.
 #pragma unroll
     for (int r = 0; r < kItems; ++r) {
         const unsigned long long idx = base + (unsigned)(wid * (kItems * 32) + r * 32 + lane);
-        const unsigned d = idx < n ? (unsigned)(key[r] >> shift) & (kDigits - 1) : (unsigned)kDigits;
-        const unsigned peers = __match_any_sync(0xffffffffu, d);
-        const unsigned lt = __popc(peers & lanemask_lt());
-        const unsigned run = d < (unsigned)kDigits ? s_whist[wid][d] : 0u;
-        rank[r] = run + lt;
-        __syncwarp();
-        if (d < (unsigned)kDigits && lt == 0) s_whist[wid][d] = run + __popc(peers);
-        __syncwarp();
+        const unsigned d = (unsigned)(key[r] >> shift) & (kDigits - 1);
+        unsigned peers = __ballot_sync(0xffffffffu, idx < n);
+#pragma unroll
+        for (int q = 0; q < kRadixBits; ++q) {
+            const bool one = (d >> q) & 1u;
+            const unsigned v = __ballot_sync(0xffffffffu, one);
+            peers &= one ? v : ~v;
+        }
+        // (a lane past the end shares no key's count: its own bit is not in `peers`)
+        const int first = __ffs((int)peers) - 1;
+        unsigned run = 0;
+        if (lane == first) run = atomicAdd(&s_whist[wid][d], (unsigned)__popc(peers));
+        run = __shfl_sync(0xffffffffu, run, first < 0 ? lane : first);
+        rank[r] = run + __popc(peers & lanemask_lt());
     }
     __syncthreads();
     // thread d: the tile's count of digit d, exclusive over warps in place
@@ -381,9 +451,12 @@ unique_diff_kernel(const uint64_t* __restrict__ a, unsigned long long na, const 
     }
     unsigned total = 0;
     const unsigned excl = block_excl_scan<unsigned>(cnt, &total);   // ends with __syncthreads
-    if (tid == 0) {
-        s_prefix = look_back(desc, 1, tile, total, epoch, err);
-        if (tile == ntiles - 1 && *(volatile int*)err == 0) *d_count = s_prefix + total;
+    if (wid == 0) {
+        const unsigned long long before = look_back_warp(desc, tile, total, epoch, err, lane);
+        if (lane == 0) {
+            s_prefix = before;
+            if (tile == ntiles - 1 && *(volatile int*)err == 0) *d_count = before + total;
+        }
     }
     unsigned pos = excl;
 #pragma unroll
@@ -632,7 +705,7 @@ cudaError_t radix_passes(const uint64_t* in, const ExpandSrc* src, unsigned long
     cudaError_t e = cudaMemsetAsync(s.ghist, 0, reset, st);
     if (e != cudaSuccess) return e;
     const ExpandSrc none{};
-    unsigned long long hb = (n + kBlock - 1) / kBlock;
+    unsigned long long hb = ((src ? src->F : n) + kBlock - 1) / kBlock;
     if (hb > 152ull * 4) hb = 152ull * 4;
     if (src) hist_all_kernel<true><<<(unsigned)hb, kBlock, 0, st>>>(nullptr, *src, n, P, lo, s.ghist);
     else hist_all_kernel<false><<<(unsigned)hb, kBlock, 0, st>>>(in, none, n, P, lo, s.ghist);
@@ -704,7 +777,7 @@ cudaError_t launch_candidate_hist(const ExpandSrc& src, int bits, const SortScra
     const unsigned long long n = src.F * (unsigned long long)src.k;
     cudaError_t e = cudaMemsetAsync(s.ghist, 0, sizeof(unsigned long long) * kSortMaxPasses * kDigits, st);
     if (e != cudaSuccess || n == 0) return e;
-    unsigned long long hb = (n + kBlock - 1) / kBlock;
+    unsigned long long hb = (src.F + kBlock - 1) / kBlock;
     if (hb > 152ull * 4) hb = 152ull * 4;
     hist_all_kernel<true><<<(unsigned)hb, kBlock, 0, st>>>(nullptr, src, n, passes_of(bits - lo < 1 ? 1 : bits - lo),
                                                           lo, s.ghist);
