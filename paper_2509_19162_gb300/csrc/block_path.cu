@@ -346,8 +346,11 @@ __device__ void block_close(BlockDev& D, Ctl* ctl) {
     __threadfence();
 }
 
+// Bound by issue and the latency of what is left between (S_12 pancake: 2.18 G warp instructions, issue
+// slots 50 % busy, DRAM at 11 % of its rate, 64 % of L2 accesses hit): four blocks an SM at 64 registers
+// are faster than three at 77 (S_12 pancake 3.27 / 3.52 ms, S_13 pancake 47.3 / 51.9 ms).
 template <int N>
-__global__ void __launch_bounds__(kBlkThreads, 3)
+__global__ void __launch_bounds__(kBlkThreads, 4)
 block_grow_kernel(BlockDev* Dp, Ctl* ctl, int max_rounds, uint64_t timeout_ns) {
     using Word = typename BlockShape<N>::Word;
     __shared__ uint4 s_map[kBlockSmemGens];
