@@ -375,11 +375,16 @@ def run_ours(args):
     # kernel names as ncu prints them: the single-job bitmap kernel with one generator in
     # flight is compiled per n (last template argument), every other variant has 0 there
     per_n = job.n if (strat_name == "bitmap" and variant == 17 and 2 <= job.n <= 14) else 0
+    # the sweep's forms in blocks of states report variant 1 (state by state: min(k, 2) generators)
+    in_blocks = strat_name == "sweep" and variant == 1 and job.k > 1
+    block_kernel = (f"block_grow_kernel<{job.n}>" if job.n >= 10 else
+                    f"cluster_grow_{'spread_kernel' if job.n >= 8 else 'small_kernel<1024>'}")
     # the sweep's block order changes its memory traffic: its ncu record names the order
     launch_settings = {"sweep_order": args.sweep_order} if strat_name == "sweep" else None
     kernel_name = {"sort": "radix sort / merge-path kernels",
-                   "sweep": f"sweep_grow_kernel<{min(variant, 2)}, {job.n}>"}.get(
-        strat_name, f"hash_grow_kernel<{variant & 7}, {variant >> 3}, 0, {per_n}>")
+                   "sweep": block_kernel if in_blocks else f"sweep_grow_kernel<{min(variant, 2)}, {job.n}>"}.get(
+        strat_name, "hash_grow_kernel<1, 3, 0, 0>" if variant == 21 else     # arrangement bitmap
+        f"hash_grow_kernel<{variant & 7}, {variant >> 3}, 0, {per_n}>")
     for i in range(args.steps):
         flush.zero_()                               # evict L2 between timed steps
         torch.cuda.synchronize()
@@ -605,8 +610,8 @@ def run_batch(args):
             "traffic": measured_traffic(f"hash_grow_kernel<{variant & 7}, {variant >> 3}, 1, 0>",
                                         f"batched-{len(jobs_all)}-random-groups-seed{wl.BATCH_SEED}",
                                         tuned["settings"] if tuned else None),
-            "kernel": f"hash_grow_kernel<{variant & 7}, {variant >> 3}, 1, 0> (multi-job, one "
-                      f"persistent launch per batch run admitting the jobs by the L2 window)",
+            "kernel": "cluster_grow_small_kernel<512> (n <= 8) and cluster_grow_kernel (n = 9, 10): a "
+                      "block or a thread-block cluster per job, drawn from a queue",
             "kernel_ms": kms, "algorithmic_bytes": bytes_step, "peak_source": peak_kind}),
         "e2e": {"value": nb_step / e2e_s, "unit": UNIT, "h2d_bytes_per_step": est["h2d_bytes"],
                 "d2h_bytes_per_step": est["d2h_bytes"], "api": "paper_2509_19162_gb300.Batch(...).run()"},
