@@ -47,9 +47,12 @@ extern "C" {
                                   cg_growth_run_noalloc (CG_NOALLOC_MAX_*)                    */
 
 /* ---- strategies (cg_growth_set_option(h, CG_OPT_STRATEGY, ...)) --------------------- */
-#define CG_STRATEGY_AUTO    0  /* library chooses: SWEEP for whole growths of large dense groups
-                                  (n >= 10) and when the states of BITMAP do not fit but the
-                                  sweep's bitmaps do, else BITMAP when eligible, else HASH     */
+#define CG_STRATEGY_AUTO    0  /* library chooses: SWEEP (in blocks of states) for dense groups
+                                  of n <= 9, for whole growths of n >= 12 (11 from 6 and 10 from
+                                  10 generators) and for limited growths once their layers are
+                                  dense, and when the states of BITMAP do not fit but the sweep's
+                                  bitmaps do; else BITMAP when eligible; else a bit per
+                                  arrangement of the start vector, or HASH                     */
 #define CG_STRATEGY_HASH    1  /* visited open-addressing hash set; any generating set        */
 #define CG_STRATEGY_SORT    2  /* sorted layers, radix sort + unique + merge-path difference
                                   against layers r and r-1; inverse-closed sets only          */
@@ -57,7 +60,7 @@ extern "C" {
                                   rank; any generating set; needs n <= 14 and a bitmap of at
                                   most half of mem_cap and 16 GiB (else CG_EINVAL at run).
                                   AUTO picks it when it fits and the group fills at least 1/512
-                                  of S_n, else HASH                                           */
+                                  of S_n                                                      */
 #define CG_STRATEGY_SWEEP   4  /* bitmask BFS (Section 3.1.3): the visited set and two
                                   layers are bitmaps over the n! Lehmer ranks (3 bits per
                                   element of S_n, nothing per state), so the whole of S_14 fits
@@ -85,6 +88,9 @@ extern "C" {
                                   1 = order of discovery; 2 = rank order (both state by state,
                                   never in blocks).  The layers are the same in every order    */
 /* batch options (cg_batch_set_option; CG_OPT_ILP and CG_OPT_GRID apply there too, 1..4)      */
+/* A batch grows its rank-bitmap jobs of n <= 10 by one block or one thread-block cluster each;
+   for those, of the options below and CG_OPT_ILP, only CG_OPT_GRID, CG_OPT_BATCH_VISITED and
+   CG_OPT_GRAPH matter.                                                                       */
 #define CG_OPT_BATCH_WAVE_L2 6 /* cap on the summed visited-set bytes of one launch:
                                   0 = half of L2 (default), -1 = none                          */
 #define CG_OPT_BATCH_VISITED 7 /* CG_STRATEGY_AUTO (rank bitmap for dense groups of n <= 12),
@@ -143,9 +149,12 @@ int cg_growth_create(int n, int k, const uint8_t* gens, int inverse_closed, int 
  * the identity.  States are packed with the narrowest element width w of 1, 2, 4 bits that
  * holds the values (4 for a permutation of n <= 16), in one 64-bit key when n * w <= 64 and
  * every generator has a one-word form, else in two words (n * w <= 128: 4-bit vectors up to
- * n = 32, 2-bit up to 64, binary up to 128; CG_EINVAL beyond).  Two-word keys run the hash
- * strategy only (AUTO or HASH; others fail at run with CG_EINVAL).  A start with repeated values
- * needs the HASH or SORT strategy (AUTO picks HASH; BITMAP then fails at run with CG_EINVAL).
+ * n = 32, 2-bit up to 64, binary up to 128; CG_EINVAL beyond).  Two-word keys take AUTO or
+ * HASH (others fail at run with CG_EINVAL).  A start with repeated values takes AUTO, HASH or SORT
+ * (BITMAP then fails at run with CG_EINVAL).  For binary one-word vectors and for two-word vectors
+ * with fewer than 2^32 arrangements of their values, AUTO keeps a visited bit per arrangement when
+ * the growth may reach at least 1/512 of them and its states and the hash table would have fitted
+ * mem_cap as well (cg_growth_stats.strategy_used is then CG_STRATEGY_BITMAP), else HASH.
  * A start whose values are all equal is fixed by every generator: its growth is {1}.  Releases
  * buffers sized for an earlier start.  Errors: CG_EINVAL (also a generator that fits neither
  * the shift-and-mask form, at most 16 distinct offsets in one word or 32 in two, nor the
@@ -207,7 +216,9 @@ typedef struct cg_growth_stats {
     uint64_t d2h_bytes;
     uint64_t state_capacity;    /* states the job's buffers hold */
     uint64_t table_slots;       /* visited-table slots (hash strategy) */
-    int strategy_used;          /* CG_STRATEGY_HASH, _SORT, _BITMAP or _SWEEP: what the run used */
+    int strategy_used;          /* CG_STRATEGY_HASH, _SORT, _BITMAP (a bit per permutation, or per
+                                   arrangement of the start) or _SWEEP (state by state, or in
+                                   blocks of states): what the run used, at its end             */
     int probe_variant;          /* kernel variant of the run (generators probed together) */
     int switched_to_sort;       /* 1: AUTO, inverse-closed set: the states stored by the hash or
                                    bitmap path outgrew mem_cap at layer sort_from + 1, and the

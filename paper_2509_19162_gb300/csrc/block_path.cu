@@ -888,11 +888,9 @@ __global__ void __launch_bounds__(kClThreads, 2) cluster_grow_kernel(const Clust
         if (job >= A.njobs) break;
         JobDev& J = A.jobs[job];
         switch (J.n) {
-#define CG_CLUSTER(n) case n: cluster_grow<n, kInL2, kClThreads>(S, A, J, ws, A.table[n], false, cl); break;
-            CG_CLUSTER(2) CG_CLUSTER(3) CG_CLUSTER(4) CG_CLUSTER(5) CG_CLUSTER(6) CG_CLUSTER(7) CG_CLUSTER(8)
-            CG_CLUSTER(9) CG_CLUSTER(10)
-#undef CG_CLUSTER
-            default: break;                 // planned for n in 2..10 only
+            case 9: cluster_grow<9, kInL2, kClThreads>(S, A, J, ws, A.table[9], false, cl); break;
+            case 10: cluster_grow<10, kInL2, kClThreads>(S, A, J, ws, A.table[10], false, cl); break;
+            default: break;                 // planned for n = 9, 10 only
         }
         cl.sync();                          // everyone is done with this job's shared state
     }
@@ -952,10 +950,10 @@ __global__ void __launch_bounds__(kSpreadThreads, 1) cluster_grow_spread_kernel(
     cl.sync();                              // nobody leaves while its words are in use
 }
 
-// Unranking tables of the cluster kernels, one for each n asked for: block idx -> nibble v = position
+// Unranking tables of cluster_grow_kernel, one for each n asked for: block idx -> nibble v = position
 // of value v.
 __global__ void cluster_prepare_kernel(const ClusterArgs A, unsigned want) {
-    for (int n = 2; n <= kClusterMaxN; ++n) {
+    for (int n = kClusterSmemN + 1; n <= kClusterMaxN; ++n) {
         if (!(want >> n & 1u)) continue;
         uint64_t* out = const_cast<uint64_t*>(A.table[n]);
         const int M = block_pairs(n);

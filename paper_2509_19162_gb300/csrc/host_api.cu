@@ -2361,7 +2361,7 @@ struct cg_batch {
         int csize = 1;
         int large = 0;
         int small_blocks = 0;      //   the others by this many blocks
-        unsigned want = 0;         // clusters: the n that occur, a bit each
+        unsigned want = 0;         // clusters: the n > kClusterSmemN that occur, a bit each
         int max_n = 0;
         bool admit = false;        // one launch admitting its jobs by the L2 window (AdmitDev)
         char* base = nullptr;      // resident plans: the wave's device buffer
@@ -2512,7 +2512,7 @@ void layout_cluster_wave(cg_batch* b, cg_batch::Wave& w, int lcap) {
         D.max_radius = J.max_radius;
         ngens += J.gsm.size();
         w.hg.insert(w.hg.end(), J.gsm.begin(), J.gsm.end());
-        w.want |= 1u << J.n;
+        if (J.n > cg::kClusterSmemN) w.want |= 1u << J.n;
         w.max_n = std::max(w.max_n, J.n);
     }
     w.o_gens = 0;
@@ -2521,7 +2521,7 @@ void layout_cluster_wave(cg_batch* b, cg_batch::Wave& w, int lcap) {
     w.o_lay = al256(w.o_ctl + sizeof(Ctl));
     w.o_tab = al256(w.o_lay + (uint64_t)nj * lcap * 8);
     uint64_t tables = 0;
-    for (int n = 2; n <= cg::kClusterMaxN; ++n)
+    for (int n = cg::kClusterSmemN + 1; n <= cg::kClusterMaxN; ++n)
         if (w.want >> n & 1u) tables += al256(cg::cluster_table_entries(n) * 8);
     w.o_keys = al256(w.o_tab + tables);
     w.bytes = al256(w.o_keys + std::max<uint64_t>((uint64_t)w.clusters * cg::cluster_words(w.max_n) * 4, 256));
@@ -2535,7 +2535,7 @@ cg::ClusterArgs cluster_args(const cg_batch::Wave& w, char* base) {
     A.words = reinterpret_cast<unsigned*>(base + w.o_keys);
     A.stride = cg::cluster_words(w.max_n);
     uint64_t o = w.o_tab;
-    for (int n = 2; n <= cg::kClusterMaxN; ++n)
+    for (int n = cg::kClusterSmemN + 1; n <= cg::kClusterMaxN; ++n)
         if (w.want >> n & 1u) {
             A.table[n] = reinterpret_cast<const uint64_t*>(base + o);
             o += al256(cg::cluster_table_entries(n) * 8);
@@ -2559,7 +2559,7 @@ cudaError_t bind_wave(cg_batch::Wave& w, char* base, cudaStream_t st) {
                                            cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(base + w.o_jobs, hj.data(), hj.size() * sizeof(JobDev), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess && w.cluster) e = cg::launch_cluster_prepare(cluster_args(w, base), w.want, st);
+    if (e == cudaSuccess && w.cluster && w.want) e = cg::launch_cluster_prepare(cluster_args(w, base), w.want, st);
     cg::AdmitDev A{};
     if (w.admit) {
         A.act[0] = reinterpret_cast<int*>(base + w.o_act);
