@@ -1565,6 +1565,11 @@ int sort_steps(cg_growth* h, cudaStream_t st, int cur, int prev, uint64_t Fcur, 
     const int lo = sort_low_bit(h);
     const int P = cg::sort_passes(bits, lo);
     const int top_shift = lo + 8 * (P - 1);
+    // Parent-edge tags above the keys, where the passes' digits leave bits 60..63 alone and every generator
+    // has one (ExpandSrc); the first layer comes without.
+    bool tags = bits <= 60 && lo + 8 * P <= 60 && h->k >= 2, cur_tagged = false;
+    for (const GenSM& g : h->gsm) tags = tags && g.inv_tag != 0;
+    const uint64_t mask = tags ? cg::kKeyBits60 : ~0ull;
     int nxt = 3 - cur - prev;
     cudaError_t e = cudaSuccess;
     int rc = CG_OK;
@@ -1599,7 +1604,7 @@ int sort_steps(cg_growth* h, cudaStream_t st, int cur, int prev, uint64_t Fcur, 
             if ((e = cudaMemcpyAsync(h->d_small, &ss, head, cudaMemcpyHostToDevice, st)) != cudaSuccess)
                 return cuda_rc(e);
             if ((e = cudaEventRecord(h->ev0, st)) != cudaSuccess) return cuda_rc(e);
-            if ((e = cg::launch_small_steps(h->d_gens, h->k, h->d_L[0], h->d_L[1], h->d_L[2], h->max_radius,
+            if ((e = cg::launch_small_steps(h->d_gens, h->k, tags ? 1 : 0, h->d_L[0], h->d_L[1], h->d_L[2], h->max_radius,
                                             h->stop_above, (int)h->sort_layers.size(), h->d_small, st)) !=
                 cudaSuccess)
                 return cuda_rc(e);
@@ -1616,6 +1621,7 @@ int sort_steps(cg_growth* h, cudaStream_t st, int cur, int prev, uint64_t Fcur, 
                 ss.prev > 2 || ss.cur == ss.prev)
                 return CG_EDEVICE;
             for (int i = 0; i < ss.nsteps; ++i) h->sort_layers.push_back(ss.sizes[i]);
+            if (ss.nsteps > 0) cur_tagged = tags;
             cur = ss.cur;
             prev = ss.prev;
             nxt = 3 - cur - prev;
@@ -1645,7 +1651,10 @@ int sort_steps(cg_growth* h, cudaStream_t st, int cur, int prev, uint64_t Fcur, 
         if (fail_mem(rc)) { status = cg::kNeedMem; break; }
         if (rc) return rc;
         cg::SortScratch sc = cg::carve_sort_scratch(h->d_sort_scratch, h->cand_cap);
-        const cg::ExpandSrc src{h->d_gens, h->k, h->d_L[cur], Fcur};
+        // (buffers, and whether chunks are needed, are planned for all k F candidates, and chunks
+        // generate them all: the memory a step needs does not depend on the tags)
+        const int each = cur_tagged && C <= h->cand_cap ? h->k - 1 : h->k;
+        const cg::ExpandSrc src{h->d_gens, h->k, h->d_L[cur], Fcur, each, mask};
         const uint64_t* bs[2] = {h->d_L[cur], h->d_L[prev]};
         const unsigned long long nbs[2] = {Fcur, Fprev};
         if ((e = cudaMemsetAsync(sc.err, 0, 4, st)) != cudaSuccess) return cuda_rc(e);
@@ -1677,7 +1686,7 @@ int sort_steps(cg_growth* h, cudaStream_t st, int cur, int prev, uint64_t Fcur, 
         bool stop_mem = false;
         for (const auto& rg : ranges) {
             if ((e = cudaEventRecord(h->ev0, st)) != cudaSuccess) return cuda_rc(e);
-            uint64_t Cc = C;
+            uint64_t Cc = (uint64_t)each * Fcur;
             if (ranges.size() == 1) {
                 if ((e = cg::launch_expand_sort(src, h->d_cand, bits, sc, st, lo)) != cudaSuccess) return cuda_rc(e);
                 h->stats.launches += 1 + P;
@@ -1693,7 +1702,7 @@ int sort_steps(cg_growth* h, cudaStream_t st, int cur, int prev, uint64_t Fcur, 
                 if ((e = cg::launch_radix_sort(h->d_cand, Cc, bits, sc, st, lo)) != cudaSuccess) return cuda_rc(e);
                 h->stats.launches += 2 + P;
             }
-            if ((e = cg::launch_unique_difference(h->d_cand, Cc, bs, nbs, 2, sc.keys_tmp, h->d_count, sc, st)) !=
+            if ((e = cg::launch_unique_difference(h->d_cand, Cc, bs, nbs, 2, sc.keys_tmp, h->d_count, sc, st, mask)) !=
                 cudaSuccess)
                 return cuda_rc(e);
             if ((e = cudaEventRecord(h->ev1, st)) != cudaSuccess) return cuda_rc(e);
@@ -1723,6 +1732,7 @@ int sort_steps(cg_growth* h, cudaStream_t st, int cur, int prev, uint64_t Fcur, 
         if (stop_mem) { status = cg::kNeedMem; break; }
         if (Fn == 0) { status = cg::kDone; break; }
         h->sort_layers.push_back(Fn);
+        cur_tagged = tags;
         ++radius;
         const int old_prev = prev;
         prev = cur;
@@ -1732,6 +1742,10 @@ int sort_steps(cg_growth* h, cudaStream_t st, int cur, int prev, uint64_t Fcur, 
         Fcur = Fn;
         if (h->stop_above > 0 && Fn > h->stop_above) { status = cg::kTruncAbove; break; }
         if ((int)h->sort_layers.size() >= cg::kMaxLayers) { status = cg::kTruncRadius; break; }
+    }
+    if (cur_tagged) {                   // the last layer is read as plain keys
+        if ((e = cg::launch_mask_keys(h->d_L[cur], Fcur, mask, st)) != cudaSuccess) return cuda_rc(e);
+        h->stats.launches += 1;
     }
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_rc(e);
     h->host_job.radius = radius;

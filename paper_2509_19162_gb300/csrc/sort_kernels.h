@@ -28,13 +28,18 @@ constexpr int kSortMaxPasses = 8;
 size_t sort_scratch_bytes(unsigned long long n);
 SortScratch carve_sort_scratch(void* scratch, unsigned long long n);
 
-// Candidates generated on the fly: candidate i of [0, k F) is generator i / F applied to
-// frontier[i % F] (expand fused into the sort's first reads).
+// Candidates generated on the fly: candidate i of [0, each F) is generator i / F applied to
+// frontier[i % F] (expand fused into the sort's first reads).  mask != ~0: the candidates carry in bits
+// 60..63 the tag of the generator that leads back (GenSM::inv_tag), `mask` is the bits below; each = k - 1:
+// so does the frontier, and a state's generator of that tag is passed over, because it leads to the state
+// the search came from, which lies in L_{r-1}.
 struct ExpandSrc {
     const GenSM* gens;
     int k;
     const uint64_t* frontier;
     unsigned long long F;
+    int each;
+    uint64_t mask;
 };
 
 cudaError_t launch_expand_all(const GenSM* d_gens, int k, const uint64_t* in, unsigned long long F,
@@ -44,14 +49,15 @@ cudaError_t launch_expand_all(const GenSM* d_gens, int k, const uint64_t* in, un
 // in place.
 cudaError_t launch_radix_sort(uint64_t* keys, unsigned long long n, int bits, const SortScratch& s,
                               cudaStream_t st, int lo = 0);
-// Generate the k F candidates of src and write them sorted to out (k F keys, not s.keys_tmp).
+// Generate the candidates of src and write them sorted to out (each F keys, not s.keys_tmp).
 cudaError_t launch_expand_sort(const ExpandSrc& src, uint64_t* out, int bits, const SortScratch& s,
                                cudaStream_t st, int lo = 0);
 // out = the keys of sorted a that are first of their run and absent from every sorted b_j (at
-// most 2 sets), in order; *d_count = their number.
+// most 2 sets), in order; *d_count = their number.  Keys are compared on the bits of mask.
 cudaError_t launch_unique_difference(const uint64_t* a, unsigned long long na, const uint64_t* const* bs,
                                      const unsigned long long* nbs, int nb_sets, uint64_t* out,
-                                     unsigned long long* d_count, const SortScratch& s, cudaStream_t st);
+                                     unsigned long long* d_count, const SortScratch& s, cudaStream_t st,
+                                     uint64_t mask = ~0ull);
 
 // 8-bit LSD passes over key bits [lo, bits).
 int sort_passes(int bits, int lo = 0);
@@ -87,8 +93,9 @@ struct SmallSteps {                 // device memory, read and written by the ke
 };
 
 // L[3]: the three layer buffers (each of at least kSmallStep keys); layers_done: layer sizes
-// recorded before this launch (the layer array holds at most kMaxLayers).
-cudaError_t launch_small_steps(const GenSM* d_gens, int k, uint64_t* L0, uint64_t* L1, uint64_t* L2,
+// recorded before this launch (the layer array holds at most kMaxLayers).  tags: the layers may carry
+// tags in bits 60..63 (see ExpandSrc), and those written do.
+cudaError_t launch_small_steps(const GenSM* d_gens, int k, int tags, uint64_t* L0, uint64_t* L1, uint64_t* L2,
                                int max_radius, unsigned long long stop_above, int layers_done,
                                SmallSteps* d_state, cudaStream_t st);
 

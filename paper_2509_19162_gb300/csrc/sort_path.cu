@@ -7,9 +7,13 @@
 // as arrays of packed keys sorted ascending.  One layer step is:
 //   histograms    one read of the candidates -- generated on the fly from L_r (every generator
 //                 on every state: the expand is fused, candidates are never written unsorted)
-//                 -- counts the 8-bit digits of every pass at once
+//                 -- counts the 8-bit digits of every pass at once.  A state carries the tag of the
+//                 generator that leads back to its parent above its key bits, where they leave room,
+//                 and that generator is passed over: its image lies in L_{r-1}.  The tag rides along
+//                 through the passes.  S_11 under L, R, X: a third fewer candidates,
+//                 a whole growth 13.27 / 12.26 ms
 //   radix passes  LSD over the w n significant key bits, one kernel per pass: each 4096-key
-//                 tile ranks its keys by digit (warp match_any, per-warp digit counts in shared
+//                 tile ranks its keys by digit (a vote per digit bit, per-warp digit counts in shared
 //                 memory), finds each digit's offset among the earlier tiles by a decoupled
 //                 look-back per digit, and writes its keys digit run by digit run (coalesced)
 //                 from a shared-memory staging copy; stable, so the passes compose
@@ -165,13 +169,20 @@ __device__ __forceinline__ T block_excl_scan(T v, T* total) {
     return excl;
 }
 
+__device__ __forceinline__ uint64_t tagged_image(const ExpandSrc& src, const GenSM& g, uint64_t s) {
+    const uint64_t t = apply_gen(g, s & src.mask);
+    return src.mask == ~0ull ? t : t | (uint64_t)g.inv_tag << 60;
+}
+
 // Candidate number i, given the generator `first` of an earlier one: a division per tile instead of one
 // per candidate.
 __device__ __forceinline__ uint64_t gen_candidate_from(const ExpandSrc& src, unsigned long long i, unsigned first) {
     unsigned long long off = i - (unsigned long long)first * src.F;
     unsigned g = first;
     while (off >= src.F) { off -= src.F; ++g; }
-    return apply_gen(src.gens[g], src.frontier[off]);
+    const uint64_t s = src.frontier[off];
+    if (src.each < src.k) g += g >= (unsigned)(s >> 60) - 1u ? 1u : 0u;      // (g <= k - 2 before)
+    return tagged_image(src, src.gens[g], s);
 }
 
 __device__ __forceinline__ uint64_t gen_candidate(const ExpandSrc& src, unsigned long long i) {
@@ -199,7 +210,8 @@ __global__ void expand_all_kernel(const GenSM* __restrict__ gens, int k, const u
 }
 
 // ---- digit histograms of every pass in one read ------------------------------------------
-// kGen: the candidates of src, a state's k together (one read of the frontier).
+// kGen: the candidates of src, a state's together (one read of the frontier).  Every generator is applied
+// in step, and the one to pass over not counted: the lanes of a warp read the same generator.
 template <bool kGen>
 __global__ void __launch_bounds__(kBlock)
 hist_all_kernel(const uint64_t* __restrict__ keys, ExpandSrc src, unsigned long long n, int passes, int lo,
@@ -210,10 +222,12 @@ hist_all_kernel(const uint64_t* __restrict__ keys, ExpandSrc src, unsigned long 
     const unsigned long long stride = (unsigned long long)gridDim.x * kBlock;
     const unsigned long long items = kGen ? src.F : n;
     const int each = kGen ? src.k : 1;
+    const bool skips = kGen && src.each < src.k;
     for (unsigned long long i = blockIdx.x * (unsigned long long)kBlock + threadIdx.x; i < items; i += stride) {
         const uint64_t in = kGen ? src.frontier[i] : keys[i];
         for (int g = 0; g < each; ++g) {
-            const uint64_t key = kGen ? apply_gen(src.gens[g], in) : in;
+            if (skips && g + 1 == (int)(in >> 60)) continue;
+            const uint64_t key = kGen ? apply_gen(src.gens[g], in & src.mask) : in;
             for (int p = 0; p < passes; ++p) atomicAdd(&s_h[p][(key >> (lo + kRadixBits * p)) & (kDigits - 1)], 1u);
         }
     }
@@ -310,19 +324,20 @@ onesweep_kernel(const uint64_t* __restrict__ in, ExpandSrc src, uint64_t* __rest
 }
 
 // ---- first of run, set difference and compaction in one pass -------------------------------
-// Lower bound of key in b[j, nb), galloping from j (the keys a thread asks for ascend).
+// Lower bound of key in b[j, nb), compared on the bits of mask, galloping from j (the keys a thread asks
+// for ascend).
 __device__ __forceinline__ unsigned long long gallop(const uint64_t* __restrict__ b, unsigned long long nb,
-                                                     unsigned long long j, uint64_t key) {
-    if (j >= nb || b[j] >= key) return j;
+                                                     unsigned long long j, uint64_t key, uint64_t mask) {
+    if (j >= nb || (b[j] & mask) >= key) return j;
     unsigned long long lo = j, step = 1;        // b[lo] < key
-    while (lo + step < nb && b[lo + step] < key) {
+    while (lo + step < nb && (b[lo + step] & mask) < key) {
         lo += step;
         step <<= 1;
     }
     unsigned long long hi = lo + step < nb ? lo + step : nb;   // b[hi] >= key or hi = nb
     while (hi - lo > 1) {
         const unsigned long long mid = lo + ((hi - lo) >> 1);
-        if (b[mid] < key) lo = mid; else hi = mid;
+        if ((b[mid] & mask) < key) lo = mid; else hi = mid;
     }
     return hi;
 }
@@ -331,19 +346,19 @@ __device__ __forceinline__ unsigned long long gallop(const uint64_t* __restrict_
 // probes 32 evenly spaced positions of the remaining interval at once (one round trip) and keeps
 // the part between the last probe below key and the first one at or above it.
 __device__ unsigned long long warp_lower_bound(const uint64_t* __restrict__ b, unsigned long long nb, uint64_t key,
-                                               int lane) {
+                                               int lane, uint64_t mask) {
     unsigned long long lo = 0, hi = nb;         // the answer lies in [lo, hi]
     while (hi - lo > 32) {
         const unsigned long long span = hi - lo;
         const unsigned long long p = lo + span * (unsigned long long)(lane + 1) / 33;   // in [lo, hi)
-        const int c = __popc(__ballot_sync(0xffffffffu, b[p] < key));                  // lanes 0..c-1
+        const int c = __popc(__ballot_sync(0xffffffffu, (b[p] & mask) < key));         // lanes 0..c-1
         const unsigned long long nlo = c ? lo + span * (unsigned long long)c / 33 + 1 : lo;
         const unsigned long long nhi = c < 32 ? lo + span * (unsigned long long)(c + 1) / 33 : hi;
         lo = nlo;
         hi = nhi;
     }
     const unsigned long long p = lo + (unsigned)lane;
-    return lo + __popc(__ballot_sync(0xffffffffu, p < hi && b[p] < key));
+    return lo + __popc(__ballot_sync(0xffffffffu, p < hi && (b[p] & mask) < key));
 }
 
 // Lower bound of key in the shared-memory slice s[j, ns), galloping from j.
@@ -370,7 +385,7 @@ constexpr int kSlice = 2048;
 __global__ void __launch_bounds__(kBlock)
 unique_diff_kernel(const uint64_t* __restrict__ a, unsigned long long na, const uint64_t* __restrict__ b0,
                    unsigned long long nb0, const uint64_t* __restrict__ b1, unsigned long long nb1,
-                   int first_of_run, uint64_t* __restrict__ out, unsigned long long* d_count,
+                   uint64_t mask, int first_of_run, uint64_t* __restrict__ out, unsigned long long* d_count,
                    unsigned long long* desc, unsigned* ticket, int ntiles, unsigned epoch, int* err) {
     // the staged slices are done with before the survivors are staged for the output
     __shared__ union {
@@ -393,8 +408,8 @@ unique_diff_kernel(const uint64_t* __restrict__ a, unsigned long long na, const 
         const int q = wid >> 1, end = wid & 1;
         const uint64_t* b = q ? b1 : b0;
         const unsigned long long nb = q ? nb1 : nb0;
-        const uint64_t key = end ? a[t1 - 1] : a[t0];
-        const unsigned long long j = (end && key == ~0ull) ? nb : warp_lower_bound(b, nb, key + (end ? 1 : 0), lane);
+        const uint64_t key = (end ? a[t1 - 1] : a[t0]) & mask;
+        const unsigned long long j = (end && key == ~0ull) ? nb : warp_lower_bound(b, nb, key + (end ? 1 : 0), lane, mask);
         if (lane == 0) s_j[q][end] = j;
     }
     __syncthreads();
@@ -409,7 +424,7 @@ unique_diff_kernel(const uint64_t* __restrict__ a, unsigned long long na, const 
         staged[q] = s_n[q] <= (unsigned long long)kSlice;
         if (staged[q]) {
             const uint64_t* b = q ? b1 : b0;
-            for (unsigned i = tid; i < (unsigned)s_n[q]; i += kBlock) s_m.slice[q][i] = b[s_lo[q] + i];
+            for (unsigned i = tid; i < (unsigned)s_n[q]; i += kBlock) s_m.slice[q][i] = b[s_lo[q] + i] & mask;
         }
     }
     __syncthreads();
@@ -418,35 +433,36 @@ unique_diff_kernel(const uint64_t* __restrict__ a, unsigned long long na, const 
     unsigned keep = 0, cnt = 0;
 #pragma unroll
     for (int i = 0; i < kItems; ++i) key[i] = p0 + i < na ? a[p0 + i] : 0;
-    uint64_t prev = (p0 > 0 && p0 - 1 < na) ? a[p0 - 1] : 0;
+    uint64_t prev = (p0 > 0 && p0 - 1 < na) ? a[p0 - 1] & mask : 0;
     bool has_prev = p0 > 0;
     unsigned long long j0 = 0, j1 = 0;         // global walks (slices too large)
     unsigned k0 = 0, k1 = 0;                   // walks in the staged slices
     if (p0 < na) {
-        if (!staged[0]) j0 = gallop(b0, nb0, s_lo[0], key[0]);
-        if (!staged[1]) j1 = gallop(b1, nb1, s_lo[1], key[0]);
+        if (!staged[0]) j0 = gallop(b0, nb0, s_lo[0], key[0] & mask, mask);
+        if (!staged[1]) j1 = gallop(b1, nb1, s_lo[1], key[0] & mask, mask);
     }
 #pragma unroll
     for (int i = 0; i < kItems; ++i) {
         if (p0 + i >= na) break;
-        bool k = !(first_of_run && has_prev && prev == key[i]);
+        const uint64_t x = key[i] & mask;
+        bool k = !(first_of_run && has_prev && prev == x);
         if (staged[0]) {
-            k0 = gallop_smem(s_m.slice[0], (unsigned)s_n[0], k0, key[i]);
-            if (k0 < (unsigned)s_n[0] && s_m.slice[0][k0] == key[i]) k = false;
+            k0 = gallop_smem(s_m.slice[0], (unsigned)s_n[0], k0, x);
+            if (k0 < (unsigned)s_n[0] && s_m.slice[0][k0] == x) k = false;
         } else {
-            j0 = gallop(b0, nb0, j0, key[i]);
-            if (j0 < nb0 && b0[j0] == key[i]) k = false;
+            j0 = gallop(b0, nb0, j0, x, mask);
+            if (j0 < nb0 && (b0[j0] & mask) == x) k = false;
         }
         if (staged[1]) {
-            k1 = gallop_smem(s_m.slice[1], (unsigned)s_n[1], k1, key[i]);
-            if (k1 < (unsigned)s_n[1] && s_m.slice[1][k1] == key[i]) k = false;
+            k1 = gallop_smem(s_m.slice[1], (unsigned)s_n[1], k1, x);
+            if (k1 < (unsigned)s_n[1] && s_m.slice[1][k1] == x) k = false;
         } else {
-            j1 = gallop(b1, nb1, j1, key[i]);
-            if (j1 < nb1 && b1[j1] == key[i]) k = false;
+            j1 = gallop(b1, nb1, j1, x, mask);
+            if (j1 < nb1 && (b1[j1] & mask) == x) k = false;
         }
         keep |= (unsigned)k << i;
         cnt += k;
-        prev = key[i];
+        prev = x;
         has_prev = true;
     }
     unsigned total = 0;
@@ -474,7 +490,7 @@ unique_diff_kernel(const uint64_t* __restrict__ a, unsigned long long na, const 
 __global__ void __launch_bounds__(kBlock)
 expand_filter_kernel(ExpandSrc src, int shift, unsigned d0, unsigned d1, uint64_t* __restrict__ out,
                      unsigned long long cap, unsigned long long* count, int* err) {
-    const unsigned long long n = src.F * (unsigned long long)src.k;
+    const unsigned long long n = src.F * (unsigned long long)src.each;
     const int lane = threadIdx.x & 31;
     const unsigned long long stride = (unsigned long long)gridDim.x * kBlock;
     for (unsigned long long w = blockIdx.x * (unsigned long long)kBlock + (threadIdx.x & ~31u); w < n; w += stride) {
@@ -520,7 +536,7 @@ __device__ __forceinline__ unsigned small_lower_bound(const uint64_t* s, unsigne
 
 // One block; dynamic shared memory: candidates | L_r | L_{r-1}, kSmallStep keys each.
 __global__ void __launch_bounds__(kSmallBlock)
-small_steps_kernel(const GenSM* __restrict__ gens, int k, uint64_t* L0, uint64_t* L1, uint64_t* L2,
+small_steps_kernel(const GenSM* __restrict__ gens, int k, int tags, uint64_t* L0, uint64_t* L1, uint64_t* L2,
                    int max_radius, unsigned long long stop_above, int layers_done, SmallSteps* S) {
     extern __shared__ uint64_t s_small[];
     uint64_t* A = s_small;
@@ -528,6 +544,10 @@ small_steps_kernel(const GenSM* __restrict__ gens, int k, uint64_t* L0, uint64_t
     uint64_t* Lp = s_small + 2 * kSmallStep;
     __shared__ unsigned s_w[kSmallBlock / 32];
     uint64_t* L[3] = {L0, L1, L2};
+    // tags: a candidate is sorted with its tag below the key (all k are generated: the sort's length is a
+    // power of two), and stored with it above
+    const int up = tags ? 4 : 0;
+    const uint64_t mask = tags ? kKeyBits60 : ~0ull;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     int cur = S->cur, prev = S->prev, radius = S->radius, nsteps = 0, status = kRunning;
     unsigned long long Fcur = S->Fcur, Fprev = S->Fprev;
@@ -542,14 +562,14 @@ small_steps_kernel(const GenSM* __restrict__ gens, int k, uint64_t* L0, uint64_t
         const unsigned nc = (unsigned)C, fc = (unsigned)Fcur, fp = (unsigned)Fprev;
         unsigned P = 1;
         while (P < nc) P <<= 1;
-        for (unsigned i = tid; i < fc; i += kSmallBlock) Lc[i] = L[cur][i];
-        for (unsigned i = tid; i < fp; i += kSmallBlock) Lp[i] = L[prev][i];
+        for (unsigned i = tid; i < fc; i += kSmallBlock) Lc[i] = L[cur][i] & mask;
+        for (unsigned i = tid; i < fp; i += kSmallBlock) Lp[i] = L[prev][i] & mask;
         __syncthreads();
         // candidate i: generator i / F on state i mod F; padding sorts last
         for (unsigned i = tid; i < P; i += kSmallBlock) {
             if (i < nc) {
                 const unsigned g = i / fc;
-                A[i] = apply_gen(gens[g], Lc[i - g * fc]);
+                A[i] = apply_gen(gens[g], Lc[i - g * fc]) << up | (tags ? gens[g].inv_tag : 0u);
             } else {
                 A[i] = ~0ull;
             }
@@ -577,8 +597,8 @@ small_steps_kernel(const GenSM* __restrict__ gens, int k, uint64_t* L0, uint64_t
         for (int q = 0; q < kSmallPer; ++q) {
             const unsigned i = (unsigned)tid * kSmallPer + q;
             if (i < nc) {
-                const uint64_t key = A[i];
-                bool kp = i == 0 || A[i - 1] != key;
+                const uint64_t key = A[i] >> up;
+                bool kp = i == 0 || A[i - 1] >> up != key;
                 if (kp) {
                     const unsigned a = small_lower_bound(Lc, fc, key);
                     if (a < fc && Lc[a] == key) kp = false;
@@ -614,7 +634,10 @@ small_steps_kernel(const GenSM* __restrict__ gens, int k, uint64_t* L0, uint64_t
         const unsigned Fn = s_w[kSmallBlock / 32 - 1];
 #pragma unroll
         for (int q = 0; q < kSmallPer; ++q)
-            if (keep >> q & 1u) L[nxt][pos++] = A[(unsigned)tid * kSmallPer + q];
+            if (keep >> q & 1u) {
+                const uint64_t a = A[(unsigned)tid * kSmallPer + q];
+                L[nxt][pos++] = tags ? a >> 4 | a << 60 : a;
+            }
         __syncthreads();                        // A, Lc, Lp and s_w are reused by the next step
         if (Fn == 0) { status = kDone; break; }
         if (tid == 0) S->sizes[nsteps] = Fn;
@@ -727,8 +750,8 @@ cudaError_t radix_passes(const uint64_t* in, const ExpandSrc* src, unsigned long
 
 }  // namespace
 
-// Sort keys[0, n) ascending on their bits [lo, bits) (higher bits must be zero; lower bits
-// decided by the others), in place; an odd number of 8-bit passes ends with one copy back.
+// Sort keys[0, n) ascending on their bits [lo, bits) (higher bits zero, or past the last pass's digit;
+// lower bits decided by the others), in place; an odd number of 8-bit passes ends with one copy back.
 cudaError_t launch_radix_sort(uint64_t* keys, unsigned long long n, int bits, const SortScratch& s,
                               cudaStream_t st, int lo) {
     (void)cudaGetLastError();   // clear a stale error: the check after the launch is about this one
@@ -746,7 +769,7 @@ cudaError_t launch_radix_sort(uint64_t* keys, unsigned long long n, int bits, co
 cudaError_t launch_expand_sort(const ExpandSrc& src, uint64_t* out, int bits, const SortScratch& s,
                                cudaStream_t st, int lo) {
     (void)cudaGetLastError();   // clear a stale error: the check after the launch is about this one
-    const unsigned long long n = src.F * (unsigned long long)src.k;
+    const unsigned long long n = src.F * (unsigned long long)src.each;
     if (n == 0) return cudaSuccess;
     uint64_t* bufs[2] = {out, s.keys_tmp};
     return radix_passes(nullptr, &src, n, bits, lo, bufs, s, st);
@@ -756,7 +779,8 @@ cudaError_t launch_expand_sort(const ExpandSrc& src, uint64_t* out, int bits, co
 // compacted in order; *d_count = their number.
 cudaError_t launch_unique_difference(const uint64_t* a, unsigned long long na, const uint64_t* const* bs,
                                      const unsigned long long* nbs, int nb_sets, uint64_t* out,
-                                     unsigned long long* d_count, const SortScratch& s, cudaStream_t st) {
+                                     unsigned long long* d_count, const SortScratch& s, cudaStream_t st,
+                                     uint64_t mask) {
     (void)cudaGetLastError();   // clear a stale error: the check after the launch is about this one
     if (na == 0) return cudaMemsetAsync(d_count, 0, 8, st);
     const int nt = tiles_of(na);
@@ -766,7 +790,7 @@ cudaError_t launch_unique_difference(const uint64_t* a, unsigned long long na, c
     const uint64_t* b0 = nb_sets > 0 ? bs[0] : a;
     const uint64_t* b1 = nb_sets > 1 ? bs[1] : a;
     const unsigned long long n0 = nb_sets > 0 ? nbs[0] : 0, n1 = nb_sets > 1 ? nbs[1] : 0;
-    unique_diff_kernel<<<nt, kBlock, 0, st>>>(a, na, b0, n0, b1, n1, 1, out, d_count, s.desc, s.ctl + 15,
+    unique_diff_kernel<<<nt, kBlock, 0, st>>>(a, na, b0, n0, b1, n1, mask, 1, out, d_count, s.desc, s.ctl + 15,
                                               nt, 15u, s.err);
     return cudaGetLastError();
 }
@@ -774,7 +798,7 @@ cudaError_t launch_unique_difference(const uint64_t* a, unsigned long long na, c
 cudaError_t launch_candidate_hist(const ExpandSrc& src, int bits, const SortScratch& s, cudaStream_t st,
                                   int lo) {
     (void)cudaGetLastError();   // clear a stale error: the check after the launch is about this one
-    const unsigned long long n = src.F * (unsigned long long)src.k;
+    const unsigned long long n = src.F * (unsigned long long)src.each;
     cudaError_t e = cudaMemsetAsync(s.ghist, 0, sizeof(unsigned long long) * kSortMaxPasses * kDigits, st);
     if (e != cudaSuccess || n == 0) return e;
     unsigned long long hb = (src.F + kBlock - 1) / kBlock;
@@ -805,7 +829,7 @@ cudaError_t launch_mask_keys(uint64_t* keys, unsigned long long n, uint64_t mask
 
 int sort_passes(int bits, int lo) { return passes_of(bits - lo < 1 ? 1 : bits - lo); }
 
-cudaError_t launch_small_steps(const GenSM* d_gens, int k, uint64_t* L0, uint64_t* L1, uint64_t* L2,
+cudaError_t launch_small_steps(const GenSM* d_gens, int k, int tags, uint64_t* L0, uint64_t* L1, uint64_t* L2,
                                int max_radius, unsigned long long stop_above, int layers_done,
                                SmallSteps* d_state, cudaStream_t st) {
     (void)cudaGetLastError();   // clear a stale error: the check after the launch is about this one
@@ -819,7 +843,7 @@ cudaError_t launch_small_steps(const GenSM* d_gens, int k, uint64_t* L0, uint64_
         if (e != cudaSuccess) return e;
         attr_set[dev] = true;
     }
-    small_steps_kernel<<<1, kSmallBlock, smem, st>>>(d_gens, k, L0, L1, L2, max_radius, stop_above, layers_done,
+    small_steps_kernel<<<1, kSmallBlock, smem, st>>>(d_gens, k, tags, L0, L1, L2, max_radius, stop_above, layers_done,
                                                       d_state);
     return cudaGetLastError();
 }

@@ -169,3 +169,28 @@ def test_sort_strategy_s12_pancake_whole(cg):
     # all 12! states through the sorted two-layer step (11 generators), against oracle B
     r = cg.growth(12, w.pancake(12), strategy="sort")
     assert r.status == 0 and r.layers == golden("s12_pancake_growth_b")
+
+
+@pytest.mark.parametrize("n,gens,start,cap", [
+    (15, "lrx", None, 19),                                  # 60-bit keys, passes to bit 60: tags
+    (15, "cyclic_coxeter", None, 5),                        # 15 generators, the largest tag
+    (16, "coxeter", None, 5),                               # 64-bit keys: no room for tags
+    (56, "lrx", [1] * 5 + [0] * 51, 60),                    # 7 passes over all 56 bits: tags
+    (57, "lrx", [1] * 5 + [0] * 52, 60),                    # an eighth pass would meet the tags: none
+    (17, "cyclic_coxeter", [1] * 8 + [0] * 9, -1),          # 17 generators: none
+    (12, "all_transpositions", [0, 0, 1, 1, 2, 2, 3, 3, 4, 4, 5, 5], 4),   # 66 generators: none
+    (12, "star", [0, 0, 1, 1, 2, 2, 3, 3, 4, 4, 5, 5], -1),  # images equal to their state
+])
+def test_sort_parent_tags(cg, n, gens, start, cap):
+    # States carry their parent edge above the key bits where there is room; the layers and the last
+    # layer's plain keys are those of the visited-set strategy.
+    rows = w.FAMILIES[gens](n)
+    out = []
+    for strategy in ("sort", "hash"):
+        g = cg.Growth(n, rows, strategy=strategy, max_radius=cap, keep_last=True, start=start)
+        r = g.run()
+        out.append((r.status, r.layers, np.sort(np.asarray(g.last_layer(), dtype=np.uint64))))
+        g.close()
+    assert out[0][0] == out[1][0] and out[0][1] == out[1][1]
+    assert max(out[0][1]) * len(rows) > 4096                # past the steps of one block
+    assert np.array_equal(out[0][2], out[1][2])
