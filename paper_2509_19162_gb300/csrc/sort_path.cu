@@ -174,19 +174,27 @@ __device__ __forceinline__ uint64_t tagged_image(const ExpandSrc& src, const Gen
     return src.mask == ~0ull ? t : t | (uint64_t)g.inv_tag << 60;
 }
 
-// Candidate number i, given the generator `first` of an earlier one: a division per tile instead of one
-// per candidate.
-__device__ __forceinline__ uint64_t gen_candidate_from(const ExpandSrc& src, unsigned long long i, unsigned first) {
+// Candidate number i, given the generator `first` of an earlier one (a division per tile instead of one
+// per candidate): its state's place in the frontier, and its number among the state's candidates.
+__device__ __forceinline__ unsigned long long candidate_state(const ExpandSrc& src, unsigned long long i, unsigned first,
+                                                              unsigned* j) {
     unsigned long long off = i - (unsigned long long)first * src.F;
     unsigned g = first;
     while (off >= src.F) { off -= src.F; ++g; }
-    const uint64_t s = src.frontier[off];
-    if (src.each < src.k) g += g >= (unsigned)(s >> 60) - 1u ? 1u : 0u;      // (g <= k - 2 before)
-    return tagged_image(src, src.gens[g], s);
+    *j = g;
+    return off;
+}
+
+// Candidate j of state s.
+__device__ __forceinline__ uint64_t candidate_of(const ExpandSrc& src, uint64_t s, unsigned j) {
+    if (src.each < src.k) j += j >= (unsigned)(s >> 60) - 1u ? 1u : 0u;      // (j <= k - 2 before)
+    return tagged_image(src, src.gens[j], s);
 }
 
 __device__ __forceinline__ uint64_t gen_candidate(const ExpandSrc& src, unsigned long long i) {
-    return gen_candidate_from(src, i, (unsigned)(i / src.F));
+    unsigned j;
+    const unsigned long long off = candidate_state(src, i, (unsigned)(i / src.F), &j);
+    return candidate_of(src, src.frontier[off], j);
 }
 
 // ---- expand (standalone: the step-level cg_expand and the memory hand-off) ----------------
@@ -266,7 +274,17 @@ onesweep_kernel(const uint64_t* __restrict__ in, ExpandSrc src, uint64_t* __rest
 #pragma unroll
     for (int r = 0; r < kItems; ++r) {
         const unsigned long long idx = base + (unsigned)(wid * (kItems * 32) + r * 32 + lane);
-        key[r] = idx < n ? (kGen ? gen_candidate_from(src, idx, s_gen) : in[idx]) : 0;
+        if (kGen) key[r] = idx < n ? src.frontier[candidate_state(src, idx, s_gen, &rank[r])] : 0;
+        else key[r] = idx < n ? in[idx] : 0;
+    }
+    // the generators after every state is on its way: applied one state at a time, each would wait for its
+    // own trip to L2 (S_11, ten star transpositions: 24.3 / 23.5 ms a growth)
+    if constexpr (kGen) {
+#pragma unroll
+        for (int r = 0; r < kItems; ++r) {
+            const unsigned long long idx = base + (unsigned)(wid * (kItems * 32) + r * 32 + lane);
+            if (idx < n) key[r] = candidate_of(src, key[r], rank[r]);
+        }
     }
     // A key's rank among the warp's keys of its digit.  The lanes of a row that share a digit are found
     // with a vote per digit bit, their first lane
