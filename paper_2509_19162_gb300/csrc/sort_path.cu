@@ -11,7 +11,7 @@
 //                 generator that leads back to its parent above its key bits, where they leave room,
 //                 and that generator is passed over: its image lies in L_{r-1}.  The tag rides along
 //                 through the passes.  S_11 under L, R, X: a third fewer candidates,
-//                 a whole growth 13.27 / 12.26 ms
+//                 a whole growth 13.0 / 10.95 ms
 //   radix passes  LSD over the w n significant key bits, one kernel per pass: each 4096-key
 //                 tile ranks its keys by digit (a vote per digit bit, per-warp digit counts in shared
 //                 memory), finds each digit's offset among the earlier tiles by a decoupled
@@ -396,9 +396,12 @@ __device__ __forceinline__ unsigned gallop_smem(const uint64_t* s, unsigned ns, 
 }
 
 // The keys of b0 and b1 that can match a tile's keys (those within the tile's first and last
-// key) are staged in shared memory when there are at most kSlice of them; each thread then walks
-// the staged slices instead of L2.  A slice larger than that falls back to the global walk.
-constexpr int kSlice = 2048;
+// key) are staged in shared memory, one after the other, while they fit kSlices; each thread then walks
+// the staged slices instead of L2.  A slice that does not fit is walked there.  With two candidates a state
+// (three generators, one passed over) a tile's 4096 keys span about 2048 states of L_r, and more of L_{r-1}
+// once the layers shrink: room for 2048 of each sent half of the tiles to
+// L2 (S_11 under L, R, X: 11.9 / 10.95 ms a growth; S_9: 2.68 / 2.53).
+constexpr int kSlices = 6080;    // with the rest of the kernel's shared memory just below 48 KB
 
 __global__ void __launch_bounds__(kBlock)
 unique_diff_kernel(const uint64_t* __restrict__ a, unsigned long long na, const uint64_t* __restrict__ b0,
@@ -408,7 +411,7 @@ unique_diff_kernel(const uint64_t* __restrict__ a, unsigned long long na, const 
     // the staged slices are done with before the survivors are staged for the output
     __shared__ union {
         uint64_t stage[kTile];
-        uint64_t slice[2][kSlice];
+        uint64_t slices[kSlices];
     } s_m;
     __shared__ int s_tile;
     __shared__ unsigned long long s_prefix;
@@ -437,14 +440,15 @@ unique_diff_kernel(const uint64_t* __restrict__ a, unsigned long long na, const 
     }
     __syncthreads();
     bool staged[2];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        staged[q] = s_n[q] <= (unsigned long long)kSlice;
-        if (staged[q]) {
-            const uint64_t* b = q ? b1 : b0;
-            for (unsigned i = tid; i < (unsigned)s_n[q]; i += kBlock) s_m.slice[q][i] = b[s_lo[q] + i] & mask;
-        }
-    }
+    staged[0] = s_n[0] <= (unsigned long long)kSlices;
+    const unsigned used = staged[0] ? (unsigned)s_n[0] : 0u;
+    staged[1] = s_n[1] <= (unsigned long long)(kSlices - used);
+    const uint64_t* slice0 = s_m.slices;
+    const uint64_t* slice1 = s_m.slices + used;
+    if (staged[0])
+        for (unsigned i = tid; i < (unsigned)s_n[0]; i += kBlock) s_m.slices[i] = b0[s_lo[0] + i] & mask;
+    if (staged[1])
+        for (unsigned i = tid; i < (unsigned)s_n[1]; i += kBlock) s_m.slices[used + i] = b1[s_lo[1] + i] & mask;
     __syncthreads();
     const unsigned long long p0 = t0 + (unsigned long long)tid * kItems;
     uint64_t key[kItems];
@@ -465,15 +469,15 @@ unique_diff_kernel(const uint64_t* __restrict__ a, unsigned long long na, const 
         const uint64_t x = key[i] & mask;
         bool k = !(first_of_run && has_prev && prev == x);
         if (staged[0]) {
-            k0 = gallop_smem(s_m.slice[0], (unsigned)s_n[0], k0, x);
-            if (k0 < (unsigned)s_n[0] && s_m.slice[0][k0] == x) k = false;
+            k0 = gallop_smem(slice0, (unsigned)s_n[0], k0, x);
+            if (k0 < (unsigned)s_n[0] && slice0[k0] == x) k = false;
         } else {
             j0 = gallop(b0, nb0, j0, x, mask);
             if (j0 < nb0 && (b0[j0] & mask) == x) k = false;
         }
         if (staged[1]) {
-            k1 = gallop_smem(s_m.slice[1], (unsigned)s_n[1], k1, x);
-            if (k1 < (unsigned)s_n[1] && s_m.slice[1][k1] == x) k = false;
+            k1 = gallop_smem(slice1, (unsigned)s_n[1], k1, x);
+            if (k1 < (unsigned)s_n[1] && slice1[k1] == x) k = false;
         } else {
             j1 = gallop(b1, nb1, j1, x, mask);
             if (j1 < nb1 && (b1[j1] & mask) == x) k = false;

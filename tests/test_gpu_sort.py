@@ -194,3 +194,26 @@ def test_sort_parent_tags(cg, n, gens, start, cap):
     assert out[0][0] == out[1][0] and out[0][1] == out[1][1]
     assert max(out[0][1]) * len(rows) > 4096                # past the steps of one block
     assert np.array_equal(out[0][2], out[1][2])
+
+
+@pytest.mark.parametrize("nb,nc", [(0, 6080), (6080, 0), (6081, 0), (6080, 1), (3040, 3040), (3040, 3041), (6081, 100),
+                                   (6081, 6081), (100, 6081)])
+def test_set_difference_slices(cg, nb, nc):
+    # One tile of 4096 keys across slices that fit the staging room of 6080 keys exactly, by one too many,
+    # and only for one of the sets.
+    import torch
+    from paper_2509_19162_gb300 import _cg
+    rng = np.random.default_rng(nb + 7 * nc)
+    top = 20000
+    a = np.sort(np.concatenate([[0, top], rng.integers(0, top + 1, size=4094)]).astype(np.uint64))
+    b, c = (np.sort(rng.choice(top + 1, size=m, replace=False)).astype(np.uint64) for m in (nb, nc))
+    da, db, dc = _dev(a), _dev(b) if nb else None, _dev(c) if nc else None
+    out = torch.empty(len(a), dtype=torch.int64, device="cuda")
+    cnt = torch.zeros(1, dtype=torch.int64, device="cuda")
+    scr, nbytes = _scratch(_cg, len(a))
+    rc = _cg.cg_set_difference(da.data_ptr(), len(a), db.data_ptr() if nb else None, nb, dc.data_ptr() if nc else None, nc,
+                               out.data_ptr(), cnt.data_ptr(), scr.data_ptr(), nbytes, None)
+    assert rc == 0
+    torch.cuda.synchronize()
+    want = np.setdiff1d(np.setdiff1d(np.unique(a), b), c)
+    assert np.array_equal(out[:int(cnt.item())].cpu().numpy().view(np.uint64), want)
