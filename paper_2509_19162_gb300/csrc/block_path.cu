@@ -876,6 +876,7 @@ __global__ void __launch_bounds__(kClThreads, 2) cluster_grow_kernel(const Clust
     const cgr::cluster_group cl = cgr::this_cluster();
     const unsigned size = cl.num_blocks();
     unsigned* ws = A.words + (uint64_t)(blockIdx.x / size) * A.stride;
+    cl.sync();                              // every block runs: block 0 may write the others' S.job
     for (;;) {
         if (cl.block_rank() == 0 && threadIdx.x < size) {
             int j = 0;
