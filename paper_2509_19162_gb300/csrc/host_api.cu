@@ -1506,6 +1506,16 @@ int run_sweep(cg_growth* h, cudaStream_t st, int* final_status) {
     return CG_OK;
 }
 
+// A run that failed gives every buffer back.  The paths take a buffer that is there for a buffer that is
+// ready (tables filled, generators uploaded, its companions allocated), which one left behind by an
+// allocation or a copy that failed half-way would not be.
+int run_failed(cg_growth* h, cudaStream_t st, int rc) {
+    if (cudaStreamSynchronize(st) != cudaSuccess) cudaGetLastError();
+    h->release(st);
+    h->mode = -1;
+    return rc;
+}
+
 // ---- sort strategy driver ------------------------------------------------------------------
 // Layers live in three rotating buffers sorted ascending; each layer step is expand, radix
 // sort, unique + merge-path difference against layers r and r-1, compaction (sort_path.cu).
@@ -1528,8 +1538,13 @@ int ensure_cand(cg_growth* h, uint64_t q, cudaStream_t st, bool shrink = false) 
     h->d_cand = (uint64_t*)dev_alloc(q * 8, st);
     h->d_sort_scratch = dev_alloc(cg::sort_scratch_bytes(q), st);
     h->cand_cap = q;
-    if (!h->d_cand || !h->d_sort_scratch) return CG_ENOMEM;
-    return CG_OK;
+    if (h->d_cand && h->d_sort_scratch) return CG_OK;
+    dev_free(h->d_cand, st);            // the two belong together: a later call finds both or neither
+    dev_free(h->d_sort_scratch, st);
+    h->d_cand = nullptr;
+    h->d_sort_scratch = nullptr;
+    h->cand_cap = 0;
+    return CG_ENOMEM;
 }
 
 // Layer buffer i with room for cap keys, keeping its first `keep` keys.
@@ -2044,7 +2059,7 @@ int cg_growth_run(cg_growth_t h, void* cuda_stream, uint64_t* layer_sizes_out, i
     int status = 0;
     if (h->wide) {
         int rc = run_wide(h, st, &status);
-        if (rc) return rc;
+        if (rc) return run_failed(h, st, rc);
         h->last_is_sweep = false;
         const int layers = h->host_job.radius + 1;
         *num_layers_out = layers;
@@ -2063,10 +2078,10 @@ int cg_growth_run(cg_growth_t h, void* cuda_stream, uint64_t* layer_sizes_out, i
     int rc = use_cluster ? run_cluster(h, st, &status)
              : use_sort ? run_sort(h, st, &status)
                       : use_sweep ? run_sweep(h, st, &status) : run_hash(h, st, &status);
-    if (rc) return rc;
+    if (rc) return run_failed(h, st, rc);
     if (!use_cluster && !use_sort && !use_sweep && status == cg::kNeedMem && h->strategy == CG_STRATEGY_AUTO &&
         h->inverse_closed) {
-        if ((rc = continue_sorted(h, st, &status))) return rc;
+        if ((rc = continue_sorted(h, st, &status))) return run_failed(h, st, rc);
     }
     const bool sorted = use_sort || h->stats.switched_to_sort;
     h->last_is_sweep = use_sweep;

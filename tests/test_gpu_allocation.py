@@ -1,0 +1,102 @@
+"""GPU tests of what a growth does with device memory: every allocation of every path failing once,
+after which the same handle grows the graph as if nothing had been, and everything given back at the
+end."""
+
+import ctypes
+
+import numpy as np
+import pytest
+
+import workloads as w
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def cg():
+    import torch
+    assert torch.cuda.is_available()
+    import paper_2509_19162_gb300 as p
+    p.build()
+    return p
+
+
+class Device:
+    """An allocator for the library: counts allocations, can fail one or all above a size, and knows
+    what is held."""
+
+    def __init__(self):
+        import torch
+        from paper_2509_19162_gb300 import _cg
+        self.fail_at, self.limit = -1, None
+        self.calls, self.live, self.held, self.peak = 0, {}, 0, 0
+
+        def alloc(nbytes, stream, ctx):
+            i, self.calls = self.calls, self.calls + 1
+            if i == self.fail_at or (self.limit is not None and nbytes > self.limit):
+                return None
+            p = int(torch.cuda.caching_allocator_alloc(int(nbytes), torch.cuda.current_device(), stream or 0))
+            self.live[p] = int(nbytes)
+            self.held += int(nbytes)
+            self.peak = max(self.peak, self.held)
+            return p
+
+        def free(p, stream, ctx):
+            if p:
+                self.held -= self.live.pop(int(p))
+                torch.cuda.caching_allocator_delete(int(p))
+
+        self._cg, self._refs = _cg, (_cg.ALLOC_FN(alloc), _cg.FREE_FN(free))
+
+    def __enter__(self):
+        self._cg.check(self._cg.cg_set_allocator(self._refs[0], self._refs[1], None), "cg_set_allocator")
+        return self
+
+    def __exit__(self, *exc):
+        self._cg.check(self._cg.cg_set_allocator(self._cg.ALLOC_FN(), self._cg.FREE_FN(), None), "cg_set_allocator")
+
+
+PATHS = {
+    "one block": (7, w.coxeter(7), {}),
+    "one cluster": (9, w.lrx(9), {}),
+    "rank bitmap": (10, w.lrx(10), {}),
+    "hash table": (9, w.lx(9), {"strategy": "hash"}),
+    "blocks": (11, w.coxeter(11), {}),
+    "blocks after a list": (11, w.pancake(11), {"max_radius": 9}),
+    "sweep": (9, w.lrx(9), {"strategy": "sweep"}),
+    "sort": (9, w.lrx(9), {"strategy": "sort"}),
+    "sort, many candidates": (10, w.coxeter(10), {"strategy": "sort"}),
+    "list, then sort": (10, w.coxeter(10), {"mem_cap": 12 << 20}),
+    "arrangement bitmap": (20, w.lrx(20), {"start": [1] * 10 + [0] * 10}),
+    "two words, arrangements": (70, w.lrx(70), {"start": [1] * 3 + [0] * 67}),
+    "two words, table": (18, w.lrx(18), {"max_radius": 9}),
+}
+
+
+@pytest.mark.parametrize("path", PATHS)
+def test_a_run_after_a_failed_allocation(cg, path):
+    # (a path took a buffer that a failed run had left for one that was ready: null tables, no maps)
+    from paper_2509_19162_gb300._cg import CgError
+    n, gens, kw = PATHS[path]
+    with Device() as dev:
+        with cg.Growth(n, gens, **kw) as g:
+            want = g.run()
+            far = np.sort(g.last_layer(), axis=0)
+        total = dev.calls
+        assert total > 0 and dev.held == 0
+        for i in range(total):
+            with cg.Growth(n, gens, **kw) as g:
+                dev.fail_at = dev.calls + i
+                try:
+                    cut = g.run()
+                    assert cut.status in (want.status, 2) and cut.layers == want.layers[:len(cut.layers)]
+                except CgError as e:
+                    assert e.code == -3
+                    assert dev.held == 0            # a failed run holds nothing
+                    with pytest.raises(CgError):
+                        g.last_layer()
+                dev.fail_at = -1
+                again = g.run()
+                assert (again.status, again.layers) == (want.status, want.layers)
+                assert np.array_equal(np.sort(g.last_layer(), axis=0), far)
+            assert dev.held == 0
