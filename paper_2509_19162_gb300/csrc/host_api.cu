@@ -897,10 +897,15 @@ bool cluster_preferred(const cg_growth* h) {
 // One buffer, one copy each way: control block | descriptor | layer sizes | generators | last layer's
 // keys.  (The call to S_8 under adjacent transpositions, with the antipodes: 312 us on the grid; by one
 // block 326 us with the growth's usual buffers, a table kernel and an export kernel, 255 us so.)
+constexpr int kHeadLayers = 256;                                // come back with the first copy
+struct ClusterHead {                                            // the buffer's first bytes
+    Ctl ctl;
+    JobDev job;
+    uint64_t layers[kHeadLayers];
+};
 int run_cluster(cg_growth* h, cudaStream_t st, int* final_status) {
-    constexpr uint64_t kHostLayers = 256;                       // come back with the first copy
-    const uint64_t o_job = al_up(sizeof(Ctl)), o_layers = o_job + al_up(sizeof(JobDev));
-    const uint64_t o_gens = o_layers + cg::kMaxLayers * sizeof(uint64_t);
+    constexpr uint64_t o_job = offsetof(ClusterHead, job), o_layers = offsetof(ClusterHead, layers);
+    const uint64_t o_gens = al_up(o_layers + cg::kMaxLayers * sizeof(uint64_t));
     const uint64_t o_last = o_gens + al_up(sizeof(GenSM) * h->k);
     cudaError_t e = cudaSuccess;
     const bool fresh_alloc = h->d_cl == nullptr;
@@ -912,8 +917,9 @@ int run_cluster(cg_growth* h, cudaStream_t st, int* final_status) {
             return cuda_rc(e);
         h->stats.h2d_bytes += sizeof(GenSM) * h->k;
     }
-    std::vector<char> head(o_layers + kHostLayers * sizeof(uint64_t), 0);
-    JobDev& J = *reinterpret_cast<JobDev*>(head.data() + o_job);
+    ClusterHead head;
+    std::memset(&head, 0, sizeof(head));
+    JobDev& J = head.job;
     fill_static(h, J);
     J.gens = reinterpret_cast<const GenSM*>(h->d_cl + o_gens);
     J.layer_sizes = reinterpret_cast<uint64_t*>(h->d_cl + o_layers);
@@ -924,7 +930,7 @@ int run_cluster(cg_growth* h, cudaStream_t st, int* final_status) {
     A.last = reinterpret_cast<uint64_t*>(h->d_cl + o_last);
     for (int i = 0; i < h->n; ++i) A.start |= (h->use_start ? (h->start_key >> (4 * i)) & 15u : (uint64_t)i) << (4 * i);
     A.ctl = reinterpret_cast<Ctl*>(h->d_cl);
-    if ((e = cudaMemcpyAsync(h->d_cl, head.data(), o_layers, cudaMemcpyHostToDevice, st)) != cudaSuccess) return cuda_rc(e);
+    if ((e = cudaMemcpyAsync(h->d_cl, &head, o_layers, cudaMemcpyHostToDevice, st)) != cudaSuccess) return cuda_rc(e);
     if (!h->ev0) {
         if ((e = cudaEventCreate(&h->ev0)) != cudaSuccess) return cuda_rc(e);
         if ((e = cudaEventCreate(&h->ev1)) != cudaSuccess) return cuda_rc(e);
@@ -934,19 +940,17 @@ int run_cluster(cg_growth* h, cudaStream_t st, int* final_status) {
     e = spread ? cg::launch_cluster_spread(A, h->n, spread, st) : cg::launch_cluster_small(A, 1, st);
     if (e != cudaSuccess) return cuda_rc(e);
     if ((e = cudaEventRecord(h->ev1, st)) != cudaSuccess) return cuda_rc(e);
-    if ((e = cudaMemcpyAsync(head.data(), h->d_cl, head.size(), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return cuda_rc(e);
+    if ((e = cudaMemcpyAsync(&head, h->d_cl, sizeof(head), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return cuda_rc(e);
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_rc(e);
     h->stats.launches += 1;
     h->stats.h2d_bytes += o_layers;
-    h->stats.d2h_bytes += head.size();
+    h->stats.d2h_bytes += sizeof(head);
     h->stats.kernel_ms += elapsed_ms(h->ev0, h->ev1);
     h->stats.rounds += J.radius + 1;
-    const Ctl& ctl = *reinterpret_cast<const Ctl*>(head.data());
-    if (ctl.err) return ctl.err;
+    if (head.ctl.err) return head.ctl.err;
     if (J.radius < 0 || J.radius >= cg::kMaxLayers) return CG_EDEVICE;
-    const uint64_t* sizes = reinterpret_cast<const uint64_t*>(head.data() + o_layers);
-    h->cl_layers.assign(sizes, sizes + std::min<uint64_t>((uint64_t)J.radius + 1, kHostLayers));
-    if ((uint64_t)J.radius + 1 > kHostLayers) {
+    h->cl_layers.assign(head.layers, head.layers + std::min(J.radius + 1, kHeadLayers));
+    if (J.radius + 1 > kHeadLayers) {
         h->cl_layers.resize((size_t)J.radius + 1);
         if ((e = cudaMemcpyAsync(h->cl_layers.data(), J.layer_sizes, sizeof(uint64_t) * h->cl_layers.size(),
                                  cudaMemcpyDeviceToHost, st)) != cudaSuccess)
