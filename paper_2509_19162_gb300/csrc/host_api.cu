@@ -605,18 +605,22 @@ struct cg_growth {
     cg_growth_stats stats{};
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
 
-    void release(cudaStream_t st) {
+    void release_small(cudaStream_t st) {
         dev_free(d_gens, st);
         dev_free(d_job, st);
         dev_free(d_ctl, st);
         dev_free(d_ubeg, st);
         dev_free(d_layers, st);
+        d_gens = nullptr; d_job = nullptr; d_ctl = nullptr; d_ubeg = nullptr; d_layers = nullptr;
+    }
+
+    void release(cudaStream_t st) {
+        release_small(st);
         dev_free(d_keys, st);
         dev_free(d_table, st);
         dev_free(d_comb, st);
         d_comb = nullptr;
-        d_gens = nullptr; d_job = nullptr; d_ctl = nullptr; d_ubeg = nullptr;
-        d_layers = nullptr; d_keys = nullptr; d_table = nullptr;
+        d_keys = nullptr; d_table = nullptr;
         keys_cap = table_slots = 0;
         dev_free(d_sweep, st);
         dev_free(d_sw, st);
@@ -668,13 +672,12 @@ int ensure_small_buffers(cg_growth* h, cudaStream_t st) {
     h->d_ctl = (Ctl*)dev_alloc(sizeof(Ctl), st);
     h->d_ubeg = (unsigned long long*)dev_alloc(sizeof(unsigned long long) * 2, st);
     h->d_layers = (uint64_t*)dev_alloc(sizeof(uint64_t) * cg::kMaxLayers, st);
-    if (!h->d_gens || !h->d_job || !h->d_ctl || !h->d_ubeg || !h->d_layers) return CG_ENOMEM;
-    if (h->k > 0 && (int)h->gsm.size() == h->k) {   // one-word forms (two-word keys: none)
-        cudaError_t e = cudaMemcpyAsync(h->d_gens, h->gsm.data(), sizeof(GenSM) * h->k,
-                                        cudaMemcpyHostToDevice, st);
-        if (e != cudaSuccess) return cuda_rc(e);
-    }
-    return CG_OK;
+    int rc = CG_OK;
+    if (!h->d_gens || !h->d_job || !h->d_ctl || !h->d_ubeg || !h->d_layers) rc = CG_ENOMEM;
+    if (rc == CG_OK && h->k > 0 && (int)h->gsm.size() == h->k)   // one-word forms (two-word keys: none)
+        rc = cuda_rc(cudaMemcpyAsync(h->d_gens, h->gsm.data(), sizeof(GenSM) * h->k, cudaMemcpyHostToDevice, st));
+    if (rc) h->release_small(st);           // all of them or none: a path that falls back asks again
+    return rc;
 }
 
 // What comb_rank counts: the ones of a binary start vector, or, negative, its zeros when they are fewer.
@@ -1008,15 +1011,12 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
                    (h->strategy == CG_STRATEGY_AUTO && h->start_is_perm &&
                     bitmap_eligible(h->n, h->order, mem)))
                       ? cg::kVisitBitmap : comb_preferred(h, mem) ? cg::kVisitComb : cg::kVisitHash;
-        h->comb.clear();
         if (h->mode == cg::kVisitComb) {
             h->comb = make_comb_table(h->n, std::abs(comb_ones(h)));
-            if (h->comb.size() > (size_t)cg::kCombMaxWords) {
-                h->comb.clear();
-                h->mode = cg::kVisitHash;
-            }
+            if (h->comb.size() > (size_t)cg::kCombMaxWords) h->mode = cg::kVisitHash;
         }
     }
+    if (h->mode != cg::kVisitComb) h->comb.clear();
     const bool bitmap = h->mode == cg::kVisitBitmap, comb = h->mode == cg::kVisitComb;
     h->last_is_block = false;
     const int ilp = comb ? cg::kVariantComb
@@ -1042,6 +1042,12 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
     }
     if (!h->d_keys) {
         rc = resize_state(h, may_block ? std::min<uint64_t>(first_cap, 1ull << 28) : list_cap, 0, st);
+        if (rc == CG_ENOMEM && comb) {
+            // the arrangement bitmap's growth takes room for every state at once; the hash table's begins
+            // with 2^24 of a large one and may need no more
+            h->mode = cg::kVisitHash;
+            return run_hash(h, st, final_status);
+        }
         if (rc) return rc;
     }
     if (comb && !h->d_comb) {
@@ -1421,10 +1427,14 @@ int run_sweep(cg_growth* h, cudaStream_t st, int* final_status) {
     if (!h->start_is_perm || h->n > 14 || h->n < 1) return CG_EINVAL;
     const uint64_t bytes = sweep_bytes(h->n);
     if (bytes > mem) return CG_EINVAL;
+    int rc = CG_OK;
     h->last_is_block = h->sweep_order == cg::kSweepOrderAuto && block_fits(h);
-    if (h->last_is_block) return run_block(h, st, final_status);
-    int rc = ensure_small_buffers(h, st);
-    if (rc) return rc;
+    if (h->last_is_block) {
+        if ((rc = run_block(h, st, final_status)) != CG_ENOMEM) return rc;
+        h->last_is_block = false;       // the device has no room for a fourth bit: three, state by state
+        h->release_block(st);
+    }
+    if ((rc = ensure_small_buffers(h, st))) return rc;
     const uint64_t nb = sweep_blocks(h->n);
     const uint64_t words = nb * 32, nsum = (nb + 31) / 32;
     if (!h->d_sw) {

@@ -100,3 +100,31 @@ def test_a_run_after_a_failed_allocation(cg, path):
                 assert (again.status, again.layers) == (want.status, want.layers)
                 assert np.array_equal(np.sort(g.last_layer(), axis=0), far)
             assert dev.held == 0
+
+
+@pytest.mark.parametrize("strategy", ["auto", "sweep"])
+def test_sweep_without_room_for_a_fourth_bit(cg, strategy):
+    # S_12 in blocks takes 240 MB, state by state 183 MB: a device with 200 MB to give still grows it
+    n, gens = 12, w.pancake(12)
+    want = cg.growth(n, gens, strategy="bitmap")
+    with Device() as dev:
+        dev.limit = 200 << 20
+        with cg.Growth(n, gens, strategy=strategy) as g:
+            for _ in range(2):
+                got = g.run()
+                assert (got.status, got.layers) == (want.status, want.layers)
+            assert len(g.last_layer()) == want.layers[-1]
+        assert dev.peak <= dev.limit and dev.held == 0
+
+
+def test_large_binary_coset_without_room_for_every_state(cg):
+    # 2.3 G arrangements of 34 bits: their keys take 18.7 GB, the first radii next to nothing
+    n, start = 34, [1] * 17 + [0] * 17
+    want = cg.growth(n, w.lrx(n), max_radius=12, strategy="hash", start=start)
+    with Device() as dev:
+        dev.limit = 4 << 30
+        with cg.Growth(n, w.lrx(n), max_radius=12, start=start) as g:
+            for _ in range(2):
+                got = g.run()
+                assert (got.status, got.layers) == (want.status, want.layers)
+        assert dev.held == 0
