@@ -598,6 +598,7 @@ struct cg_growth {
     bool last_is_block = false;
     char* d_cl = nullptr;                        // one-block growth: its one buffer (run_cluster)
     std::vector<uint64_t> cl_layers;             // and its layer sizes
+    int route = -1;                              // path of the last run (cg_growth_run)
     bool served = false;                         // grown for a server: the share bounds its states
 
     JobDev host_job{};
@@ -622,11 +623,7 @@ struct cg_growth {
         d_comb = nullptr;
         d_keys = nullptr; d_table = nullptr;
         keys_cap = table_slots = 0;
-        dev_free(d_sweep, st);
-        dev_free(d_sw, st);
-        d_sweep = nullptr;
-        d_sw = nullptr;
-        sw_bytes = 0;
+        release_sweep(st);
         release_block(st);
         dev_free(d_cl, st);
         d_cl = nullptr;
@@ -642,6 +639,14 @@ struct cg_growth {
         have_last = false;                 // the last layer lived in the freed buffers
         last_layer_ptr = nullptr;
         last_layer_n = 0;
+    }
+
+    void release_sweep(cudaStream_t st) {
+        dev_free(d_sweep, st);
+        dev_free(d_sw, st);
+        d_sweep = nullptr;
+        d_sw = nullptr;
+        sw_bytes = 0;
     }
 
     void release_block(cudaStream_t st) {
@@ -1034,6 +1039,7 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
                      (h->stop_above == 0 || h->stop_above >= std::max(h->order / 64, block_check(h))) &&
                      block_group(h) &&
                      block_layout(h->n, h->k).bytes + bm_bytes + first_cap * 8 + (1 << 20) <= mem;
+    if (!may_block) h->release_block(st);       // blocks that an earlier run went on in
     uint64_t list_cap = h->states_bound;
     {
         const uint64_t need = comb ? 0 : bitmap ? list_cap * 8 + bm_bytes : bytes_for(list_cap);
@@ -1163,9 +1169,9 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
                 rc = run_block(h, st, final_status, &J, h->served ? max_cap : 0);
                 if (rc != CG_ENOMEM) return rc;
                 h->last_is_block = false;       // no room on the device: stay on the list
-                h->release_block(st);
             }
             if (!over) {
+                h->release_block(st);
                 if (h->keys_cap < list_cap) {   // room for the whole list, as without the check
                     rc = resize_state(h, list_cap, J.hi, st);
                     if (rc && rc != CG_ENOMEM) return rc;
@@ -1429,11 +1435,12 @@ int run_sweep(cg_growth* h, cudaStream_t st, int* final_status) {
     if (bytes > mem) return CG_EINVAL;
     int rc = CG_OK;
     h->last_is_block = h->sweep_order == cg::kSweepOrderAuto && block_fits(h);
-    if (h->last_is_block) {
+    if (h->last_is_block) {             // (a handle holds one form's bitmaps at a time: mem_cap bounds both)
+        h->release_sweep(st);
         if ((rc = run_block(h, st, final_status)) != CG_ENOMEM) return rc;
         h->last_is_block = false;       // the device has no room for a fourth bit: three, state by state
-        h->release_block(st);
     }
+    h->release_block(st);
     if ((rc = ensure_small_buffers(h, st))) return rc;
     const uint64_t nb = sweep_blocks(h->n);
     const uint64_t words = nb * 32, nsum = (nb + 31) / 32;
@@ -2089,6 +2096,11 @@ int cg_growth_run(cg_growth_t h, void* cuda_stream, uint64_t* layer_sizes_out, i
     const bool use_cluster = cluster_preferred(h) && small_blocks(dev) > 0;
     const bool use_sweep = !use_cluster && (h->strategy == CG_STRATEGY_SWEEP ||
                                             (h->strategy == CG_STRATEGY_AUTO && sweep_preferred(h)));
+    // another path than the last run's (an option changed): its buffers beside the new ones would be more
+    // than mem_cap
+    const int route = use_cluster ? 0 : use_sort ? 1 : use_sweep ? 2 : 3;
+    if (h->route >= 0 && h->route != route) h->release(st);
+    h->route = route;
     int rc = use_cluster ? run_cluster(h, st, &status)
              : use_sort ? run_sort(h, st, &status)
                       : use_sweep ? run_sweep(h, st, &status) : run_hash(h, st, &status);

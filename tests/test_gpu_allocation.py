@@ -128,3 +128,23 @@ def test_large_binary_coset_without_room_for_every_state(cg):
                 got = g.run()
                 assert (got.status, got.layers) == (want.status, want.layers)
         assert dev.held == 0
+
+
+def test_one_handle_stays_within_its_memory_cap(cg):
+    # S_12: blocks 240 MB, state by state 183 MB, a list what it is given; never two of them at once
+    from paper_2509_19162_gb300 import _cg
+    n, gens, cap = 12, w.pancake(12), 300 << 20
+    whole = cg.growth(n, gens, strategy="bitmap").layers
+    with Device() as dev:
+        with cg.Growth(n, gens, strategy="sweep", mem_cap=cap) as g:
+            for order in ("auto", "rank", "auto"):
+                g.set_sweep_order(order)
+                assert g.run().layers == whole
+                assert dev.peak <= cap
+        with cg.Growth(n, gens, mem_cap=cap) as g:
+            for stop in (0, 1000, 0):
+                assert _cg.cg_growth_set_option(g._h, _cg.CG_OPT_STOP_ABOVE, stop) == 0
+                got = g.run().layers
+                assert got == whole[:len(got)] and (len(got) == len(whole) if not stop else got[-1] > stop)
+                assert dev.peak <= cap
+        assert dev.held == 0
