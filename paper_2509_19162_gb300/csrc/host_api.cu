@@ -3198,7 +3198,15 @@ int server_init_device(cg_server* s, cudaStream_t st) {
     s->d_ctl = (Ctl*)dev_alloc(sizeof(Ctl), st);
     s->d_gens = (GenSM*)dev_alloc(sizeof(GenSM) * kSrvMaxGens * m, st);
     s->d_layers = (uint64_t*)dev_alloc(8ull * kSrvLayers * m, st);
-    if (!s->d_jobs || !s->d_ubeg || !s->d_ctl || !s->d_gens || !s->d_layers) return CG_ENOMEM;
+    if (!s->d_jobs || !s->d_ubeg || !s->d_ctl || !s->d_gens || !s->d_layers) {
+        dev_free(s->d_jobs, st);        // all or none: the next step asks again
+        dev_free(s->d_ubeg, st);
+        dev_free(s->d_ctl, st);
+        dev_free(s->d_gens, st);
+        dev_free(s->d_layers, st);
+        s->d_jobs = nullptr; s->d_ubeg = nullptr; s->d_ctl = nullptr; s->d_gens = nullptr; s->d_layers = nullptr;
+        return CG_ENOMEM;
+    }
     s->h_jobs.assign(m, JobDev{});
     for (auto& J : s->h_jobs) {
         std::memset(&J, 0, sizeof(J));

@@ -148,3 +148,22 @@ def test_one_handle_stays_within_its_memory_cap(cg):
                 assert got == whole[:len(got)] and (len(got) == len(whole) if not stop else got[-1] > stop)
                 assert dev.peak <= cap
         assert dev.held == 0
+
+
+def test_a_server_step_after_a_failed_allocation(cg):
+    from paper_2509_19162_gb300._cg import CgError
+    from paper_2509_19162_gb300.serve import Server
+    want = cg.growth(8, w.lrx(8)).layers
+    with Device() as dev:
+        for i in range(6):              # the server's own five buffers, the job's
+            with Server() as s:
+                job = s.submit(8, w.lrx(8))
+                dev.fail_at = dev.calls + i
+                with pytest.raises(CgError) as e:
+                    s.step()
+                assert e.value.code == -3
+                dev.fail_at = -1
+                while job not in s.finished():
+                    s.step()
+                assert s.result(job).layers == want
+            assert dev.held == 0
