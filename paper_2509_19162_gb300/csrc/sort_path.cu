@@ -180,7 +180,13 @@ __device__ __forceinline__ unsigned long long candidate_state(const ExpandSrc& s
                                                               unsigned* j) {
     unsigned long long off = i - (unsigned long long)first * src.F;
     unsigned g = first;
-    while (off >= src.F) { off -= src.F; ++g; }
+    if (src.F >= (unsigned long long)kTile) {           // at most one generator further
+        if (off >= src.F) { off -= src.F; ++g; }
+    } else {                                            // (off < F + kTile)
+        const unsigned more = (unsigned)off / (unsigned)src.F;
+        off = (unsigned)off - more * (unsigned)src.F;
+        g += more;
+    }
     *j = g;
     return off;
 }
@@ -218,22 +224,25 @@ __global__ void expand_all_kernel(const GenSM* __restrict__ gens, int k, const u
 }
 
 // ---- digit histograms of every pass in one read ------------------------------------------
-// kGen: the candidates of src, a state's together (one read of the frontier).  Every generator is applied
-// in step, and the one to pass over not counted: the lanes of a warp read the same generator.
+// kGen: the candidates of src, `span` generators of a state together (few reads of the frontier).  Every
+// generator is applied in step, and the one to pass over not counted: the lanes of a warp read the same
+// generator.
 template <bool kGen>
 __global__ void __launch_bounds__(kBlock)
-hist_all_kernel(const uint64_t* __restrict__ keys, ExpandSrc src, unsigned long long n, int passes, int lo,
+hist_all_kernel(const uint64_t* __restrict__ keys, ExpandSrc src, int span, unsigned long long n, int passes, int lo,
                 unsigned long long* __restrict__ ghist) {
     __shared__ unsigned s_h[kSortMaxPasses][kDigits];
     for (int i = threadIdx.x; i < kSortMaxPasses * kDigits; i += kBlock) (&s_h[0][0])[i] = 0;
     __syncthreads();
     const unsigned long long stride = (unsigned long long)gridDim.x * kBlock;
-    const unsigned long long items = kGen ? src.F : n;
-    const int each = kGen ? src.k : 1;
+    const bool split = kGen && span < src.k;
+    const unsigned long long items = !kGen ? n : split ? src.F * (unsigned)((src.k + span - 1) / span) : src.F;
     const bool skips = kGen && src.each < src.k;
     for (unsigned long long i = blockIdx.x * (unsigned long long)kBlock + threadIdx.x; i < items; i += stride) {
-        const uint64_t in = kGen ? src.frontier[i] : keys[i];
-        for (int g = 0; g < each; ++g) {
+        const unsigned part = split ? (unsigned)(i / src.F) : 0u;
+        const uint64_t in = kGen ? src.frontier[i - (unsigned long long)part * src.F] : keys[i];
+        const int g0 = (int)part * span, g1 = !kGen ? 1 : min(g0 + span, src.k);
+        for (int g = g0; g < g1; ++g) {
             if (skips && g + 1 == (int)(in >> 60)) continue;
             const uint64_t key = kGen ? apply_gen(src.gens[g], in & src.mask) : in;
             for (int p = 0; p < passes; ++p) atomicAdd(&s_h[p][(key >> (lo + kRadixBits * p)) & (kDigits - 1)], 1u);
@@ -739,6 +748,22 @@ cudaError_t launch_expand_all(const GenSM* d_gens, int k, const uint64_t* in, un
 
 namespace {
 
+// Histograms of the candidates of src.  While the states are fewer than the threads of a full grid their
+// generators are spread over several threads: one thread a state left most of the chip idle in thin
+// layers with many generators (whole growths: S_8 under 112 three-cycles 1.14 ms so, 0.88 ms spread;
+// S_8 under all 28 transpositions 0.98 / 0.89, S_8 under adjacent ones 2.31 / 2.23).
+constexpr unsigned kHistBlocks = 152u * 4;
+cudaError_t launch_hist_gen(const ExpandSrc& src, int passes, int lo, unsigned long long* ghist, cudaStream_t st) {
+    const unsigned long long full = (unsigned long long)kHistBlocks * kBlock;
+    const unsigned long long parts = src.F >= full ? 1ull : (full + src.F - 1) / src.F;
+    const int span = parts >= (unsigned long long)src.k ? 1 : (int)(((unsigned long long)src.k + parts - 1) / parts);
+    const unsigned long long items = src.F * (unsigned long long)((src.k + span - 1) / span);
+    const unsigned long long hb = (items + kBlock - 1) / kBlock;
+    hist_all_kernel<true><<<hb > kHistBlocks ? kHistBlocks : (unsigned)hb, kBlock, 0, st>>>(nullptr, src, span, 0, passes,
+                                                                                           lo, ghist);
+    return cudaGetLastError();
+}
+
 // The passes of one sort, over key bits [lo, bits).  Input: `in` keys, or the candidates of src
 // (gen).  Pass p writes bufs[(P - 1 - p) & 1], so the last pass writes bufs[0].  The error word
 // and the descriptors are cleared first (one memset); the caller zeroes nothing.
@@ -750,10 +775,13 @@ cudaError_t radix_passes(const uint64_t* in, const ExpandSrc* src, unsigned long
     cudaError_t e = cudaMemsetAsync(s.ghist, 0, reset, st);
     if (e != cudaSuccess) return e;
     const ExpandSrc none{};
-    unsigned long long hb = ((src ? src->F : n) + kBlock - 1) / kBlock;
-    if (hb > 152ull * 4) hb = 152ull * 4;
-    if (src) hist_all_kernel<true><<<(unsigned)hb, kBlock, 0, st>>>(nullptr, *src, n, P, lo, s.ghist);
-    else hist_all_kernel<false><<<(unsigned)hb, kBlock, 0, st>>>(in, none, n, P, lo, s.ghist);
+    if (src) {
+        if ((e = launch_hist_gen(*src, P, lo, s.ghist, st)) != cudaSuccess) return e;
+    } else {
+        unsigned long long hb = (n + kBlock - 1) / kBlock;
+        if (hb > kHistBlocks) hb = kHistBlocks;
+        hist_all_kernel<false><<<(unsigned)hb, kBlock, 0, st>>>(in, none, 1, n, P, lo, s.ghist);
+    }
     const uint64_t* cur = in;
     for (int p = 0; p < P; ++p) {
         uint64_t* dst = bufs[(P - 1 - p) & 1];
@@ -823,11 +851,7 @@ cudaError_t launch_candidate_hist(const ExpandSrc& src, int bits, const SortScra
     const unsigned long long n = src.F * (unsigned long long)src.each;
     cudaError_t e = cudaMemsetAsync(s.ghist, 0, sizeof(unsigned long long) * kSortMaxPasses * kDigits, st);
     if (e != cudaSuccess || n == 0) return e;
-    unsigned long long hb = (src.F + kBlock - 1) / kBlock;
-    if (hb > 152ull * 4) hb = 152ull * 4;
-    hist_all_kernel<true><<<(unsigned)hb, kBlock, 0, st>>>(nullptr, src, n, passes_of(bits - lo < 1 ? 1 : bits - lo),
-                                                          lo, s.ghist);
-    return cudaGetLastError();
+    return launch_hist_gen(src, passes_of(bits - lo < 1 ? 1 : bits - lo), lo, s.ghist, st);
 }
 
 cudaError_t launch_expand_filter(const ExpandSrc& src, int shift, unsigned d0, unsigned d1, uint64_t* out,
