@@ -1779,10 +1779,7 @@ int sort_steps(cg_growth* h, cudaStream_t st, int cur, int prev, uint64_t Fcur, 
         if (h->stop_above > 0 && Fn > h->stop_above) { status = cg::kTruncAbove; break; }
         if ((int)h->sort_layers.size() >= cg::kMaxLayers) { status = cg::kTruncRadius; break; }
     }
-    if (cur_tagged) {                   // the last layer is read as plain keys
-        if ((e = cg::launch_mask_keys(h->d_L[cur], Fcur, mask, st)) != cudaSuccess) return cuda_rc(e);
-        h->stats.launches += 1;
-    }
+    // (cg_growth_last_layer strips the tags of the last layer, as it does a list's)
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_rc(e);
     h->host_job.radius = radius;
     h->host_job.status = status;
