@@ -23,6 +23,7 @@
 //                 decoupled look-back over tiles: layer r+1, sorted, and its size
 // The same primitives back the step-level entry points cg_sort_unique and cg_set_difference.
 #include <cstdint>
+#include <type_traits>
 
 #include "cg_device.cuh"
 #include "sort_kernels.h"
@@ -176,13 +177,14 @@ __device__ __forceinline__ uint64_t tagged_image(const ExpandSrc& src, const Gen
 
 // Candidate number i, given the generator `first` of an earlier one (a division per tile instead of one
 // per candidate): its state's place in the frontier, and its number among the state's candidates.
+template <bool kThin>
 __device__ __forceinline__ unsigned long long candidate_state(const ExpandSrc& src, unsigned long long i, unsigned first,
                                                               unsigned* j) {
     unsigned long long off = i - (unsigned long long)first * src.F;
     unsigned g = first;
-    if (src.F >= (unsigned long long)kTile) {           // at most one generator further
+    if constexpr (!kThin) {                             // F >= kTile: at most one generator further
         if (off >= src.F) { off -= src.F; ++g; }
-    } else {                                            // (off < F + kTile)
+    } else {                                            // off < F + kTile
         const unsigned more = (unsigned)off / (unsigned)src.F;
         off = (unsigned)off - more * (unsigned)src.F;
         g += more;
@@ -199,7 +201,7 @@ __device__ __forceinline__ uint64_t candidate_of(const ExpandSrc& src, uint64_t 
 
 __device__ __forceinline__ uint64_t gen_candidate(const ExpandSrc& src, unsigned long long i) {
     unsigned j;
-    const unsigned long long off = candidate_state(src, i, (unsigned)(i / src.F), &j);
+    const unsigned long long off = candidate_state<false>(src, i, (unsigned)(i / src.F), &j);
     return candidate_of(src, src.frontier[off], j);
 }
 
@@ -280,12 +282,16 @@ onesweep_kernel(const uint64_t* __restrict__ in, ExpandSrc src, uint64_t* __rest
     const unsigned long long base = (unsigned long long)tile * kTile;
     uint64_t key[kItems];
     unsigned rank[kItems];
+    auto load = [&](auto thin) {
 #pragma unroll
-    for (int r = 0; r < kItems; ++r) {
-        const unsigned long long idx = base + (unsigned)(wid * (kItems * 32) + r * 32 + lane);
-        if (kGen) key[r] = idx < n ? src.frontier[candidate_state(src, idx, s_gen, &rank[r])] : 0;
-        else key[r] = idx < n ? in[idx] : 0;
-    }
+        for (int r = 0; r < kItems; ++r) {
+            const unsigned long long idx = base + (unsigned)(wid * (kItems * 32) + r * 32 + lane);
+            if (kGen) key[r] = idx < n ? src.frontier[candidate_state<thin.value>(src, idx, s_gen, &rank[r])] : 0;
+            else key[r] = idx < n ? in[idx] : 0;
+        }
+    };
+    if (kGen && src.F < (unsigned long long)kTile) load(std::true_type{});
+    else load(std::false_type{});
     // the generators after every state is on its way: applied one state at a time, each would wait for its
     // own trip to L2 (S_11, ten star transpositions: 24.3 / 23.5 ms a growth)
     if constexpr (kGen) {
