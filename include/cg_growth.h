@@ -153,8 +153,9 @@ int cg_growth_create(int n, int k, const uint8_t* gens, int inverse_closed, int 
  * HASH (others fail at run with CG_EINVAL).  A start with repeated values takes AUTO, HASH or SORT
  * (BITMAP then fails at run with CG_EINVAL).  For binary one-word vectors and for two-word vectors
  * with fewer than 2^32 arrangements of their values, AUTO keeps a visited bit per arrangement when
- * the growth may reach at least 1/512 of them and its states and the hash table would have fitted
- * mem_cap as well (cg_growth_stats.strategy_used is then CG_STRATEGY_BITMAP), else HASH.
+ * the growth may reach at least 1/512 of them (and, with two words, 512 states) and its states and the
+ * hash table would have fitted mem_cap as well (cg_growth_stats.strategy_used is then
+ * CG_STRATEGY_BITMAP), else HASH.
  * A start whose values are all equal is fixed by every generator: its growth is {1}.  Releases
  * buffers sized for an earlier start.  Errors: CG_EINVAL (also a generator that fits neither
  * the shift-and-mask form, at most 16 distinct offsets in one word or 32 in two, nor the

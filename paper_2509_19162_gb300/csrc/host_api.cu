@@ -1292,11 +1292,15 @@ int run_wide(cg_growth* h, cudaStream_t st, int* final_status) {
     // them where their number and the ranking tables allow it, and only where the hash table and every
     // state would have fitted as well, so that nothing else would have stopped the growth.  40 elements
     // of four values under L, R, X: 19.7 M states, 2.5 MB of bitmap in L2 for a table of 1 GB, kernel 3.68 / 2.20 ms.
+    // Small orbits don't earn the tables (made on the host, copied, read by every block): a one among 65, 99
+    // and 127 zeros under L, R, X takes 405, 536 and 694 us with the hash table, 424, 606 and 717 with them, two
+    // ones among 64 zeros (2145 states) 845 and 747.
+    constexpr uint64_t kRankMinStates = 512;
     const bool whole = h->states_bound <= max_cap && h->states_bound * 48 <= std::min<uint64_t>(mem, kExactAllocLimit);
     if (!h->d_wkeys) {
         h->wrank = cg::WideRank{};
         if (h->strategy == CG_STRATEGY_AUTO && h->use_start && whole && !(h->rearrangements >> 32) &&
-            h->rearrangements <= 512 * h->states_bound)
+            h->states_bound >= kRankMinStates && h->rearrangements <= 512 * h->states_bound)
             h->wrank_table = make_wide_rank(h->start_values.data(), h->n, h->width, h->wrank);
     }
     if (h->wrank.steps && !h->d_wrank) {
