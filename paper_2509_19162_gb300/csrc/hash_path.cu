@@ -346,12 +346,15 @@ __device__ void close_round_single(JobDev* jobs, unsigned long long* ubeg, Ctl* 
 // has queued: with half the entries a growth bound by random DRAM accesses ran 15 % longer (S_14,
 // six random generators to radius 12: 20.1 against 23.2 ms), while a rank-bitmap launch that reads
 // visited words before its atomics finds few new states and has the better use of the room as L1
-// (S_12 pancake 28.9 against 30.3 ms).  Launches of several jobs keep selectors or generators per
-// warp as well and have to stay within 48 KB, or a quarter of the SM.
-constexpr int kStage = 512, kStageTest = 256, kStageMulti = 448;
+// (S_12 pancake 28.9 against 30.3 ms).  In launches of several jobs a warp's room also holds its
+// current job's generators and pending candidates, and has to stay within 48 KB a block, or a
+// quarter of the SM: kStageBitmap or kStageHash entries, of which a job takes what it needs and
+// leaves the rest to its staged states (room_gens): four growths of S_11 under L, X 5.24 ms with
+// fixed parts, 256 entries for the states; 4.70 so.
+constexpr int kStage = 512, kStageTest = 256, kStageBitmap = 664, kStageHash = 728;
 
 __host__ __device__ __forceinline__ int stage_entries(bool multi, bool bitmap, bool test) {
-    return multi ? (bitmap ? kStageTest : kStageMulti) : (bitmap && test ? kStageTest : kStage);
+    return multi ? (bitmap ? kStageBitmap : kStageHash) : (bitmap && test ? kStageTest : kStage);
 }
 
 // The static fields of one job as the work loops use them.  A single-job launch receives them
@@ -386,6 +389,14 @@ __host__ __device__ __forceinline__ bool bitmap_test_first(unsigned long long fr
                                                            int k, int closed) {
     return 4 * fresh < expanded * (unsigned long long)(k - (closed ? 1 : 0));
 }
+
+// Frontier [lo, hi) and units [u0, u1) of the job a warp works on, in a launch of several jobs: in shared
+// memory with its JobConst, because the loop around the units has no registers to spare (spilled, they
+// and the unit numbers in 64 bits cost 24 M local accesses in the launch below, more than its keys).
+struct JobRange {
+    unsigned long long lo, hi;
+    unsigned u0, u1;
+};
 
 __device__ __forceinline__ JobConst job_const(const JobDev* J, int stage) {
     JobConst c;
@@ -706,9 +717,9 @@ __device__ __forceinline__ void bitmap_drain(BitmapCand& prev, uint64_t* buf, in
 }
 
 // Next work unit of the block for the calling warp (one shared-memory atomic per warp).
-__device__ __forceinline__ unsigned long long draw_unit(unsigned long long& counter, int lane) {
-    unsigned long long u = 0;
-    if (lane == 0) u = atomicAdd(&counter, 1ull);
+__device__ __forceinline__ unsigned draw_unit(unsigned& counter, int lane) {
+    unsigned u = 0;
+    if (lane == 0) u = atomicAdd(&counter, 1u);
     return __shfl_sync(0xffffffffu, u, 0);
 }
 
@@ -852,6 +863,14 @@ constexpr int kWarpGens = 10;
 // this many; of a warp's current job, as many as fit where its kWarpGens generators would go.
 constexpr int kSmemSels = 64;
 constexpr int kWarpSels = kWarpGens * (int)sizeof(GenSM) / (kSelWords * 4);
+// 8-byte words of a warp's room (stage_entries) that a job's k generators take, 0 when they stay in
+// global memory.  Both sizes are multiples of 16 bytes, as is the room's.
+__device__ __forceinline__ int room_gens(int k, bool bitmap) {
+    return bitmap ? (k <= kWarpSels ? k * kSelWords / 2 : 0) : (k <= kWarpGens ? k * (int)sizeof(GenSM) / 8 : 0);
+}
+static_assert(kStageBitmap % 2 == 0 && kStageHash % 2 == 0 && kSelWords % 4 == 0, "a warp's room: 16-byte parts");
+static_assert(kStageBitmap - kWarpGens * (int)sizeof(GenSM) / 8 - kPend * 2 >= kStageTest, "room for staged states");
+static_assert(kStageHash - kWarpGens * (int)sizeof(GenSM) / 8 >= 448, "room for staged states");
 constexpr int kGenStride = (int)sizeof(GenSM) / 4;
 
 // kMulti = false: the launch has exactly one job (the single-job path only is compiled, which
@@ -862,13 +881,14 @@ __global__ void __launch_bounds__(kGrowBlock, kMode >= 2 ? 4 : ((kMode == 1 && k
 hash_grow_kernel(JobDev* jobs, int njobs, unsigned long long* ubeg, Ctl* ctl, int max_rounds,
                  uint64_t timeout_ns, const AdmitDev* adm, const JobConst jc) {
     constexpr bool kBitmap = kMode == kVisitBitmap, kComb = kMode == kVisitComb;
-    extern __shared__ uint64_t s_stage[];       // jc.stage entries a warp
-    __shared__ uint4 s_pend[kBitmap || kComb ? kGrowBlock / 32 : 1][kBitmap || kComb ? kPend : 1];
+    extern __shared__ __align__(16) uint64_t s_stage[];   // jc.stage entries a warp
+    constexpr bool kPends = !kMulti && (kBitmap || kComb);
+    __shared__ uint4 s_pend[kPends ? kGrowBlock / 32 : 1][kPends ? kPend : 1];
     __shared__ GenSM s_gens[!kMulti && !kBitmap ? kSmemGens : 1];
     __shared__ alignas(16) uint32_t s_selw[!kMulti && kBitmap ? kSmemSels * kSelWords : 4];
-    __shared__ unsigned long long s_unit;
+    __shared__ unsigned s_unit;
     __shared__ JobConst s_jc[kMulti ? kGrowBlock / 32 : 1];
-    __shared__ GenSM s_wgens[kMulti ? kGrowBlock / 32 : 1][kMulti ? kWarpGens : 1];
+    __shared__ JobRange s_range[kMulti ? kGrowBlock / 32 : 1];
     const GenSM* single_gens = jobs[0].gens;
     if (!kMulti && !kBitmap && jobs[0].k <= kSmemGens) {
         for (int j = threadIdx.x; j < jobs[0].k; j += blockDim.x) s_gens[j] = jobs[0].gens[j];
@@ -882,7 +902,7 @@ hash_grow_kernel(JobDev* jobs, int njobs, unsigned long long* ubeg, Ctl* ctl, in
     }
     const int lane = threadIdx.x & 31;
     uint64_t* buf = s_stage + (threadIdx.x >> 5) * jc.stage;
-    uint4* pend = s_pend[kBitmap || kComb ? threadIdx.x >> 5 : 0];
+    uint4* pend = s_pend[kPends ? threadIdx.x >> 5 : 0];
     // binary vectors: the ranking table, behind the staged states
     const uint32_t* comb = nullptr;
     if constexpr (kComb) {
@@ -942,7 +962,7 @@ hash_grow_kernel(JobDev* jobs, int njobs, unsigned long long* ubeg, Ctl* ctl, in
         const bool shared_tail = total >= 16ull * gridDim.x;
         const unsigned long long stat = shared_tail ? static_units(total) : total;
         if (kMulti) {
-            if (threadIdx.x == 0) s_unit = stat * blockIdx.x / gridDim.x;   // this block's first unit
+            if (threadIdx.x == 0) s_unit = (unsigned)(stat * blockIdx.x / gridDim.x);   // this block's first unit
             __syncthreads();
         }
         int cnt = 0;
@@ -954,7 +974,6 @@ hash_grow_kernel(JobDev* jobs, int njobs, unsigned long long* ubeg, Ctl* ctl, in
                                                : (unsigned long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
             single_phase(test, w0, W, lo, hi);
         } else {
-            int cur = -1;
             JobDev* J = nullptr;
             // the current job's static fields, one copy per warp in shared memory (read where
             // used, which keeps them out of the registers)
@@ -968,35 +987,35 @@ hash_grow_kernel(JobDev* jobs, int njobs, unsigned long long* ubeg, Ctl* ctl, in
             prev.lo = prev.hi = prev.w = prev.b = prev.word = 0;
             int pcnt = 0;
             int ovf = 0;                            // the current job's overflow flag, read a unit ago
-            unsigned long long lo = 0, hi = 0, u0 = 0;
-            const unsigned long long ue = stat * (blockIdx.x + 1) / gridDim.x;
-            unsigned long long pending = ~0ull;
+            JobRange& jr = s_range[threadIdx.x >> 5];   // its frontier and its units
+            // (unit numbers fit 32 bits: a unit is 32 states of 8 bytes)
+            const unsigned ue = (unsigned)(stat * (blockIdx.x + 1) / gridDim.x);
+            unsigned pending = ~0u;
             // a batch launch (adm): units map to slots of the active list, 32 * unit_mult
             // frontier states each; otherwise to jobs, 32 states each
             const int nj = adm ? s_nact : njobs;
             const int* act = adm ? adm->act[s_sel] : nullptr;
             const int umult = adm ? adm->unit_mult : 1;
             // the block's range, then (large rounds) the shared half, two units per draw
-            auto next_unit = [&]() -> unsigned long long {
-                const unsigned long long u = draw_unit(s_unit, lane);
+            auto next_unit = [&]() -> unsigned {
+                const unsigned u = draw_unit(s_unit, lane);
                 if (u < ue) return u;
-                if (pending != ~0ull) {
-                    const unsigned long long p = pending;
-                    pending = ~0ull;
+                if (pending != ~0u) {
+                    const unsigned p = pending;
+                    pending = ~0u;
                     return p;
                 }
-                if (!shared_tail) return ~0ull;
-                unsigned long long d = 0;
-                if (lane == 0) d = atomicAdd(&ctl->dyn_next, 2ull);
+                if (!shared_tail) return ~0u;
+                unsigned d = 0;
+                if (lane == 0) d = (unsigned)atomicAdd(&ctl->dyn_next, 2ull);
                 d = __shfl_sync(0xffffffffu, d, 0);
-                if (d >= total) return ~0ull;
-                if (d + 1 < total) pending = d + 1;
+                if (d >= (unsigned)total) return ~0u;
+                if (d + 1 < (unsigned)total) pending = d + 1;
                 return d;
             };
-            unsigned long long u1 = 0;              // units of slot cur: [u0, u1)
-            for (unsigned long long u = next_unit(); u != ~0ull; u = next_unit()) {
+            for (unsigned u = next_unit(); u != ~0u; u = next_unit()) {
                 // a warp's units mostly stay within one job: search the table only on leaving it
-                if (cur >= 0 && u >= u0 && u < u1) {
+                if (J && u >= jr.u0 && u < jr.u1) {
                     // same job as the previous unit
                 } else {
                     const int slot = find_job(ubeg, nj, u);
@@ -1004,27 +1023,39 @@ hash_grow_kernel(JobDev* jobs, int njobs, unsigned long long* ubeg, Ctl* ctl, in
                         if (jbitmap) bitmap_drain(prev, buf, cnt, pend, pcnt, J, c, c.test != 0, lane);
                         stage_flush(buf, cnt, J, c, lane);
                     }
-                    cur = slot;
                     J = jobs + (act ? __ldcg(act + slot) : slot);
-                    if (lane == 0) c = job_const(J, jc.stage);
+                    if (lane == 0) {                // (one trip to L2 for all that changes by round)
+                        const JobRange r{ld_relaxed_ull(&J->lo), ld_relaxed_ull(&J->hi),
+                                         (unsigned)ld_relaxed_ull(ubeg + slot), (unsigned)ld_relaxed_ull(ubeg + slot + 1)};
+                        c = job_const(J, jc.stage);
+                        jr = r;
+                    }
                     __syncwarp();
                     ovf = 0;
                     jg = J->gens;
                     jbitmap = kBitmap && c.mode == kVisitBitmap;
+                    // the warp's room (nothing is staged or pending in it now): the job's generators,
+                    // candidates pending, staged states
+                    uint64_t* room = s_stage + (threadIdx.x >> 5) * jc.stage;
+                    const int gwords = room_gens(c.k, jbitmap), pwords = jbitmap && c.test ? kPend * 2 : 0;
+                    pend = reinterpret_cast<uint4*>(room + gwords);
+                    buf = room + gwords + pwords;
+                    if (lane == 0) c.stage = jc.stage - gwords - pwords;
+                    __syncwarp();
                     if (jbitmap) {
                         jsel = jg->sel;
                         jstride = kGenStride;
-                        if (c.k <= kWarpSels) {
-                            uint32_t* to = reinterpret_cast<uint32_t*>(s_wgens[threadIdx.x >> 5]);
+                        if (gwords > 0) {
+                            uint32_t* to = reinterpret_cast<uint32_t*>(room);
                             for (int i = lane; i < c.k * kSelWords; i += 32)
                                 to[i] = jg[i / kSelWords].sel[i % kSelWords];
                             __syncwarp();
                             jsel = to;
                             jstride = kSelWords;
                         }
-                    } else if (c.k <= kWarpGens) {
-                        // copy them into this warp's shared slots, word by word across the lanes
-                        GenSM* dst = s_wgens[threadIdx.x >> 5];
+                    } else if (gwords > 0) {
+                        // copy them into the warp's room, word by word across the lanes
+                        GenSM* dst = reinterpret_cast<GenSM*>(room);
                         const unsigned words = (unsigned)c.k * (unsigned)(sizeof(GenSM) / 4);
                         const unsigned* from = reinterpret_cast<const unsigned*>(jg);
                         unsigned* to = reinterpret_cast<unsigned*>(dst);
@@ -1032,10 +1063,6 @@ hash_grow_kernel(JobDev* jobs, int njobs, unsigned long long* ubeg, Ctl* ctl, in
                         __syncwarp();
                         jg = dst;
                     }
-                    lo = ld_relaxed_ull(&J->lo);
-                    hi = ld_relaxed_ull(&J->hi);
-                    u0 = ld_relaxed_ull(ubeg + slot);
-                    u1 = ld_relaxed_ull(ubeg + slot + 1);
                 }
                 // A job whose buffers ran full stops expanding (the host grows them or reports
                 // the exact layers so far): its flag, read while the previous unit of the same
@@ -1044,7 +1071,8 @@ hash_grow_kernel(JobDev* jobs, int njobs, unsigned long long* ubeg, Ctl* ctl, in
                 ovf = ld_relaxed_int(&J->overflow);
                 // the unit's unit_mult groups of 32 states, the next group's keys loaded while one
                 // is expanded
-                unsigned long long first = lo + (((u - u0) * (unsigned long long)umult) << 5);
+                const unsigned long long hi = jr.hi;
+                unsigned long long first = jr.lo + (((u - jr.u0) * (unsigned long long)umult) << 5);
                 uint64_t s_nx = first + lane < hi ? __ldcg(c.keys + first + lane) : 0;
                 for (int sub = 0; sub < umult && first < hi; ++sub) {
                     const unsigned long long idx = first + lane;
