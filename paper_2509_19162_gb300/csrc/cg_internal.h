@@ -146,9 +146,9 @@ constexpr int kVisitComb = 3;           // bitmap over the C(n, m) binary vector
 constexpr int kVariantComb = 21;        // its kernel variant
 constexpr int kCombMaxWords = 6144;     // ranking table: at most 96 rows of 64
 
-// Generators beyond the parent edge from which a rank-bitmap job reads a visited word before its
-// atomic as long as nothing better is known (a single job decides by its last round's yield, see
-// bitmap_test_first in hash_path.cu).
+// Generators beyond the parent edge from which a single rank-bitmap job's first round reads a visited
+// word before its atomic (later rounds, and those of several jobs, go by the last round's yield: see
+// bitmap_test_first and job_reads_first in hash_path.cu).
 constexpr int kTestMinDegree = 4;
 
 enum JobStatus : int {
@@ -197,7 +197,8 @@ struct alignas(128) JobDev {
     int radius;                // radius of the frontier layer
     int status;                // JobStatus
     int overflow;              // set during a round: keys or table ran out
-    int pad;
+    int reads_first;           // rank bitmap, one of several jobs: this round reads visited words
+                               //    before its atomics
 };
 // The round close loads (lo, hi) and (tail, radius | status << 32) as two 16-byte vectors.
 static_assert(offsetof(JobDev, lo) % 16 == 0 && offsetof(JobDev, hi) == offsetof(JobDev, lo) + 8,

@@ -51,6 +51,27 @@ __host__ __device__ __forceinline__ unsigned long long static_units(unsigned lon
     return total - total / 2;
 }
 
+// Rank bitmap, read before the atomic or not: with `fresh` new states out of `expanded` last round,
+// whether less than a quarter of the candidates were new.  A read costs L2 about half of what an
+// atomic does (287 G/s against 133 G/s on a bitmap in L2), so it pays while most bits are found set:
+// S_12 pancake 28.8 ms, 41.2 ms without; S_11 under L, R, X, half of whose candidates are new, 1.04 ms
+// by this rule and 1.13 ms with the line at a half.
+__host__ __device__ __forceinline__ bool bitmap_test_first(unsigned long long fresh, unsigned long long expanded,
+                                                           int k, int closed) {
+    return 4 * fresh < expanded * (unsigned long long)(k - (closed ? 1 : 0));
+}
+
+// The same for one of several jobs.  Its thin rounds would pay a read's trip and the atomic's (sixteen S_10
+// under adjacent transpositions 6.45 ms from 2^15 states on, 6.11 from 2^18), and the line lies at a third
+// (four S_11 under ten random generators 9.42 ms at a quarter, 9.11 at a third; under L, X 4.62, 4.64, and
+// 5.04 at a half).  By the out-degree alone, as it once was, layers of mostly new states paid for reads that
+// found nothing: eight S_11 under four random generators to radius 14 2.23 ms against 1.53, 32 of S_12 under
+// ten to radius 9 246 against 143.
+constexpr unsigned long long kTestMinStates = 1ull << 18;
+__device__ __forceinline__ int job_reads_first(const JobDev& J, unsigned long long fresh, unsigned long long expanded) {
+    return fresh >= kTestMinStates && 3 * fresh < expanded * (unsigned long long)(J.k - J.closed) ? 1 : 0;
+}
+
 // Phase B, executed by the block that arrives last at the round's barrier: close the layer of
 // every running job and lay out the work of the next round.  ubeg has njobs + 1 entries.
 __device__ void close_round(JobDev* jobs, int njobs, unsigned long long* ubeg, Ctl* ctl) {
@@ -87,6 +108,7 @@ __device__ void close_round(JobDev* jobs, int njobs, unsigned long long* ubeg, C
                         V.radius = radius;
                         V.lo = hi;
                         V.hi = tail;
+                        V.reads_first = job_reads_first(J, fresh, hi - lo);
                         if (J.max_radius >= 0 && radius >= J.max_radius) status = kTruncRadius;
                         else if (J.stop_above > 0 && fresh > J.stop_above) status = kTruncAbove;
                         else if (radius + 1 >= J.layers_cap) status = kTruncRadius;
@@ -95,7 +117,6 @@ __device__ void close_round(JobDev* jobs, int njobs, unsigned long long* ubeg, C
                 }
                 if (status != kRunning) V.status = status;
             }
-            (void)lo;
         }
         // block-wide exclusive scan of units
         unsigned long long v = units;
@@ -187,7 +208,6 @@ __device__ void close_round_admit(JobDev* jobs, unsigned long long* ubeg, Ctl* c
             const int overflow = ld_relaxed_int(&J.overflow);
             int radius = (int)(unsigned)(rs & 0xffffffffull);
             int status = (int)(unsigned)(rs >> 32);
-            (void)lo;
             if (status == kRunning) {
                 volatile JobDev& V = jobs[j];
                 if (overflow) {
@@ -202,6 +222,7 @@ __device__ void close_round_admit(JobDev* jobs, unsigned long long* ubeg, Ctl* c
                         V.radius = radius;
                         V.lo = hi;
                         V.hi = tail;
+                        V.reads_first = job_reads_first(J, fresh, hi - lo);
                         if (J.max_radius >= 0 && radius >= J.max_radius) status = kTruncRadius;
                         else if (J.stop_above > 0 && fresh > J.stop_above) status = kTruncAbove;
                         else if (radius + 1 >= J.layers_cap) status = kTruncRadius;
@@ -380,15 +401,6 @@ struct JobConst {
     int stage;             // staged states a warp holds
 };
 
-// Rank bitmap, read before the atomic or not: with `fresh` new states out of `expanded` last round,
-// whether less than a quarter of the candidates were new.  A read costs L2 about half of what an
-// atomic does (287 G/s against 133 G/s on a bitmap in L2), so it pays while most bits are found set:
-// S_12 pancake 28.8 ms, 41.2 ms without; S_11 under L, R, X, half of whose candidates are new, 1.04 ms
-// by this rule and 1.13 ms with the line at a half.
-__host__ __device__ __forceinline__ bool bitmap_test_first(unsigned long long fresh, unsigned long long expanded,
-                                                           int k, int closed) {
-    return 4 * fresh < expanded * (unsigned long long)(k - (closed ? 1 : 0));
-}
 
 // Frontier [lo, hi) and units [u0, u1) of the job a warp works on, in a launch of several jobs: in shared
 // memory with its JobConst, because the loop around the units has no registers to spare (spilled, they
@@ -410,7 +422,7 @@ __device__ __forceinline__ JobConst job_const(const JobDev* J, int stage) {
     c.tagged = J->tagged;
     c.mode = J->mode;
     c.closed = J->closed;
-    c.test = c.k - (c.closed ? 1 : 0) >= kTestMinDegree;     // several jobs: by the out-degree alone
+    c.test = ld_relaxed_int(&J->reads_first);       // several jobs: set by the block that closed the round
     c.stage = stage;
     return c;
 }
@@ -1166,6 +1178,7 @@ __device__ void init_job(JobDev& J) {
     J.tail = 1;
     J.radius = 0;
     J.overflow = 0;
+    J.reads_first = 0;
     J.status = kRunning;
     if (J.max_radius == 0) J.status = kTruncRadius;
 }

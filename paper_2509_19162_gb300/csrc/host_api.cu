@@ -685,6 +685,13 @@ int ensure_small_buffers(cg_growth* h, cudaStream_t st) {
     return rc;
 }
 
+// 1: every generator's inverse is in the set, and has a tag.
+int all_closed(const std::vector<GenSM>& gens) {
+    for (const GenSM& g : gens)
+        if (g.inv_tag == 0) return 0;
+    return 1;
+}
+
 // What comb_rank counts: the ones of a binary start vector, or, negative, its zeros when they are fewer.
 int comb_ones(const cg_growth* h) {
     const int m = __builtin_popcountll(h->start_key);
@@ -757,8 +764,7 @@ void fill_static(cg_growth* h, JobDev& J) {
     J.use_start = h->use_start ? 1 : 0;
     J.start_key = h->start_key;
     J.tagged = h->n * h->width <= 60 ? 1 : 0;
-    J.closed = 1;
-    for (const GenSM& g : h->gsm) J.closed &= g.inv_tag != 0 ? 1 : 0;
+    J.closed = all_closed(h->gsm);
     J.test = h->k - J.closed >= cg::kTestMinDegree ? 1 : 0;
     J.comb = h->d_comb;
     J.comb_words = (int)h->comb.size();
@@ -2541,6 +2547,7 @@ void layout_wave(cg_batch* b, cg_batch::Wave& w, int lcap) {
         D.mode = J.mode;
         D.bitmap_words = J.mode == cg::kVisitBitmap ? bitmap_words(J.n) : 0;
         D.tagged = J.n <= 15 ? 1 : 0;
+        D.closed = all_closed(J.gsm);
     }
 }
 
@@ -3256,6 +3263,7 @@ int server_admit(cg_server* s, cudaStream_t st) {
         D.mode = J.mode;
         D.bitmap_words = J.mode == cg::kVisitBitmap ? bitmap_words(J.n) : 0;
         D.tagged = J.n <= 15 ? 1 : 0;
+        D.closed = all_closed(J.gsm);
         D.status = cg::kFresh;
         s->h_jobs[free_slot] = D;
         cudaError_t e;
