@@ -88,9 +88,10 @@ extern "C" {
                                   1 = order of discovery; 2 = rank order (both state by state,
                                   never in blocks).  The layers are the same in every order    */
 /* batch options (cg_batch_set_option; CG_OPT_ILP and CG_OPT_GRID apply there too, 1..4)      */
-/* A batch grows its rank-bitmap jobs of n <= 10 by one block or one thread-block cluster each;
-   for those, of the options below and CG_OPT_ILP, only CG_OPT_GRID, CG_OPT_BATCH_VISITED and
-   CG_OPT_GRAPH matter.                                                                       */
+/* A batch grows its rank-bitmap jobs of n <= 10 by one block or one thread-block cluster each (of n = 9
+   and 10 not those that reach little of S_n, when there are many, nor up to four of S_10 under few
+   generators); for those, of the options below and CG_OPT_ILP, only CG_OPT_GRID,
+   CG_OPT_BATCH_VISITED and CG_OPT_GRAPH matter.                                              */
 #define CG_OPT_BATCH_WAVE_L2 6 /* cap on the summed visited-set bytes of one launch:
                                   0 = half of L2 (default), -1 = none                          */
 #define CG_OPT_BATCH_VISITED 7 /* CG_STRATEGY_AUTO (rank bitmap for dense groups of n <= 12),

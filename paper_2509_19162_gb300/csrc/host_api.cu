@@ -692,6 +692,8 @@ int all_closed(const std::vector<GenSM>& gens) {
     return 1;
 }
 
+uint64_t predict_states(int k, uint64_t order, int max_radius, bool inverse_closed);   // (serving, below)
+
 // What comb_rank counts: the ones of a binary start vector, or, negative, its zeros when they are fewer.
 int comb_ones(const cg_growth* h) {
     const int m = __builtin_popcountll(h->start_key);
@@ -2708,6 +2710,23 @@ int collect_wave(cg_batch* b, const cg_batch::Wave& w, const char* hres, int lca
     return rc;
 }
 
+// A job of n = 9 or 10 whose growth is too little for a cluster when there are many like it: a cluster goes
+// through all words of S_n every round, a list through its states.  `reach` states (the group's order,
+// or fewer by the radius) under k generators.  1024 jobs each, list against clusters: n = 10, S_9 under
+// eight adjacent transpositions 29.7 / 25.7 ms, under L, X 14.5 / 17.5, S_8 x S_2 10.8 / 14.8, S_7 x S_2 5.3 / 8.6,
+// six random generators to radius 3 1.0 / 1.6 ms, to radius 8 8.2 / 7.2; n = 9, S_8 3.9 / 5.4, S_6 1.1 / 1.9.
+// A few of them are best off in clusters, which run side by side without a common round (plan_batch takes
+// as many as run at once, twice as many when n = 9 is the largest): 38 of S_8 in S_9 0.77 / 0.39 ms, 152
+// 1.05 / 1.01, 228 1.31 / 1.38; 32 of S_7 x S_2 in S_10 0.56 / 0.38, 76 0.66 / 0.87.
+uint64_t job_reach(const cg_batch::Job& J) {
+    return predict_states(J.k, J.order, J.max_radius, all_closed(J.gsm) != 0);
+}
+bool cluster_thin(const cg_batch::Job& J) {
+    return job_reach(J) * (uint64_t)J.k < factorial(J.n) / (J.n == 10 ? 2 : 1);
+}
+
+int cluster_size(int max_n) { return max_n >= 10 ? 8 : 4; }
+
 // The wave of the jobs marked `cluster` (b->waves[0]), in at most `bytes` of device memory; false when
 // it cannot be had.  Jobs of n <= kClusterSmemN take a block each, the larger ones a cluster: eight
 // blocks for S_10, whose rounds go through 113,400 words and of which then few enough run at once for
@@ -2724,7 +2743,7 @@ bool plan_cluster_wave(cg_batch* b, int dev, int lcap, uint64_t bytes) {
         }
     if (w.ids.empty()) return true;
     w.cluster = true;
-    w.csize = max_n >= 10 ? 8 : 4;
+    w.csize = cluster_size(max_n);
     int fit = w.large ? cluster_clusters(dev, w.csize) : 0, small_fit = small_blocks(dev);
     if (b->grid_override > 0) {
         fit = std::min(fit, std::max(1, b->grid_override / w.csize));
@@ -2785,6 +2804,22 @@ int plan_batch(cg_batch* b, int dev, int cap, cudaStream_t st) {
     // wherever it runs and does not count.  Jobs with no work (no generator, radius 0) are
     // answered on the host.
     const int lcap = cap + 1;
+    int thin = 0, max_n = 0, large = 0, whole = 0, whole_k = 0;
+    for (const auto& J : b->jobs)
+        if (J.k > 0 && J.max_radius != 0 && J.mode == cg::kVisitBitmap && J.n <= cg::kClusterMaxN) {
+            max_n = std::max(max_n, J.n);
+            if (J.n <= cg::kClusterSmemN) continue;
+            ++large;
+            thin += cluster_thin(J) ? 1 : 0;
+            if (J.n == 10 && 4 * job_reach(J) >= factorial(10)) { ++whole; whole_k += J.k + 1; }
+        }
+    // A handful of S_10 under few generators, and nothing else of their size, leave most of the GPU idle in
+    // eight blocks each: as lists on the whole grid, L, R, X once 0.73 ms against 1.17, four times 0.99 / 1.19, eight
+    // 1.34 / 1.19; L, X four times 1.19 / 1.15; four random generators twice 0.54 / 0.72, four times 0.76 / 0.72;
+    // twelve once 0.58 / 0.76, twice 0.85 / 0.76.  (n = 9: clusters even for one, L, R, X 0.56 / 0.47.)
+    const bool few = whole > 0 && whole == large && whole <= 4 && whole_k <= 16;
+    const int csize = cluster_size(max_n);
+    const bool thin_clusters = thin <= (max_n >= 10 ? 1 : 2) * cluster_clusters(dev, csize);
     std::vector<uint64_t> need_of(b->jobs.size(), 0), vis_of(b->jobs.size(), 0);
     uint64_t all_need = 0;
     int with_work = 0;
@@ -2794,7 +2829,8 @@ int plan_batch(cg_batch* b, int dev, int cap, cudaStream_t st) {
         J.cap = std::max<uint64_t>(1, std::min<uint64_t>(J.order, per_job_max));
         const uint64_t set_bytes = J.mode == cg::kVisitBitmap ? bitmap_words(J.n) * 4
                                                                : table_slots_for(J.cap) * 8;
-        J.cluster = J.mode == cg::kVisitBitmap && J.n >= 2 && J.n <= cg::kClusterMaxN;
+        J.cluster = J.mode == cg::kVisitBitmap && J.n >= 2 && J.n <= cg::kClusterMaxN &&
+                    (J.n <= cg::kClusterSmemN || (!few && (thin_clusters || !cluster_thin(J))));
         if (J.cluster) continue;
         need_of[j] = J.cap * 8 + set_bytes + sizeof(GenSM) * J.gsm.size() + sizeof(JobDev) +
                      (uint64_t)lcap * 8 + 1024;

@@ -64,3 +64,50 @@ def test_reading_first_or_not(cg, n, k, radius):
             s.step()
             done |= set(s.finished())
         assert [s.result(i).layers for i in ids] == want
+
+
+def product(n, parts, seed):
+    """Adjacent transpositions of S_a x S_b x .. on consecutive elements, renamed at random."""
+    gens, o = [], 0
+    for m in parts:
+        gens += [w.families.transposition(n, o + i, o + i + 1) for i in range(m - 1)]
+        o += m
+    s = np.random.default_rng(seed).permutation(n).tolist()
+    si = w.inverse(s)
+    return [[si[g[s[i]]] for i in range(n)] for g in gens]
+
+
+@pytest.mark.parametrize("count", [2, 30, 170])
+@pytest.mark.parametrize("n", [9, 10])
+def test_thin_growths_few_and_many(cg, n, count):
+    # groups that fill little of S_n and growths cut off early, in clusters when they are few and as lists
+    # when they are many, beside others that fill it
+    kinds = [lambda j: (n, product(n, (n - 3, 2), j), True, -1), lambda j: (n, product(n, (n - 4, 3), j), True, 6),
+             lambda j: (n, w.inverse_closure(w.random_perms(np.random.default_rng(j), n, 3)), True, 3),
+             lambda j: (n, [list(g) + list(range(n - 2, n)) for g in w.lx(n - 2)], False, -1)]
+    jobs = [kinds[j % 4](j) for j in range(count)]
+    jobs[count // 2:count // 2] = [(n, w.lrx(n), True, -1), (8, product(8, (5, 2), 1), True, -1)]
+    want = {}
+    with cg.Batch(jobs) as b:
+        for _ in range(2):
+            for i, r in enumerate(b.run()):
+                j = jobs[i]
+                key = i if j[3] == 3 else str(sorted(map(tuple, j[1]))) + str(j[3])
+                if key not in want:
+                    want[key] = cg.growth(*j, strategy="hash")
+                assert (r.layers, r.status) == (want[key].layers, want[key].status)
+
+
+@pytest.mark.parametrize("sets", [("lrx",), ("lrx",) * 4, ("lrx",) * 5, ("lx", "coxeter"), ("coxeter", "lx", "lrx"),
+                                  ("pancake", "coxeter")])
+def test_a_handful_of_whole_s10(cg, sets):
+    # few generators in all: lists on the whole grid; more: clusters; beside small jobs or one of n = 9 too
+    def whole(n, f):
+        return (n, w.FAMILIES[f](n), f != "lx", -1)
+    for rest in ([], [whole(7, "coxeter")] * 3, [whole(9, "lrx")]):
+        jobs = [whole(10, f) for f in sets] + rest
+        with cg.Batch(jobs) as b:
+            for _ in range(2):
+                for j, r in zip(jobs, b.run()):
+                    x = cg.growth(*j, strategy="hash")
+                    assert (r.layers, r.status) == (x.layers, x.status)
