@@ -1440,13 +1440,27 @@ bool sweep_preferred(const cg_growth* h) {
     return h->states_bound * 8 + bitmap_words(h->n) * 4 > mem;
 }
 
+// The sweep's block form against state by state.  Beyond L2 it begins by clearing a fourth bit of every
+// element (n = 14: 1.6 ms more) and goes through more flags each round (0.5 ms), which a growth that stops
+// while its layers are sparse does not earn back.  Calls state by state / in blocks: S_14 pancake to radius 3
+// 4.5 / 7.6 ms, 7 8.0 / 10.1; four random generators to the first layer above 2^18 5.1 / 12.7, above 2^24
+// 12.0 / 17.0, above 2^25 (85 M states) 23.5 / 23.8, above 2^26 51.9 / 40.5; S_13 pancake to radius 3 0.57 /
+// 0.67, 5 (0.16 M) 0.88 / 0.75; S_12 to radius 3 0.27 / 0.22.  The lines are on what the limits allow.
+bool sweep_in_blocks(const cg_growth* h) {
+    if (h->sweep_order != cg::kSweepOrderAuto || !block_fits(h)) return false;
+    if (h->n < 13) return true;
+    uint64_t reach = predict_states(h->k, h->order, h->max_radius, h->inverse_closed != 0);
+    if (h->stop_above > 0 && h->stop_above < reach / (uint64_t)(h->k + 1)) reach = h->stop_above * (uint64_t)(h->k + 1);
+    return reach >= (h->n == 13 ? 1ull << 17 : 1ull << 27);
+}
+
 int run_sweep(cg_growth* h, cudaStream_t st, int* final_status) {
     const uint64_t mem = h->mem_cap ? h->mem_cap : kDefaultMemCap;
     if (!h->start_is_perm || h->n > 14 || h->n < 1) return CG_EINVAL;
     const uint64_t bytes = sweep_bytes(h->n);
     if (bytes > mem) return CG_EINVAL;
     int rc = CG_OK;
-    h->last_is_block = h->sweep_order == cg::kSweepOrderAuto && block_fits(h);
+    h->last_is_block = sweep_in_blocks(h);
     if (h->last_is_block) {             // (a handle holds one form's bitmaps at a time: mem_cap bounds both)
         h->release_sweep(st);
         if ((rc = run_block(h, st, final_status)) != CG_ENOMEM) return rc;
