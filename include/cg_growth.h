@@ -67,9 +67,9 @@ extern "C" {
                                   in 33.4 GB; any generating set; start with distinct values;
                                   needs n <= 14 and the bitmaps within mem_cap (else CG_EINVAL
                                   at run).  For 10 <= n, when a fourth bit fits (43.8 GB for
-                                   S_14) and, for n >= 13, the radius and layer limits allow
-                                   more than sparse layers, the states are expanded in blocks
-                                   that the generators move together                            */
+                                  S_14) and, for n >= 13, the radius and layer limits allow
+                                  more than sparse layers, the states are expanded in blocks
+                                  that the generators move together                            */
 
 /* ---- options ------------------------------------------------------------------------ */
 #define CG_OPT_STRATEGY     1  /* one of CG_STRATEGY_*                                        */

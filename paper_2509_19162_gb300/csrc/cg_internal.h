@@ -143,7 +143,8 @@ constexpr uint64_t kKeyBits60 = (1ull << 60) - 1;
 constexpr int kVisitHash = 0;
 constexpr int kVisitBitmap = 2;
 constexpr int kVisitComb = 3;           // bitmap over the C(n, m) binary vectors (comb_rank)
-constexpr int kVariantComb = 21;        // its kernel variant
+constexpr int kVariantBitmap = 17;      // kernel variants of the rank bitmap (one form, whatever CG_OPT_ILP says)
+constexpr int kVariantComb = 21;        // and of the arrangement bitmap
 constexpr int kCombMaxWords = 6144;     // ranking table: at most 96 rows of 64
 
 // Generators beyond the parent edge from which a single rank-bitmap job's first round reads a visited

@@ -1287,7 +1287,7 @@ int hash_grow_block() { return kGrowBlock; }
 namespace {
 using GrowFn = void (*)(JobDev*, int, unsigned long long*, Ctl*, int, uint64_t, const AdmitDev*, const JobConst);
 // Kernel variants: `ilp` generators per thread (1..4); +8 selects whole-sector table probing,
-// +16 the rank bitmap; multi = launches of several jobs.
+// kVariantBitmap the rank bitmap; multi = launches of several jobs.
 template <bool M>
 GrowFn grow_fn_t(int variant) {
     switch (variant) {
@@ -1316,7 +1316,7 @@ GrowFn grow_fn_bitmap_n(int n, std::integer_sequence<int, Ns...>) {
 }
 
 GrowFn grow_fn(int variant, bool multi, int n) {
-    if (variant >= 17 && variant != kVariantComb && !multi && n >= 2 && n <= 14)
+    if (variant == kVariantBitmap && !multi && n >= 2 && n <= 14)
         return grow_fn_bitmap_n<1>(n, std::make_integer_sequence<int, 13>{});
     return grow_fn(variant, multi);
 }

@@ -472,7 +472,7 @@ int status_to_rc(int status) {
 int device_grid_cache[64][32][2] = {};
 
 // Blocks of the persistent kernel that fit co-resident on device `dev` (variant: ILP 1..4, +8
-// for whole-sector table probing, +16 for the rank bitmap; multi: several jobs per launch).
+// for whole-sector table probing, kVariantBitmap, kVariantComb; multi: several jobs per launch).
 int grow_grid(int dev, int ilp, bool multi = false) {
     if (dev < 0 || dev >= 64 || ilp < 1 || ilp > cg::kVariantComb) return 0;
     int& c = device_grid_cache[dev][ilp][multi ? 1 : 0];
@@ -511,10 +511,9 @@ int spread_blocks(int dev, int n, int k) {
     return c > 0 ? size : 0;
 }
 
-// Generators probed together per thread.  Hash tables (random DRAM probes): all of them when
-// k <= 4, else 4.  Rank bitmap (L2-resident, one atomic per probe): 1 -- measured fastest, and
-// the only bitmap variant that fits 64 registers without spilling.
-int default_ilp(int k, bool bitmap = false) { return bitmap ? 1 : std::max(1, std::min(4, k)); }
+// Generators probed together per thread in a hash table (random DRAM probes): all of them when
+// k <= 4, else 4.
+int default_ilp(int k) { return std::max(1, std::min(4, k)); }
 
 }  // namespace
 
@@ -1033,7 +1032,8 @@ int run_hash(cg_growth* h, cudaStream_t st, int* final_status) {
     const bool bitmap = h->mode == cg::kVisitBitmap, comb = h->mode == cg::kVisitComb;
     h->last_is_block = false;
     const int ilp = comb ? cg::kVariantComb
-                         : (h->ilp_override > 0 ? h->ilp_override : default_ilp(h->k, bitmap)) + (bitmap ? 16 : 0);
+                    : bitmap ? cg::kVariantBitmap
+                    : h->ilp_override > 0 ? h->ilp_override : default_ilp(h->k);
     const uint64_t avail = mem > (1 << 20) ? mem - (1 << 20) : mem;
     const uint64_t bm_bytes = bitmap ? bitmap_words(h->n) * 4 : 0;
     const uint64_t max_cap = std::min<uint64_t>(
@@ -2793,8 +2793,7 @@ int plan_batch(cg_batch* b, int dev, int cap, cudaStream_t st) {
         any_bitmap |= J.mode == cg::kVisitBitmap;
     }
     // The rank-bitmap kernel variant also runs hash-table jobs of the same launch.
-    const int base_ilp = b->ilp_override > 0 ? b->ilp_override : default_ilp(maxk, any_bitmap);
-    b->ilp = base_ilp + (any_bitmap ? 16 : 0);
+    b->ilp = any_bitmap ? cg::kVariantBitmap : b->ilp_override > 0 ? b->ilp_override : default_ilp(maxk);
     b->stats.strategy_used = any_bitmap ? CG_STRATEGY_BITMAP : CG_STRATEGY_HASH;
     b->stats.probe_variant = b->ilp;
     const int grid_max = grow_grid(dev, b->ilp, true);
@@ -3451,7 +3450,7 @@ int cg_server_step(cg_server_t s, void* cuda_stream, int* active_out, int* finis
                 maxk = std::max(maxk, sl.job.k);
                 any_bitmap |= sl.job.mode == cg::kVisitBitmap;
             }
-        const int variant = default_ilp(maxk, any_bitmap) + (any_bitmap ? 16 : 0);
+        const int variant = any_bitmap ? cg::kVariantBitmap : default_ilp(maxk);
         const int grid = grow_grid(s->device, variant, true);
         if (grid <= 0) return CG_ECUDA;
         cudaError_t e;
