@@ -1001,7 +1001,7 @@ cudaError_t launch_cluster_prepare(const ClusterArgs& A, unsigned want, cudaStre
     return cudaGetLastError();
 }
 
-int cluster_max_clusters(int device, int size) {
+int cluster_max_clusters(int size) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)size);
     cfg.blockDim = dim3(kClThreads);
@@ -1010,12 +1010,6 @@ int cluster_max_clusters(int device, int size) {
     attr[0].val.clusterDim = {(unsigned)size, 1, 1};
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    (void)device;
-    if (size > 8 &&
-        cudaFuncSetAttribute(cluster_grow_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return 0;
-    }
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, cluster_grow_kernel, &cfg) != cudaSuccess) {
         (void)cudaGetLastError();

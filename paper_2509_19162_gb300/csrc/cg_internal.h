@@ -181,7 +181,6 @@ struct alignas(128) JobDev {
     int max_radius;            // < 0: unlimited
     int mode;                  // visited set: 0 hash table, 2 rank bitmap (kVisitBitmap)
     int use_start;             // 1: grow from start_key (a central state), 0: from the identity
-    uint64_t bitmap_words;     // bitmap mode: 32-bit words in `table` (ceil(n!/32))
     uint64_t start_key;        // packed start vector when use_start
     int tagged;                // 1: keys leave bits 60-63 free for the parent-edge tag
     int closed;                // 1: every generator's inverse is in the set (every state but

@@ -87,7 +87,7 @@ cudaError_t launch_block_export(const BlockDev& host, int which, uint64_t* out, 
 uint64_t cluster_words(int n);
 uint64_t cluster_table_entries(int n);
 cudaError_t launch_cluster_prepare(const ClusterArgs& A, unsigned want, cudaStream_t st);
-int cluster_max_clusters(int device, int size);
+int cluster_max_clusters(int size);
 cudaError_t launch_cluster_grow(const ClusterArgs& A, int clusters, int size, cudaStream_t st);
 int cluster_small_blocks(int device);
 // one growth of n = 8 or 9 by a cluster of `size` blocks, and whether the device runs such a cluster

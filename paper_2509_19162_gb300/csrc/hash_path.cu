@@ -387,7 +387,6 @@ struct JobConst {
     unsigned long long keys_cap;
     uint64_t* table;
     uint64_t table_mask;
-    unsigned long long bitmap_words;
     int k;
     int n;
     int tagged;
@@ -416,7 +415,6 @@ __device__ __forceinline__ JobConst job_const(const JobDev* J, int stage) {
     c.keys_cap = J->keys_cap;
     c.table = J->table;
     c.table_mask = J->table_mask;
-    c.bitmap_words = J->bitmap_words;
     c.k = J->k;
     c.n = J->n;
     c.tagged = J->tagged;
@@ -1375,7 +1373,6 @@ cudaError_t launch_hash_grow(JobDev* d_jobs, int njobs, unsigned long long* d_ub
         jc.keys_cap = host_job->keys_cap;
         jc.table = host_job->table;
         jc.table_mask = host_job->table_mask;
-        jc.bitmap_words = host_job->bitmap_words;
         jc.k = host_job->k;
         jc.n = host_job->n;
         jc.tagged = host_job->tagged;

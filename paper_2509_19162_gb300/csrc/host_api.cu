@@ -481,11 +481,11 @@ int grow_grid(int dev, int ilp, bool multi = false) {
 }
 
 // Clusters of `size` blocks of the cluster kernel that device `dev` runs at once (0: none).
-int cluster_cache[64][17] = {};
+int cluster_cache[64][9] = {};
 int cluster_clusters(int dev, int size) {
-    if (dev < 0 || dev >= 64 || size < 1 || size > 16) return 0;
+    if (dev < 0 || dev >= 64 || size < 1 || size > 8) return 0;
     int& c = cluster_cache[dev][size];
-    if (!c) c = 1 + cg::cluster_max_clusters(dev, size);
+    if (!c) c = 1 + cg::cluster_max_clusters(size);
     return c - 1;
 }
 
@@ -761,7 +761,6 @@ void fill_static(cg_growth* h, JobDev& J) {
     J.layers_cap = cg::kMaxLayers;
     J.max_radius = h->max_radius;
     J.mode = h->mode;
-    J.bitmap_words = h->mode == cg::kVisitBitmap ? bitmap_words(h->n) : 0;
     J.use_start = h->use_start ? 1 : 0;
     J.start_key = h->start_key;
     J.tagged = h->n * h->width <= 60 ? 1 : 0;
@@ -2561,7 +2560,6 @@ void layout_wave(cg_batch* b, cg_batch::Wave& w, int lcap) {
         D.layers_cap = lcap;
         D.max_radius = J.max_radius;
         D.mode = J.mode;
-        D.bitmap_words = J.mode == cg::kVisitBitmap ? bitmap_words(J.n) : 0;
         D.tagged = J.n <= 15 ? 1 : 0;
         D.closed = all_closed(J.gsm);
     }
@@ -3310,7 +3308,6 @@ int server_admit(cg_server* s, cudaStream_t st) {
         D.layers_cap = kSrvLayers;
         D.max_radius = J.max_radius;
         D.mode = J.mode;
-        D.bitmap_words = J.mode == cg::kVisitBitmap ? bitmap_words(J.n) : 0;
         D.tagged = J.n <= 15 ? 1 : 0;
         D.closed = all_closed(J.gsm);
         D.status = cg::kFresh;
