@@ -102,6 +102,20 @@ def with_dram_rate(roof):
     return roof
 
 
+def batch_kernels(stats):
+    """What grew the jobs of a batch run with these stats: (name of the one kernel that did, or None,
+    and a description).  Small rank-bitmap groups take a block or a cluster each (one or two launches,
+    strategy 4 when there is nothing else); the others a launch of the list kernel, admitted by two."""
+    variant = stats["probe_variant"]
+    clusters = ("cluster_grow_small_kernel<512> (n <= 8) and cluster_grow_kernel (n = 9, 10): a block or a "
+                "thread-block cluster per job, drawn from a queue")
+    if stats["strategy_used"] == 4:
+        return None, clusters
+    lists = f"hash_grow_kernel<{variant & 7}, {variant >> 3}, 1, 0>"
+    text = f"{lists} (multi-job, one persistent launch per batch run admitting the jobs by the L2 window)"
+    return (lists, text) if stats["launches"] <= 2 else (None, f"{clusters}; {text}")
+
+
 def algorithmic_bytes(layers, k, complete):
     """Bytes the layer steps must move (per-step model B_r): read the frontier (8 F_r), write and
     read back each candidate key (16 k F_r), read layers r and r-1 for the set difference
@@ -514,10 +528,11 @@ def measure_batch(cg, spec, stream, flush, steps, warmup, autotune=True, tune_ta
         launches += st["launches"]
         if [r.layers for r in out] != layers:
             raise RuntimeError("batched layer counts changed between steps")
-    variant = batch.stats()["probe_variant"]
+    kernel, kernel_text = batch_kernels(batch.stats())
     batch.close()
     return {"layers": layers, "statuses": [r.status for r in res], "total_ms": total_ms,
-            "kernel_ms": kernel_ms, "launches": launches, "variant": variant, "tuned": tuned}
+            "kernel_ms": kernel_ms, "launches": launches, "kernel": kernel, "kernel_text": kernel_text,
+            "tuned": tuned}
 
 
 def one_at_a_time(cg, jobs, stream, mem_cap=0, strategies=None, per_job=None):
@@ -586,7 +601,6 @@ def run_batch(args):
     peak, peak_kind = load_peaks()
     kms = m["kernel_ms"] / args.steps
     achieved = bytes_step / (kms / 1000.0) / 1e9
-    variant = m["variant"]
     if rank != 0:
         return 0
     out = {
@@ -607,11 +621,9 @@ def run_batch(args):
         "roofline": with_dram_rate({
             "bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak,
-            "traffic": measured_traffic(f"hash_grow_kernel<{variant & 7}, {variant >> 3}, 1, 0>",
-                                        f"batched-{len(jobs_all)}-random-groups-seed{wl.BATCH_SEED}",
-                                        tuned["settings"] if tuned else None),
-            "kernel": "cluster_grow_small_kernel<512> (n <= 8) and cluster_grow_kernel (n = 9, 10): a "
-                      "block or a thread-block cluster per job, drawn from a queue",
+            "traffic": measured_traffic(m["kernel"], f"batched-{len(jobs_all)}-random-groups-seed{wl.BATCH_SEED}",
+                                        tuned["settings"] if tuned else None) if m["kernel"] else None,
+            "kernel": m["kernel_text"],
             "kernel_ms": kms, "algorithmic_bytes": bytes_step, "peak_source": peak_kind}),
         "e2e": {"value": nb_step / e2e_s, "unit": UNIT, "h2d_bytes_per_step": est["h2d_bytes"],
                 "d2h_bytes_per_step": est["d2h_bytes"], "api": "paper_2509_19162_gb300.Batch(...).run()"},

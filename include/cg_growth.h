@@ -293,7 +293,9 @@ int cg_batch_set_wave_l2(cg_batch_t b, uint64_t bytes);
  */
 int cg_batch_set_option(cg_batch_t b, int option, int64_t value);
 
-/* Measurements of the last cg_batch_run (as cg_growth_get_stats).  Errors: CG_EINVAL. */
+/* Measurements of the last cg_batch_run (as cg_growth_get_stats).  strategy_used is the visited set of
+ * the jobs grown as lists of states, CG_STRATEGY_BITMAP or _HASH, and CG_STRATEGY_SWEEP when every job
+ * was grown by a block or a cluster.  Errors: CG_EINVAL. */
 int cg_batch_get_stats(cg_batch_t b, cg_growth_stats* out);
 
 /* Release the batch and its device buffers.  NULL is accepted. */

@@ -2697,6 +2697,11 @@ cudaError_t enqueue_wave(cg_batch* b, cg_batch::Wave& w, char* base, char* hout,
     return e;
 }
 
+// Kernels that enqueue_wave launches: clusters and blocks, or (admit_first | init_jobs + init_units) + grow.
+int wave_launches(const cg_batch::Wave& w) {
+    return w.cluster ? (w.large > 0) + (w.small_blocks > 0) : w.admit ? 2 : 3;
+}
+
 // Read one wave's results from host memory into the caller's arrays.
 int collect_wave(cg_batch* b, const cg_batch::Wave& w, const char* hres, int lcap, int cap,
                  uint64_t* layer_out, int* nl_out, int* status_out) {
@@ -2792,8 +2797,6 @@ int plan_batch(cg_batch* b, int dev, int cap, cudaStream_t st) {
     }
     // The rank-bitmap kernel variant also runs hash-table jobs of the same launch.
     b->ilp = any_bitmap ? cg::kVariantBitmap : b->ilp_override > 0 ? b->ilp_override : default_ilp(maxk);
-    b->stats.strategy_used = any_bitmap ? CG_STRATEGY_BITMAP : CG_STRATEGY_HASH;
-    b->stats.probe_variant = b->ilp;
     const int grid_max = grow_grid(dev, b->ilp, true);
     if (grid_max <= 0) return CG_ECUDA;
     b->grid = b->grid_override > 0 ? std::min(grid_max, b->grid_override) : grid_max;
@@ -3000,10 +3003,11 @@ int cg_batch_run(cg_batch_t b, void* cuda_stream, uint64_t* layer_sizes_out, int
     int rc = CG_OK;
     if (!b->planned || b->plan_cap != cap || b->device != dev) {
         if ((rc = plan_batch(b, dev, cap, st)) != CG_OK) return rc;
-    } else {
-        b->stats.strategy_used = b->ilp >= 16 ? CG_STRATEGY_BITMAP : CG_STRATEGY_HASH;
-        b->stats.probe_variant = b->ilp;
     }
+    // jobs that a launch of the list kernel grew, or, when there are none, blocks and clusters
+    const bool lists = b->waves.empty() || !b->waves.back().cluster;
+    b->stats.strategy_used = !lists ? CG_STRATEGY_SWEEP : b->ilp >= 16 ? CG_STRATEGY_BITMAP : CG_STRATEGY_HASH;
+    b->stats.probe_variant = lists ? b->ilp : 1;
     const int lcap = cap + 1;
     if (b->resident) {
         if (b->use_graph > 0 && !b->gexec) {
@@ -3044,8 +3048,7 @@ int cg_batch_run(cg_batch_t b, void* cuda_stream, uint64_t* layer_sizes_out, int
         }
         b->stats.kernel_ms += elapsed_ms(b->ev0, b->ev1);
         for (auto& w : b->waves) {
-            b->stats.launches += w.cluster ? (w.large > 0) + (w.small_blocks > 0)
-                                           : w.admit ? 2 : 3;     // (admit_first | init_jobs + init_units) + grow
+            b->stats.launches += wave_launches(w);
             b->stats.d2h_bytes += wave_result_bytes(w, lcap);
             int r = collect_wave(b, w, b->h_pinned + w.h_off, lcap, cap, layer_sizes_out,
                                  num_layers_out, status_out);
@@ -3067,7 +3070,7 @@ int cg_batch_run(cg_batch_t b, void* cuda_stream, uint64_t* layer_sizes_out, int
         dev_free(base, st);
         cudaStreamSynchronize(st);
         if (e != cudaSuccess) return cuda_rc(e);
-        b->stats.launches += 3;
+        b->stats.launches += wave_launches(w) + (w.cluster && w.want ? 1 : 0);     // (unranking tables)
         b->stats.d2h_bytes += wave_result_bytes(w, lcap);
         int r = collect_wave(b, w, b->h_pinned + w.h_off, lcap, cap, layer_sizes_out, num_layers_out,
                              status_out);
