@@ -23,6 +23,6 @@ def __getattr__(name):
         from . import api as _g
         return getattr(_g, name)
     if name == "serve":
-        from . import serve as _s
-        return _s
+        import importlib
+        return importlib.import_module(".serve", __name__)     # (`from . import` would ask here again)
     raise AttributeError(name)
