@@ -2733,8 +2733,10 @@ int collect_wave(cg_batch* b, const cg_batch::Wave& w, const char* hres, int lca
 // eight adjacent transpositions 29.7 / 25.7 ms, under L, X 14.5 / 17.5, S_8 x S_2 10.8 / 14.8, S_7 x S_2 5.3 / 8.6,
 // six random generators to radius 3 1.0 / 1.6 ms, to radius 8 8.2 / 7.2; n = 9, S_8 3.9 / 5.4, S_6 1.1 / 1.9.
 // A few of them are best off in clusters, which run side by side without a common round (plan_batch takes
-// as many as run at once, twice as many when n = 9 is the largest): 38 of S_8 in S_9 0.77 / 0.39 ms, 152
-// 1.05 / 1.01, 228 1.31 / 1.38; 32 of S_7 x S_2 in S_10 0.56 / 0.38, 76 0.66 / 0.87.
+// as many as run at once, twice as many when n = 9 is the largest, and twice that beside growths that take
+// clusters anyway): 38 of S_8 in S_9 0.77 / 0.39 ms, 152 1.05 / 1.01, 228 1.31 / 1.38; 32 of S_7 x S_2 in S_10 0.56 /
+// 0.38, 76 0.66 / 0.87; beside sixteen whole S_10, 48 of S_7 x S_2 1.33 / 1.25, 96 1.40 / 1.79, 192 of S_6 in S_9 1.22 /
+// 1.06, 384 1.42 / 1.43.
 uint64_t job_reach(const cg_batch::Job& J) {
     return predict_states(J.k, J.order, J.max_radius, all_closed(J.gsm) != 0);
 }
@@ -2818,13 +2820,13 @@ int plan_batch(cg_batch* b, int dev, int cap, cudaStream_t st) {
     // wherever it runs and does not count.  Jobs with no work (no generator, radius 0) are
     // answered on the host.
     const int lcap = cap + 1;
-    int thin = 0, max_n = 0, large = 0, whole = 0, whole_k = 0;
+    int thin9 = 0, thin10 = 0, max_n = 0, large = 0, whole = 0, whole_k = 0;
     for (const auto& J : b->jobs)
         if (J.k > 0 && J.max_radius != 0 && J.mode == cg::kVisitBitmap && J.n <= cg::kClusterMaxN) {
             max_n = std::max(max_n, J.n);
             if (J.n <= cg::kClusterSmemN) continue;
             ++large;
-            thin += cluster_thin(J) ? 1 : 0;
+            if (cluster_thin(J)) ++(J.n == 10 ? thin10 : thin9);
             if (J.n == 10 && 4 * job_reach(J) >= factorial(10)) { ++whole; whole_k += J.k + 1; }
         }
     // A handful of S_10 under few generators, and nothing else of their size, leave most of the GPU idle in
@@ -2832,8 +2834,10 @@ int plan_batch(cg_batch* b, int dev, int cap, cudaStream_t st) {
     // 1.34 / 1.19; L, X four times 1.19 / 1.15; four random generators twice 0.54 / 0.72, four times 0.76 / 0.72;
     // twelve once 0.58 / 0.76, twice 0.85 / 0.76.  (n = 9: clusters even for one, L, R, X 0.56 / 0.47.)
     const bool few = whole > 0 && whole == large && whole <= 4 && whole_k <= 16;
-    const int csize = cluster_size(max_n);
-    const bool thin_clusters = thin <= (max_n >= 10 ? 1 : 2) * cluster_clusters(dev, csize);
+    // how many thin ones clusters take, in quarters of a job of the largest n, and twice as many beside others,
+    // where a launch for the lists is extra
+    const int csize = cluster_size(max_n), room = 4 * cluster_clusters(dev, csize) * (max_n >= 10 ? 1 : 2);
+    const bool thin_clusters = 4 * thin10 + (max_n >= 10 ? 1 : 4) * thin9 <= room * (large > thin9 + thin10 ? 2 : 1);
     std::vector<uint64_t> need_of(b->jobs.size(), 0), vis_of(b->jobs.size(), 0);
     uint64_t all_need = 0;
     int with_work = 0;
