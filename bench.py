@@ -130,6 +130,23 @@ def algorithmic_bytes(layers, k, complete):
     return total
 
 
+def block_bytes(n, layers, in_cluster):
+    """Bytes a growth of S_n in blocks of 2^M states moves in its own layout: per round the words of the
+    layer are read, those of the layer before cleared, the new states' visited words read and written
+    and their layer's words written, a word a block at most (in a cluster or one block: every word of
+    the layer read and of the layer before cleared), and on the grid the two layers' flags, a byte per
+    32 blocks.  (algorithmic_bytes counts candidates written and read back, which no block does: as a
+    share of the copy rate it comes out above one for these kernels.)"""
+    pairs = 6 if n >= 12 else n // 2
+    blocks, word = math.factorial(n) >> pairs, 8 if pairs == 6 else 4
+    words = [min(f, blocks) for f in layers] + [0]
+    total = 0
+    for r in range(len(layers)):
+        scanned = 2 * blocks if in_cluster else words[r] + (words[r - 1] if r else 0)
+        total += word * (scanned + 3 * words[r + 1]) + (0 if in_cluster else 2 * ((blocks + 31) // 32))
+    return total
+
+
 def neighbours(layers, k, complete):
     """The metric's unit count: the graph's edges out of every expanded layer, k * sum F_r."""
     expanded = len(layers) if complete else len(layers) - 1
@@ -367,7 +384,6 @@ def run_ours(args):
     complete = res.status == 0
     layers = res.layers
     nb_step = neighbours(layers, job.k, complete)
-    bytes_step = algorithmic_bytes(layers, job.k, complete)
 
     def barrier():
         if world > 1:
@@ -393,6 +409,8 @@ def run_ours(args):
     in_blocks = strat_name == "sweep" and variant == 1 and job.k > 1
     block_kernel = (f"block_grow_kernel<{job.n}>" if job.n >= 10 else
                     f"cluster_grow_{'spread_kernel' if job.n >= 8 else 'small_kernel<1024>'}")
+    bytes_step = (block_bytes(job.n, layers, job.n < 10) if in_blocks
+                  else algorithmic_bytes(layers, job.k, complete))
     # the sweep's block order changes its memory traffic: its ncu record names the order
     launch_settings = {"sweep_order": args.sweep_order} if strat_name == "sweep" else None
     kernel_name = {"sort": "radix sort / merge-path kernels",
@@ -457,9 +475,9 @@ def run_ours(args):
                    "layers": len(layers), "neighbours_per_step": nb_step,
                    "generated_per_step": generated_candidates(job.n, job.gens, layers, complete,
                                                               strat_name in ("bitmap", "hash")),
-                   "counting": "value and roofline count k * sum F_r neighbours (every edge out of "
-                               "every expanded layer) and the algorithmic bytes of that growth; "
-                               "generated_per_step is what the kernel expands after skipping each "
+                   "counting": "value counts k * sum F_r neighbours (every edge out of every expanded "
+                               "layer), roofline the algorithmic bytes of that growth, or, in blocks of "
+                               "states, the bytes of the blocks' words; generated_per_step is what the kernel expands after skipping each "
                                "state's parent edge",
                    "strategy": strat_name + {
                        "sort": " (sorted layers: expand, radix sort, merge-path difference)",
@@ -579,7 +597,9 @@ def run_batch(args):
     clocks = sampler.stop() if sampler else None
     layers, tuned, launches = m["layers"], m["tuned"], m["launches"]
     nb_step = sum(len(j.gens) * sum(l) for j, l in zip(jobs, layers))
-    bytes_step = sum(algorithmic_bytes(l, len(j.gens), True) for j, l in zip(jobs, layers))
+    # (jobs of n <= 10 on a rank bitmap: all but a few go through blocks' words)
+    bytes_step = sum(block_bytes(j.n, l, True) if m["kernel"] is None else algorithmic_bytes(l, len(j.gens), True)
+                     for j, l in zip(jobs, layers))
     total_ms = m["total_ms"]
     if world > 1:
         total_ms, nb_all = combine_ranks(total_ms, nb_step)
@@ -758,7 +778,9 @@ def quick_growth(cg, job, stream, flush, steps=3, warmup=2):
     return {"workload": job.name, "value": nb / (t / 1000.0), "unit": UNIT, "ms_per_step": t,
             "kernel_ms": kt, "layers": len(r.layers), "states": sum(r.layers), "status": r.status,
             "strategy": {1: "hash", 2: "sort", 3: "bitmap", 4: "sweep"}.get(st["strategy_used"], "?"),
-            "roofline_frac": algorithmic_bytes(r.layers, job.k, complete) / (kt / 1000.0) / 1e9 / peak,
+            "roofline_frac": (block_bytes(job.n, r.layers, job.n < 10)
+                              if st["strategy_used"] == 4 and st["probe_variant"] == 1 and job.k > 1
+                              else algorithmic_bytes(r.layers, job.k, complete)) / (kt / 1000.0) / 1e9 / peak,
             "steps": steps}
 
 

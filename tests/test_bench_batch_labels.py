@@ -41,3 +41,14 @@ def test_stats_say_which_kernels_ran():
             name, text = bench.batch_kernels(st)
             assert ("cluster" in text) == (visited == "auto" and len(jobs) + (jobs[0] is small) > 1)
             assert (name is None) == ("cluster" in text)
+
+
+def test_block_bytes_by_hand():
+    # S_4 in 6 blocks of 4 states, a 4-byte word each: layers 1, 3, 5, 6, 5, 3, 1 under adjacent transpositions
+    layers = [1, 3, 5, 6, 5, 3, 1]
+    grid = sum(4 * (a + b + 3 * c) + 2 for a, b, c in zip(layers, [0] + layers, layers[1:] + [0]))
+    assert bench.block_bytes(4, layers, False) == grid
+    assert bench.block_bytes(4, layers, True) == sum(4 * (2 * 6 + 3 * c) for c in layers[1:] + [0])
+    # a layer takes a word a block at most: whole S_12 pancake, 12!/64 words of 8 bytes
+    big = bench.block_bytes(12, [1, 10 ** 9], False)
+    assert big == 8 * (1 + 3 * 7484400) + 8 * (7484400 + 1) + 4 * ((7484400 + 31) // 32)
