@@ -502,6 +502,8 @@ int small_blocks(int dev) {
 // transpositions 165 against 96 / 98 / 110 us, all transpositions (k = 28) 141 against 75 / 79 / 95; S_9
 // L, X 262 against 162 / 190 / 262, adjacent transpositions 258 against 198 / 247 / 364, all
 // transpositions (k = 36) 236 against 309 (sixteen SMs' issue rate); S_10 L, X 395 against 490 / - / -.
+// Up to the line, whole calls with the list of the time before and so: S_9 under nine cyclic adjacent
+// transpositions 315 / 255 us, ten and twelve random generators 250 / 232 and 278 / 244.
 int spread_cache[64][2] = {};
 int spread_blocks(int dev, int n, int k) {
     if (dev < 0 || dev >= 64 || n < 8 || n > 9 || (n == 9 && k > 12)) return 0;
@@ -1422,7 +1424,9 @@ int run_wide(cg_growth* h, cudaStream_t st, int* final_status) {
 // 28 / 5.9, all transpositions 169 / 16.5, S_13 pancake 688 / 52; in smaller groups a round's fixed
 // cost (12 us) counts and the line is the generators' number: S_11 LRX 1.00 / 1.28 ms (k = 3),
 // adjacent transpositions 2.59 / 1.51 (k = 10), S_10 adjacent transpositions 0.53 / 0.59 (k = 9),
-// pancake 0.30 / 0.19 (k = 9), all transpositions 1.01 / 0.31 (k = 45).  (2) The states, stored as
+// pancake 0.30 / 0.19 (k = 9: few rounds; the number of generators does not see them), ten cyclic
+// adjacent transpositions 0.66 / 0.51, L's powers and X (k = 10) 0.76 / 0.72, all transpositions 1.01 / 0.31
+// (k = 45).  (2) The states, stored as
 // keys beside a rank bitmap, would not fit the memory cap while the sweep's bitmaps do.
 // A layer-size limit of at least a state per block does not change (1): S_14 pancake to the first layer
 // above 2^31 142 / 58 ms; with a bitmap in L2 (n <= 12) it takes more, S_12 under six random generators

@@ -11,7 +11,7 @@
 //                 generator that leads back to its parent above its key bits, where they leave room,
 //                 and that generator is passed over: its image lies in L_{r-1}.  The tag rides along
 //                 through the passes.  S_11 under L, R, X: a third fewer candidates,
-//                 a whole growth 13.0 / 10.95 ms
+//                 a whole growth 13.27 / 12.26 ms
 //   radix passes  LSD over the w n significant key bits, one kernel per pass: each 4096-key
 //                 tile ranks its keys by digit (a vote per digit bit, per-warp digit counts in shared
 //                 memory), finds each digit's offset among the earlier tiles by a decoupled
