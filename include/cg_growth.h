@@ -48,7 +48,7 @@ extern "C" {
 
 /* ---- strategies (cg_growth_set_option(h, CG_OPT_STRATEGY, ...)) --------------------- */
 #define CG_STRATEGY_AUTO    0  /* library chooses: SWEEP (in blocks of states) for dense groups
-                                  of n <= 9, for whole growths of n >= 12 (11 from 6 and 10 from
+                                  of n <= 9 (n = 9: up to 12 generators), for whole growths of n >= 12 (11 from 6 and 10 from
                                   10 generators) and for limited growths once their layers are
                                   dense, and when the states of BITMAP do not fit but the sweep's
                                   bitmaps do; else BITMAP when eligible; else a bit per
