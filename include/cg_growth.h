@@ -48,11 +48,12 @@ extern "C" {
 
 /* ---- strategies (cg_growth_set_option(h, CG_OPT_STRATEGY, ...)) --------------------- */
 #define CG_STRATEGY_AUTO    0  /* library chooses: SWEEP (in blocks of states) for dense groups
-                                  of n <= 9 (n = 9: up to 12 generators), for whole growths of n >= 12 (11 from 6 and 10 from
-                                  10 generators) and for limited growths once their layers are
-                                  dense, and when the states of BITMAP do not fit but the sweep's
-                                  bitmaps do; else BITMAP when eligible; else a bit per
-                                  arrangement of the start vector, or HASH                     */
+                                  of n <= 9 (n = 9: up to 12 generators), for whole growths of
+                                  n >= 12 (11 from 6 and 10 from 10 generators) and for limited
+                                  growths once their layers are dense, and when the states of
+                                  BITMAP do not fit but the sweep's bitmaps do; else BITMAP
+                                  when eligible; else a bit per arrangement of the start vector,
+                                  or HASH                                                      */
 #define CG_STRATEGY_HASH    1  /* visited open-addressing hash set; any generating set        */
 #define CG_STRATEGY_SORT    2  /* sorted layers, radix sort + unique + merge-path difference
                                   against layers r and r-1; inverse-closed sets only          */

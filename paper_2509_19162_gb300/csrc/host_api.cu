@@ -3339,8 +3339,7 @@ int server_admit(cg_server* s, cudaStream_t st) {
 // set and per-job share the batched launch would give it (so the same layers), no hand-off to
 // the sorted step.  Its result joins the finished list.
 int server_run_solo(cg_server* s, cudaStream_t st) {
-    cg_server::Job J = std::move(s->queue.front());
-    s->queue.pop_front();
+    const cg_server::Job& J = s->queue.front();     // (stays at the head when its growth fails)
     cg_growth_t g = nullptr;
     // a served job keeps at most kSrvLayers layers, as in the batched launch
     const int rad = (J.max_radius < 0 || J.max_radius > kSrvLayers - 1) ? kSrvLayers - 1 : J.max_radius;
@@ -3359,6 +3358,7 @@ int server_run_solo(cg_server* s, cudaStream_t st) {
     R.status = rc;
     s->results[J.id] = std::move(R);
     s->finished.push_back(J.id);
+    s->queue.pop_front();
     return CG_OK;
 }
 

@@ -167,3 +167,23 @@ def test_a_server_step_after_a_failed_allocation(cg):
                     s.step()
                 assert s.result(job).layers == want
             assert dev.held == 0
+
+
+def test_a_solo_job_after_a_failed_allocation(cg):
+    # a job that the server grows alone stays queued when its growth fails
+    from paper_2509_19162_gb300._cg import CgError
+    from paper_2509_19162_gb300.serve import Server
+    n, radius, share = 12, 20, 1 << 30
+    want = cg.growth(n, w.pancake(n), max_radius=radius, strategy="bitmap", mem_cap=share)   # as far as its share goes
+    with Device() as dev:
+        with Server(job_mem_cap=share) as s:
+            job = s.submit(n, w.pancake(n), max_radius=radius)
+            dev.fail_at = dev.calls + 5         # behind the server's own five buffers
+            with pytest.raises(CgError) as e:
+                s.step()
+            assert e.value.code == -3 and s.load()[0] == 1
+            dev.fail_at = -1
+            while job not in s.finished():
+                s.step()
+            assert s.result(job).layers == want.layers
+        assert dev.held == 0
